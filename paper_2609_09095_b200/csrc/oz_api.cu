@@ -11,7 +11,7 @@ namespace oz {
 // ------------------------------------------------------------------------------------------
 // per-device objects: plane lookup tables and the sticky status word
 // ------------------------------------------------------------------------------------------
-__device__ uint32_t g_lut[kNumSets][3][kLutWords];
+__device__ uint32_t g_lut[kNumSets][2][kLutWords];
 // status block: [0] sticky condition bits; [1], [2] smallest flatness code of the lines of A / B seen
 // since the last query (exponent-span check); [3] the threshold of the modulus set last used
 __device__ unsigned int g_status[5];
@@ -65,7 +65,6 @@ int floor_mod(int a, int b) { int r = a % b; return r < 0 ? r + b : r; }
 uint32_t lut_entry(int u, int m, int substrate)
 {
     int d = (2 * u >= m) ? u - m : u;        // centred, -m/2 included
-    if (substrate == 2) return static_cast<uint32_t>(d & 0xFF);   // native INT8: the residue is the operand
     int s = square_root(m);
     int dig[3] = {0, 0, 0};
     if (s) {
@@ -208,17 +207,16 @@ oz_status_t ensure_device_ready()
     if (dev < 0 || dev >= kMaxDevices) return OZ_ERR_CUDA;
     std::lock_guard<std::mutex> lock(g_mutex);
     if (g_ready[dev]) return OZ_OK;
-    static uint32_t host_lut[kNumSets][3][kLutWords];
+    static uint32_t host_lut[kNumSets][2][kLutWords];
     for (int set = 0; set < kNumSets; ++set)
-        for (int sub = 0; sub < 3; ++sub) {
-            int off = 0;
+        for (int sub = 0; sub < 2; ++sub)
             for (int i = 0; i < set_r(set); ++i) {
-                int m = modulus(set, i);
-                for (int u = 0; u < kLutSpan * m; ++u) host_lut[set][sub][off + u] = lut_entry(u % m, m, sub);
-                off += kLutSpan * m;
+                const int m = modulus(set, i), span = lut_span(m);
+                // entry u: the canonical residue u of a power of two, the balanced residue u - kLutGuard - m/2 otherwise
+                for (int u = 0; u < span; ++u)
+                    host_lut[set][sub][lut_offset(set, i) + u] =
+                        lut_entry(floor_mod(span == m ? u : u - kLutGuard - m / 2, m), m, sub);
             }
-            for (; off < kLutWords; ++off) host_lut[set][sub][off] = 0;
-        }
     OZ_CUDA_CHECK(cudaMemcpyToSymbol(g_lut, host_lut, sizeof(host_lut)));
     OZ_CUDA_CHECK(cudaMemcpyToSymbol(g_status, kStatusReset, sizeof(kStatusReset)));
     void *p = nullptr;
@@ -260,7 +258,7 @@ const uint32_t *device_lut(int set, int substrate)
 {
     int dev = 0;
     cudaGetDevice(&dev);
-    return g_lut_addr[dev] + (static_cast<size_t>(set) * 3 + substrate) * kLutWords;
+    return g_lut_addr[dev] + (static_cast<size_t>(set) * 2 + (substrate == 0 ? 0 : 1)) * kLutWords;
 }
 
 unsigned int *device_status_word()

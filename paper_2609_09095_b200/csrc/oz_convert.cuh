@@ -41,92 +41,224 @@ __device__ __forceinline__ long long quantise(double x, int sigma, bool tz)
     return (bits >> 63) ? -static_cast<long long>(q) : static_cast<long long>(q);
 }
 
-// One modulus (compile-time index I of set SET) for four consecutive inner-dimension elements:
-// residues, table look-up, byte transposition, 2 or 3 four-byte plane stores.
-template <int SET, int LAYOUT, int I>
-__device__ __forceinline__ void convert_modulus(const uint32_t (&l0)[4], const uint32_t (&l1)[4],
-                                                const uint32_t (&l2)[4], const uint32_t (&l3)[4],
-                                                const uint32_t *__restrict__ lut, uint8_t *out,
-                                                int64_t plane_stride)
+// ---- residues in FP32 ---------------------------------------------------------------------------
+// The quantised integer is cut into four BALANCED limbs at bits 0, 16, 31 and 45 (16, 15, 14 bits and
+// the signed rest), each held exactly in FP32, and
+//     v = l0 + c1 l1 + c2 l2 + c3 l3,   c_q = 2^(bit q) mod m, balanced,
+// is an integer below 2^24 in magnitude: three fused multiply-adds, exact.  rint(v / m) comes from a
+// multiplication by the rounded reciprocal and the 1.5 * 2^23 constant, one more multiply-add leaves the
+// balanced residue r.  The quotient is the nearest integer as long as |v| |m inv - 1| < 1/2 (v / m is never
+// closer than 1 / (2m) to a half-integer for odd m), which residue_exact() checks for every modulus.
+// Every instruction works on a packed pair of elements: six for two residues, where 16-bit integer limbs
+// take seven for one.  What bounds the conversion is instruction issue (and the look-ups' shared-memory
+// wavefronts), so both the packed arithmetic and the digits of the odd squares, which need no table,
+// come straight off its time: 204 -> 125 thread-instructions per element on set S.
+constexpr int kLimbBit1 = 16, kLimbBit2 = 31, kLimbBit3 = 45;
+// Largest |a'|, as 2^q, of an element whose product does not vanish: CS and MAXEXP stay below sqrt(M/2); the
+// accurate rule reaches sqrt(32) 2^(L/2) with L = floor(log2 of its budget) = 110, 112, 116.  (Elements
+// that only meet zeros may be larger under the accurate rule; their residues then are arbitrary but
+// bounded, see kLutGuard.)
+__host__ __device__ constexpr double max_operand(int set)
 {
-    constexpr uint32_t m = modulus(SET, I);
-    constexpr uint32_t c1 = pow2_mod(16, m), c2 = pow2_mod(32, m), c3 = pow2_mod(48, m);
-    // a' = l0 + l1 2^16 + l2 2^32 + l3 2^48 with the top limb SIGNED; `bias` (a multiple of m not
-    // below 2^15 c3) keeps the limb sum non-negative, so no separate sign correction is needed.
-    constexpr uint32_t bias = ((32768u * c3 + m - 1) / m) * m;
-    static_assert(65535ull * (1ull + c1 + c2) + 32767ull * c3 + bias < (1ull << 28), "limb sum below 2^28");
-    // Everything is carried four times too large, so that the remainder is the BYTE offset of the
-    // table entry: v = 4 (limb sum) < 2^30, and floor(v / 4m) = (v * ceil(2^(32+s) / 4m)) >> (32+s)
-    // exactly for s = ceil(log2 m) (the multiplier stays below 2^31).
-    // Per element: four multiply-adds, one multiply-high, a shift, one multiply-subtract, one look-up.
-    constexpr uint32_t m4 = 4u * m;
-    constexpr int s = ceil_log2(m);
-    constexpr uint32_t magic = static_cast<uint32_t>(((1ull << (32 + s)) + m4 - 1) / m4);
-    static_assert(static_cast<unsigned long long>(m4) << 30 <= (1ull << (32 + s)), "exact quotient for v < 2^30");
-    constexpr int off = lut_offset(SET, I);
-    constexpr int plane = first_plane(SET, I, LAYOUT);
-    const unsigned char *table = reinterpret_cast<const unsigned char *>(lut + off);
-    uint32_t w[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        uint32_t v = l3[e] * (4u * c3) + 4u * bias;      // l3 holds the signed limb in two's complement
-        v = l2[e] * (4u * c2) + v;
-        v = l1[e] * (4u * c1) + v;
-        v = l0[e] * 4u + v;
-        const uint32_t r4 = v - (__umulhi(v, magic) >> s) * m4;        // 4 (a' mod m), canonical
-        w[e] = *reinterpret_cast<const uint32_t *>(table + r4);
-    }
-    uint32_t t01 = __byte_perm(w[0], w[1], 0x5140);
-    uint32_t t23 = __byte_perm(w[2], w[3], 0x5140);
-    const uint32_t first = __byte_perm(t01, t23, 0x5410), second = __byte_perm(t01, t23, 0x7632);
-    if (LAYOUT == kLayoutNative) {            // one plane: the centred residue itself
-        *reinterpret_cast<uint32_t *>(out + plane * plane_stride) = first;
-        return;
-    }
-    if (planes_of(m) == 3) {
-        // bytes 2 and 3 of the table words: d0+d1 and the byte the merged layouts swap in
-        // (FP8: the pre-scaled -16*d1 for d1; INT8: -d0 for d0, with 4*d1 made by a byte-wise shift)
-        uint32_t u01 = __byte_perm(w[0], w[1], 0x7362);
-        uint32_t u23 = __byte_perm(w[2], w[3], 0x7362);
-        const uint32_t extra = __byte_perm(u01, u23, 0x7632);
-        constexpr bool kI8 = LAYOUT == kLayoutMergedI8A || LAYOUT == kLayoutMergedI8B;
-        *reinterpret_cast<uint32_t *>(out + plane * plane_stride) = LAYOUT == kLayoutMergedI8A ? extra : first;
-        *reinterpret_cast<uint32_t *>(out + (plane + 1) * plane_stride) =
-            LAYOUT == kLayoutMerged ? extra : (kI8 ? ((second << 2) & 0xFCFCFCFCu) : second);
-        *reinterpret_cast<uint32_t *>(out + (plane + 2) * plane_stride) = __byte_perm(u01, u23, 0x5410);
-    } else {
-        *reinterpret_cast<uint32_t *>(out + plane * plane_stride) = first;
-        *reinterpret_cast<uint32_t *>(out + (plane + 1) * plane_stride) = second;
-    }
+    constexpr double sqrt_half = 0.7071067811865476;
+    return sqrt_half * (set == 0 ? 0x1p58 : (set == 1 ? 0x1p59 : 0x1p61));
+}
+__host__ __device__ constexpr float inv_of(uint32_t m) { return 1.0f / static_cast<float>(m); }
+__host__ __device__ constexpr int balanced_pow2(int e, uint32_t m)
+{
+    const int v = static_cast<int>(pow2_mod(e, m));
+    return 2 * v > static_cast<int>(m) ? v - static_cast<int>(m) : v;
+}
+__host__ __device__ constexpr double abs_d(double x) { return x < 0 ? -x : x; }
+__host__ __device__ constexpr bool residue_exact(int set, uint32_t m)
+{
+    const double v = 32768.0 + 16384.0 * abs_d(balanced_pow2(kLimbBit1, m)) + 8192.0 * abs_d(balanced_pow2(kLimbBit2, m)) +
+                     (max_operand(set) * 0x1p-45 + 1.0) * abs_d(balanced_pow2(kLimbBit3, m));
+    const double delta = abs_d(static_cast<double>(inv_of(m)) * m - 1.0);
+    return v < 16777216.0 && v * delta < 0.5;
 }
 
-template <int SET, int LAYOUT, int... I>
-__device__ __forceinline__ void convert_all_moduli(std::integer_sequence<int, I...>,
-                                                   const uint32_t (&l0)[4], const uint32_t (&l1)[4],
-                                                   const uint32_t (&l2)[4], const uint32_t (&l3)[4],
-                                                   const uint32_t *__restrict__ lut, uint8_t *out,
-                                                   int64_t plane_stride)
-{
-    (convert_modulus<SET, LAYOUT, I>(l0, l1, l2, l3, lut, out, plane_stride), ...);
-}
+constexpr float kRintF = 12582912.0f;        // 1.5 * 2^23: the low mantissa bits of x + kRintF hold rint(x)
 
-// The four 16-bit limbs (top one signed) of the quantised values of four elements.
-__device__ __forceinline__ void split_limbs4(const double (&x)[4], int sigma, bool tz, uint32_t (&l0)[4],
-                                             uint32_t (&l1)[4], uint32_t (&l2)[4], uint32_t (&l3)[4])
+// NP pairs of consecutive elements: pair q holds elements 2q and 2q + 1
+template <int NP>
+struct Limbs {
+    float2 l0[NP], l1[NP], l2[NP], l3[NP];
+    uint32_t low[2 * NP];                    // bits 0..14 are those of a' (the power-of-two moduli)
+};
+
+// limbs of the quantised values of 2 NP elements
+template <int NP>
+__device__ __forceinline__ void split_limbs(const double (&x)[2 * NP], int sigma, bool tz, Limbs<NP> &L)
 {
     // 2^sigma as a double when it is a normal number (always, except for lines of subnormals)
     const bool fast = sigma >= -1000 && sigma <= 1000;
     const double scale = __hiloint2double((1023 + (fast ? sigma : 0)) << 20, 0);
+    constexpr unsigned long long kBias = (1ull << 15) + (1ull << 30) + (1ull << 44) + (1ull << 63);
+    constexpr float k23 = 8388608.0f;
+    const float2 o0 = make_float2(-(k23 + 32768.0f), -(k23 + 32768.0f)), o1 = make_float2(-(k23 + 16384.0f), -(k23 + 16384.0f));
+    const float2 o2 = make_float2(-(k23 + 8192.0f), -(k23 + 8192.0f)), o3 = make_float2(-(k23 + 262144.0f), -(k23 + 262144.0f));
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        long long a = fast ? quantise_fp(x[e], scale, tz) : quantise(x[e], sigma, tz);
-        unsigned long long p = static_cast<unsigned long long>(a);
-        uint32_t lo = static_cast<uint32_t>(p), hi = static_cast<uint32_t>(p >> 32);
-        l0[e] = lo & 0xFFFFu;
-        l1[e] = lo >> 16;
-        l2[e] = hi & 0xFFFFu;
-        l3[e] = static_cast<uint32_t>(static_cast<int32_t>(hi) >> 16);   // signed top limb
+    for (int q = 0; q < NP; ++q) {
+        float f0[2], f1[2], f2[2], f3[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const long long a = fast ? quantise_fp(x[2 * q + e], scale, tz) : quantise(x[2 * q + e], sigma, tz);
+            const unsigned long long p = static_cast<unsigned long long>(a) + kBias;
+            const uint32_t lo = static_cast<uint32_t>(p), hi = static_cast<uint32_t>(p >> 32);
+            // a field OR 2^23's exponent is the float 2^23 + field
+            const uint32_t u0 = __byte_perm(lo, 0x4B000000u, 0x7610);
+            L.low[2 * q + e] = u0;
+            f0[e] = __uint_as_float(u0);
+            f1[e] = __uint_as_float(((lo >> 16) & 0x7FFFu) | 0x4B000000u);
+            f2[e] = __uint_as_float((__funnelshift_r(lo, hi, 31) & 0x3FFFu) | 0x4B000000u);
+            f3[e] = __uint_as_float((hi >> 13) | 0x4B000000u);
+        }
+        L.l0[q] = __fadd2_rn(make_float2(f0[0], f0[1]), o0);
+        L.l1[q] = __fadd2_rn(make_float2(f1[0], f1[1]), o1);
+        L.l2[q] = __fadd2_rn(make_float2(f2[0], f2[1]), o2);
+        L.l3[q] = __fadd2_rn(make_float2(f3[0], f3[1]), o3);
     }
+}
+
+__device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
+
+// balanced residues of a pair
+template <int SET, int I, int NP>
+__device__ __forceinline__ float2 residue_pair(const Limbs<NP> &L, int q)
+{
+    constexpr uint32_t m = modulus(SET, I);
+    static_assert(residue_exact(SET, m), "exact limb sum and quotient");
+    constexpr float c1 = balanced_pow2(kLimbBit1, m), c2 = balanced_pow2(kLimbBit2, m), c3 = balanced_pow2(kLimbBit3, m);
+    float2 v = __ffma2_rn(L.l1[q], dup(c1), L.l0[q]);
+    v = __ffma2_rn(L.l2[q], dup(c2), v);
+    v = __ffma2_rn(L.l3[q], dup(c3), v);
+    const float2 quot = __fadd2_rn(__ffma2_rn(v, dup(inv_of(m)), dup(kRintF)), dup(-kRintF));
+    return __ffma2_rn(quot, dup(-static_cast<float>(m)), v);
+}
+
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
+{
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));      // the table is written once, before a block barrier
+    return v;
+}
+
+// two E4M3 bytes (x in the low one); every digit is representable, so nothing is rounded
+__device__ __forceinline__ uint32_t e4m3_pair(float2 d)
+{
+    uint16_t h;
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(h) : "f"(d.y), "f"(d.x));
+    return h;
+}
+
+// four values whose low bytes are wanted -> one word
+__device__ __forceinline__ uint32_t pack_low_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+
+template <int N>
+__device__ __forceinline__ void store_words(uint8_t *out, const uint32_t (&w)[N])
+{
+    if constexpr (N == 2) *reinterpret_cast<uint2 *>(out) = make_uint2(w[0], w[1]);
+    else *reinterpret_cast<uint32_t *>(out) = w[0];
+}
+
+// One modulus (compile-time index I of set SET) for 2 NP consecutive inner-dimension elements: residues,
+// digits, and 1, 2 or 3 plane stores of 2 NP bytes.  Digits come from the table for the power-of-two and the
+// non-square moduli (Lemma 1's carry makes the latter irregular) and from one more rounded division for the
+// odd squares.  lut: shared-memory address of the set's table.
+template <int SET, int LAYOUT, int I, int NP>
+__device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut, uint8_t *out, int64_t plane_stride)
+{
+    static_assert(NP % 2 == 0, "whole words");
+    constexpr uint32_t m = modulus(SET, I);
+    constexpr int plane = first_plane(SET, I, LAYOUT);
+    constexpr bool pow2 = (m & (m - 1)) == 0;
+    constexpr int s = square_root(m);
+    constexpr int NW = NP / 2;                       // plane words
+    constexpr bool e4m3 = LAYOUT == kLayoutDigits || LAYOUT == kLayoutMerged;      // else INT8 digits
+    if constexpr (LAYOUT == kLayoutNative) {         // one plane: the centred residue itself
+        uint32_t w[NW];
+#pragma unroll
+        for (int g = 0; g < NW; ++g) {
+            if constexpr (pow2) {
+                static_assert(!pow2 || m == 256, "the low byte of a' is its centred residue modulo 256");
+                w[g] = pack_low_bytes(L.low[4 * g], L.low[4 * g + 1], L.low[4 * g + 2], L.low[4 * g + 3]);
+            } else {
+                const float2 r0 = __fadd2_rn(residue_pair<SET, I>(L, 2 * g), dup(kRintF));
+                const float2 r1 = __fadd2_rn(residue_pair<SET, I>(L, 2 * g + 1), dup(kRintF));
+                w[g] = pack_low_bytes(__float_as_uint(r0.x), __float_as_uint(r0.y), __float_as_uint(r1.x), __float_as_uint(r1.y));
+            }
+        }
+        store_words(out + plane * plane_stride, w);
+    } else if constexpr (s != 0 && !pow2) {
+        // odd square: d1 = rint(r / s), d0 = r - s d1, both balanced and free of ties
+        uint32_t w0[NW], w1[NW];
+#pragma unroll
+        for (int g = 0; g < NW; ++g) {
+            float2 d0[2], d1[2], t1[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float2 r = residue_pair<SET, I>(L, 2 * g + h);
+                t1[h] = __ffma2_rn(r, dup(inv_of(s)), dup(kRintF));
+                d1[h] = __fadd2_rn(t1[h], dup(-kRintF));
+                d0[h] = __ffma2_rn(d1[h], dup(-static_cast<float>(s)), r);
+            }
+            if constexpr (e4m3) {
+                w0[g] = e4m3_pair(d0[0]) | (e4m3_pair(d0[1]) << 16);
+                w1[g] = e4m3_pair(d1[0]) | (e4m3_pair(d1[1]) << 16);
+            } else {
+                const float2 u0 = __fadd2_rn(d0[0], dup(kRintF)), u1 = __fadd2_rn(d0[1], dup(kRintF));
+                w0[g] = pack_low_bytes(__float_as_uint(u0.x), __float_as_uint(u0.y), __float_as_uint(u1.x), __float_as_uint(u1.y));
+                w1[g] = pack_low_bytes(__float_as_uint(t1[0].x), __float_as_uint(t1[0].y), __float_as_uint(t1[1].x), __float_as_uint(t1[1].y));
+            }
+        }
+        store_words(out + plane * plane_stride, w0);
+        store_words(out + (plane + 1) * plane_stride, w1);
+    } else {
+        // table word: byte 0 = d0, 1 = d1, 2 = d0+d1, 3 = the byte the merged layouts swap in (FP8: the pre-scaled
+        // -16*d1 for d1; INT8: -d0 for d0, with 4*d1 made by a byte-wise shift)
+        uint32_t w0[NW], w1[NW], w2[NW];
+#pragma unroll
+        for (int g = 0; g < NW; ++g) {
+            uint32_t t[4];
+            if constexpr (pow2) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    t[e] = lds_u32(lut + 4 * lut_offset(SET, I) + ((L.low[4 * g + e] & (m - 1)) << 2));
+            } else {
+                // byte offset 4 (r + bias) as the bits of a denormal: one multiply-add, no conversion
+                constexpr int bias = static_cast<int>(m / 2) + kLutGuard;
+                const float2 base = dup(__uint_as_float(lut + 4 * (lut_offset(SET, I) + bias)));
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 a = __ffma2_rn(residue_pair<SET, I>(L, 2 * g + h), dup(0x1p-147f), base);
+                    t[2 * h] = lds_u32(__float_as_uint(a.x));
+                    t[2 * h + 1] = lds_u32(__float_as_uint(a.y));
+                }
+            }
+            const uint32_t t01 = __byte_perm(t[0], t[1], 0x5140), t23 = __byte_perm(t[2], t[3], 0x5140);
+            const uint32_t first = __byte_perm(t01, t23, 0x5410), second = __byte_perm(t01, t23, 0x7632);
+            const uint32_t u01 = __byte_perm(t[0], t[1], 0x7362), u23 = __byte_perm(t[2], t[3], 0x7362);
+            const uint32_t extra = __byte_perm(u01, u23, 0x7632);
+            constexpr bool kI8 = s == 0 && (LAYOUT == kLayoutMergedI8A || LAYOUT == kLayoutMergedI8B);
+            w0[g] = s == 0 && LAYOUT == kLayoutMergedI8A ? extra : first;
+            w1[g] = s == 0 && LAYOUT == kLayoutMerged ? extra : (kI8 ? ((second << 2) & 0xFCFCFCFCu) : second);
+            w2[g] = __byte_perm(u01, u23, 0x5410);
+        }
+        store_words(out + plane * plane_stride, w0);
+        store_words(out + (plane + 1) * plane_stride, w1);
+        if constexpr (s == 0) store_words(out + (plane + 2) * plane_stride, w2);
+    }
+}
+
+template <int SET, int LAYOUT, int NP, int... I>
+__device__ __forceinline__ void convert_all_moduli(std::integer_sequence<int, I...>, const Limbs<NP> &L, uint32_t lut,
+                                                   uint8_t *out, int64_t plane_stride)
+{
+    (convert_modulus<SET, LAYOUT, I>(L, lut, out, plane_stride), ...);
 }
 
 }  // namespace

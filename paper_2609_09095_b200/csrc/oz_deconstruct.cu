@@ -11,14 +11,9 @@
 // The scan is split over the inner dimension with integer atomics (max / or / add), so its
 // result does not depend on the order of the partial results: the shifts are bit-reproducible.
 //
-// Residue of a 64-bit two's-complement integer a' modulo m (the paper's byte-plane identity of
-// paragraph "O2", applied to 16-bit limbs so that every partial sum stays below 2^32):
-//   a' mod m = (l0 + l1 (2^16 mod m) + l2 (2^32 mod m) + l3 (2^48 mod m) + bias_m) mod m
-// with the top limb l3 taken SIGNED (this replaces the paper's (-2^64) mod m sign correction) and
-// bias_m a multiple of m that keeps the sum non-negative, followed by one exact multiply-high
-// division by m.  The digit split, the Lemma 1 carry and the
-// E4M3 / INT8 encoding are folded into a per-modulus table indexed by the canonical residue
-// (built on the host at set-up), held in shared memory.
+// The residues modulo every m_i and their digits come from FP32 arithmetic on balanced limbs and a small
+// per-modulus table in shared memory (oz_convert.cuh; the paper's byte-plane identity of paragraph "O2" on
+// limbs of 14 to 16 bits).
 #include <utility>
 
 #include "oz_internal.h"
@@ -28,9 +23,9 @@ namespace oz {
 namespace {
 
 constexpr int kConvThreads = 256;
-constexpr int kChunk = 128;            // inner-dimension bytes handled per warp step (4 per lane)
-constexpr int kTileLines = 32;         // side 0: lines per shared-memory transposition tile
-constexpr int kTilePitch = kChunk + 1; // doubles per tile row (+1: conflict-free column writes)
+constexpr int kChunk = 128;            // inner-dimension elements of a conversion tile
+constexpr int kTileLines = 16;         // lines of a conversion tile: two per warp
+constexpr int kTilePitch = kChunk + 2; // doubles per tile row: an odd number of 16-byte chunks
 
 struct ScanScratch {
     unsigned long long *sumsq;  // [lines]  sum of squared magnitudes (accurate rule: maximum of the bound product)
@@ -372,77 +367,147 @@ __global__ void accurate_finalize_kernel(ScanScratch s, int64_t lines, int L, in
     shift[i] = ((L - clog) >> 1) + 4 - E;
 }
 
-// Four consecutive inner-dimension elements of one line -> 4 bytes of every stored plane.
+// Eight consecutive inner-dimension elements of one line -> 8 bytes of every stored plane.
 template <int SET, int LAYOUT>
-__device__ __forceinline__ void convert4(const double (&x)[4], int sigma, bool tz,
-                                         const uint32_t *__restrict__ lut, uint8_t *out,
+__device__ __forceinline__ void convert8(const double (&x)[8], int sigma, bool tz, uint32_t lut, uint8_t *out,
                                          int64_t plane_stride)
 {
-    uint32_t l0[4], l1[4], l2[4], l3[4];
-    split_limbs4(x, sigma, tz, l0, l1, l2, l3);
-    convert_all_moduli<SET, LAYOUT>(std::make_integer_sequence<int, set_r(SET)>{}, l0, l1, l2, l3, lut, out,
-                            plane_stride);
+    Limbs<4> L;
+    split_limbs<4>(x, sigma, tz, L);
+    convert_all_moduli<SET, LAYOUT>(std::make_integer_sequence<int, set_r(SET)>{}, L, lut, out, plane_stride);
 }
 
+// copies the digit table to shared memory (16-byte pieces)
+template <int SET, int LAYOUT>
+__device__ __forceinline__ void load_table(uint32_t *lut, const uint32_t *__restrict__ lut_global, int tid, int nthreads)
+{
+    for (int i = tid; i < lut_words_of(SET, LAYOUT) / 4; i += nthreads)
+        reinterpret_cast<uint4 *>(lut)[i] = reinterpret_cast<const uint4 *>(lut_global)[i];
+}
+
+// 16-byte chunk of a tile row that holds the element pair c: the eight lanes of a quarter warp, which read
+// chunks 4 l + e (l = 0..7), then hit eight different bank groups
+__device__ __forceinline__ int tile_chunk(int c) { return c ^ ((c >> 3) & 3); }
+
+// asynchronous copies of one (8 bytes) or two (16 bytes) elements; nothing is read and zeros are written when !live
+__device__ __forceinline__ void copy8(uint32_t dst, const double *src, bool live)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(live ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void copy16(uint32_t dst, const double *src, int bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+
+// A block takes tiles of 16 lines x 128 inner indices through shared memory (on side 0 that is the
+// transposition: loads run along the lines, plane stores along k) and a thread converts eight consecutive
+// elements of one line, so that half a warp stores 128 contiguous bytes of every plane.  The next tile's
+// elements are copied asynchronously while this one is converted.  Whole deconstruction of a 32768 x 4096
+// operand, integer limbs and a table for every modulus before -> now: native residues 1.77 -> 1.23 ms (side 0), 1.37 -> 1.06
+// (side 1); set S on FP8 1.76 -> 1.62 and 1.50 -> 1.52, where the 30 planes' scattered 128-byte writes (3.3 TB/s) bound it.
 template <int SET, int SIDE, int LAYOUT>
-__global__ void __launch_bounds__(kConvThreads)
+__global__ void __launch_bounds__(kConvThreads, 3)
 convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
                const int32_t *__restrict__ shift, const uint32_t *__restrict__ lut_global,
                uint8_t *__restrict__ planes, int64_t plane_stride, int64_t row_pitch, int tz)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw);
-    for (int i = threadIdx.x; i < lut_words(SET); i += kConvThreads) lut[i] = lut_global[i];
-    __syncthreads();
+    double *tile = reinterpret_cast<double *>(smem_raw + lut_words_of(SET, LAYOUT) * 4);
+    const uint32_t lut_addr = static_cast<uint32_t>(__cvta_generic_to_shared(lut));
+    const uint32_t tile_addr = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
+    constexpr int kTileDoubles = kTileLines * kTilePitch;
+    load_table<SET, LAYOUT>(lut, lut_global, threadIdx.x, kConvThreads);
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // work items are numbered in 32 bits (checked on the host): cheap division
     const uint32_t nchunks = static_cast<uint32_t>((row_pitch + kChunk - 1) / kChunk);
+    const uint32_t ltiles = static_cast<uint32_t>((lines + kTileLines - 1) / kTileLines);
+    const uint32_t items = ltiles * nchunks;
+    const bool pairs = SIDE == 1 && (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
 
-    if (SIDE == 1) {
-        const uint32_t items = static_cast<uint32_t>(lines) * nchunks;
-        for (uint32_t item = blockIdx.x * 8u + warp; item < items; item += gridDim.x * 8u) {
-            const uint32_t uline = item / nchunks;
-            const int64_t line = uline;
-            int64_t kb = static_cast<int64_t>(item - uline * nchunks) * kChunk + lane * 4;
-            if (kb >= row_pitch) continue;
-            int sigma = shift[line];
-            bool dead = sigma == OZ_NONFINITE_SHIFT;
-            double x[4];
+    // side 0: neighbouring blocks take neighbouring lines; side 1: neighbouring inner indices
+    auto place = [&](uint32_t item, int64_t &line0, int64_t &k0) {
+        const uint32_t q = item / (SIDE == 0 ? ltiles : nchunks), rest = item - q * (SIDE == 0 ? ltiles : nchunks);
+        line0 = static_cast<int64_t>(SIDE == 0 ? rest : q) * kTileLines;
+        k0 = static_cast<int64_t>(SIDE == 0 ? q : rest) * kChunk;
+    };
+    auto request = [&](uint32_t item, int buf) {
+        int64_t line0, k0;
+        place(item, line0, k0);
+        const int kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);        // <= 0: padding only
+        const uint32_t base = tile_addr + buf * (kTileDoubles * 8);
+        if (SIDE == 0) {
+            // 16 lanes take the lines of one inner index, a warp two indices at a time
+            const int l = lane & 15;
+            const int64_t line = line0 + l;
+            const bool live = line < lines && shift[line] != OZ_NONFINITE_SHIFT;
+            const int kk0 = 2 * warp + (lane >> 4);
+            const double *src = X + (live ? line : 0) + (k0 + kk0) * ldx;
 #pragma unroll
-            for (int e = 0; e < 4; ++e)
-                x[e] = (!dead && kb + e < k) ? X[kb + e + line * ldx] : 0.0;
-            convert4<SET, LAYOUT>(x, dead ? 0 : sigma, tz != 0, lut, planes + line * row_pitch + kb, plane_stride);
-        }
-    } else {
-        double *tile = reinterpret_cast<double *>(smem_raw + lut_words(SET) * 4);
-        const uint32_t ltiles = static_cast<uint32_t>((lines + kTileLines - 1) / kTileLines);
-        const uint32_t items = ltiles * nchunks;
-        for (uint32_t item = blockIdx.x; item < items; item += gridDim.x) {
-            const uint32_t ukc = item / ltiles;
-            const int64_t kc = ukc;
-            const int64_t lt = item - ukc * ltiles;  // neighbouring blocks read neighbouring rows
-            int64_t line_l = lt * kTileLines + lane;
-            for (int kk = warp; kk < kChunk; kk += kConvThreads / 32) {
-                int64_t kg = kc * kChunk + kk;
-                tile[lane * kTilePitch + kk] =
-                    (line_l < lines && kg < k) ? X[line_l + kg * ldx] : 0.0;
+            for (int u = 0; u < kChunk / 16; ++u) {
+                const int kk = kk0 + 16 * u;
+                const bool in = live && kk < kleft;
+                copy8(base + l * (kTilePitch * 8) + tile_chunk(warp + 8 * u) * 16 + (lane >> 4) * 8, in ? src + (16 * u) * ldx : X, in);
             }
-            __syncthreads();
-            int64_t kb = kc * kChunk + lane * 4;
-#pragma unroll 1
-            for (int li = warp * 4; li < warp * 4 + 4; ++li) {
-                int64_t line = lt * kTileLines + li;
-                if (line >= lines || kb >= row_pitch) continue;
-                int sigma = shift[line];
-                bool dead = sigma == OZ_NONFINITE_SHIFT;
-                double x[4];
+        } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) x[e] = dead ? 0.0 : tile[li * kTilePitch + lane * 4 + e];
-                convert4<SET, LAYOUT>(x, dead ? 0 : sigma, tz != 0, lut, planes + line * row_pitch + kb, plane_stride);
+            for (int h = 0; h < 2; ++h) {
+                const int li = warp * 2 + h;
+                const int64_t line = line0 + li;
+                const bool live = line < lines && shift[line] != OZ_NONFINITE_SHIFT;
+                const double *src = X + (live ? line : 0) * ldx + k0;
+                const uint32_t row = base + li * (kTilePitch * 8);
+                if (pairs) {
+#pragma unroll
+                    for (int u = 0; u < kChunk / 64; ++u) {
+                        const int c = lane + 32 * u;
+                        const int left = live ? (kleft - 2 * c) * 8 : 0;
+                        const int bytes = left >= 16 ? 16 : (left > 0 ? left : 0);
+                        copy16(row + tile_chunk(c) * 16, bytes ? src + 2 * c : X, bytes);
+                    }
+                } else {
+#pragma unroll
+                    for (int u = 0; u < kChunk / 32; ++u) {
+                        const int kk = lane + 32 * u;
+                        const bool in = live && kk < kleft;
+                        copy8(row + tile_chunk(kk >> 1) * 16 + (kk & 1) * 8, in ? src + kk : X, in);
+                    }
+                }
             }
-            __syncthreads();
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    int buf = 0;
+    if (blockIdx.x < items) request(blockIdx.x, 0);
+    for (uint32_t item = blockIdx.x; item < items; item += gridDim.x, buf ^= 1) {
+        const bool more = items - item > gridDim.x;
+        if (more) {
+            request(item + gridDim.x, buf ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();                 // this tile (and, the first time, the table) is there
+        int64_t line0, k0;
+        place(item, line0, k0);
+        const int li = warp * 2 + (lane >> 4);
+        const int64_t line = line0 + li, kb = k0 + (lane & 15) * 8;
+        if (line < lines && kb < row_pitch) {
+            const int sigma_raw = shift[line];
+            const int sigma = sigma_raw == OZ_NONFINITE_SHIFT ? 0 : sigma_raw;     // such a line is zero in the tile
+            const double2 *row = reinterpret_cast<const double2 *>(tile + buf * kTileDoubles + li * kTilePitch);
+            double x[8];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const double2 v = row[tile_chunk((lane & 15) * 4 + e)];
+                x[2 * e] = v.x;
+                x[2 * e + 1] = v.y;
+            }
+            convert8<SET, LAYOUT>(x, sigma, tz != 0, lut_addr, planes + line * row_pitch + kb, plane_stride);
+        }
+        __syncthreads();                 // the tile may be overwritten
     }
 }
 
@@ -458,7 +523,7 @@ struct FusedParams {
     const double *X;
     int64_t ldx, lines, k;
     int group;                 // lines per thread block pass
-    int pitch;                 // doubles per line in shared memory (k + 1: conflict-free for both sides)
+    int pitch;                 // doubles per line in shared memory: odd (conflict-free across lines)
     int side, rule, tbits, tz;
     unsigned long long g2lo, g2hi;
     unsigned int esc_threshold;
@@ -468,6 +533,11 @@ struct FusedParams {
     int32_t *shift;
     unsigned int *status;
 };
+
+// position of inner index kk in a line's buffer: one spare double behind every eight, so that threads that read
+// eight consecutive elements each (stride 9) touch all banks
+__host__ __device__ constexpr int padded(int kk) { return kk + (kk >> 3); }
+__host__ __device__ constexpr int fused_pitch(int k) { return padded(k) | 1; }
 
 struct FusedLine {             // per-line results in shared memory
     unsigned long long sumsq;
@@ -481,10 +551,11 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw);
-    double *buf = reinterpret_cast<double *>(smem_raw + lut_words(SET) * 4);
+    const uint32_t lut_addr = static_cast<uint32_t>(__cvta_generic_to_shared(lut));
+    double *buf = reinterpret_cast<double *>(smem_raw + lut_words_of(SET, LAYOUT) * 4);
     FusedLine *res = reinterpret_cast<FusedLine *>(buf + static_cast<size_t>(p.group) * p.pitch);
     const int nthreads = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
-    for (int i = tid; i < lut_words(SET); i += nthreads) lut[i] = p.lut_global[i];
+    load_table<SET, LAYOUT>(lut, p.lut_global, tid, nthreads);
     const int64_t ngroups = (p.lines + p.group - 1) / p.group;
     const int k = static_cast<int>(p.k);
     for (int64_t g = blockIdx.x; g < ngroups; g += gridDim.x) {
@@ -507,7 +578,7 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int e = e0 + u * nthreads, kk = e >> gshift, l = e & gmask;
-                    if (e < total && l < nl) buf[l * p.pitch + kk] = v[u];
+                    if (e < total && l < nl) buf[l * p.pitch + padded(kk)] = v[u];
                 }
             }
         } else {
@@ -519,7 +590,7 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
                     for (int u = 0; u < 4; ++u) v[u] = l0 + u < nl ? p.X[kk + (line0 + l0 + u) * p.ldx] : 0.0;
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
-                        if (l0 + u < nl) buf[(l0 + u) * p.pitch + kk] = v[u];
+                        if (l0 + u < nl) buf[(l0 + u) * p.pitch + padded(kk)] = v[u];
                 }
         }
         if (tid < nl) {
@@ -538,7 +609,7 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
             int emax = INT32_MIN, bad = 0;
             for (int kk = k0 + lane; kk < k1; kk += 32) {
                 int e;
-                const int c = classify(buf[l * p.pitch + kk], &e);
+                const int c = classify(buf[l * p.pitch + padded(kk)], &e);
                 if (c == 2) bad = 1;
                 if (c == 1 && e > emax) emax = e;
             }
@@ -564,7 +635,7 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
                 unsigned long long acc = 0ull;
                 unsigned int l1 = 0u;
                 for (int kk = k0 + lane; kk < k1; kk += 32) {
-                    const double x = buf[l * p.pitch + kk];
+                    const double x = buf[l * p.pitch + padded(kk)];
                     unsigned long long abar;
                     if (fast_scale) {
                         const double y = fabs(x) * scale9;
@@ -625,16 +696,16 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
             p.shift[line0 + tid] = sh;
         }
         __syncthreads();
-        // ---- conversion: a thread takes four consecutive inner indices of one line
-        const int quads = static_cast<int>(p.row_pitch >> 2);          // row_pitch is a multiple of 16
-        for (int it = tid; it < nl * quads; it += nthreads) {
-            const int l = it / quads, kb = (it - l * quads) * 4;
+        // ---- conversion: a thread takes eight consecutive inner indices of one line
+        const int octs = static_cast<int>(p.row_pitch >> 3);           // row_pitch is a multiple of 16
+        for (int it = tid; it < nl * octs; it += nthreads) {
+            const int l = it / octs, kb = (it - l * octs) * 8;
             const int sigma = res[l].shift;
             const bool dead = sigma == OZ_NONFINITE_SHIFT;
-            double x[4];
+            double x[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) x[e] = (!dead && kb + e < k) ? buf[l * p.pitch + kb + e] : 0.0;
-            convert4<SET, LAYOUT>(x, dead ? 0 : sigma, p.tz != 0, lut, p.planes + (line0 + l) * p.row_pitch + kb,
+            for (int e = 0; e < 8; ++e) x[e] = (!dead && kb + e < k) ? buf[l * p.pitch + padded(kb) + e] : 0.0;
+            convert8<SET, LAYOUT>(x, dead ? 0 : sigma, p.tz != 0, lut_addr, p.planes + (line0 + l) * p.row_pitch + kb,
                                   p.plane_stride);
         }
     }
@@ -647,15 +718,15 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
 #endif
 struct FusedShape { int group, threads, grid; size_t smem; };
 
-FusedShape fused_shape(int set, int side, int64_t lines, int64_t k, int sms)
+FusedShape fused_shape(int set, int layout, int side, int64_t lines, int64_t k, int sms)
 {
     FusedShape f{0, 0, 0, 0};
     if (k < 1 || k > 32768 || lines < 1) return f;
     // The one-kernel form wins where the call is bound by launch latency; larger operands keep the
     // three-pass kernels, whose many small blocks hide the memory latency better.
     if (lines * k > OZ_FUSED_MAX_ELEMS) return f;
-    const size_t line_bytes = static_cast<size_t>(k + 1) * 8;
-    const size_t fixed = lut_words(set) * 4 + 64 * sizeof(FusedLine) + 64;
+    const size_t line_bytes = static_cast<size_t>(fused_pitch(static_cast<int>(k))) * 8;
+    const size_t fixed = lut_words_of(set, layout) * 4 + 64 * sizeof(FusedLine) + 64;
     // two blocks per SM when lines are short enough for that, else one block with more threads
     const size_t budget2 = 110 * 1024, budget1 = 224 * 1024;
     int group = static_cast<int>((budget2 - fixed) / line_bytes);
@@ -711,14 +782,13 @@ oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t 
                            const int32_t *shift, const uint32_t *lut, uint8_t *planes,
                            int64_t plane_stride, int64_t row_pitch, int tz, cudaStream_t stream)
 {
-    size_t smem = lut_words(SET) * 4 + (SIDE == 0 ? sizeof(double) * kTileLines * kTilePitch : 0);
+    const size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * sizeof(double) * kTileLines * kTilePitch;
     OZ_CUDA_CHECK(cudaFuncSetAttribute(convert_kernel<SET, SIDE, LAYOUT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
     int64_t nchunks = (row_pitch + kChunk - 1) / kChunk;
     if (lines * nchunks >= 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;   // item numbers are 32-bit
-    int64_t need = SIDE == 1 ? (lines * nchunks + 7) / 8
-                             : ((lines + kTileLines - 1) / kTileLines) * nchunks;
+    const int64_t need = ((lines + kTileLines - 1) / kTileLines) * nchunks;
     int dev = 0, sms = 148;
     OZ_CUDA_CHECK(cudaGetDevice(&dev));
     OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -836,10 +906,10 @@ oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const doub
     launch_convert<SET_, SIDE_, LAYOUT_>(X, ldx, lines, k, shift, lut, planes, plane_stride, row_pitch, \
                                          rt.quant, stream)
 #define OZ_CONVERT_SET(SET_)                                                                             \
-    (side == 1 ? (layout == kLayoutMergedI8B ? OZ_CONVERT(SET_, 1, kLayoutMergedI8B)                    \
+    (side == 1 ? (layout == kLayoutMergedI8B ? OZ_CONVERT(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_CONVERT(SET_, 1, kLayoutDigitsI8)                    \
                                              : OZ_CONVERT(SET_, 1, kLayoutDigits))                      \
                : (layout == kLayoutMerged      ? OZ_CONVERT(SET_, 0, kLayoutMerged)                     \
-                  : layout == kLayoutMergedI8A ? OZ_CONVERT(SET_, 0, kLayoutMergedI8A)                  \
+                  : layout == kLayoutMergedI8A ? OZ_CONVERT(SET_, 0, kLayoutMergedI8A) : layout == kLayoutDigitsI8 ? OZ_CONVERT(SET_, 0, kLayoutDigitsI8)                  \
                                                : OZ_CONVERT(SET_, 0, kLayoutDigits)))
     const int layout = rt.layout(side);
     if (layout == kLayoutNative) return side == 0 ? OZ_CONVERT(2, 0, kLayoutNative) : OZ_CONVERT(2, 1, kLayoutNative);
@@ -859,12 +929,12 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
     int dev = 0, sms = 148;
     OZ_CUDA_CHECK(cudaGetDevice(&dev));
     OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const FusedShape f = fused_shape(rt.layout(side) == kLayoutNative ? 2 : set, side, lines, k, sms);
+    const FusedShape f = fused_shape(set, rt.layout(side), side, lines, k, sms);
     if (f.group > 0 && !rt.fallback) {      // the row check reads the scan results of the three-pass form
         FusedParams p{};
         p.X = X; p.ldx = ldx; p.lines = lines; p.k = k;
         p.group = f.group;
-        p.pitch = static_cast<int>(k + 1);
+        p.pitch = fused_pitch(static_cast<int>(k));
         p.side = side; p.rule = rt.rule; p.tz = rt.quant;
         int tA = 0, tB = 0;
         budget_maxexp(set, k, &tA, &tB);
@@ -880,10 +950,10 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
         const int layout = rt.layout(side);
 #define OZ_FUSED(SET_, SIDE_, LAYOUT_) launch_fused<SET_, SIDE_, LAYOUT_>(p, f, stream)
 #define OZ_FUSED_SET(SET_)                                                                      \
-    (side == 1 ? (layout == kLayoutMergedI8B ? OZ_FUSED(SET_, 1, kLayoutMergedI8B)             \
+    (side == 1 ? (layout == kLayoutMergedI8B ? OZ_FUSED(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_FUSED(SET_, 1, kLayoutDigitsI8)             \
                                              : OZ_FUSED(SET_, 1, kLayoutDigits))               \
                : (layout == kLayoutMerged      ? OZ_FUSED(SET_, 0, kLayoutMerged)              \
-                  : layout == kLayoutMergedI8A ? OZ_FUSED(SET_, 0, kLayoutMergedI8A)           \
+                  : layout == kLayoutMergedI8A ? OZ_FUSED(SET_, 0, kLayoutMergedI8A) : layout == kLayoutDigitsI8 ? OZ_FUSED(SET_, 0, kLayoutDigitsI8)           \
                                                : OZ_FUSED(SET_, 0, kLayoutDigits)))
         if (layout == kLayoutNative) return side == 0 ? OZ_FUSED(2, 0, kLayoutNative) : OZ_FUSED(2, 1, kLayoutNative);
         if (set == 0) return OZ_FUSED_SET(0);

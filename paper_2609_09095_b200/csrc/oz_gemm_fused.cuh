@@ -1,7 +1,7 @@
 // Fused mode of the residue products for tall-skinny shapes (Sec. "Storage Modes", mode F; "O4:
 // pipelining"): the planes of A are never written to memory.  The kernel reads FP64 A and the shifts
 // of its rows, converts each tile of A into plane bytes inside the shared-memory ring that feeds the
-// tensor core (quantise -> limbs -> residues -> table look-up, the same arithmetic as the
+// tensor core (quantise -> limbs -> residues -> digits, the same arithmetic as the
 // deconstruction kernels), and multiplies it with B's planes, which are materialised as always and
 // stream from L2.  Included by oz_gemm_sm100.cu inside its anonymous namespace.
 //
@@ -79,22 +79,19 @@ __host__ __device__ constexpr uint32_t fused_instr_desc()
 // planes of the moduli 4G .. 4G+3 of the set for one quad of elements, written at their position
 // inside the stage (plane index relative to the first plane of the pass)
 template <int SET, int LAYOUT, int G, int... S>
-__device__ __forceinline__ void convert_pass_moduli(std::integer_sequence<int, S...>, const uint32_t (&l0)[4],
-                                                    const uint32_t (&l1)[4], const uint32_t (&l2)[4],
-                                                    const uint32_t (&l3)[4], const uint32_t *lut, uint8_t *out)
+__device__ __forceinline__ void convert_pass_moduli(std::integer_sequence<int, S...>, const Limbs<2> &L, uint32_t lut,
+                                                    uint8_t *out)
 {
     constexpr int first = first_plane(SET, F_GROUP * G, LAYOUT);
-    (convert_modulus<SET, LAYOUT, F_GROUP * G + S>(l0, l1, l2, l3, lut, out - first * F_A_PLANE, F_A_PLANE), ...);
+    (convert_modulus<SET, LAYOUT, F_GROUP * G + S>(L, lut, out - first * F_A_PLANE, F_A_PLANE), ...);
 }
 
 template <int SET, int LAYOUT, int G>
-__device__ __forceinline__ void convert_pass(const uint32_t (&l0)[4], const uint32_t (&l1)[4],
-                                             const uint32_t (&l2)[4], const uint32_t (&l3)[4],
-                                             const uint32_t *lut, uint8_t *out)
+__device__ __forceinline__ void convert_pass(const Limbs<2> &L, uint32_t lut, uint8_t *out)
 {
     constexpr int left = set_r(SET) - F_GROUP * G;
     constexpr int count = left < F_GROUP ? (left > 0 ? left : 0) : F_GROUP;
-    convert_pass_moduli<SET, LAYOUT, G>(std::make_integer_sequence<int, count>{}, l0, l1, l2, l3, lut, out);
+    convert_pass_moduli<SET, LAYOUT, G>(std::make_integer_sequence<int, count>{}, L, lut, out);
 }
 
 template <int SUB, int SET, int LAYOUT_A>
@@ -341,16 +338,16 @@ fused_gemm_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constan
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         xn[e] = (!dead && ks + 1 < f.nks && kn + e < p.k) ? src[(static_cast<int64_t>(ks + 1) * F_K + e) * f.lda] : 0.0;
-                    uint32_t l0[4], l1[4], l2[4], l3[4];
-                    split_limbs4(x, sigma, tz, l0, l1, l2, l3);
+                    Limbs<2> L;
+                    split_limbs<2>(x, sigma, tz, L);
                     ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status));
                     if (!ok) break;
                     uint8_t *out = ring_gen + stage * F_STAGE + (h * F_LINES + r) * 16 + kq * 4;
                     switch (g) {
-                    case 0: convert_pass<SET, LAYOUT_A, 0>(l0, l1, l2, l3, lut, out); break;
-                    case 1: convert_pass<SET, LAYOUT_A, 1>(l0, l1, l2, l3, lut, out); break;
-                    case 2: convert_pass<SET, LAYOUT_A, 2>(l0, l1, l2, l3, lut, out); break;
-                    default: convert_pass<SET, LAYOUT_A, 3>(l0, l1, l2, l3, lut, out); break;
+                    case 0: convert_pass<SET, LAYOUT_A, 0>(L, lut_addr, out); break;
+                    case 1: convert_pass<SET, LAYOUT_A, 1>(L, lut_addr, out); break;
+                    case 2: convert_pass<SET, LAYOUT_A, 2>(L, lut_addr, out); break;
+                    default: convert_pass<SET, LAYOUT_A, 3>(L, lut_addr, out); break;
                     }
                     // the tensor core reads shared memory through the asynchronous proxy
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");

@@ -11,9 +11,11 @@ namespace oz {
 
 constexpr int kMaxR = 15;          // moduli in the largest supported set (A)
 constexpr int kMaxPlanes = 44;     // stored planes of set A with two-limb digits
-// The plane look-up table of a set holds, per modulus, the packed plane bytes of the residues 0 .. m-1.
-constexpr int kLutSpan = 1;
-constexpr int kLutWords = 8208;    // >= sum of the moduli of any set (S: 8069, E: 6736, A: 3478)
+// The plane look-up table of a set: the packed plane bytes of the residues of the moduli whose digits are not
+// computed (lut_span() words each).  kLutGuard: entries in front of and behind those of the balanced residues, so that an
+// operand element beyond the exact range of the conversion (see max_operand()) still indexes the table.
+constexpr int kLutGuard = 8;
+constexpr int kLutWords = 4160;    // >= lut_words() of any set (S: 4132, E: 2808, A: 3704)
 
 // ---- modulus sets (Sec. 2 step (ii) for S; "Candidate E" and "Candidate A" paragraphs) ---
 constexpr int kNumSets = 3;
@@ -48,8 +50,9 @@ __host__ __device__ constexpr int square_root(int m)
 //   kLayoutMergedI8A / kLayoutMergedI8B  the same schedule on INT8 digit planes, where -16*d1 does
 //                  not fit a byte: both operands carry 4*d1 in place of d1 and the A operand -d0
 //                  in place of d0, so that (-d0) e0 + (4 d1)(4 e1) = -(d0 e0 - 16 d1 e1)
+//   kLayoutDigitsI8  kLayoutDigits with INT8 instead of E4M3 bytes
 constexpr int kLayoutDigits = 0, kLayoutNative = 1, kLayoutMerged = 2, kLayoutMergedI8A = 3,
-              kLayoutMergedI8B = 4;
+              kLayoutMergedI8B = 4, kLayoutDigitsI8 = 5;
 
 __host__ __device__ constexpr int planes_of(int m, int layout = kLayoutDigits)
 {
@@ -72,15 +75,26 @@ __host__ __device__ constexpr int p_store(int set, int layout = kLayoutDigits)
 // reaches 4095 on the 9-bit tail of S and 1088 on byte moduli
 __host__ __device__ constexpr int64_t merged_k_limit(int set) { return set == 0 ? 4097 : 15420; }
 
+// table words of one modulus: canonical residues of a power of two, balanced residues between two guards of a
+// non-square, none for an odd square (its digits are computed)
+__host__ __device__ constexpr int lut_span(int m)
+{
+    return (m & (m - 1)) == 0 ? m : (square_root(m) ? 0 : m + 2 * kLutGuard);
+}
+
 __host__ __device__ constexpr int lut_offset(int set, int i)
 {
     int o = 0;
-    for (int j = 0; j < i; ++j) o += kLutSpan * modulus(set, j);
+    for (int j = 0; j < i; ++j) o += lut_span(modulus(set, j));
     return o;
 }
 
 // words of a set's table, rounded up to whole 16-byte groups
 __host__ __device__ constexpr int lut_words(int set) { return (lut_offset(set, set_r(set)) + 3) / 4 * 4; }
+static_assert(lut_words(0) <= kLutWords && lut_words(1) <= kLutWords && lut_words(2) <= kLutWords, "table size");
+
+// table words that a conversion into `layout` needs: native residues need none
+__host__ __device__ constexpr int lut_words_of(int set, int layout) { return layout == kLayoutNative ? 0 : lut_words(set); }
 
 // 2^e mod m
 __host__ __device__ constexpr uint32_t pow2_mod(int e, uint32_t m)
@@ -88,14 +102,6 @@ __host__ __device__ constexpr uint32_t pow2_mod(int e, uint32_t m)
     uint32_t v = 1 % m;
     for (int j = 0; j < e; ++j) v = (v * 2u) % m;
     return v;
-}
-
-// smallest s with 2^s >= m
-__host__ __device__ constexpr int ceil_log2(uint32_t m)
-{
-    int s = 0;
-    while ((1u << s) < m) ++s;
-    return s;
 }
 
 // floor(2^32 / m)
@@ -116,7 +122,7 @@ struct Route {
     int layout(int side) const
     {
         if (native()) return kLayoutNative;
-        if (!merged()) return kLayoutDigits;
+        if (!merged()) return substrate == 1 ? kLayoutDigitsI8 : kLayoutDigits;
         if (substrate == 1) return side == 0 ? kLayoutMergedI8A : kLayoutMergedI8B;
         return side == 0 ? kLayoutMerged : kLayoutDigits;
     }
@@ -135,7 +141,7 @@ oz_status_t resolve_schedule(int set, int64_t k, int64_t n, bool automatic, Rout
 oz_status_t ensure_device_ready();
 
 // device addresses of the per-device objects (valid after ensure_device_ready())
-const uint32_t *device_lut(int set, int substrate);  // kLutWords packed plane bytes
+const uint32_t *device_lut(int set, int substrate);  // substrate 0, 1: kLutWords packed plane bytes
 unsigned int *device_status_word();
 
 void count_launch(int n = 1);

@@ -1,0 +1,44 @@
+"""The conversion's FP32 limb arithmetic where it can go wrong: quantised values at the edges of every
+limb (bits 0, 16, 31, 45) and at the largest magnitude of the scale rule, planes bit for bit against the
+oracle, from the one-kernel form and from the large-operand kernels, at ragged sizes and odd strides."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import oz_oracle as ozo
+
+pytestmark = pytest.mark.gpu
+
+OSET = {"S": ozo.SET_S, "E": ozo.SET_E, "A": ozo.SET_A}
+OSUB = {"fp8": ozo.SUB_FP8, "int8": ozo.SUB_INT8, "int8n": ozo.SUB_INT8_NATIVE}
+
+
+def _limb_edges(rng, lines, k, side, t):
+    """Every line holds +-(1 - 2^-53), so that MAXEXP with a budget of t bits scales by 2^t; the other entries are
+    sums of up to three +-2^(b - t), b around the limb boundaries, and single bits anywhere in the range."""
+    b = rng.choice([0, 1, 14, 15, 16, 17, 29, 30, 31, 32, 43, 44, 45, 46], size=(lines, k, 3))
+    X = (rng.choice([-1.0, 0.0, 1.0], size=b.shape) * np.exp2(b - float(t))).sum(axis=2)
+    X += rng.choice([0.0, 0.0, 1.0, -1.0], size=(lines, k)) * np.exp2(-rng.integers(1, t, size=(lines, k)).astype(float))
+    X = np.clip(X, -0.75, 0.75)
+    X[np.arange(lines), rng.integers(0, k, size=lines)] = rng.choice([1.0, -1.0], size=lines) * (1.0 - 2.0 ** -53)
+    X = X * np.exp2(rng.integers(-300, 300, size=lines).astype(float))[:, None]
+    return np.asfortranarray(X if side == 0 else X.T)
+
+
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("S", "int8"), ("E", "fp8"), ("E", "int8"), ("A", "fp8"),
+                                          ("A", "int8"), ("A", "int8n")])
+@pytest.mark.parametrize("side,lines,k", [(0, 37, 131), (1, 37, 131), (0, 1, 1), (0, 2101, 2051), (1, 2101, 2051),
+                                          (1, 33, 131100)])
+def test_limb_edges_bit_exact(side, lines, k, set_name, sub):
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(1000 * lines + k + side)
+    t = ozo.budget_maxexp(OSET[set_name], k)[side]
+    X = _limb_edges(rng, lines, k, side, t)
+    for rule, quant in (("MAXEXP", "RN"), ("CS", "TZ")):
+        got, shift, st = gh.deconstruct(side, X, set_name, gh.route(sub, quant, rule))
+        want_shift = ozo.shifts(side, X, OSET[set_name], getattr(ozo, "SCALE_" + rule), t)
+        Q = ozo.quantise(side, X, want_shift, getattr(ozo, "QUANT_" + quant))
+        want = ozo.planes(ozo.residues(Q, OSET[set_name]), OSET[set_name], OSUB[sub])
+        assert st == 0 and (shift == want_shift).all()
+        assert got.shape == want.shape and (got == want).all()
