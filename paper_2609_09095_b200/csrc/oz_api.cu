@@ -470,10 +470,10 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         if (st == OZ_OK) st = launch_accurate_finalize(m, a.scratch, budget, a.shift, stream);
         if (st == OZ_OK) st = launch_accurate_finalize(n, b.scratch, budget, b.shift, stream);
         if (st == OZ_OK)
-            st = launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, a.stride, a.pitch, a.shift, stream);
+            st = launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, stream);
         if (ev && st == OZ_OK) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
         if (st == OZ_OK)
-            st = launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, b.stride, b.pitch, b.shift, stream);
+            st = launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, stream);
         if (st != OZ_OK) return st;
         return product_impl(m, n, k, alpha, a, b, beta, C, ldc, set, rt, stream, ws + L.R, dev, plan);
     }
@@ -483,7 +483,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         if (rt.fallback || rt.hosted || plan || !fused_gemm_applies(m, n, k, set, rt)) return OZ_ERR_UNSUPPORTED;
         OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
         OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
-        st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, b.stride, b.pitch, b.shift, b.scratch, side);
+        st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, side);
         if (st != OZ_OK) return st;
         OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
         st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, stream);
@@ -503,10 +503,10 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     }
     OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
     OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
-    st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, b.stride, b.pitch, b.shift, b.scratch, side);
+    st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, side);
     if (st != OZ_OK) return st;
     OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-    st = launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, a.stride, a.pitch, a.shift, a.scratch, stream);
+    st = launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, stream);
     if (st != OZ_OK) return st;
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
     OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
@@ -748,7 +748,7 @@ oz_status_t oz_prepare_operand(int side, int64_t lines, int64_t k, const double 
     oz_status_t st = ensure_device_ready();
     if (st != OZ_OK) return st;
     const OperandView v = operand_view(static_cast<char *>(operand), o);
-    return launch_deconstruct(side, lines, k, X, ldx, set, rt, v.planes, v.stride, v.pitch, v.shift, v.scratch,
+    return launch_deconstruct(side, lines, k, X, ldx, set, rt, v.planes, private_planes(lines, v.pitch), v.shift, v.scratch,
                               static_cast<cudaStream_t>(stream));
 }
 
@@ -805,7 +805,7 @@ oz_status_t oz_deconstruct(int side, int64_t lines, int64_t k, const double *X, 
     if (k > 0 && ldx < (side == 0 ? lines : k)) return OZ_ERR_INVALID_ARG;
     oz_status_t st = ensure_device_ready();
     if (st != OZ_OK) return st;
-    return launch_deconstruct(side, lines, k, X, ldx, set, rt, planes, plane_stride, row_pitch, shift,
+    return launch_deconstruct(side, lines, k, X, ldx, set, rt, planes, public_planes(plane_stride, row_pitch), shift,
                               scratch, static_cast<cudaStream_t>(stream));
 }
 

@@ -409,8 +409,9 @@ template <int SET, int SIDE, int LAYOUT>
 __global__ void __launch_bounds__(kConvThreads, 3)
 convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
                const int32_t *__restrict__ shift, const uint32_t *__restrict__ lut_global,
-               uint8_t *__restrict__ planes, int64_t plane_stride, int64_t row_pitch, int tz)
+               uint8_t *__restrict__ planes, const __grid_constant__ PlaneGeom geom, int tz)
 {
+    const int64_t row_pitch = geom.row_pitch;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw);
     double *tile = reinterpret_cast<double *>(smem_raw + lut_words_of(SET, LAYOUT) * 4);
@@ -505,7 +506,8 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
                 x[2 * e] = v.x;
                 x[2 * e + 1] = v.y;
             }
-            convert8<SET, LAYOUT>(x, sigma, tz != 0, lut_addr, planes + line * row_pitch + kb, plane_stride);
+            convert8<SET, LAYOUT>(x, sigma, tz != 0, lut_addr,
+                                 planes + (k0 >> 7) * geom.chunk_stride + line * geom.line_stride + (kb & 127), geom.plane_stride);
         }
         __syncthreads();                 // the tile may be overwritten
     }
@@ -529,7 +531,7 @@ struct FusedParams {
     unsigned int esc_threshold;
     const uint32_t *lut_global;
     uint8_t *planes;
-    int64_t plane_stride, row_pitch;
+    PlaneGeom geom;
     int32_t *shift;
     unsigned int *status;
 };
@@ -697,7 +699,7 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
         }
         __syncthreads();
         // ---- conversion: a thread takes eight consecutive inner indices of one line
-        const int octs = static_cast<int>(p.row_pitch >> 3);           // row_pitch is a multiple of 16
+        const int octs = static_cast<int>(p.geom.row_pitch >> 3);           // row_pitch is a multiple of 16
         for (int it = tid; it < nl * octs; it += nthreads) {
             const int l = it / octs, kb = (it - l * octs) * 8;
             const int sigma = res[l].shift;
@@ -705,8 +707,9 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
             double x[8];
 #pragma unroll
             for (int e = 0; e < 8; ++e) x[e] = (!dead && kb + e < k) ? buf[l * p.pitch + padded(kb) + e] : 0.0;
-            convert8<SET, LAYOUT>(x, dead ? 0 : sigma, p.tz != 0, lut_addr, p.planes + (line0 + l) * p.row_pitch + kb,
-                                  p.plane_stride);
+            convert8<SET, LAYOUT>(x, dead ? 0 : sigma, p.tz != 0, lut_addr,
+                                  p.planes + (kb >> 7) * p.geom.chunk_stride + (line0 + l) * p.geom.line_stride + (kb & 127),
+                                  p.geom.plane_stride);
         }
     }
 }
@@ -780,13 +783,13 @@ oz_status_t launch_fused(const FusedParams &p, const FusedShape &f, cudaStream_t
 template <int SET, int SIDE, int LAYOUT>
 oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t k,
                            const int32_t *shift, const uint32_t *lut, uint8_t *planes,
-                           int64_t plane_stride, int64_t row_pitch, int tz, cudaStream_t stream)
+                           const PlaneGeom &geom, int tz, cudaStream_t stream)
 {
     const size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * sizeof(double) * kTileLines * kTilePitch;
     OZ_CUDA_CHECK(cudaFuncSetAttribute(convert_kernel<SET, SIDE, LAYOUT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem)));
-    int64_t nchunks = (row_pitch + kChunk - 1) / kChunk;
+    const int64_t nchunks = (geom.row_pitch + kChunk - 1) / kChunk;
     if (lines * nchunks >= 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;   // item numbers are 32-bit
     const int64_t need = ((lines + kTileLines - 1) / kTileLines) * nchunks;
     int dev = 0, sms = 148;
@@ -799,7 +802,7 @@ oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t 
     int64_t cap = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
     int grid = static_cast<int>(need < cap ? need : cap);
     convert_kernel<SET, SIDE, LAYOUT><<<grid, kConvThreads, smem, stream>>>(
-        X, ldx, lines, k, shift, lut, planes, plane_stride, row_pitch, tz);
+        X, ldx, lines, k, shift, lut, planes, geom, tz);
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
@@ -898,13 +901,12 @@ oz_status_t upload_bound_codes(const unsigned char *codes33)
 
 // quantise, reduce, look up, store: the planes of one operand from its shifts
 oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
-                                  int set, const Route &rt, uint8_t *planes, int64_t plane_stride,
-                                  int64_t row_pitch, const int32_t *shift, cudaStream_t stream)
+                                  int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
+                                  const int32_t *shift, cudaStream_t stream)
 {
     const uint32_t *lut = device_lut(set, rt.substrate);
 #define OZ_CONVERT(SET_, SIDE_, LAYOUT_)                                                                 \
-    launch_convert<SET_, SIDE_, LAYOUT_>(X, ldx, lines, k, shift, lut, planes, plane_stride, row_pitch, \
-                                         rt.quant, stream)
+    launch_convert<SET_, SIDE_, LAYOUT_>(X, ldx, lines, k, shift, lut, planes, geom, rt.quant, stream)
 #define OZ_CONVERT_SET(SET_)                                                                             \
     (side == 1 ? (layout == kLayoutMergedI8B ? OZ_CONVERT(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_CONVERT(SET_, 1, kLayoutDigitsI8)                    \
                                              : OZ_CONVERT(SET_, 1, kLayoutDigits))                      \
@@ -921,9 +923,8 @@ oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const doub
 }
 
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
-                               int set, const Route &rt, uint8_t *planes, int64_t plane_stride,
-                               int64_t row_pitch, int32_t *shift, void *scratch,
-                               cudaStream_t stream)
+                               int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
+                               int32_t *shift, void *scratch, cudaStream_t stream)
 {
     if (rt.rule == 2) return OZ_ERR_UNSUPPORTED;      // the accurate rule needs both operands
     int dev = 0, sms = 148;
@@ -944,7 +945,7 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
         p.g2lo = g2lo; p.g2hi = g2hi;
         p.esc_threshold = esc_threshold(set);
         p.lut_global = device_lut(set, rt.substrate);
-        p.planes = planes; p.plane_stride = plane_stride; p.row_pitch = row_pitch;
+        p.planes = planes; p.geom = geom;
         p.shift = shift;
         p.status = device_status_word();
         const int layout = rt.layout(side);
@@ -964,7 +965,7 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
     }
     oz_status_t st = launch_scan(side, lines, k, X, ldx, set, rt, shift, scratch, stream);
     if (st != OZ_OK) return st;
-    return launch_convert_planes(side, lines, k, X, ldx, set, rt, planes, plane_stride, row_pitch, shift, stream);
+    return launch_convert_planes(side, lines, k, X, ldx, set, rt, planes, geom, shift, stream);
 }
 
 // flags, ordered list and number of the rows that go to the native FP64 path, from the scan results

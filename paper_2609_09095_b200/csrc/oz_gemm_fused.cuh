@@ -43,6 +43,7 @@ struct FusedGemmParams {
     const double *A;                // FP64 operand, column-major m x k
     int64_t lda;
     const int32_t *shiftA;
+    int chunksB;                    // K chunks of 128 bytes per plane of B
     const uint32_t *lut_global;     // plane table of (set, substrate)
     int tz;
     int tiles;                      // tiles of 64 rows
@@ -160,8 +161,9 @@ fused_gemm_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constan
                         const uint32_t sb = ring + stage * F_STAGE + F_A_BYTES;
                         mbar_expect_tx(fb, static_cast<uint32_t>(np) * F_B_PLANE);
                         for (int lp = 0; lp < np; ++lp) {
-                            tma_load_3d(sb + lp * F_B_PLANE, &mapB, fb, ks * F_K, 0, firstB + lp);
-                            tma_load_3d(sb + lp * F_B_PLANE + F_B_PLANE / 2, &mapB, fb, ks * F_K + 16, 0, firstB + lp);
+                            const int x = (ks * F_K) % BLOCK_K, z = (firstB + lp) * f.chunksB + ks * F_K / BLOCK_K;
+                            tma_load_3d(sb + lp * F_B_PLANE, &mapB, fb, x, 0, z);
+                            tma_load_3d(sb + lp * F_B_PLANE + F_B_PLANE / 2, &mapB, fb, x + 16, 0, z);
                         }
                         if (++stage == F_STAGES) { stage = 0; phase ^= 1u; }
                     }

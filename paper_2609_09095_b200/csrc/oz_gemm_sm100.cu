@@ -122,6 +122,7 @@ struct GemmParams {
     int64_t m, n, k;
     int tiles_m, tiles_n, nk;       // tiles of 256 rows / 128 columns of C; nk = K chunks of BLOCK_K
     int vec_store;                  // R rows 16-byte aligned: use vector stores
+    int kc_x, plane_z, kc_z;        // TMA coordinates of chunk kc of a plane: x = kc * kc_x, z = plane * plane_z + kc * kc_z
     int stall_producer;             // test hook: the producer issues no copy, so every wait runs out
     int r;
     int64_t total_items;
@@ -540,16 +541,16 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                             uint32_t sa = tiles + stage * STAGE_BYTES;
                             if (CG == 1) {
                                 mbar_expect_tx(fb, STAGE_BYTES);
-                                tma_load_3d(sa, &mapB, fb, kc * BLOCK_K, it.tn * BLOCK_M, pb);
-                                tma_load_3d(sa + A_BYTES, &mapA, fb, kc * BLOCK_K, it.tm * BLOCK_N, pa);
+                                tma_load_3d(sa, &mapB, fb, kc * p.kc_x, it.tn * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
+                                tma_load_3d(sa + A_BYTES, &mapA, fb, kc * p.kc_x, it.tm * BLOCK_N, pa * p.plane_z + kc * p.kc_z);
                             } else {
                                 // both CTAs' copies complete on the leader's barrier
                                 if (rank == 0) mbar_expect_tx(fb, 2 * STAGE_BYTES);
                                 const uint32_t fb_leader = map_to_cta(fb, 0);
-                                tma_load_3d_pair(sa, &mapB, fb_leader, kc * BLOCK_K,
-                                                 it.tn * Tile<CG>::TILE_J + static_cast<int>(rank) * BLOCK_M, pb);
-                                tma_load_3d_pair(sa + A_BYTES, &mapA, fb_leader, kc * BLOCK_K,
-                                                 it.tm * BLOCK_N + static_cast<int>(rank) * Tile<CG>::B_LINES, pa);
+                                tma_load_3d_pair(sa, &mapB, fb_leader, kc * p.kc_x,
+                                                 it.tn * Tile<CG>::TILE_J + static_cast<int>(rank) * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
+                                tma_load_3d_pair(sa + A_BYTES, &mapA, fb_leader, kc * p.kc_x,
+                                                 it.tm * BLOCK_N + static_cast<int>(rank) * Tile<CG>::B_LINES, pa * p.plane_z + kc * p.kc_z);
                             }
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                         }
@@ -894,8 +895,8 @@ EncodeTiledFn encode_tiled_fn()
     return fn;
 }
 
-// 3-D map over planes[plane][line][kbyte]; box = 128 bytes x box_lines lines x 1 plane,
-// 128-byte swizzle, out-of-range elements read as zero.
+// 3-D map over planes[plane][line][kbyte] (private layout: planes[plane * chunks + chunk][line][128 bytes]);
+// box = 128 bytes x box_lines lines x 1 plane, 128-byte swizzle, out-of-range elements read as zero.
 bool make_plane_map(CUtensorMap *map, const uint8_t *base, int64_t lines, int64_t pitch,
                     int64_t plane_stride, int planes, int box_lines)
 {
@@ -912,16 +913,16 @@ bool make_plane_map(CUtensorMap *map, const uint8_t *base, int64_t lines, int64_
     return rc == CUDA_SUCCESS;
 }
 
-// 3-D map over planes[plane][line][kbyte] for the fused kernel: box = 16 bytes x 128 lines x 1 plane,
-// no swizzle (8 rows x 16 bytes land as one contiguous core matrix), out-of-range elements read as zero.
-bool make_core_matrix_map(CUtensorMap *map, const uint8_t *base, int64_t lines, int64_t pitch,
-                          int64_t plane_stride, int planes)
+// 3-D map over private-layout planes[plane * chunks + chunk][line][128 bytes] for the fused kernel: box = 16 bytes x
+// 128 lines x 1 chunk, no swizzle (8 rows x 16 bytes land as one contiguous core matrix), out-of-range
+// elements read as zero.
+bool make_core_matrix_map(CUtensorMap *map, const uint8_t *base, int64_t lines, int64_t chunks_total)
 {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
-    cuuint64_t dims[3] = {static_cast<cuuint64_t>(pitch), static_cast<cuuint64_t>(lines),
-                          static_cast<cuuint64_t>(planes)};
-    cuuint64_t strides[2] = {static_cast<cuuint64_t>(pitch), static_cast<cuuint64_t>(plane_stride)};
+    cuuint64_t dims[3] = {static_cast<cuuint64_t>(BLOCK_K), static_cast<cuuint64_t>(lines),
+                          static_cast<cuuint64_t>(chunks_total)};
+    cuuint64_t strides[2] = {static_cast<cuuint64_t>(BLOCK_K), static_cast<cuuint64_t>(BLOCK_K * lines)};
     cuuint32_t box[3] = {16, 128, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult rc = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t *>(base), dims, strides,
@@ -1119,9 +1120,19 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     fill_mod_info(p, set, rt, k);
 
     CUtensorMap mapA, mapB;
-    if (!make_plane_map(&mapA, PA, m, pitchA, strideA, p_store(set, rt.layout(0)), BLOCK_N / cg) ||
-        !make_plane_map(&mapB, PB, n, pitchB, strideB, p_store(set, rt.layout(1)), BLOCK_M))
-        return OZ_ERR_CUDA;
+    const int planesA = p_store(set, rt.layout(0)), planesB = p_store(set, rt.layout(1));
+    bool maps;
+    if (tiled) {       // private layout: one 128-byte column of lines per (plane, chunk); both operands have the same pitch
+        const int chunks = static_cast<int>(pitchA / BLOCK_K);
+        p.kc_x = 0; p.plane_z = chunks; p.kc_z = 1;
+        maps = make_plane_map(&mapA, PA, m, BLOCK_K, BLOCK_K * m, planesA * chunks, BLOCK_N / cg) &&
+               make_plane_map(&mapB, PB, n, BLOCK_K, BLOCK_K * n, planesB * chunks, BLOCK_M);
+    } else {
+        p.kc_x = BLOCK_K; p.plane_z = 1; p.kc_z = 0;
+        maps = make_plane_map(&mapA, PA, m, pitchA, strideA, planesA, BLOCK_N / cg) &&
+               make_plane_map(&mapB, PB, n, pitchB, strideB, planesB, BLOCK_M);
+    }
+    if (!maps) return OZ_ERR_CUDA;
 
     int dev = 0, sms = 148;
     OZ_CUDA_CHECK(cudaGetDevice(&dev));
@@ -1182,7 +1193,8 @@ oz_status_t launch_fused_gemm(int64_t m, int64_t n, int64_t k, const double *A, 
     f.passes = (p.r + F_GROUP - 1) / F_GROUP;
     f.nks = static_cast<int>((k + F_K - 1) / F_K);
     CUtensorMap mapB;
-    if (!make_core_matrix_map(&mapB, PB, n, pitchB, strideB, p_store(set, rt.layout(1)))) return OZ_ERR_CUDA;
+    f.chunksB = static_cast<int>(pitchB / BLOCK_K);
+    if (!make_core_matrix_map(&mapB, PB, n, static_cast<int64_t>(p_store(set, rt.layout(1))) * f.chunksB)) return OZ_ERR_CUDA;
     int dev = 0, sms = 148;
     OZ_CUDA_CHECK(cudaGetDevice(&dev));
     OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1213,6 +1225,7 @@ oz_status_t launch_bound_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *GA
     p.total_items = static_cast<int64_t>(p.tiles_m) * p.tiles_n;
     if (p.total_items >= 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;
     p.stall_producer = 0;
+    p.kc_x = BLOCK_K; p.plane_z = 1; p.kc_z = 0;
     p.status = device_status_word();
     p.rowmax = rowmax;
     p.colmax = colmax;

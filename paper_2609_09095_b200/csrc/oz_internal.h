@@ -150,11 +150,22 @@ void count_launch(int n = 1);
 void budget_maxexp(int set, int64_t k, int *tA, int *tB);
 void cs_bound_squared(int set, int64_t k, uint64_t *lo, uint64_t *hi);  // G^2 as 128 bits
 
+// Where a plane keeps byte (line, kk): (kk / 128) chunk_stride + line line_stride + kk % 128.
+//   public:   lines of row_pitch bytes (line_stride = row_pitch, chunk_stride = 128)
+//   private:  K chunk by K chunk, the 128-byte pieces of all lines one behind the other (line_stride = 128,
+//             chunk_stride = 128 lines; row_pitch = k rounded up to 128, so the size is that of the public layout).
+//             A 128-line TMA box is then 16 KiB of consecutive bytes, and so is what a conversion tile stores: with
+//             128-byte pieces a row pitch apart the plane writes stopped at 3.3 TB/s.
+struct PlaneGeom {
+    int64_t plane_stride, row_pitch, line_stride, chunk_stride;
+};
+inline PlaneGeom public_planes(int64_t plane_stride, int64_t row_pitch) { return {plane_stride, row_pitch, row_pitch, 128}; }
+inline PlaneGeom private_planes(int64_t lines, int64_t pitch) { return {lines * pitch, pitch, 128, 128 * lines}; }
+
 // ---- stage launchers (host side of each .cu) ---------------------------------------------
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
-                               int set, const Route &rt, uint8_t *planes, int64_t plane_stride,
-                               int64_t row_pitch, int32_t *shift, void *scratch,
-                               cudaStream_t stream);
+                               int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
+                               int32_t *shift, void *scratch, cudaStream_t stream);
 
 // Tile-ordered private residue array of the whole-method calls.  The output is cut into tiles of
 // 256 rows x tile_cols columns (128, or 256 when CTA pairs are used); a tile is 16 blocks (32 with
@@ -171,14 +182,14 @@ struct ResidueTiling {
 };
 ResidueTiling residue_tiling(int64_t m, int64_t n, int set);
 
-// loose: residues in [0, 2 m_i) (two-byte sets); tiled: R is the tile-ordered private array
-// (ldr and mod_stride are then ignored)
+// loose: residues in [0, 2 m_i) (two-byte sets); tiled: R is the tile-ordered private array (ldr and
+// mod_stride are then ignored) and the planes are in the private layout
 // pieces of launch_deconstruct, and the steps of the accurate rule between them
 oz_status_t launch_scan(int side, int64_t lines, int64_t k, const double *X, int64_t ldx, int set,
                         const Route &rt, int32_t *shift, void *scratch, cudaStream_t stream);
 oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
-                                  int set, const Route &rt, uint8_t *planes, int64_t plane_stride,
-                                  int64_t row_pitch, const int32_t *shift, cudaStream_t stream);
+                                  int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
+                                  const int32_t *shift, cudaStream_t stream);
 oz_status_t launch_bound_plane(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                void *scratch, uint8_t *plane, int64_t pitch, cudaStream_t stream);
 unsigned int *bound_maxima(void *scratch, int64_t lines);      // one word per line, word stride 2
