@@ -11,94 +11,147 @@
 // emulated rows.  C(i,j) = alpha P (beta = 0) or C(i,j) + alpha P (beta = 1) from the caller's old
 // C: the reconstruction leaves the re-issued rows untouched.
 //
-// Work distribution: the re-issued rows come as an ascending list; a thread block takes 64 of
-// them x 64 columns, stages 16 inner indices at a time in shared memory, and each thread carries a
-// 4 x 4 block of (acc, comp) pairs.  The grid is sized for the worst case (every row re-issued),
-// blocks beyond the list's end return at once: the number of rows is known on the device only.
+// Work distribution: the re-issued rows come as an ascending list whose length only the device knows.  Resident
+// blocks (two per SM) walk tiles of S x S outputs, S = 32 (2 x 2 a thread) or 16 (one a thread), chosen from the
+// length by small_tiles().  1024 / S inner indices are staged in shared memory at a time and the next ones
+// are requested before the arithmetic.  Bound: the FP64 pipe, ten instructions per multiply-add, 0.88 of it
+// when every row is re-issued (3000 x 3000 x 1500: 8.56 ms; 8.53 with 64 x 64 tiles in one pass over the grid).  With few
+// rows those tiles left most SMs idle; now 60 of 2003 rows x 1999 x 1501 take 0.20 instead of 0.71 ms, 85 of
+// 3000 rows x 3000 x 3000 0.60 instead of 1.39, 3 of 300 rows x 300 x 3000 0.13 instead of 1.35.
 #include "oz_internal.h"
 
 namespace oz {
 namespace {
 
-constexpr int kFbRows = 64, kFbCols = 64, kFbK = 16, kFbThreads = 256;
+constexpr int kFbThreads = 256, kFbBlocksPerSm = 2;
+constexpr int kFbStage = 1024;                   // elements of each operand per stage
+constexpr int kFbStageDoubles = 64 * (16 + 2);   // one staged operand: the larger of (1024 / S) (S + 2)
+static_assert(32 * (32 + 2) <= kFbStageDoubles, "stage size");
 
-__global__ void __launch_bounds__(kFbThreads)
-native_rows_kernel(int64_t m, int64_t n, int64_t k, const double *__restrict__ A, int64_t lda,
-                   const double *__restrict__ B, int64_t ldb, const int *__restrict__ list,
-                   const unsigned int *__restrict__ count, const int32_t *__restrict__ shiftB,
-                   double alpha, double beta, double *__restrict__ C, int64_t ldc)
+struct NativeParams {
+    int64_t m, n, k, lda, ldb, ldc;
+    const double *A, *B;
+    const int *list;
+    const unsigned int *count;
+    const int32_t *shiftB;
+    double alpha, beta;
+    double *C;
+};
+
+// A round of 32 x 32 tiles over the resident blocks takes 0.20 us per inner index whether one or both blocks of an
+// SM have a tile (the chains of dependent additions bound it), a round of 16 x 16 tiles 0.066 us: the smaller tiles
+// win while their rounds are fewer than three times those of the larger.
+__device__ __forceinline__ bool small_tiles(int64_t rows, int64_t n, int64_t slots)
 {
-    const int64_t rows = *count;
-    const int64_t r0 = static_cast<int64_t>(blockIdx.y) * kFbRows;
-    if (r0 >= rows) return;
-    const int64_t c0 = static_cast<int64_t>(blockIdx.x) * kFbCols;
-    __shared__ __align__(16) double As[kFbK][kFbRows + 2];     // +2: rows stay 16-byte aligned for the pair loads
-    __shared__ __align__(16) double Bs[kFbK][kFbCols + 2];
-    __shared__ int64_t row_of[kFbRows];
+    const int64_t tiles32 = ((rows + 31) / 32) * ((n + 31) / 32), tiles16 = ((rows + 15) / 16) * ((n + 15) / 16);
+    return (tiles16 + slots - 1) / slots < 3 * ((tiles32 + slots - 1) / slots);
+}
+
+template <int S>
+__device__ __forceinline__ void native_tiles(const NativeParams &p, int64_t rows, double *As, double *Bs, int64_t *row_of)
+{
+    constexpr int T = S / 16;                    // outputs of a thread per direction
+    constexpr int K = kFbStage / S;              // inner indices per stage
+    constexpr int kUnroll = T == 1 ? 16 : 8;      // keeps several inner indices' chains in flight
+    constexpr int P = S + 2;                     // doubles per staged index: rows stay 16-byte aligned
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    if (tid < kFbRows) row_of[tid] = r0 + tid < rows ? list[r0 + tid] : -1;
-    __syncthreads();
+    const int64_t tcols = (p.n + S - 1) / S, tiles = tcols * ((rows + S - 1) / S);
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int64_t r0 = t / tcols * S, c0 = (t - t / tcols * tcols) * S;
+        __syncthreads();                         // the previous tile's rows have been used
+        if (tid < S) row_of[tid] = r0 + tid < rows ? p.list[r0 + tid] : -1;
+        __syncthreads();
 
-    double acc[4][4], comp[4][4];
+        double acc[T][T], comp[T][T];
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < T; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = comp[r][c] = 0.0;
+            for (int c = 0; c < T; ++c) acc[r][c] = comp[r][c] = 0.0;
 
-    for (int64_t k0 = 0; k0 < k; k0 += kFbK) {
-        const int kn = k - k0 < kFbK ? static_cast<int>(k - k0) : kFbK;
-        // A: consecutive threads take consecutive re-issued rows of one inner index
-#pragma unroll
-        for (int u = 0; u < kFbRows * kFbK / kFbThreads; ++u) {
-            const int r = tid & (kFbRows - 1), kk = (tid >> 6) + 4 * u;
-            const int64_t row = row_of[r];
-            As[kk][r] = (row >= 0 && kk < kn) ? A[row + (k0 + kk) * lda] : 0.0;
-        }
+        // A: consecutive threads take consecutive re-issued rows of one inner index;
         // B: consecutive threads take consecutive inner indices of one column
+        const int ar = tid & (S - 1), ak = tid / S, bk = tid & (K - 1), bc = tid / K;
+        const int64_t arow = row_of[ar];
+        double av[4], bv[4];
+        auto request = [&](int64_t k0) {
 #pragma unroll
-        for (int u = 0; u < kFbCols * kFbK / kFbThreads; ++u) {
-            const int kk = tid & (kFbK - 1), c = (tid >> 4) + 16 * u;
-            Bs[kk][c] = (c0 + c < n && kk < kn) ? B[(k0 + kk) + (c0 + c) * ldb] : 0.0;
-        }
-        __syncthreads();
-        for (int kk = 0; kk < kn; ++kk) {
-            const double2 a01 = *reinterpret_cast<const double2 *>(&As[kk][ty * 4]);
-            const double2 a23 = *reinterpret_cast<const double2 *>(&As[kk][ty * 4 + 2]);
-            const double2 b01 = *reinterpret_cast<const double2 *>(&Bs[kk][tx * 4]);
-            const double2 b23 = *reinterpret_cast<const double2 *>(&Bs[kk][tx * 4 + 2]);
-            const double a[4] = {a01.x, a01.y, a23.x, a23.y}, b[4] = {b01.x, b01.y, b23.x, b23.y};
+            for (int u = 0; u < 4; ++u) {
+                const int64_t kk = k0 + ak + u * (kFbThreads / S);
+                av[u] = (arow >= 0 && kk < p.k) ? p.A[arow + kk * p.lda] : 0.0;
+                const int64_t c = c0 + bc + u * (kFbThreads / K);
+                bv[u] = (c < p.n && k0 + bk < p.k) ? p.B[(k0 + bk) + c * p.ldb] : 0.0;
+            }
+        };
+        request(0);
+        for (int64_t k0 = 0; k0 < p.k; k0 += K) {
+            const int kn = p.k - k0 < K ? static_cast<int>(p.k - k0) : K;
+            if (k0) __syncthreads();             // the previous stage has been read
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            for (int u = 0; u < 4; ++u) {
+                As[(ak + u * (kFbThreads / S)) * P + ar] = av[u];
+                Bs[bk * P + bc + u * (kFbThreads / K)] = bv[u];
+            }
+            __syncthreads();
+            if (k0 + K < p.k) request(k0 + K);
+#pragma unroll kUnroll
+            for (int kk = 0; kk < kn; ++kk) {
+                double a[T], b[T];
+                if constexpr (T == 1) {
+                    a[0] = As[kk * P + ty];
+                    b[0] = Bs[kk * P + tx];
+                } else {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const double p = __dmul_rn(a[r], b[c]);
-                    const double pe = __fma_rn(a[r], b[c], -p);
-                    const double s = __dadd_rn(acc[r][c], p);
-                    const double bb = __dsub_rn(s, acc[r][c]);
-                    const double se = __dadd_rn(__dsub_rn(acc[r][c], __dsub_rn(s, bb)), __dsub_rn(p, bb));
-                    comp[r][c] = __dadd_rn(comp[r][c], __dadd_rn(pe, se));
-                    acc[r][c] = s;
+                    for (int h = 0; h < T; h += 2) {
+                        const double2 a2 = *reinterpret_cast<const double2 *>(As + kk * P + ty * T + h);
+                        const double2 b2 = *reinterpret_cast<const double2 *>(Bs + kk * P + tx * T + h);
+                        a[h] = a2.x; a[h + 1] = a2.y;
+                        b[h] = b2.x; b[h + 1] = b2.y;
+                    }
                 }
+#pragma unroll
+                for (int r = 0; r < T; ++r)
+#pragma unroll
+                    for (int c = 0; c < T; ++c) {
+                        const double q = __dmul_rn(a[r], b[c]);
+                        const double qe = __fma_rn(a[r], b[c], -q);
+                        const double s = __dadd_rn(acc[r][c], q);
+                        const double bb = __dsub_rn(s, acc[r][c]);
+                        const double se = __dadd_rn(__dsub_rn(acc[r][c], __dsub_rn(s, bb)), __dsub_rn(q, bb));
+                        comp[r][c] = __dadd_rn(comp[r][c], __dadd_rn(qe, se));
+                        acc[r][c] = s;
+                    }
+            }
         }
-        __syncthreads();
-    }
 
-    const double nan = __longlong_as_double(0x7FF8000000000000ll);
+        const double nan = __longlong_as_double(0x7FF8000000000000ll);
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const int64_t j = c0 + tx * 4 + c;
-        if (j >= n) continue;
-        const bool bad = shiftB[j] == OZ_NONFINITE_SHIFT;
+        for (int c = 0; c < T; ++c) {
+            const int64_t j = c0 + tx * T + c;
+            if (j >= p.n) continue;
+            const bool bad = p.shiftB[j] == OZ_NONFINITE_SHIFT;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int64_t row = row_of[ty * 4 + r];
-            if (row < 0) continue;
-            const double v = bad ? nan : __dadd_rn(acc[r][c], comp[r][c]);
-            double *out = C + row + j * ldc;
-            const double t = __dmul_rn(alpha, v);
-            *out = beta != 0.0 ? __dadd_rn(*out, t) : t;
+            for (int r = 0; r < T; ++r) {
+                const int64_t row = row_of[ty * T + r];
+                if (row < 0) continue;
+                const double v = bad ? nan : __dadd_rn(acc[r][c], comp[r][c]);
+                double *out = p.C + row + j * p.ldc;
+                const double x = __dmul_rn(p.alpha, v);
+                *out = p.beta != 0.0 ? __dadd_rn(*out, x) : x;
+            }
         }
     }
+}
+
+__global__ void __launch_bounds__(kFbThreads, kFbBlocksPerSm)
+native_rows_kernel(const __grid_constant__ NativeParams p, int sms)
+{
+    const int64_t rows = *p.count;
+    if (rows == 0) return;
+    __shared__ __align__(16) double As[kFbStageDoubles];
+    __shared__ __align__(16) double Bs[kFbStageDoubles];
+    __shared__ int64_t row_of[32];
+    if (small_tiles(rows, p.n, static_cast<int64_t>(kFbBlocksPerSm) * sms)) native_tiles<16>(p, rows, As, Bs, row_of);
+    else native_tiles<32>(p, rows, As, Bs, row_of);
 }
 
 }  // namespace
@@ -108,11 +161,15 @@ oz_status_t launch_native_rows(int64_t m, int64_t n, int64_t k, const double *A,
                                const int32_t *shiftB, double alpha, double beta, double *C, int64_t ldc,
                                cudaStream_t stream)
 {
-    const int64_t gy = (m + kFbRows - 1) / kFbRows, gx = (n + kFbCols - 1) / kFbCols;
-    if (gy > 65535 || gx > 2147483647ll) return OZ_ERR_UNSUPPORTED;
-    dim3 grid(static_cast<unsigned>(gx), static_cast<unsigned>(gy));
-    native_rows_kernel<<<grid, kFbThreads, 0, stream>>>(m, n, k, A, lda, B, ldb, list, count, shiftB, alpha, beta,
-                                                       C, ldc);
+    // refused as ever: more than 65535 groups of 64 rows, or 2^31 groups of 64 columns
+    if ((m + 63) / 64 > 65535 || (n + 63) / 64 > 2147483647ll) return OZ_ERR_UNSUPPORTED;
+    int dev = 0, sms = 148;
+    OZ_CUDA_CHECK(cudaGetDevice(&dev));
+    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    NativeParams p{m, n, k, lda, ldb, ldc, A, B, list, count, shiftB, alpha, beta, C};
+    // as many blocks as are resident at once, or fewer where even the smallest tiles are fewer
+    const int64_t most = ((m + 15) / 16) * ((n + 15) / 16), cap = static_cast<int64_t>(kFbBlocksPerSm) * sms;
+    native_rows_kernel<<<static_cast<unsigned>(most < cap ? most : cap), kFbThreads, 0, stream>>>(p, sms);
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;

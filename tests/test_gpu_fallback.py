@@ -149,3 +149,24 @@ def test_fallback_unsupported_combinations():
     # the workspace of the route is larger than that of the plain one, and the call checks it
     plain, fb = (oz.oz_workspace_bytes(4096, n, k, oz.OZ_SET_S, gh.route("fp8", fallback=f)) for f in (False, True))
     assert fb > plain
+
+
+@pytest.mark.parametrize("m,n,k,sigma", [
+    (33, 17, 65, 3.0),          # one tile and a remainder of each edge, one index past a stage of the small tiles
+    (16, 16, 64, 3.0),          # exactly one small tile and one stage
+    (900, 1100, 40, 3.0),       # enough tiles for the large ones: 32 x 32, more than one round, ragged edges
+    (640, 992, 33, 3.0),        # large tiles exactly, one index past a stage of theirs
+])
+def test_native_rows_tiles(m, n, k, sigma):
+    """Both tile sizes of the native path with every row re-issued, at and around their edges: the matrix is
+    the oracle's bit for bit (the order over k is fixed, so no tolerance)."""
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m + n + k)
+    A, B = _wide(rng, m, k, sigma), _wide(rng, k, n, sigma)
+    C0 = np.asfortranarray(rng.standard_normal((m, n)))
+    oz.oz_query_fallback_rows()
+    got, st = gh.dgemm(A, B, "S", gh.route("fp8", "RN", "CS", fallback=True), -1.0, 1.0, C0)
+    want, flag = ozo.dgemm_fallback(A, B, ozo.SET_S, ozo.QUANT_RN, -1.0, 1.0, C0)
+    assert st == 0 and oz.oz_query_fallback_rows() == int(flag.sum()) and flag.mean() > 0.9
+    assert (got == want).all()
