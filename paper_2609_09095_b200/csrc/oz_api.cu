@@ -98,20 +98,49 @@ uint32_t lut_entry(int u, int m, int substrate)
     return word;
 }
 
-unsigned __int128 set_product(int set)
+constexpr unsigned __int128 set_product(int set)
 {
     unsigned __int128 M = 1;
     for (int i = 0; i < set_r(set); ++i) M *= static_cast<unsigned>(modulus(set, i));
     return M;
 }
 
-uint64_t isqrt_u128(unsigned __int128 v)
+// floor(sqrt(v)), bit by bit
+constexpr uint64_t isqrt_u128(unsigned __int128 v)
 {
-    uint64_t r = static_cast<uint64_t>(sqrtl(static_cast<long double>(v)));
-    while (static_cast<unsigned __int128>(r) * r > v) --r;
-    while (static_cast<unsigned __int128>(r + 1) * (r + 1) <= v) ++r;
+    uint64_t r = 0;
+    for (int b = 63; b >= 0; --b) {
+        const uint64_t t = r | (1ull << b);
+        if (static_cast<unsigned __int128>(t) * t <= v) r = t;
+    }
     return r;
 }
+
+constexpr int floor_log2_u128(unsigned __int128 v)
+{
+    int L = -1;
+    while (v) { ++L; v >>= 1; }
+    return L;
+}
+
+// per-set constants of the scale rules and checks, fixed at compile time
+struct SetConst {
+    unsigned __int128 half;     // (M - 1) / 2
+    uint64_t root_half;         // floor(sqrt(half))
+    int accurate_log2;
+    unsigned int esc;
+};
+constexpr SetConst set_const(int set)
+{
+    SetConst c{};
+    c.half = (set_product(set) - 1) / 2;
+    c.root_half = isqrt_u128(c.half);
+    c.accurate_log2 = floor_log2_u128((c.half / 129) * 128);
+    const unsigned __int128 t = ((static_cast<unsigned __int128>(1) << 120) / 3) / (c.half >> 20);
+    c.esc = t > 0xFFFFFFFFu ? 0xFFFFFFFFu : static_cast<unsigned int>(t);
+    return c;
+}
+constexpr SetConst kSetConst[kNumSets] = {set_const(0), set_const(1), set_const(2)};
 
 }  // namespace
 
@@ -162,40 +191,28 @@ oz_status_t resolve_schedule(int set, int64_t k, int64_t n, bool automatic, Rout
 
 void budget_maxexp(int set, int64_t k, int *tA, int *tB)
 {
-    unsigned __int128 v = (set_product(set) - 1) / 2 / static_cast<unsigned __int128>(k > 0 ? k : 1);
-    int T = -1;
-    while (v) { ++T; v >>= 1; }
+    const int T = floor_log2_u128(kSetConst[set].half / static_cast<unsigned __int128>(k > 0 ? k : 1));
     *tB = T / 2;
     *tA = T - T / 2;
 }
 
 // floor(log2 H') of the accurate rule: H' = floor(((M-1)/2) / 129) * 128
-int accurate_budget_log2(int set)
-{
-    unsigned __int128 v = ((set_product(set) - 1) / 2 / 129) * 128;
-    int L = -1;
-    while (v) { ++L; v >>= 1; }
-    return L;
-}
+int accurate_budget_log2(int set) { return kSetConst[set].accurate_log2; }
 
 // Exponent-span check: a call is flagged when  qA qB < floor(floor(2^120 / 3) / (((M-1)/2) >> 20)),
 // i.e. phiA^2 phiB^2 < (16/3) 2^104 / ((M-1)/2), with q = floor(2^16 phi^2) the smallest flatness of an
-// operand's lines (see scan_finalize_kernel).
-unsigned int esc_threshold(int set)
-{
-    unsigned __int128 H = (set_product(set) - 1) / 2;
-    unsigned __int128 t = ((static_cast<unsigned __int128>(1) << 120) / 3) / (H >> 20);
-    return t > 0xFFFFFFFFu ? 0xFFFFFFFFu : static_cast<unsigned int>(t);
-}
+// operand's lines (see line_flatness() in oz_deconstruct.cu).
+unsigned int esc_threshold(int set) { return kSetConst[set].esc; }
 
 void cs_bound_squared(int set, int64_t k, uint64_t *lo, uint64_t *hi)
 {
-    uint64_t bnd = isqrt_u128((set_product(set) - 1) / 2);
-    uint64_t kk = static_cast<uint64_t>(k > 0 ? k : 1);
-    uint64_t s = isqrt_u128(kk);
-    uint64_t g = (s * s == kk) ? (s + 1) / 2 : s / 2 + 1;   // ceil(sqrt(k)/2)
-    unsigned __int128 G = bnd - g;
-    unsigned __int128 G2 = G * G;
+    const uint64_t kk = static_cast<uint64_t>(k > 0 ? k : 1);
+    uint64_t s = static_cast<uint64_t>(std::sqrt(static_cast<double>(kk)));       // k <= 2^20: within one of floor(sqrt(k))
+    while (s * s > kk) --s;
+    while ((s + 1) * (s + 1) <= kk) ++s;
+    const uint64_t g = (s * s == kk) ? (s + 1) / 2 : s / 2 + 1;   // ceil(sqrt(k)/2)
+    const unsigned __int128 G = kSetConst[set].root_half - g;
+    const unsigned __int128 G2 = G * G;
     *lo = static_cast<uint64_t>(G2);
     *hi = static_cast<uint64_t>(G2 >> 64);
 }
@@ -268,6 +285,18 @@ unsigned int *device_status_word()
     return g_status_addr[dev];
 }
 
+int sm_count()
+{
+    static std::atomic<int> known[kMaxDevices];
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return sms;
+    const int v = known[dev].load(std::memory_order_relaxed);
+    if (v) return v;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+        known[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
 void count_launch(int n) { g_launches.fetch_add(static_cast<uint64_t>(n)); }
 
 namespace {
@@ -299,7 +328,7 @@ OperandLayout operand_layout(int side, int64_t lines, int64_t k, int set, const 
     o.shift = c.take(4 * static_cast<size_t>(lines));
     o.scratch = c.take(16 * static_cast<size_t>(lines) + 256);
     // storage mode F keeps no planes of A: they exist only inside the product kernel's shared memory
-    o.planes = c.take((whole_method && rt.fused && side == 0) ? 0 : static_cast<size_t>(p_store(set, rt.layout(side))) * o.stride);
+    o.planes = c.take((whole_method && rt.fused && side == 0) ? 0 : static_cast<size_t>(kSetTables.first[set][rt.layout(side)][set_r(set)]) * o.stride);
     o.total = c.off;
     return o;
 }
@@ -444,9 +473,9 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     if (st != OZ_OK) return st;
     const OperandView a = operand_view(ws + L.offA, L.A), b = operand_view(ws + L.offB, L.B);
 
-    // The two operands are deconstructed side by side: B's chain of short kernels runs on an
-    // internal stream that forks from and joins the caller's (their scratch, planes and shifts are
-    // disjoint).  Stage event [1] marks the end of A's chain, [2] the join.
+    // The two operands are deconstructed side by side: in one launch when both fit the one-kernel form, else B's
+    // chain of short kernels runs on an internal stream that forks from and joins the caller's (their scratch,
+    // planes and shifts are disjoint).  Stage event [1] marks the end of A's chain, [2] the join.
     int dev = 0;
     OZ_CUDA_CHECK(cudaGetDevice(&dev));
     st = ensure_side_stream(dev);
@@ -459,8 +488,8 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         // of each operand, which the conversion overwrites afterwards), the bound product on the
         // tensor cores, the shifts from its row and column maxima, then the conversion as usual.
         if (k > kBoundKMax) return OZ_ERR_UNSUPPORTED;
-        st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, stream);
-        if (st == OZ_OK) st = launch_scan(1, n, k, B, ldb, set, rt, b.shift, b.scratch, stream);
+        st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, true, stream);
+        if (st == OZ_OK) st = launch_scan(1, n, k, B, ldb, set, rt, b.shift, b.scratch, true, stream);
         if (st == OZ_OK) st = launch_bound_plane(0, m, k, A, lda, a.scratch, a.planes, a.pitch, stream);
         if (st == OZ_OK) st = launch_bound_plane(1, n, k, B, ldb, b.scratch, b.planes, b.pitch, stream);
         if (st == OZ_OK)
@@ -470,10 +499,10 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         if (st == OZ_OK) st = launch_accurate_finalize(m, a.scratch, budget, a.shift, stream);
         if (st == OZ_OK) st = launch_accurate_finalize(n, b.scratch, budget, b.shift, stream);
         if (st == OZ_OK)
-            st = launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, stream);
+            st = launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, true, stream);
         if (ev && st == OZ_OK) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
         if (st == OZ_OK)
-            st = launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, stream);
+            st = launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, true, stream);
         if (st != OZ_OK) return st;
         return product_impl(m, n, k, alpha, a, b, beta, C, ldc, set, rt, stream, ws + L.R, dev, plan);
     }
@@ -483,10 +512,10 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         if (rt.fallback || rt.hosted || plan || !fused_gemm_applies(m, n, k, set, rt)) return OZ_ERR_UNSUPPORTED;
         OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
         OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
-        st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, side);
+        st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
         if (st != OZ_OK) return st;
         OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-        st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, stream);
+        st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, false, stream);
         if (st != OZ_OK) return st;
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
         OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
@@ -501,12 +530,20 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][4], stream));
         return OZ_OK;
     }
+    bool both = false;
+    st = launch_deconstruct_pair({m, A, lda, a.planes, private_planes(m, a.pitch), a.shift},
+                                 {n, B, ldb, b.planes, private_planes(n, b.pitch), b.shift}, k, set, rt, &both, stream);
+    if (st != OZ_OK) return st;
+    if (both) {
+        if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
+        return product_impl(m, n, k, alpha, a, b, beta, C, ldc, set, rt, stream, ws + L.R, dev, plan);
+    }
     OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
     OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
-    st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, side);
+    st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
     if (st != OZ_OK) return st;
     OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-    st = launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, stream);
+    st = launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, false, stream);
     if (st != OZ_OK) return st;
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
     OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
@@ -748,7 +785,7 @@ oz_status_t oz_prepare_operand(int side, int64_t lines, int64_t k, const double 
     oz_status_t st = ensure_device_ready();
     if (st != OZ_OK) return st;
     const OperandView v = operand_view(static_cast<char *>(operand), o);
-    return launch_deconstruct(side, lines, k, X, ldx, set, rt, v.planes, private_planes(lines, v.pitch), v.shift, v.scratch,
+    return launch_deconstruct(side, lines, k, X, ldx, set, rt, v.planes, private_planes(lines, v.pitch), v.shift, v.scratch, true,
                               static_cast<cudaStream_t>(stream));
 }
 
@@ -806,7 +843,7 @@ oz_status_t oz_deconstruct(int side, int64_t lines, int64_t k, const double *X, 
     oz_status_t st = ensure_device_ready();
     if (st != OZ_OK) return st;
     return launch_deconstruct(side, lines, k, X, ldx, set, rt, planes, public_planes(plane_stride, row_pitch), shift,
-                              scratch, static_cast<cudaStream_t>(stream));
+                              scratch, true, static_cast<cudaStream_t>(stream));
 }
 
 oz_status_t oz_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA, int64_t strideA,

@@ -68,6 +68,8 @@ __device__ __forceinline__ int classify(double x, int *e)
 
 __global__ void scan_init_kernel(ScanScratch s, int64_t lines)
 {
+    dependency_release();
+    dependency_wait();
     int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     if (i < lines) {
         s.sumsq[i] = 0ull;
@@ -84,6 +86,8 @@ __global__ void __launch_bounds__(256)
 scan_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k, int64_t kspan,
             ScanScratch s)
 {
+    dependency_release();
+    dependency_wait();
     int64_t k0 = static_cast<int64_t>(blockIdx.y) * kspan;
     int64_t k1 = k0 + kspan < k ? k0 + kspan : k;
     int lane = threadIdx.x & 31;
@@ -175,12 +179,37 @@ scan_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
     }
 }
 
+// Largest p with 4^p S <= G^2 (S = sum of squares > 0, G^2 as two words): from the bit lengths, and one comparison.
+__device__ __forceinline__ int norm_exponent(unsigned long long S, unsigned long long g2lo, unsigned long long g2hi)
+{
+    const int bits_g = g2hi ? 128 - __clzll(static_cast<long long>(g2hi)) : 64 - __clzll(static_cast<long long>(g2lo));
+    const int p = (bits_g - (64 - __clzll(static_cast<long long>(S)))) >> 1;      // G^2 has at least as many bits as S
+    const unsigned __int128 scaled = static_cast<unsigned __int128>(S) << (2 * p);
+    const unsigned __int128 G2 = (static_cast<unsigned __int128>(g2hi) << 64) | g2lo;
+    return scaled <= G2 ? p : p - 1;
+}
+
+// Flatness of a line, floor(2^16 l1^2 / (k S)), at most 2^16 since l1^2 <= k S (l1 < 2^30, S <= 2^40): the quotient of
+// the rounded FP64 values is off by less than 2^-30 of one, so the exact floor is its integer part or a neighbour.
+__device__ __forceinline__ unsigned int line_flatness(unsigned int l1, unsigned long long S, int64_t k)
+{
+    const unsigned __int128 num = static_cast<unsigned __int128>(static_cast<unsigned long long>(l1) * l1) << 16;
+    const unsigned long long den = static_cast<unsigned long long>(k) * S;
+    const double approx = static_cast<double>(static_cast<unsigned long long>(l1) * l1) * 65536.0 / static_cast<double>(den);
+    unsigned long long q = static_cast<unsigned long long>(approx);
+    if (static_cast<unsigned __int128>(q) * den > num) --q;
+    else if (static_cast<unsigned __int128>(q + 1) * den <= num) ++q;
+    return static_cast<unsigned int>(q);
+}
+
 // shift[line]: MAXEXP  t - 1 - E;  CS  p + 9 - E with p the largest integer such that
 // 4^p * S <= G^2  (G^2 passed as two 64-bit words).
 __global__ void scan_finalize_kernel(ScanScratch s, int64_t lines, int64_t k, int side, int rule, int tbits,
                                      unsigned long long g2lo, unsigned long long g2hi,
                                      unsigned int esc_threshold, int32_t *shift, unsigned int *status)
 {
+    dependency_release();
+    dependency_wait();
     int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     if (i >= lines) return;
     if (s.nonfinite[i] < 0) {
@@ -191,19 +220,10 @@ __global__ void scan_finalize_kernel(ScanScratch s, int64_t lines, int64_t k, in
     int E = s.emax[i];
     if (E == INT32_MIN) { shift[i] = 0; return; }
     if (rule == 0) { shift[i] = tbits - 1 - E; return; }
-    unsigned __int128 G2 = (static_cast<unsigned __int128>(g2hi) << 64) | g2lo;
-    unsigned __int128 q = G2 / static_cast<unsigned __int128>(s.sumsq[i]);   // >= 4^p  <=>  4^p S <= G^2
-    unsigned long long qhi = static_cast<unsigned long long>(q >> 64);
-    unsigned long long qlo = static_cast<unsigned long long>(q);
-    int top = qhi ? 127 - __clzll(static_cast<long long>(qhi)) : 63 - __clzll(static_cast<long long>(qlo));
-    shift[i] = (top >> 1) + 9 - E;
-    // Exponent-span check (Algorithm 1, "ESC check"): flatness of the line,
-    // floor(2^16 (sum abar)^2 / (k sum abar^2)); the smallest value of each operand is kept in the
-    // device status block and judged against the set's threshold when the status is queried.
-    const unsigned long long l1 = static_cast<unsigned int>(s.nonfinite[i]);
-    const unsigned __int128 flat = ((static_cast<unsigned __int128>(l1 * l1)) << 16) /
-                                   (static_cast<unsigned __int128>(static_cast<unsigned long long>(k)) * s.sumsq[i]);
-    atomicMin(status + 1 + side, static_cast<unsigned int>(flat));
+    shift[i] = norm_exponent(s.sumsq[i], g2lo, g2hi) + 9 - E;
+    // Exponent-span check (Algorithm 1, "ESC check"): the smallest flatness of each operand's lines is kept in
+    // the device status block and judged against the set's threshold when the status is queried.
+    atomicMin(status + 1 + side, line_flatness(static_cast<unsigned int>(s.nonfinite[i]), s.sumsq[i], k));
     status[3] = esc_threshold;
 }
 
@@ -215,10 +235,7 @@ __device__ __forceinline__ unsigned int scanned_flatness(const ScanScratch &s, i
 {
     const int nf = s.nonfinite[i];
     if (nf < 0 || s.emax[i] == INT32_MIN) return 0xFFFFFFFFu;
-    const unsigned long long l1 = static_cast<unsigned int>(nf);
-    const unsigned __int128 flat = ((static_cast<unsigned __int128>(l1 * l1)) << 16) /
-                                   (static_cast<unsigned __int128>(static_cast<unsigned long long>(k)) * s.sumsq[i]);
-    const unsigned int q = static_cast<unsigned int>(flat);
+    const unsigned int q = line_flatness(static_cast<unsigned int>(nf), s.sumsq[i], k);
     return q > 65536u ? 65536u : q;
 }
 
@@ -231,6 +248,8 @@ esc_rows_kernel(ScanScratch sA, int64_t m, ScanScratch sB, int64_t n, int64_t k,
 {
     __shared__ unsigned int red[32];
     __shared__ unsigned int base;
+    dependency_release();
+    dependency_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned int qb = 0xFFFFFFFFu;
     for (int64_t j = tid; j < n; j += blockDim.x) qb = min(qb, scanned_flatness(sB, j, k));
@@ -305,6 +324,8 @@ bound_plane_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int
                    uint8_t *__restrict__ out, int64_t pitch)
 {
     __shared__ unsigned char tile[32][36];
+    dependency_release();
+    dependency_wait();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;      // 32 x 8
     const int64_t kchunks = (pitch + 31) / 32;
     const int64_t ltiles = (lines + 31) / 32;
@@ -353,6 +374,10 @@ bound_plane_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int
 __global__ void accurate_finalize_kernel(ScanScratch s, int64_t lines, int L, int32_t *shift,
                                          unsigned int *status)
 {
+    dependency_release();
+    dependency_wait();
+    dependency_release();
+    dependency_wait();
     int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
     if (i >= lines) return;
     if (s.nonfinite[i] < 0) {
@@ -418,7 +443,9 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
     const uint32_t lut_addr = static_cast<uint32_t>(__cvta_generic_to_shared(lut));
     const uint32_t tile_addr = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
     constexpr int kTileDoubles = kTileLines * kTilePitch;
-    load_table<SET, LAYOUT>(lut, lut_global, threadIdx.x, kConvThreads);
+    dependency_release();
+    load_table<SET, LAYOUT>(lut, lut_global, threadIdx.x, kConvThreads);      // written once, before any call
+    dependency_wait();
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // work items are numbered in 32 bits (checked on the host): cheap division
@@ -547,20 +574,50 @@ struct FusedLine {             // per-line results in shared memory
     unsigned int l1;
 };
 
-template <int SET, int SIDE, int LAYOUT>
-__global__ void __launch_bounds__(1024, 1)
-deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
+// ceil(|x| 2^(9-E)) in integer arithmetic (lines of subnormals, where 2^(9-E) is no normal double)
+__device__ __forceinline__ unsigned int scaled_magnitude(double x, int E)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
+    const int be = static_cast<int>((bits >> 52) & 0x7FF);
+    const unsigned long long frac = bits & 0xFFFFFFFFFFFFFull;
+    if (be == 0x7FF || (be == 0 && frac == 0)) return 0u;
+    const unsigned long long sig = be ? (frac | (1ull << 52)) : frac;
+    const int ex = be ? be - 1023 : -1022;
+    const int sh = 43 + E - ex;                           // |x| 2^(9-E) = sig / 2^sh
+    if (sh >= 64) return 1u;
+    if (sh <= 0) return static_cast<unsigned int>(sig << (-sh));
+    return static_cast<unsigned int>((sig >> sh) + ((sig & ((1ull << sh) - 1ull)) ? 1ull : 0ull));
+}
+
+// The shift of a line from its scan results, with its contribution to the device status block
+__device__ __forceinline__ int line_shift(const FusedParams &p, const FusedLine &r)
+{
+    if (r.bad) {
+        atomicOr(p.status, 1u << OZ_ERR_NONFINITE_INPUT);
+        return OZ_NONFINITE_SHIFT;
+    }
+    if (r.emax == INT32_MIN) return 0;
+    if (p.rule == 0) return p.tbits - 1 - r.emax;
+    atomicMin(p.status + 1 + p.side, line_flatness(r.l1, r.sumsq, p.k));
+    p.status[3] = p.esc_threshold;
+    return norm_exponent(r.sumsq, p.g2lo, p.g2hi) + 9 - r.emax;
+}
+
+// line groups block, block + nblocks, .. of one operand
+template <int SET, int SIDE, int LAYOUT>
+__device__ __forceinline__ void deconstruct_lines(const FusedParams &p, int block, int nblocks, unsigned char *smem_raw)
+{
     uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw);
     const uint32_t lut_addr = static_cast<uint32_t>(__cvta_generic_to_shared(lut));
     double *buf = reinterpret_cast<double *>(smem_raw + lut_words_of(SET, LAYOUT) * 4);
     FusedLine *res = reinterpret_cast<FusedLine *>(buf + static_cast<size_t>(p.group) * p.pitch);
     const int nthreads = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = nthreads >> 5;
-    load_table<SET, LAYOUT>(lut, p.lut_global, tid, nthreads);
+    dependency_release();
+    load_table<SET, LAYOUT>(lut, p.lut_global, tid, nthreads);      // written once, before any call
+    dependency_wait();
     const int64_t ngroups = (p.lines + p.group - 1) / p.group;
     const int k = static_cast<int>(p.k);
-    for (int64_t g = blockIdx.x; g < ngroups; g += gridDim.x) {
+    for (int64_t g = block; g < ngroups; g += nblocks) {
         const int64_t line0 = g * p.group;
         const int nl = static_cast<int>(p.lines - line0 < p.group ? p.lines - line0 : p.group);
         __syncthreads();                 // the previous group's conversion has finished with buf / res
@@ -608,21 +665,25 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
         for (int item = warp; item < nl * segs; item += nwarps) {
             const int l = item / segs, seg = item - l * segs;
             const int k0 = seg * span, k1 = min(k, k0 + span);
-            int emax = INT32_MIN, bad = 0;
-            for (int kk = k0 + lane; kk < k1; kk += 32) {
-                int e;
-                const int c = classify(buf[l * p.pitch + padded(kk)], &e);
-                if (c == 2) bad = 1;
-                if (c == 1 && e > emax) emax = e;
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                emax = max(emax, __shfl_xor_sync(0xFFFFFFFFu, emax, o));
-                bad |= __shfl_xor_sync(0xFFFFFFFFu, bad, o);
+            // the high words of |x| order like the exponents
+            unsigned int top = 0u;
+            for (int kk = k0 + lane; kk < k1; kk += 32)
+                top = max(top, static_cast<unsigned int>(__double2hiint(buf[l * p.pitch + padded(kk)])) & 0x7FFFFFFFu);
+            top = __reduce_max_sync(0xFFFFFFFFu, top);
+            int emax = INT32_MIN;
+            if (top >= 0x00100000u) {
+                emax = static_cast<int>(top >> 20) - 1023;
+            } else {
+                // zeros and subnormals only: exponents from the whole words
+                for (int kk = k0 + lane; kk < k1; kk += 32) {
+                    int e;
+                    if (classify(buf[l * p.pitch + padded(kk)], &e) == 1 && e > emax) emax = e;
+                }
+                emax = __reduce_max_sync(0xFFFFFFFFu, emax);
             }
             if (lane == 0) {
-                if (emax != INT32_MIN) atomicMax(&res[l].emax, emax);
-                if (bad) atomicOr(&res[l].bad, 1);
+                if (top >= 0x7FF00000u) atomicOr(&res[l].bad, 1);
+                else if (emax != INT32_MIN) atomicMax(&res[l].emax, emax);
             }
         }
         __syncthreads();
@@ -638,25 +699,15 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
                 unsigned int l1 = 0u;
                 for (int kk = k0 + lane; kk < k1; kk += 32) {
                     const double x = buf[l * p.pitch + padded(kk)];
-                    unsigned long long abar;
+                    unsigned int abar;
                     if (fast_scale) {
-                        const double y = fabs(x) * scale9;
-                        abar = static_cast<unsigned long long>(__double2ll_ru(y));
-                        if (abar == 0ull && x != 0.0) abar = 1ull;
+                        abar = __double2uint_ru(fabs(x) * scale9);
+                        if (abar == 0u && x != 0.0) abar = 1u;
                     } else {
-                        unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
-                        int be = static_cast<int>((bits >> 52) & 0x7FF);
-                        unsigned long long frac = bits & 0xFFFFFFFFFFFFFull;
-                        if (be == 0 && frac == 0) continue;
-                        unsigned long long sig = be ? (frac | (1ull << 52)) : frac;
-                        int ex = be ? be - 1023 : -1022;
-                        int sh = 43 + E - ex;                 // |x| 2^(9-E) = sig / 2^sh
-                        if (sh >= 64) abar = 1;
-                        else if (sh <= 0) abar = sig << (-sh);
-                        else abar = (sig >> sh) + ((sig & ((1ull << sh) - 1)) ? 1ull : 0ull);
+                        abar = scaled_magnitude(x, E);
                     }
-                    acc += abar * abar;
-                    l1 += static_cast<unsigned int>(abar);
+                    acc += static_cast<unsigned long long>(abar) * abar;
+                    l1 += abar;
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
@@ -672,29 +723,8 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
         }
         // ---- the shift of every line (same arithmetic as scan_finalize_kernel)
         if (tid < nl) {
-            FusedLine &r = res[tid];
-            int sh = 0;
-            if (r.bad) {
-                sh = OZ_NONFINITE_SHIFT;
-                atomicOr(p.status, 1u << OZ_ERR_NONFINITE_INPUT);
-            } else if (r.emax != INT32_MIN) {
-                if (p.rule == 0) {
-                    sh = p.tbits - 1 - r.emax;
-                } else {
-                    unsigned __int128 G2 = (static_cast<unsigned __int128>(p.g2hi) << 64) | p.g2lo;
-                    unsigned __int128 q = G2 / static_cast<unsigned __int128>(r.sumsq);
-                    unsigned long long qhi = static_cast<unsigned long long>(q >> 64);
-                    unsigned long long qlo = static_cast<unsigned long long>(q);
-                    int top = qhi ? 127 - __clzll(static_cast<long long>(qhi)) : 63 - __clzll(static_cast<long long>(qlo));
-                    sh = (top >> 1) + 9 - r.emax;
-                    const unsigned long long l1 = r.l1;
-                    const unsigned __int128 flat = ((static_cast<unsigned __int128>(l1 * l1)) << 16) /
-                                                   (static_cast<unsigned __int128>(static_cast<unsigned long long>(p.k)) * r.sumsq);
-                    atomicMin(p.status + 1 + p.side, static_cast<unsigned int>(flat));
-                    p.status[3] = p.esc_threshold;
-                }
-            }
-            r.shift = sh;
+            const int sh = line_shift(p, res[tid]);
+            res[tid].shift = sh;
             p.shift[line0 + tid] = sh;
         }
         __syncthreads();
@@ -712,6 +742,31 @@ deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
                                   p.geom.plane_stride);
         }
     }
+}
+
+template <int SET, int SIDE, int LAYOUT>
+__global__ void __launch_bounds__(1024, 1)
+deconstruct_fused_kernel(const __grid_constant__ FusedParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    deconstruct_lines<SET, SIDE, LAYOUT>(p, blockIdx.x, gridDim.x, smem_raw);
+}
+
+// Both operands of a product: the first `blocksA` blocks take A, the others B.  One launch in place of two on two
+// streams with their fork and join.
+struct PairParams {
+    FusedParams a, b;
+    int blocksA;
+};
+
+template <int SET, int LAYOUTA, int LAYOUTB>
+__global__ void __launch_bounds__(1024, 1)
+deconstruct_pair_kernel(const __grid_constant__ PairParams p)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int block = blockIdx.x;
+    if (block < p.blocksA) deconstruct_lines<SET, 0, LAYOUTA>(p.a, block, p.blocksA, smem_raw);
+    else deconstruct_lines<SET, 1, LAYOUTB>(p.b, block - p.blocksA, gridDim.x - p.blocksA, smem_raw);
 }
 
 // Lines per thread-block pass of the fused kernel and its launch shape; group = 0: not applicable
@@ -770,39 +825,65 @@ FusedShape fused_shape(int set, int layout, int side, int64_t lines, int64_t k, 
 }
 
 template <int SET, int SIDE, int LAYOUT>
-oz_status_t launch_fused(const FusedParams &p, const FusedShape &f, cudaStream_t stream)
+oz_status_t launch_fused(const FusedParams &p, const FusedShape &f, bool alone, cudaStream_t stream)
 {
-    auto kernel = deconstruct_fused_kernel<SET, SIDE, LAYOUT>;
-    OZ_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(f.smem)));
-    kernel<<<f.grid, f.threads, f.smem, stream>>>(p);
+    static std::atomic<unsigned long long> ready{0};
+    OZ_CUDA_CHECK(allow_shared(deconstruct_fused_kernel<SET, SIDE, LAYOUT>, kMaxShared, ready));
+    OZ_CUDA_CHECK(launch_if(alone, deconstruct_fused_kernel<SET, SIDE, LAYOUT>, dim3(f.grid), f.threads, f.smem, stream, p));
     count_launch();
-    OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
+}
+
+template <int SET, int LAYOUTA, int LAYOUTB>
+oz_status_t launch_pair(const PairParams &p, const FusedShape &fa, const FusedShape &fb, cudaStream_t stream)
+{
+    static std::atomic<unsigned long long> ready{0};
+    OZ_CUDA_CHECK(allow_shared(deconstruct_pair_kernel<SET, LAYOUTA, LAYOUTB>, kMaxShared, ready));
+    OZ_CUDA_CHECK(launch(deconstruct_pair_kernel<SET, LAYOUTA, LAYOUTB>, dim3(fa.grid + fb.grid), fa.threads,
+                         fa.smem > fb.smem ? fa.smem : fb.smem, stream, p));
+    count_launch();
+    return OZ_OK;
+}
+
+// parameters of the one-kernel form for one operand
+FusedParams fused_params(int side, int64_t lines, int64_t k, const double *X, int64_t ldx, int set, const Route &rt,
+                         uint8_t *planes, const PlaneGeom &geom, int32_t *shift, int group)
+{
+    FusedParams p{};
+    p.X = X; p.ldx = ldx; p.lines = lines; p.k = k;
+    p.group = group;
+    p.pitch = fused_pitch(static_cast<int>(k));
+    p.side = side; p.rule = rt.rule; p.tz = rt.quant;
+    int tA = 0, tB = 0;
+    budget_maxexp(set, k, &tA, &tB);
+    p.tbits = side == 0 ? tA : tB;
+    uint64_t g2lo = 0, g2hi = 0;
+    cs_bound_squared(set, k, &g2lo, &g2hi);
+    p.g2lo = g2lo; p.g2hi = g2hi;
+    p.esc_threshold = esc_threshold(set);
+    p.lut_global = device_lut(set, rt.substrate);
+    p.planes = planes; p.geom = geom;
+    p.shift = shift;
+    p.status = device_status_word();
+    return p;
 }
 
 template <int SET, int SIDE, int LAYOUT>
 oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t k,
                            const int32_t *shift, const uint32_t *lut, uint8_t *planes,
-                           const PlaneGeom &geom, int tz, cudaStream_t stream)
+                           const PlaneGeom &geom, int tz, bool alone, cudaStream_t stream)
 {
-    const size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * sizeof(double) * kTileLines * kTilePitch;
-    OZ_CUDA_CHECK(cudaFuncSetAttribute(convert_kernel<SET, SIDE, LAYOUT>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem)));
+    constexpr size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * sizeof(double) * kTileLines * kTilePitch;
+    static std::atomic<unsigned long long> ready{0};
+    OZ_CUDA_CHECK(allow_shared(convert_kernel<SET, SIDE, LAYOUT>, smem, ready));
     const int64_t nchunks = (geom.row_pitch + kChunk - 1) / kChunk;
     if (lines * nchunks >= 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;   // item numbers are 32-bit
     const int64_t need = ((lines + kTileLines - 1) / kTileLines) * nchunks;
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     // persistent blocks: as many as are resident at once (each copies the table once)
-    int per_sm = 1;
-    OZ_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, convert_kernel<SET, SIDE, LAYOUT>,
-                                                                kConvThreads, smem));
-    int64_t cap = static_cast<int64_t>(sms) * (per_sm > 0 ? per_sm : 1);
+    const int64_t cap = 3ll * sm_count();
     int grid = static_cast<int>(need < cap ? need : cap);
-    convert_kernel<SET, SIDE, LAYOUT><<<grid, kConvThreads, smem, stream>>>(
-        X, ldx, lines, k, shift, lut, planes, geom, tz);
+    OZ_CUDA_CHECK(launch_if(alone, convert_kernel<SET, SIDE, LAYOUT>, dim3(grid), kConvThreads, smem, stream,
+                         X, ldx, lines, k, shift, lut, planes, geom, tz));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
@@ -813,12 +894,12 @@ oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t 
 // scan_init + the scan passes of the route's scale rule [+ the shifts, except for the accurate rule,
 // whose shifts come later from the bound product]
 oz_status_t launch_scan(int side, int64_t lines, int64_t k, const double *X, int64_t ldx, int set,
-                        const Route &rt, int32_t *shift, void *scratch, cudaStream_t stream)
+                        const Route &rt, int32_t *shift, void *scratch, bool alone, cudaStream_t stream)
 {
     ScanScratch s = carve_scratch(scratch, lines);
     unsigned int *status = device_status_word();
     int blocks1d = static_cast<int>((lines + 255) / 256);
-    scan_init_kernel<<<blocks1d, 256, 0, stream>>>(s, lines);
+    OZ_CUDA_CHECK(launch_if(alone, scan_init_kernel, dim3(blocks1d), 256, 0, stream, s, lines));
     count_launch();
 
     // split the inner dimension so that the scan fills the machine even for few lines
@@ -838,18 +919,16 @@ oz_status_t launch_scan(int side, int64_t lines, int64_t k, const double *X, int
 
     if (k > 0) {
         dim3 grid(static_cast<unsigned>(line_blocks), static_cast<unsigned>(split));
-        if (side == 0) scan_kernel<0, 0><<<grid, 256, 0, stream>>>(X, ldx, lines, k, kspan, s);
-        else scan_kernel<1, 0><<<grid, 256, 0, stream>>>(X, ldx, lines, k, kspan, s);
+        OZ_CUDA_CHECK(launch_if(alone, side == 0 ? scan_kernel<0, 0> : scan_kernel<1, 0>, grid, 256, 0, stream, X, ldx, lines, k, kspan, s));
         count_launch();
         if (rt.rule == 1) {
-            if (side == 0) scan_kernel<0, 1><<<grid, 256, 0, stream>>>(X, ldx, lines, k, kspan, s);
-            else scan_kernel<1, 1><<<grid, 256, 0, stream>>>(X, ldx, lines, k, kspan, s);
+            OZ_CUDA_CHECK(launch_if(alone, side == 0 ? scan_kernel<0, 1> : scan_kernel<1, 1>, grid, 256, 0, stream, X, ldx, lines, k, kspan, s));
             count_launch();
         }
     }
     if (rt.rule != 2) {
-        scan_finalize_kernel<<<blocks1d, 256, 0, stream>>>(s, lines, k, side, rt.rule, side == 0 ? tA : tB, g2lo,
-                                                           g2hi, esc_threshold(set), shift, status);
+        OZ_CUDA_CHECK(launch_if(alone, scan_finalize_kernel, dim3(blocks1d), 256, 0, stream, s, lines, k, side, rt.rule,
+                             side == 0 ? tA : tB, g2lo, g2hi, esc_threshold(set), shift, status));
         count_launch();
     }
     OZ_CUDA_CHECK(cudaGetLastError());
@@ -861,14 +940,12 @@ oz_status_t launch_bound_plane(int side, int64_t lines, int64_t k, const double 
                                void *scratch, uint8_t *plane, int64_t pitch, cudaStream_t stream)
 {
     ScanScratch s = carve_scratch(scratch, lines);
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = sm_count();
     const int64_t need = ((lines + 31) / 32) * ((pitch + 31) / 32);
     const int64_t cap = static_cast<int64_t>(sms) * 8;
     const int grid = static_cast<int>(need < cap ? need : cap);
-    if (side == 0) bound_plane_kernel<0><<<grid, 256, 0, stream>>>(X, ldx, lines, k, s, plane, pitch);
-    else bound_plane_kernel<1><<<grid, 256, 0, stream>>>(X, ldx, lines, k, s, plane, pitch);
+    OZ_CUDA_CHECK(launch(side == 0 ? bound_plane_kernel<0> : bound_plane_kernel<1>, dim3(grid), 256, 0, stream,
+                         X, ldx, lines, k, s, plane, pitch));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
@@ -886,8 +963,8 @@ oz_status_t launch_accurate_finalize(int64_t lines, void *scratch, int budget_lo
                                      cudaStream_t stream)
 {
     ScanScratch s = carve_scratch(scratch, lines);
-    accurate_finalize_kernel<<<static_cast<int>((lines + 255) / 256), 256, 0, stream>>>(s, lines, budget_log2, shift,
-                                                                                         device_status_word());
+    OZ_CUDA_CHECK(launch(accurate_finalize_kernel, dim3(static_cast<unsigned>((lines + 255) / 256)), 256, 0, stream,
+                         s, lines, budget_log2, shift, device_status_word()));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
@@ -902,11 +979,11 @@ oz_status_t upload_bound_codes(const unsigned char *codes33)
 // quantise, reduce, look up, store: the planes of one operand from its shifts
 oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                   int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
-                                  const int32_t *shift, cudaStream_t stream)
+                                  const int32_t *shift, bool alone, cudaStream_t stream)
 {
     const uint32_t *lut = device_lut(set, rt.substrate);
 #define OZ_CONVERT(SET_, SIDE_, LAYOUT_)                                                                 \
-    launch_convert<SET_, SIDE_, LAYOUT_>(X, ldx, lines, k, shift, lut, planes, geom, rt.quant, stream)
+    launch_convert<SET_, SIDE_, LAYOUT_>(X, ldx, lines, k, shift, lut, planes, geom, rt.quant, alone, stream)
 #define OZ_CONVERT_SET(SET_)                                                                             \
     (side == 1 ? (layout == kLayoutMergedI8B ? OZ_CONVERT(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_CONVERT(SET_, 1, kLayoutDigitsI8)                    \
                                              : OZ_CONVERT(SET_, 1, kLayoutDigits))                      \
@@ -924,32 +1001,15 @@ oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const doub
 
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
-                               int32_t *shift, void *scratch, cudaStream_t stream)
+                               int32_t *shift, void *scratch, bool alone, cudaStream_t stream)
 {
     if (rt.rule == 2) return OZ_ERR_UNSUPPORTED;      // the accurate rule needs both operands
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = sm_count();
     const FusedShape f = fused_shape(set, rt.layout(side), side, lines, k, sms);
     if (f.group > 0 && !rt.fallback) {      // the row check reads the scan results of the three-pass form
-        FusedParams p{};
-        p.X = X; p.ldx = ldx; p.lines = lines; p.k = k;
-        p.group = f.group;
-        p.pitch = fused_pitch(static_cast<int>(k));
-        p.side = side; p.rule = rt.rule; p.tz = rt.quant;
-        int tA = 0, tB = 0;
-        budget_maxexp(set, k, &tA, &tB);
-        p.tbits = side == 0 ? tA : tB;
-        uint64_t g2lo = 0, g2hi = 0;
-        cs_bound_squared(set, k, &g2lo, &g2hi);
-        p.g2lo = g2lo; p.g2hi = g2hi;
-        p.esc_threshold = esc_threshold(set);
-        p.lut_global = device_lut(set, rt.substrate);
-        p.planes = planes; p.geom = geom;
-        p.shift = shift;
-        p.status = device_status_word();
+        const FusedParams p = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, f.group);
         const int layout = rt.layout(side);
-#define OZ_FUSED(SET_, SIDE_, LAYOUT_) launch_fused<SET_, SIDE_, LAYOUT_>(p, f, stream)
+#define OZ_FUSED(SET_, SIDE_, LAYOUT_) launch_fused<SET_, SIDE_, LAYOUT_>(p, f, alone, stream)
 #define OZ_FUSED_SET(SET_)                                                                      \
     (side == 1 ? (layout == kLayoutMergedI8B ? OZ_FUSED(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_FUSED(SET_, 1, kLayoutDigitsI8)             \
                                              : OZ_FUSED(SET_, 1, kLayoutDigits))               \
@@ -963,9 +1023,33 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
 #undef OZ_FUSED_SET
 #undef OZ_FUSED
     }
-    oz_status_t st = launch_scan(side, lines, k, X, ldx, set, rt, shift, scratch, stream);
+    oz_status_t st = launch_scan(side, lines, k, X, ldx, set, rt, shift, scratch, alone, stream);
     if (st != OZ_OK) return st;
-    return launch_convert_planes(side, lines, k, X, ldx, set, rt, planes, geom, shift, stream);
+    return launch_convert_planes(side, lines, k, X, ldx, set, rt, planes, geom, shift, alone, stream);
+}
+
+oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, int64_t k, int set, const Route &rt,
+                                    bool *taken, cudaStream_t stream)
+{
+    *taken = false;
+    if (rt.rule == 2 || rt.fallback) return OZ_OK;      // shifts from both operands; the row check's scan results
+    const int sms = sm_count();
+    const FusedShape fa = fused_shape(set, rt.layout(0), 0, a.lines, k, sms), fb = fused_shape(set, rt.layout(1), 1, b.lines, k, sms);
+    if (fa.group <= 0 || fb.group <= 0 || fa.threads != fb.threads) return OZ_OK;
+    PairParams p;
+    p.a = fused_params(0, a.lines, k, a.X, a.ldx, set, rt, a.planes, a.geom, a.shift, fa.group);
+    p.b = fused_params(1, b.lines, k, b.X, b.ldx, set, rt, b.planes, b.geom, b.shift, fb.group);
+    p.blocksA = fa.grid;
+    *taken = true;
+    const int layout = rt.layout(0);
+#define OZ_PAIR(SET_)                                                                                       \
+    (layout == kLayoutMerged      ? launch_pair<SET_, kLayoutMerged, kLayoutDigits>(p, fa, fb, stream)      \
+     : layout == kLayoutMergedI8A ? launch_pair<SET_, kLayoutMergedI8A, kLayoutMergedI8B>(p, fa, fb, stream) \
+     : layout == kLayoutDigitsI8  ? launch_pair<SET_, kLayoutDigitsI8, kLayoutDigitsI8>(p, fa, fb, stream)  \
+                                  : launch_pair<SET_, kLayoutDigits, kLayoutDigits>(p, fa, fb, stream))
+    if (layout == kLayoutNative) return launch_pair<2, kLayoutNative, kLayoutNative>(p, fa, fb, stream);
+    return set == 0 ? OZ_PAIR(0) : set == 1 ? OZ_PAIR(1) : OZ_PAIR(2);
+#undef OZ_PAIR
 }
 
 // flags, ordered list and number of the rows that go to the native FP64 path, from the scan results
@@ -973,8 +1057,8 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
 oz_status_t launch_esc_rows(void *scratchA, int64_t m, void *scratchB, int64_t n, int64_t k, int set,
                             unsigned char *flag, int *list, unsigned int *count, cudaStream_t stream)
 {
-    esc_rows_kernel<<<1, 1024, 0, stream>>>(carve_scratch(scratchA, m), m, carve_scratch(scratchB, n), n, k,
-                                            esc_threshold(set), flag, list, count, device_status_word());
+    OZ_CUDA_CHECK(launch(esc_rows_kernel, dim3(1), 1024, 0, stream, carve_scratch(scratchA, m), m,
+                         carve_scratch(scratchB, n), n, k, esc_threshold(set), flag, list, count, device_status_word()));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;

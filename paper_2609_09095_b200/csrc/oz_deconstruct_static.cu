@@ -73,5 +73,5 @@ extern "C" oz_status_t oz_deconstruct_static(int side, int64_t lines, int64_t k,
     // The scan kernels clear the part of the scratch they use before accumulating into it, so the
     // previous call's contents never leak into this one.
     return oz::launch_deconstruct(side, lines, k, X, ldx, set, rt, planes,
-                                  oz::public_planes(plane_stride, row_pitch), shift, scratch, static_cast<cudaStream_t>(stream));
+                                  oz::public_planes(plane_stride, row_pitch), shift, scratch, true, static_cast<cudaStream_t>(stream));
 }

@@ -145,6 +145,8 @@ __device__ __forceinline__ void native_tiles(const NativeParams &p, int64_t rows
 __global__ void __launch_bounds__(kFbThreads, kFbBlocksPerSm)
 native_rows_kernel(const __grid_constant__ NativeParams p, int sms)
 {
+    dependency_release();
+    dependency_wait();
     const int64_t rows = *p.count;
     if (rows == 0) return;
     __shared__ __align__(16) double As[kFbStageDoubles];
@@ -163,13 +165,11 @@ oz_status_t launch_native_rows(int64_t m, int64_t n, int64_t k, const double *A,
 {
     // refused as ever: more than 65535 groups of 64 rows, or 2^31 groups of 64 columns
     if ((m + 63) / 64 > 65535 || (n + 63) / 64 > 2147483647ll) return OZ_ERR_UNSUPPORTED;
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = sm_count();
     NativeParams p{m, n, k, lda, ldb, ldc, A, B, list, count, shiftB, alpha, beta, C};
     // as many blocks as are resident at once, or fewer where even the smallest tiles are fewer
     const int64_t most = ((m + 15) / 16) * ((n + 15) / 16), cap = static_cast<int64_t>(kFbBlocksPerSm) * sms;
-    native_rows_kernel<<<static_cast<unsigned>(most < cap ? most : cap), kFbThreads, 0, stream>>>(p, sms);
+    OZ_CUDA_CHECK(launch(native_rows_kernel, dim3(static_cast<unsigned>(most < cap ? most : cap)), kFbThreads, 0, stream, p, sms));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;

@@ -240,6 +240,11 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
+__device__ __forceinline__ void prefetch_map(const CUtensorMap *map)
+{
+    asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
 // CTA-pair copy: same as tma_load_3d, but the mbarrier may live in the peer CTA (cluster address)
 __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar_cluster,
                                                  int c0, int c1, int c2)
@@ -499,7 +504,10 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    dependency_release();
     if (threadIdx.x == 0) {
+        prefetch_map(&mapA);
+        prefetch_map(&mapB);
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar + 8 * s, 1);
             mbar_init(empty_bar + 8 * s, 1);
@@ -516,6 +524,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     __syncthreads();
     if (CG == 2) cluster_sync_all();      // the peer's barriers exist before anything signals them
     tc_fence_after();
+    dependency_wait();                    // the planes are there, and the previous readers of the residues are done
     const uint32_t tmem_base = *tmem_base_ptr;
 
     if (warp < FIRST_EPI_WARP) {
@@ -952,8 +961,8 @@ oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, con
 {
     static_assert(!LOOSE || RB == 2, "a representative below 2m needs the two-byte element");
     auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, LOOSE, TILED, BOUND>;
-    OZ_CUDA_CHECK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(SMEM_BYTES)));
+    static std::atomic<unsigned long long> ready{0};
+    OZ_CUDA_CHECK(allow_shared(kernel, SMEM_BYTES, ready));
     int64_t groups = sms / CG;                                    // CTAs, or CTA pairs
     if (p.total_items < groups) groups = p.total_items;
     cudaLaunchConfig_t cfg = {};
@@ -961,13 +970,15 @@ oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, con
     cfg.blockDim = dim3(NUM_THREADS);
     cfg.dynamicSmemBytes = SMEM_BYTES;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = CG;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     OZ_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, mapA, mapB, p));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
@@ -1010,7 +1021,7 @@ static int take_stall_flag()
 static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k)
 {
     for (int i = 0; i < p.r; ++i) {
-        int mi = modulus(set, i), s = square_root(mi);
+        const int mi = modulus(set, i), s = kSetTables.root[set][i];
         p.mod[i].m = static_cast<float>(mi);
         p.mod[i].inv_m = 1.0f / static_cast<float>(mi);
         // Exact range of the running combination.  Digits are bounded by |d0| <= 14 (16 for
@@ -1027,8 +1038,8 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k)
         mo.bias = static_cast<uint32_t>((((1ull << 31) + mi - 1) / mi) * mi);
         mo.magic39 = mi > 128 ? static_cast<uint32_t>(((1ull << 39) + mi - 1) / mi) : 0u;
         mo.bias30 = static_cast<uint32_t>((((1ull << 30) + mi - 1) / mi) * mi);
-        mo.planeA0 = first_plane(set, i, rt.layout(0));
-        mo.planeB0 = first_plane(set, i, rt.layout(1));
+        mo.planeA0 = kSetTables.first[set][rt.layout(0)][i];
+        mo.planeB0 = kSetTables.first[set][rt.layout(1)][i];
         mo.nseg = 1;
         mo.seg_len = p.nk;
         // exact depth of one accumulator, in chunks of BLOCK_K: the largest term is 2 * 16 * 16 (the
@@ -1120,7 +1131,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     fill_mod_info(p, set, rt, k);
 
     CUtensorMap mapA, mapB;
-    const int planesA = p_store(set, rt.layout(0)), planesB = p_store(set, rt.layout(1));
+    const int planesA = kSetTables.first[set][rt.layout(0)][p.r], planesB = kSetTables.first[set][rt.layout(1)][p.r];
     bool maps;
     if (tiled) {       // private layout: one 128-byte column of lines per (plane, chunk); both operands have the same pitch
         const int chunks = static_cast<int>(pitchA / BLOCK_K);
@@ -1134,9 +1145,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     }
     if (!maps) return OZ_ERR_CUDA;
 
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = sm_count();
     // substrate 0: FP8 planes; otherwise INT8 planes (two-limb digits or native residues)
 #define OZ_LAUNCH(SUB, RB, DIRECT, LOOSE, TILED)                                                    \
     (cg == 2 ? launch_variant<SUB, 2, RB, DIRECT, LOOSE, TILED>(mapA, mapB, p, sms, stream)        \
@@ -1195,9 +1204,7 @@ oz_status_t launch_fused_gemm(int64_t m, int64_t n, int64_t k, const double *A, 
     CUtensorMap mapB;
     f.chunksB = static_cast<int>(pitchB / BLOCK_K);
     if (!make_core_matrix_map(&mapB, PB, n, static_cast<int64_t>(p_store(set, rt.layout(1))) * f.chunksB)) return OZ_ERR_CUDA;
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = sm_count();
 #define OZ_FUSED_GEMM(SET_) \
     (rt.substrate == 0 ? launch_fused_variant<0, SET_>(mapB, p, f, sms, stream) : launch_fused_variant<1, SET_>(mapB, p, f, sms, stream))
     if (set == 0) return OZ_FUSED_GEMM(0);
@@ -1243,9 +1250,7 @@ oz_status_t launch_bound_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *GA
     if (!make_plane_map(&mapA, GA, m, pitchA, m * pitchA, 1, BLOCK_N / cg) ||
         !make_plane_map(&mapB, GB, n, pitchB, n * pitchB, 1, BLOCK_M))
         return OZ_ERR_CUDA;
-    int dev = 0, sms = 148;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int sms = sm_count();
     return cg == 2 ? launch_variant<0, 2, 2, true, false, false, true>(mapA, mapB, p, sms, stream)
                    : launch_variant<0, 1, 2, true, false, false, true>(mapA, mapB, p, sms, stream);
 }

@@ -2,6 +2,7 @@
 // Nothing here is part of the public ABI (see include/oz.h).
 #pragma once
 
+#include <atomic>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -70,6 +71,25 @@ __host__ __device__ constexpr int p_store(int set, int layout = kLayoutDigits)
 {
     return first_plane(set, set_r(set), layout);
 }
+
+// The same, tabulated at compile time for the host code that runs on every call (the functions above walk the
+// set and search square roots).
+struct SetTables {
+    int root[3][kMaxR];                         // square root of a square modulus, 0 otherwise
+    int first[3][6][kMaxR + 1];                 // first plane of modulus i per layout; [r]: the number of planes
+};
+constexpr SetTables make_set_tables()
+{
+    SetTables t{};
+    for (int set = 0; set < 3; ++set)
+        for (int i = 0; i < set_r(set); ++i) {
+            t.root[set][i] = square_root(modulus(set, i));
+            for (int layout = 0; layout < 6; ++layout)
+                t.first[set][layout][i + 1] = t.first[set][layout][i] + (layout == kLayoutNative ? 1 : (t.root[set][i] ? 2 : 3));
+        }
+    return t;
+}
+constexpr SetTables kSetTables = make_set_tables();
 
 // largest k for which the merged accumulator d0 e0 - 16 d1 e1 stays exact in FP32: the merged term
 // reaches 4095 on the 9-bit tail of S and 1088 on byte moduli
@@ -162,10 +182,11 @@ struct PlaneGeom {
 inline PlaneGeom public_planes(int64_t plane_stride, int64_t row_pitch) { return {plane_stride, row_pitch, row_pitch, 128}; }
 inline PlaneGeom private_planes(int64_t lines, int64_t pitch) { return {lines * pitch, pitch, 128, 128 * lines}; }
 
+// `alone`: no other chain of kernels runs beside this one (see launch_if())
 // ---- stage launchers (host side of each .cu) ---------------------------------------------
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
-                               int32_t *shift, void *scratch, cudaStream_t stream);
+                               int32_t *shift, void *scratch, bool alone, cudaStream_t stream);
 
 // Tile-ordered private residue array of the whole-method calls.  The output is cut into tiles of
 // 256 rows x tile_cols columns (128, or 256 when CTA pairs are used); a tile is 16 blocks (32 with
@@ -184,12 +205,25 @@ ResidueTiling residue_tiling(int64_t m, int64_t n, int set);
 
 // loose: residues in [0, 2 m_i) (two-byte sets); tiled: R is the tile-ordered private array (ldr and
 // mod_stride are then ignored) and the planes are in the private layout
+// Both operands of a product in one launch, when the one-kernel form takes both (*taken says whether it did);
+// otherwise nothing is launched
+struct OperandJob {
+    int64_t lines;
+    const double *X;
+    int64_t ldx;
+    uint8_t *planes;
+    PlaneGeom geom;
+    int32_t *shift;
+};
+oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, int64_t k, int set, const Route &rt,
+                                    bool *taken, cudaStream_t stream);
+
 // pieces of launch_deconstruct, and the steps of the accurate rule between them
 oz_status_t launch_scan(int side, int64_t lines, int64_t k, const double *X, int64_t ldx, int set,
-                        const Route &rt, int32_t *shift, void *scratch, cudaStream_t stream);
+                        const Route &rt, int32_t *shift, void *scratch, bool alone, cudaStream_t stream);
 oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                   int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
-                                  const int32_t *shift, cudaStream_t stream);
+                                  const int32_t *shift, bool alone, cudaStream_t stream);
 oz_status_t launch_bound_plane(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                void *scratch, uint8_t *plane, int64_t pitch, cudaStream_t stream);
 unsigned int *bound_maxima(void *scratch, int64_t lines);      // one word per line, word stride 2
@@ -249,6 +283,60 @@ oz_status_t launch_native_rows(int64_t m, int64_t n, int64_t k, const double *A,
                                const double *B, int64_t ldb, const int *list, const unsigned int *count,
                                const int32_t *shiftB, double alpha, double beta, double *C, int64_t ldc,
                                cudaStream_t stream);
+
+// ---- launching ---------------------------------------------------------------------------
+// The kernels of a call are launched as programmatic dependents of their predecessors on the stream: their blocks may
+// become resident, and set up what needs no global memory, while the predecessor's last blocks run.  In return every
+// kernel executes dependency_wait() before its first access to global memory and on every path (so
+// that its own completion implies its predecessor's), and lets its successor in with dependency_release() at
+// once.  256^3: 23 -> 15 us of GPU time a call together with the joint deconstruction of both operands.
+#ifdef __CUDACC__
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// dependent = false: an ordinary launch, for the chains of kernels that run beside another stream's: there the blocks that
+// wait early would hold the registers and shared memory that the other chain needs (2003 x 1999 x 1501 with the row
+// check: 505 -> 621 us, 6912 x 6912 x 1024: 2.25 -> 2.34 ms).
+template <class... Params, class... Args>
+cudaError_t launch_if(bool dependent, void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+template <class... Params, class... Args>
+cudaError_t launch(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, Args... args)
+{
+    return launch_if(true, kernel, grid, threads, smem, stream, args...);
+}
+
+// Opts a kernel in to dynamic shared memory beyond 48 KiB, once per device (one flag per call site's kernel).
+template <class Kernel>
+cudaError_t allow_shared(Kernel kernel, size_t bytes, std::atomic<unsigned long long> &done)
+{
+    int dev = 0;
+    cudaError_t rc = cudaGetDevice(&dev);
+    if (rc != cudaSuccess) return rc;
+    const unsigned long long bit = 1ull << (dev & 63);
+    if (done.load(std::memory_order_relaxed) & bit) return cudaSuccess;
+    rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    if (rc == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return rc;
+}
+#endif
+constexpr size_t kMaxShared = 227 * 1024;      // dynamic shared memory a block may have
+
+// multiprocessors of the current device (read once per device)
+int sm_count();
 
 #define OZ_CUDA_CHECK(expr)                                  \
     do {                                                     \

@@ -208,6 +208,8 @@ reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride,
                    int64_t n, const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
                    double alpha, double beta, double *__restrict__ C, int64_t ldc, int vecR, int vecC)
 {
+    dependency_release();
+    dependency_wait();
     constexpr int RB = residue_bytes(SET), ROWS = 4 / RB, r = set_r(SET);
     // grid.x covers the row groups of a column, grid.y (and .z beyond 65535) the columns: no division
     const int64_t row = (blockIdx.x * 256ll + threadIdx.x) * ROWS;
@@ -256,6 +258,8 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
                          double alpha, double beta, double *__restrict__ C, int64_t ldc, int vecC,
                          const unsigned char *__restrict__ skip)
 {
+    dependency_release();
+    dependency_wait();
     constexpr int RB = residue_bytes(SET), ROWS = 4 / RB, r = set_r(SET);
     constexpr int kBlockWords = 64 * 32 * RB / 4;          // words of one 32 x 64 block: 1024 or 512
     constexpr int kColWords = 64 / ROWS;                   // words of one column of the block: 32 or 16
@@ -338,15 +342,8 @@ oz_status_t launch_reconstruct(int64_t m, int64_t n, const void *R, int64_t ldr,
     if (n > 65535ll * 65535ll) return OZ_ERR_UNSUPPORTED;
     dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(n < 65535 ? n : 65535),
               static_cast<unsigned>((n + 65534) / 65535));
-    if (set == 2)
-        reconstruct_kernel<2><<<grid, 256, 0, stream>>>(R, ldr, mod_stride, m, n, shiftA, shiftB, alpha,
-                                                        beta, C, ldc, vecR, vecC);
-    else if (set == 0)
-        reconstruct_kernel<0><<<grid, 256, 0, stream>>>(R, ldr, mod_stride, m, n, shiftA, shiftB, alpha,
-                                                        beta, C, ldc, vecR, vecC);
-    else
-        reconstruct_kernel<1><<<grid, 256, 0, stream>>>(R, ldr, mod_stride, m, n, shiftA, shiftB, alpha,
-                                                        beta, C, ldc, vecR, vecC);
+    auto kernel = set == 2 ? reconstruct_kernel<2> : set == 0 ? reconstruct_kernel<0> : reconstruct_kernel<1>;
+    OZ_CUDA_CHECK(launch(kernel, grid, 256, 0, stream, R, ldr, mod_stride, m, n, shiftA, shiftB, alpha, beta, C, ldc, vecR, vecC));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
@@ -366,11 +363,12 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     const int vecC = ((ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0) ? 1 : 0;
     const dim3 grid(static_cast<unsigned>(pieces * 16 * t.cg), static_cast<unsigned>(ntn),
                     static_cast<unsigned>(t.tiles_m));
-#define OZ_RECON_TILED(SET_)                                                                               \
-    (skip ? reconstruct_tiled_kernel<SET_, true><<<grid, 256, 0, stream>>>(                                \
-                R, t.cg, t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, vecC, skip) \
-          : reconstruct_tiled_kernel<SET_, false><<<grid, 256, 0, stream>>>(                               \
-                R, t.cg, t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, vecC, nullptr))
+    // Blocks that become resident beside the GEMM's keep the multiprocessor's memory split at the GEMM's (28 KiB of L1) for
+    // the whole kernel: worth the overlapped launch up to a million outputs only (16384 x 16384: 11.4 -> 11.9 ms a call)
+    const bool early = m * n <= (1ll << 20);
+#define OZ_RECON_TILED(SET_)                                                                                         \
+    OZ_CUDA_CHECK(launch_if(early, skip ? reconstruct_tiled_kernel<SET_, true> : reconstruct_tiled_kernel<SET_, false>, grid, 256, 0, \
+                         stream, R, t.cg, t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, vecC, skip))
     if (set == 2) OZ_RECON_TILED(2);
     else if (set == 0) OZ_RECON_TILED(0);
     else OZ_RECON_TILED(1);
