@@ -66,6 +66,21 @@ __device__ __forceinline__ int classify(double x, int *e)
     return 1;
 }
 
+// ceil(|x| 2^(9-E)) in integer arithmetic (lines of subnormals, where 2^(9-E) is no normal double)
+__device__ __forceinline__ unsigned int scaled_magnitude(double x, int E)
+{
+    const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
+    const int be = static_cast<int>((bits >> 52) & 0x7FF);
+    const unsigned long long frac = bits & 0xFFFFFFFFFFFFFull;
+    if (be == 0x7FF || (be == 0 && frac == 0)) return 0u;
+    const unsigned long long sig = be ? (frac | (1ull << 52)) : frac;
+    const int ex = be ? be - 1023 : -1022;
+    const int sh = 43 + E - ex;                           // |x| 2^(9-E) = sig / 2^sh
+    if (sh >= 64) return 1u;
+    if (sh <= 0) return static_cast<unsigned int>(sig << (-sh));
+    return static_cast<unsigned int>((sig >> sh) + ((sig & ((1ull << sh) - 1ull)) ? 1ull : 0ull));
+}
+
 __global__ void scan_init_kernel(ScanScratch s, int64_t lines)
 {
     dependency_release();
@@ -103,11 +118,12 @@ scan_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
         kstep = 32;
     }
     bool live = line < lines;
-    int emax = INT32_MIN, bad = 0;
+    int emax = INT32_MIN;
+    unsigned int top = 0u;        // PASS 0: largest high word of |x|
     unsigned long long acc = 0;
     unsigned int l1 = 0;          // sum of the magnitudes abar <= 2^10 (exponent-span check): below 2^30 for k <= 2^20
     int E = 0;
-    if (PASS == 1 && live) E = s.emax[line];
+    if (PASS == 1 && live) E = s.nonfinite[line] < 0 ? INT32_MIN : s.emax[line];      // INT32_MIN: nothing to add
     // 2^(9-E) as a double, when it is a normal number (not for lines of subnormals only)
     const bool fast_scale = PASS == 1 && E != INT32_MIN && 9 - E >= -1000 && 9 - E <= 1000;
     const double scale9 = __hiloint2double((1023 + (fast_scale ? 9 - E : 0)) << 20, 0);
@@ -120,59 +136,52 @@ scan_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
                 int64_t kk = kb + u * kstep;
                 xs[u] = kk < k1 ? *element(X, ldx, SIDE, line, kk) : 0.0;
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                double x = xs[u];
-                if (PASS == 0) {
-                    int e;
-                    int c = classify(x, &e);
-                    if (c == 2) bad = 1;
-                    if (c == 1 && e > emax) emax = e;
-                } else if (fast_scale) {
-                    // ceil(|x| 2^(9-E)) through an exact FP64 scaling and a round-up conversion; a
-                    // non-zero x whose scaled value underflows to zero still counts as 1
-                    double y = fabs(x) * scale9;
-                    unsigned long long abar = static_cast<unsigned long long>(__double2ll_ru(y));
-                    if (abar == 0ull && x != 0.0) abar = 1ull;
-                    if (!(y < 2048.0)) abar = 0ull;       // Inf/NaN: the line is flagged, value unused
-                    acc += abar * abar;
-                    l1 += static_cast<unsigned int>(abar);
-                } else {
-                    unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
-                    int be = static_cast<int>((bits >> 52) & 0x7FF);
-                    unsigned long long frac = bits & 0xFFFFFFFFFFFFFull;
-                    if (be == 0x7FF || (be == 0 && frac == 0)) continue;
-                    unsigned long long sig = be ? (frac | (1ull << 52)) : frac;
-                    int ex = be ? be - 1023 : -1022;
-                    int sh = 43 + E - ex;                 // |x| 2^(9-E) = sig / 2^sh
-                    unsigned long long abar;
-                    if (sh >= 64) abar = 1;
-                    else if (sh <= 0) abar = sig << (-sh);
-                    else abar = (sig >> sh) + ((sig & ((1ull << sh) - 1)) ? 1ull : 0ull);
-                    acc += abar * abar;
-                    l1 += static_cast<unsigned int>(abar);
-                }
-            }
-        }
-    }
-    if (SIDE == 1) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
             if (PASS == 0) {
-                int other = __shfl_xor_sync(0xFFFFFFFFu, emax, o);
-                emax = other > emax ? other : emax;
-                bad |= __shfl_xor_sync(0xFFFFFFFFu, bad, o);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) top = max(top, static_cast<unsigned int>(__double2hiint(xs[u])) & 0x7FFFFFFFu);
             } else {
-                acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
-                l1 += __shfl_xor_sync(0xFFFFFFFFu, l1, o);
+                unsigned int part = 0u;           // eight terms of at most 2^20
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const double x = xs[u];
+                    unsigned int abar;
+                    if (fast_scale) {
+                        // ceil(|x| 2^(9-E)) through an exact FP64 scaling and a round-up conversion; a non-zero x whose
+                        // scaled value underflows to zero still counts as 1
+                        abar = __double2uint_ru(fabs(x) * scale9);
+                        if (abar == 0u && x != 0.0) abar = 1u;
+                    } else {
+                        abar = scaled_magnitude(x, E);
+                    }
+                    part += abar * abar;
+                    l1 += abar;
+                }
+                acc += part;
             }
         }
-        if (lane != 0) live = false;
     }
-    if (!live) return;
     if (PASS == 0) {
-        if (emax != INT32_MIN) atomicMax(&s.emax[line], emax);
-        if (bad) atomicOr(&s.nonfinite[line], kNonfiniteBit);
+        // The high words order like the exponents; where only zeros and subnormals were seen, the exponents come
+        // from the whole words.
+        if (SIDE == 1) top = __reduce_max_sync(0xFFFFFFFFu, top);
+        if (top >= 0x00100000u) {
+            emax = static_cast<int>(top >> 20) - 1023;
+        } else if (live) {
+            for (int64_t kk = kstart; kk < k1; kk += kstep) {
+                int e;
+                if (classify(*element(X, ldx, SIDE, line, kk), &e) == 1 && e > emax) emax = e;
+            }
+            if (SIDE == 1) emax = __reduce_max_sync(0xFFFFFFFFu, emax);
+        }
+    } else if (SIDE == 1) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+        l1 = __reduce_add_sync(0xFFFFFFFFu, l1);
+    }
+    if (!live || (SIDE == 1 && lane != 0)) return;
+    if (PASS == 0) {
+        if (top >= 0x7FF00000u) atomicOr(&s.nonfinite[line], kNonfiniteBit);
+        else if (emax != INT32_MIN) atomicMax(&s.emax[line], emax);
     } else if (acc) {
         atomicAdd(&s.sumsq[line], acc);
         atomicAdd(&s.nonfinite[line], static_cast<int>(l1));     // never reaches bit 31
@@ -574,21 +583,6 @@ struct FusedLine {             // per-line results in shared memory
     unsigned int l1;
 };
 
-// ceil(|x| 2^(9-E)) in integer arithmetic (lines of subnormals, where 2^(9-E) is no normal double)
-__device__ __forceinline__ unsigned int scaled_magnitude(double x, int E)
-{
-    const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
-    const int be = static_cast<int>((bits >> 52) & 0x7FF);
-    const unsigned long long frac = bits & 0xFFFFFFFFFFFFFull;
-    if (be == 0x7FF || (be == 0 && frac == 0)) return 0u;
-    const unsigned long long sig = be ? (frac | (1ull << 52)) : frac;
-    const int ex = be ? be - 1023 : -1022;
-    const int sh = 43 + E - ex;                           // |x| 2^(9-E) = sig / 2^sh
-    if (sh >= 64) return 1u;
-    if (sh <= 0) return static_cast<unsigned int>(sig << (-sh));
-    return static_cast<unsigned int>((sig >> sh) + ((sig & ((1ull << sh) - 1ull)) ? 1ull : 0ull));
-}
-
 // The shift of a line from its scan results, with its contribution to the device status block
 __device__ __forceinline__ int line_shift(const FusedParams &p, const FusedLine &r)
 {
@@ -771,56 +765,49 @@ deconstruct_pair_kernel(const __grid_constant__ PairParams p)
 
 // Lines per thread-block pass of the fused kernel and its launch shape; group = 0: not applicable
 // (the lines are too long for shared memory).
-#ifndef OZ_FUSED_MAX_ELEMS
-#define OZ_FUSED_MAX_ELEMS (1ll << 22)
-#endif
+// Largest operand of the one-kernel form.  Above, the three-pass kernels win (2500 x 2500 x 1024: equal; 1500^3: 171
+// against 165 us a call; 4000 x 1000 x 1000: 217 against 229).
+constexpr int64_t kFusedMaxElems = 1ll << 22;
 struct FusedShape { int group, threads, grid; size_t smem; };
 
-FusedShape fused_shape(int set, int layout, int side, int64_t lines, int64_t k, int sms)
+// `big`: one block of 1024 threads per SM instead of two of 512 (lines too long for two); `slots`: resident blocks
+// that this operand may count on
+FusedShape fused_shape(int set, int layout, int side, int64_t lines, int64_t k, bool big, int64_t slots)
 {
     FusedShape f{0, 0, 0, 0};
     if (k < 1 || k > 32768 || lines < 1) return f;
     // The one-kernel form wins where the call is bound by launch latency; larger operands keep the
     // three-pass kernels, whose many small blocks hide the memory latency better.
-    if (lines * k > OZ_FUSED_MAX_ELEMS) return f;
-    const size_t line_bytes = static_cast<size_t>(fused_pitch(static_cast<int>(k))) * 8;
-    const size_t fixed = lut_words_of(set, layout) * 4 + 64 * sizeof(FusedLine) + 64;
-    // two blocks per SM when lines are short enough for that, else one block with more threads
-    const size_t budget2 = 110 * 1024, budget1 = 224 * 1024;
-    int group = static_cast<int>((budget2 - fixed) / line_bytes);
-    int threads = 512;
-    const int min_group = side == 0 ? 4 : 1;         // side 0 loads `group` consecutive doubles per inner index
-    if (group < (side == 0 ? 8 : 2)) {
-        group = static_cast<int>((budget1 - fixed) / line_bytes);
-        threads = 1024;
-    }
-    if (group < min_group) return f;
+    if (lines * k > kFusedMaxElems) return f;
+    const int64_t line_bytes = static_cast<int64_t>(fused_pitch(static_cast<int>(k))) * 8;
+    const int64_t fixed = lut_words_of(set, layout) * 4 + 64 * static_cast<int64_t>(sizeof(FusedLine)) + 64;
+    int64_t group = ((big ? 224 : 110) * 1024 - fixed) / line_bytes;
+    // side 0 loads `group` consecutive doubles per inner index
+    if (group < (side == 0 ? (big ? 4 : 8) : (big ? 1 : 2))) return f;
     if (group > 32) group = 32;
     // small operands: fewer lines per block, so that the blocks cover the machine (a 256 x 256 operand
     // with 32 lines per block would run on 8 SMs)
-#ifndef OZ_FUSED_SPREAD_MIN
-#define OZ_FUSED_SPREAD_MIN 8
-#endif
-    {
-        const int64_t blocks_wanted = static_cast<int64_t>(sms) * (threads == 512 ? 2 : 1);
-        int64_t spread = (lines + blocks_wanted - 1) / blocks_wanted;
-        const int floor_group = side == 0 ? OZ_FUSED_SPREAD_MIN : 1;
-        if (spread < floor_group) spread = floor_group;
-        if (spread < group) group = static_cast<int>(spread);
-    }
+    if (slots < 1) slots = 1;
+    int64_t spread = (lines + slots - 1) / slots;
+    // side 0: at least four consecutive lines (whole 32-byte sectors), eight where few blocks are enough
+    // (500^3: 24.7 us a call with four, 28.0 with eight; 256^3: 20.2 and 19.0)
+    const int floor_group = side == 0 ? (lines * k >= (1ll << 17) ? 4 : 8) : 1;
+    if (spread < floor_group) spread = floor_group;
+    if (spread < group) group = spread;
     if (side == 0) {
         int pow2 = 1;
         while (pow2 * 2 <= group) pow2 *= 2;
+        // up rather than down: a second round costs more than fuller blocks (1300 x 300 x 1400: 70.9 and 78.0 us)
+        if (group > pow2 && (pow2 * 2) * line_bytes + fixed <= (big ? 224 : 110) * 1024 && pow2 < 32) pow2 *= 2;
         group = pow2;
     } else if (group > lines) {
-        group = static_cast<int>(lines);
+        group = lines;
     }
-    f.group = group;
-    f.threads = threads;
-    f.smem = fixed + static_cast<size_t>(group) * line_bytes;
+    f.group = static_cast<int>(group);
+    f.threads = big ? 1024 : 512;
+    f.smem = static_cast<size_t>(fixed + group * line_bytes);
     const int64_t ngroups = (lines + group - 1) / group;
-    const int64_t cap = static_cast<int64_t>(sms) * (threads == 512 ? 2 : 1);
-    f.grid = static_cast<int>(ngroups < cap ? ngroups : cap);
+    f.grid = static_cast<int>(ngroups < slots ? ngroups : slots);
     return f;
 }
 
@@ -1005,7 +992,8 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
 {
     if (rt.rule == 2) return OZ_ERR_UNSUPPORTED;      // the accurate rule needs both operands
     const int sms = sm_count();
-    const FusedShape f = fused_shape(set, rt.layout(side), side, lines, k, sms);
+    FusedShape f = fused_shape(set, rt.layout(side), side, lines, k, false, 2ll * sms);
+    if (f.group <= 0) f = fused_shape(set, rt.layout(side), side, lines, k, true, sms);
     if (f.group > 0 && !rt.fallback) {      // the row check reads the scan results of the three-pass form
         const FusedParams p = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, f.group);
         const int layout = rt.layout(side);
@@ -1034,8 +1022,20 @@ oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, in
     *taken = false;
     if (rt.rule == 2 || rt.fallback) return OZ_OK;      // shifts from both operands; the row check's scan results
     const int sms = sm_count();
-    const FusedShape fa = fused_shape(set, rt.layout(0), 0, a.lines, k, sms), fb = fused_shape(set, rt.layout(1), 1, b.lines, k, sms);
-    if (fa.group <= 0 || fb.group <= 0 || fa.threads != fb.threads) return OZ_OK;
+    // The resident blocks are shared out by the operands' sizes.  Taken when both operands then finish in one round
+    // (1009 x 983 x 1021: 77.0 -> 68.8 us a call; 1300 x 300 x 1400, one large block per SM: 81.5 -> 70.8); with more rounds the
+    // two streams do as well or better (1800^3: 286 against 309).
+    FusedShape fa, fb;
+    bool one_round = false;
+    for (const bool big : {false, true}) {
+        const int64_t slots = (big ? 1 : 2) * static_cast<int64_t>(sms);
+        fa = fused_shape(set, rt.layout(0), 0, a.lines, k, big, slots * a.lines / (a.lines + b.lines));
+        fb = fused_shape(set, rt.layout(1), 1, b.lines, k, big, slots - fa.grid);
+        one_round = fa.group > 0 && fb.group > 0 && static_cast<int64_t>(fa.grid) * fa.group >= a.lines &&
+                    static_cast<int64_t>(fb.grid) * fb.group >= b.lines;
+        if (one_round) break;
+    }
+    if (!one_round) return OZ_OK;
     PairParams p;
     p.a = fused_params(0, a.lines, k, a.X, a.ldx, set, rt, a.planes, a.geom, a.shift, fa.group);
     p.b = fused_params(1, b.lines, k, b.X, b.ldx, set, rt, b.planes, b.geom, b.shift, fb.group);

@@ -42,3 +42,40 @@ def test_limb_edges_bit_exact(side, lines, k, set_name, sub):
         want = ozo.planes(ozo.residues(Q, OSET[set_name]), OSET[set_name], OSUB[sub])
         assert st == 0 and (shift == want_shift).all()
         assert got.shape == want.shape and (got == want).all()
+
+
+@pytest.mark.parametrize("m,n,k", [
+    (1, 1, 1), (3, 2, 5),            # less than one group of lines
+    (9, 300, 64), (300, 9, 64),      # very unequal shares of the resident blocks
+    (517, 403, 260),                 # groups of four lines on side 0, ragged
+    (1301, 299, 1400),               # one large block per SM
+    (1500, 1490, 1500),              # more rounds than one: two streams
+    (150, 2100, 2051),               # one operand too large for the one-kernel form
+])
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("A", "int8n")])
+def test_joint_deconstruction_shapes(m, n, k, set_name, sub):
+    """Whole calls on either side of every rule that decides how the two operands are deconstructed together,
+    against the call on operands that were prepared one by one (bit for bit: same shifts, same planes)."""
+    import paper_2609_09095_b200 as oz
+    import torch
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m + 3 * n + k)
+    A, B = np.asfortranarray(rng.standard_normal((m, k))), np.asfortranarray(rng.standard_normal((k, n)))
+    A[0, 0] = 0.0
+    if m > 8:
+        A[5, :] = 0.0
+        A[7, :] *= 2.0 ** -1060                       # a row of subnormals
+    if n > 4:
+        B[:, 3] *= 2.0 ** 700
+    got, st = gh.dgemm(A, B, set_name, gh.route(sub))
+    rt, S = gh.route(sub), gh.SETS[set_name]
+    opA = torch.empty(oz.oz_operand_bytes(0, m, k, S, rt), dtype=torch.uint8, device="cuda")
+    opB = torch.empty(oz.oz_operand_bytes(1, n, k, S, rt), dtype=torch.uint8, device="cuda")
+    oz.check(oz.oz_prepare_operand(0, m, k, gh.to_dev(A), m, S, rt, opA), "prepare A")
+    oz.check(oz.oz_prepare_operand(1, n, k, gh.to_dev(B), k, S, rt, opB), "prepare B")
+    dC = torch.full((n, m), 7.0, dtype=torch.float64, device="cuda")
+    oz.check(oz.oz_dgemm_prepared(m, n, k, 1.0, opA, opB, 0.0, dC, m, S, rt), "product")
+    assert st == 0 and gh.sync_status() == 0
+    assert (got == gh.from_dev(dC)).all()
+    if m * n <= 200000:
+        assert (got == ozo.dgemm(A, B, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS)).all()
