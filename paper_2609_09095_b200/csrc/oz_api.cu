@@ -383,6 +383,7 @@ bool valid_set(int set) { return set == OZ_SET_S || set == OZ_SET_E || set == OZ
 // overlap the transfers of C with the computation: before panel p the stream waits for before[p]
 // (when wait_before), after it the stream records after[p].
 constexpr int kMaxPanels = 16;
+constexpr int64_t kPanelColumns = 256;      // panels of whole GEMM tiles
 struct PanelPlan {
     int np;
     int64_t col0[kMaxPanels + 1];
@@ -560,11 +561,54 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     return launch_native_rows(m, n, k, A, lda, B, ldb, list, count, b.shift, alpha, beta, C, ldc, stream);
 }
 
+// The product of the host-buffer entry point column panel by column panel, on operands that arrive in that order:
+// A is deconstructed once, a panel's columns of B when b_ready[p] says that they are there, and its residues reuse
+// one region.  Every stage runs on `stream`, so no panel overtakes another.  Same bits as the undivided call: shifts,
+// planes, residues and outputs of a column depend on A and on that column alone.
+oz_status_t dgemm_panels(int64_t m, int64_t n, int64_t k, double alpha, const double *A, const double *B, double beta,
+                         double *C, int set, const Route &rt, cudaStream_t stream, char *ws, int dev,
+                         const PanelPlan &plan, const cudaEvent_t *b_ready)
+{
+    if (!(alpha == 1.0 || alpha == -1.0) || !(beta == 0.0 || beta == 1.0)) return OZ_ERR_UNSUPPORTED;
+    const Layout L = make_layout(m, n, k, set, rt);
+    oz_status_t st = ensure_device_ready();
+    if (st != OZ_OK) return st;
+    const OperandView a = operand_view(ws + L.offA, L.A), b = operand_view(ws + L.offB, L.B);
+    const bool ev = g_stage_events_on[dev];
+    if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][0], stream));
+    st = launch_deconstruct(0, m, k, A, m, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, true, stream);
+    if (st != OZ_OK) return st;
+    if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
+    for (int p = 0; p < plan.np; ++p) {
+        const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
+        // the panel's share of B's block: every array of it is proportional to the lines
+        OperandView bp = b;
+        bp.shift = b.shift + j0;
+        bp.scratch = static_cast<char *>(b.scratch) + 16 * j0;
+        bp.planes = b.planes + static_cast<int64_t>(kSetTables.first[set][rt.layout(1)][set_r(set)]) * j0 * b.pitch;
+        bp.stride = cols * b.pitch;
+        OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, b_ready[p], 0));
+        st = launch_deconstruct(1, cols, k, B + j0 * k, k, set, rt, bp.planes, private_planes(cols, b.pitch), bp.shift, bp.scratch,
+                                true, stream);
+        if (st != OZ_OK) return st;
+        PanelPlan one{};
+        one.np = 1;
+        one.col0[0] = 0;
+        one.col0[1] = cols;
+        one.wait_before = plan.wait_before;
+        one.before = plan.before + p;
+        one.after = plan.after + p;
+        st = product_impl(m, cols, k, alpha, a, bp, beta, C + j0 * m, m, set, rt, stream, ws + L.R, dev, &one);
+        if (st != OZ_OK) return st;
+    }
+    return OZ_OK;
+}
+
 // Side streams and events of the host-buffer entry point, created once per device.
 struct HostPipe {
     bool ready;
     cudaStream_t in, out;
-    cudaEvent_t start, ab, done, c[kMaxPanels], r[kMaxPanels];
+    cudaEvent_t start, ab, done, b[kMaxPanels], c[kMaxPanels], r[kMaxPanels];
 };
 HostPipe g_pipe[kMaxDevices];
 
@@ -578,6 +622,7 @@ oz_status_t ensure_pipe(int dev, HostPipe **out)
         cudaEvent_t *single[3] = {&hp.start, &hp.ab, &hp.done};
         for (cudaEvent_t *e : single) OZ_CUDA_CHECK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
         for (int p = 0; p < kMaxPanels; ++p) {
+            OZ_CUDA_CHECK(cudaEventCreateWithFlags(&hp.b[p], cudaEventDisableTiming));
             OZ_CUDA_CHECK(cudaEventCreateWithFlags(&hp.c[p], cudaEventDisableTiming));
             OZ_CUDA_CHECK(cudaEventCreateWithFlags(&hp.r[p], cudaEventDisableTiming));
         }
@@ -694,38 +739,62 @@ oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const d
     double *dA = reinterpret_cast<double *>(ws + offA);
     double *dB = reinterpret_cast<double *>(ws + offB);
     double *dC = reinterpret_cast<double *>(ws + offC);
-    // Large outputs: C travels in column panels on two side streams, so that its upload overlaps
-    // the deconstruction and the residue GEMMs, and the download of a finished panel overlaps the
-    // upload and the reconstruction of the next ones (PCIe is full duplex).  The caller's stream
-    // waits for both side streams before the call's work counts as done on it.
-    int np = static_cast<int>(bytesC >> 26);                 // panels of at least 64 MiB
+    // C travels in column panels on two side streams, so that its upload overlaps the computation and the download
+    // of a finished panel overlaps the upload of the next ones (PCIe is full duplex).  The caller's stream
+    // waits for both side streams before the call's work counts as done on it.  Up to eight panels of at least
+    // 4 MiB of traffic, more only of 64 MiB each: a copy costs some microseconds of the link (4096 x 4096 x 1024 update:
+    // 5070 us in two panels, 4513 in eight, 4626 in sixteen; 5000 x 300 x 300: 822 undivided, 690; 16384 x 16384 x
+    // 1024: 54.8 ms, 53.0 in eight, 50.7 in sixteen).
+    const size_t moved = bytesB + (beta != 0.0 ? 2 : 1) * bytesC;
+    // the routes that take the undivided call only: panels from 64 MiB of C each, where they have always been refused
+    const bool undivided = rt.fallback || rt.fused;
+    const size_t few = moved >> 22 < 8 ? moved >> 22 : 8, many = moved >> 26;
+    int np = static_cast<int>(undivided ? bytesC >> 26 : (many > few ? (many < kMaxPanels ? many : kMaxPanels) : few));
     if (np > kMaxPanels) np = kMaxPanels;
     if (np > n) np = static_cast<int>(n);
     if (k > 0 && np >= 2) {
         HostPipe *hp = nullptr;
-        oz_status_t pst = ensure_pipe(dev, &hp);
-        if (pst != OZ_OK) return pst;
+        oz_status_t st = ensure_pipe(dev, &hp);
+        if (st != OZ_OK) return st;
+        // The columns of C are independent of one another except under the accurate rule (shifts of A from all of B):
+        // with enough of them the whole product runs panel by panel behind the upload of its columns of B.
+        const bool by_panel = rt.rule != 2 && !undivided && n >= 2 * kPanelColumns;
         PanelPlan plan{};
+        if (by_panel && np > n / kPanelColumns) np = static_cast<int>(n / kPanelColumns);      // at least one whole tile each
         plan.np = np;
-        for (int p = 0; p <= np; ++p) plan.col0[p] = n * p / np;
+        for (int p = 0; p <= np; ++p) {
+            plan.col0[p] = n * p / np;
+            if (by_panel) plan.col0[p] = plan.col0[p] / kPanelColumns * kPanelColumns;
+        }
+        plan.col0[np] = n;
         plan.wait_before = beta != 0.0;
         plan.before = hp->c;
         plan.after = hp->r;
+        auto upload_c = [&](int p) {
+            const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
+            return cudaMemcpy2DAsync(dC + j0 * m, 8 * m, C_host + j0 * ldc, 8 * ldc, 8 * m, cols, cudaMemcpyHostToDevice, hp->in);
+        };
         OZ_CUDA_CHECK(cudaEventRecord(hp->start, s));          // the workspace may still be in use on s
         OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->in, hp->start, 0));
         OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->out, hp->start, 0));
         OZ_CUDA_CHECK(cudaMemcpy2DAsync(dA, 8 * m, A_host, 8 * lda, 8 * m, k, cudaMemcpyHostToDevice, hp->in));
-        OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB, 8 * k, B_host, 8 * ldb, 8 * k, n, cudaMemcpyHostToDevice, hp->in));
+        if (!by_panel) OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB, 8 * k, B_host, 8 * ldb, 8 * k, n, cudaMemcpyHostToDevice, hp->in));
         OZ_CUDA_CHECK(cudaEventRecord(hp->ab, hp->in));
-        if (beta != 0.0)
-            for (int p = 0; p < np; ++p) {
+        // B runs one panel ahead of C, so that a panel's products are ready when its old C arrives
+        for (int p = 0; p <= np; ++p) {
+            if (by_panel && p < np) {
                 const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
-                OZ_CUDA_CHECK(cudaMemcpy2DAsync(dC + j0 * m, 8 * m, C_host + j0 * ldc, 8 * ldc, 8 * m, cols,
-                                                cudaMemcpyHostToDevice, hp->in));
-                OZ_CUDA_CHECK(cudaEventRecord(hp->c[p], hp->in));
+                OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB + j0 * k, 8 * k, B_host + j0 * ldb, 8 * ldb, 8 * k, cols, cudaMemcpyHostToDevice, hp->in));
+                OZ_CUDA_CHECK(cudaEventRecord(hp->b[p], hp->in));
             }
+            if (beta != 0.0 && p > 0) {
+                OZ_CUDA_CHECK(upload_c(p - 1));
+                OZ_CUDA_CHECK(cudaEventRecord(hp->c[p - 1], hp->in));
+            }
+        }
         OZ_CUDA_CHECK(cudaStreamWaitEvent(s, hp->ab, 0));
-        oz_status_t st = dgemm_impl(m, n, k, alpha, dA, m, dB, kk, beta, dC, m, set, route, s, ws, core, &plan);
+        if (by_panel) st = dgemm_panels(m, n, k, alpha, dA, dB, beta, dC, set, rt, s, ws, dev, plan, hp->b);
+        else st = dgemm_impl(m, n, k, alpha, dA, m, dB, kk, beta, dC, m, set, route, s, ws, core, &plan);
         if (st != OZ_OK) return st;
         for (int p = 0; p < np; ++p) {
             const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
