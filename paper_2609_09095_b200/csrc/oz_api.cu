@@ -606,7 +606,7 @@ oz_status_t dgemm_panels(int64_t m, int64_t n, int64_t k, double alpha, const do
 
 // Side streams and events of the host-buffer entry point, created once per device.
 struct HostPipe {
-    bool ready;
+    std::atomic<bool> ready;
     cudaStream_t in, out;
     cudaEvent_t start, ab, done, b[kMaxPanels], c[kMaxPanels], r[kMaxPanels];
 };
@@ -752,6 +752,12 @@ oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const d
     int np = static_cast<int>(undivided ? bytesC >> 26 : (many > few ? (many < kMaxPanels ? many : kMaxPanels) : few));
     if (np > kMaxPanels) np = kMaxPanels;
     if (np > n) np = static_cast<int>(n);
+    // nothing is created inside a capture for a size that has always been taken undivided
+    if (np >= 2 && bytesC < (2ull << 26) && !g_pipe[dev].ready.load()) {
+        cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+        OZ_CUDA_CHECK(cudaStreamIsCapturing(s, &capturing));
+        if (capturing != cudaStreamCaptureStatusNone) np = 1;
+    }
     if (k > 0 && np >= 2) {
         HostPipe *hp = nullptr;
         oz_status_t st = ensure_pipe(dev, &hp);
