@@ -11,7 +11,8 @@
 //   non-square, merged accumulators (FP8): job 0 = [D0|-16 D1].[E0|E1] (-15); job 1 = DS.ES (16)
 //                -- the regrouping discussed under Table "tuples" (N_acc = 2); one TMEM drain
 //                fewer per modulus, and the drains are what the epilogue pays for at small k
-// Three MMA K-loops per modulus either way (p_mma = 3r).
+// Three MMA K-loops per modulus either way (p_mma = 3r); the three of a square run as one loop over its four
+// tiles per K chunk, into both accumulator slots (pair_squares).
 //
 // Split-K inside the kernel: a job whose K range exceeds the exact depth of its accumulator (4097
 // or 15420 for the merged job 0, 32768 for every other FP32 accumulator, 2^31 / term size in
@@ -123,6 +124,7 @@ struct GemmParams {
     int tiles_m, tiles_n, nk;       // tiles of 256 rows / 128 columns of C; nk = K chunks of BLOCK_K
     int vec_store;                  // R rows 16-byte aligned: use vector stores
     int kc_x, plane_z, kc_z;        // TMA coordinates of chunk kc of a plane: x = kc * kc_x, z = plane * plane_z + kc * kc_z
+    int pair_squares;               // squares: both jobs in one K-loop
     int stall_producer;             // test hook: the producer issues no copy, so every wait runs out
     int r;
     int64_t total_items;
@@ -536,16 +538,9 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             for (int64_t item = first_item; ok && !p.stall_producer && item < p.total_items; item += item_step) {
                 Item it = decode_item(item, p);
                 const ModInfo &mi = p.mod[it.mod];
-                for (int job = 0; ok && job < mi.njobs; ++job)
-                for (int seg = 0, nseg = job_segments(mi, job); ok && seg < nseg; ++seg) {
-                    int npairs = job_pairs(mi, job), kc0, kc1;
-                    segment_range(mi, job, seg, p.nk, &kc0, &kc1);
-                    for (int pair = 0; ok && pair < npairs; ++pair) {
-                        int pa, pb;
-                        job_planes(mi, job, pair, &pa, &pb);
-                        for (int kc = kc0; kc < kc1; ++kc) {
-                            ok = mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status);
-                            if (!ok) break;
+                // one stage: 128 bytes of K of plane pa of A and pb of B
+                auto load = [&](int pa, int pb, int kc) {
+                            if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) return false;
                             uint32_t fb = full_bar + 8 * stage;
                             uint32_t sa = tiles + stage * STAGE_BYTES;
                             if (CG == 1) {
@@ -562,7 +557,22 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                                                  it.tm * BLOCK_N + static_cast<int>(rank) * Tile<CG>::B_LINES, pa * p.plane_z + kc * p.kc_z);
                             }
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                        }
+                            return true;
+                };
+                if (!DIRECT && p.pair_squares && mi.kind == 0) {
+                    // the two planes of a chunk in two stages, side by side
+                    for (int kc = 0; ok && kc < p.nk; ++kc)
+                        ok = load(mi.planeA0, mi.planeB0, kc) && load(mi.planeA0 + 1, mi.planeB0 + 1, kc);
+                    continue;
+                }
+                for (int job = 0; ok && job < mi.njobs; ++job)
+                for (int seg = 0, nseg = job_segments(mi, job); ok && seg < nseg; ++seg) {
+                    int npairs = job_pairs(mi, job), kc0, kc1;
+                    segment_range(mi, job, seg, p.nk, &kc0, &kc1);
+                    for (int pair = 0; ok && pair < npairs; ++pair) {
+                        int pa, pb;
+                        job_planes(mi, job, pair, &pa, &pb);
+                        for (int kc = kc0; ok && kc < kc1; ++kc) ok = load(pa, pb, kc);
                     }
                 }
             }
@@ -582,6 +592,42 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             for (int64_t item = first_item; ok && item < p.total_items; item += item_step) {
                 Item it = decode_item(item, p);
                 const ModInfo &mi = p.mod[it.mod];
+                if (!DIRECT && p.pair_squares && mi.kind == 0) {
+                    // d0 e0 into one slot, d1 e0 + d0 e1 into the other, from the four tiles of a chunk
+                    for (int h = 0; ok && h < 2; ++h)
+                        ok = mbar_wait(tempty_bar + 8 * (slot ^ h), ((slot_phase >> (slot ^ h)) & 1u) ^ 1u, abort_flag, p.status);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t d0 = tmem_base + static_cast<uint32_t>(slot * BLOCK_N);
+                    const uint32_t d1 = tmem_base + static_cast<uint32_t>((slot ^ 1) * BLOCK_N);
+                    for (int kc = 0; kc < p.nk; ++kc) {
+                        const int s0 = stage, s1 = stage + 1 == STAGES ? 0 : stage + 1;
+                        ok = mbar_wait(full_bar + 8 * s0, phase, abort_flag, p.status);
+                        if (!ok) break;
+                        ok = mbar_wait(full_bar + 8 * s1, s1 == 0 ? phase ^ 1u : phase, abort_flag, p.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t t0 = tiles + s0 * STAGE_BYTES, t1 = tiles + s1 * STAGE_BYTES;
+                        const uint64_t e0 = smem_desc(t0), a0 = smem_desc(t0 + A_BYTES), e1 = smem_desc(t1), a1 = smem_desc(t1 + A_BYTES);
+#pragma unroll
+                        for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
+                            const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
+                            const uint32_t accumulate = kc > 0 || ks > 0 ? 1u : 0u;
+                            umma<SUB, CG>(d0, e0 + o, a0 + o, idesc, accumulate);
+                            umma<SUB, CG>(d1, e0 + o, a1 + o, idesc, accumulate);
+                            umma<SUB, CG>(d1, e1 + o, a0 + o, idesc, 1u);
+                        }
+                        umma_commit<CG>(empty_bar + 8 * s0);
+                        umma_commit<CG>(empty_bar + 8 * s1);
+                        for (int h = 0; h < 2; ++h)
+                            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    }
+                    if (!ok) break;
+                    umma_commit<CG>(tfull_bar + 8 * slot);
+                    umma_commit<CG>(tfull_bar + 8 * (slot ^ 1));
+                    slot_phase ^= 3u;
+                    continue;
+                }
                 for (int job = 0; ok && job < mi.njobs; ++job)
                 for (int seg = 0, nseg = job_segments(mi, job); ok && seg < nseg; ++seg) {
                     ok = mbar_wait(tempty_bar + 8 * slot, ((slot_phase >> slot) & 1u) ^ 1u, abort_flag, p.status);
@@ -1129,6 +1175,12 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     p.stall_producer = take_stall_flag();
     p.status = device_status_word();
     fill_mod_info(p, set, rt, k);
+    // Squares in one K-loop: the products of a square read d0 and e0 twice, so job after job a K chunk costs six tiles;
+    // with both accumulators open it costs four.  The drains of the two slots no longer hide behind each other's K-loop,
+    // which costs less than the tiles at every size measured: 10240 x 64 x 10240 with a kept operator (DRAM) 680 -> 620 us a
+    // call, 131072 x 128 x 4096 9159 -> 8801, 16384 x 16384 x 1024 (power) 11.52 -> 11.10 ms, 4096^3 2371 -> 2358 us.  Not
+    // with K segments, whose accumulators take the slots in turn.
+    p.pair_squares = !rt.native() && p.mod[0].nseg_all == 1;
 
     CUtensorMap mapA, mapB;
     const int planesA = kSetTables.first[set][rt.layout(0)][p.r], planesB = kSetTables.first[set][rt.layout(1)][p.r];
