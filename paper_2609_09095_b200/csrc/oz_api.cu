@@ -453,6 +453,17 @@ oz_status_t check_product_args(int64_t m, int64_t n, int64_t k, double alpha, do
     return OZ_OK;
 }
 
+// Whether the method takes the call (valid arguments, k > 0); asked before anything is enqueued.  `panels`: C travels
+// in column panels.
+bool method_applies(int64_t m, int64_t n, int64_t k, int set, const Route &rt, bool panels)
+{
+    // out-of-range rows on the native path: defined on the norm scan, FP64 reconstruction, one panel
+    if (rt.fallback && (rt.rule != 1 || rt.hosted || panels)) return false;
+    // accurate rule: planes of both operands for the bound product, within its exact depth
+    if (rt.rule == 2 && (rt.fused || k > kBoundKMax)) return false;
+    return !rt.fused || !(rt.fallback || rt.hosted || panels || !fused_gemm_applies(m, n, k, set, rt));
+}
+
 oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const double *A, int64_t lda,
                        const double *B, int64_t ldb, double beta, double *C, int64_t ldc, int set,
                        uint32_t route, cudaStream_t stream, char *ws, size_t ws_bytes,
@@ -465,9 +476,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     if (!A || !B || lda < m || ldb < k || (reinterpret_cast<uintptr_t>(A) & 7u) ||
         (reinterpret_cast<uintptr_t>(B) & 7u))
         return OZ_ERR_INVALID_ARG;
-    // out-of-range rows on the native path: defined on the norm scan, FP64 reconstruction, one panel
-    if (rt.fallback && (rt.rule != 1 || rt.hosted || plan)) return OZ_ERR_UNSUPPORTED;
-    if (rt.fused && rt.rule == 2) return OZ_ERR_UNSUPPORTED;
+    if (!method_applies(m, n, k, set, rt, plan != nullptr)) return OZ_ERR_UNSUPPORTED;
     Layout L = make_layout(m, n, k, set, rt);
     if (!ws || ws_bytes < L.total) return OZ_ERR_WORKSPACE;
     st = ensure_device_ready();
@@ -488,7 +497,6 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         // Accurate mode: exponent scans, one magnitude plane per operand (kept in the first plane slot
         // of each operand, which the conversion overwrites afterwards), the bound product on the
         // tensor cores, the shifts from its row and column maxima, then the conversion as usual.
-        if (k > kBoundKMax) return OZ_ERR_UNSUPPORTED;
         st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, true, stream);
         if (st == OZ_OK) st = launch_scan(1, n, k, B, ldb, set, rt, b.shift, b.scratch, true, stream);
         if (st == OZ_OK) st = launch_bound_plane(0, m, k, A, lda, a.scratch, a.planes, a.pitch, stream);
@@ -510,7 +518,6 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     if (rt.fused) {
         // Storage mode F: only the scan of A runs ahead of the product kernel, which converts A's tiles
         // itself; B is deconstructed as always (side stream); residues in the public layout
-        if (rt.fallback || rt.hosted || plan || !fused_gemm_applies(m, n, k, set, rt)) return OZ_ERR_UNSUPPORTED;
         OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
         OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
         st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
@@ -569,7 +576,6 @@ oz_status_t dgemm_panels(int64_t m, int64_t n, int64_t k, double alpha, const do
                          double *C, int set, const Route &rt, cudaStream_t stream, char *ws, int dev,
                          const PanelPlan &plan, const cudaEvent_t *b_ready)
 {
-    if (!(alpha == 1.0 || alpha == -1.0) || !(beta == 0.0 || beta == 1.0)) return OZ_ERR_UNSUPPORTED;
     const Layout L = make_layout(m, n, k, set, rt);
     oz_status_t st = ensure_device_ready();
     if (st != OZ_OK) return st;
@@ -716,9 +722,6 @@ oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const d
                           double *C_host, int64_t ldc, oz_modset_t set, uint32_t route,
                           void *stream)
 {
-    int dev = 0;
-    OZ_CUDA_CHECK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices) return OZ_ERR_CUDA;
     Route rt;
     if (!valid_set(set) || !decode_route_for_set(set, route, &rt)) return OZ_ERR_INVALID_ARG;
     if (m < 0 || n < 0 || k < 0) return OZ_ERR_INVALID_ARG;
@@ -726,19 +729,10 @@ oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const d
     if (m == 0 || n == 0) return OZ_OK;
     if (!C_host || ldc < m || (k > 0 && (!A_host || !B_host || lda < m || ldb < k)))
         return OZ_ERR_INVALID_ARG;
-    cudaStream_t s = static_cast<cudaStream_t>(stream);
-    char *ws = nullptr;
-    size_t ws_have = 0;
-    registered_workspace(dev, &ws, &ws_have);
+    if (!(alpha == 1.0 || alpha == -1.0) || !(beta == 0.0 || beta == 1.0)) return OZ_ERR_UNSUPPORTED;
     int64_t kk = k > 0 ? k : 1;
-    size_t core = make_layout(m, n, kk, set, rt).total;
     size_t bytesA = 8 * static_cast<size_t>(m) * kk, bytesB = 8 * static_cast<size_t>(kk) * n;
     size_t bytesC = 8 * static_cast<size_t>(m) * n;
-    size_t offA = core, offB = offA + round_up(bytesA, 256), offC = offB + round_up(bytesB, 256);
-    if (!ws || ws_have < offC + bytesC) return OZ_ERR_WORKSPACE;
-    double *dA = reinterpret_cast<double *>(ws + offA);
-    double *dB = reinterpret_cast<double *>(ws + offB);
-    double *dC = reinterpret_cast<double *>(ws + offC);
     // C travels in column panels on two side streams, so that its upload overlaps the computation and the download
     // of a finished panel overlaps the upload of the next ones (PCIe is full duplex).  The caller's stream
     // waits for both side streams before the call's work counts as done on it.  Up to eight panels of at least
@@ -752,6 +746,21 @@ oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const d
     int np = static_cast<int>(undivided ? bytesC >> 26 : (many > few ? (many < kMaxPanels ? many : kMaxPanels) : few));
     if (np > kMaxPanels) np = kMaxPanels;
     if (np > n) np = static_cast<int>(n);
+    if (k > 0 && !method_applies(m, n, k, set, rt, np >= 2)) return OZ_ERR_UNSUPPORTED;
+
+    int dev = 0;
+    OZ_CUDA_CHECK(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevices) return OZ_ERR_CUDA;
+    cudaStream_t s = static_cast<cudaStream_t>(stream);
+    char *ws = nullptr;
+    size_t ws_have = 0;
+    registered_workspace(dev, &ws, &ws_have);
+    size_t core = make_layout(m, n, kk, set, rt).total;
+    size_t offA = core, offB = offA + round_up(bytesA, 256), offC = offB + round_up(bytesB, 256);
+    if (!ws || ws_have < offC + bytesC) return OZ_ERR_WORKSPACE;
+    double *dA = reinterpret_cast<double *>(ws + offA);
+    double *dB = reinterpret_cast<double *>(ws + offB);
+    double *dC = reinterpret_cast<double *>(ws + offC);
     // nothing is created inside a capture for a size that has always been taken undivided
     if (np >= 2 && bytesC < (2ull << 26) && !g_pipe[dev].ready.load()) {
         cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -780,37 +789,48 @@ oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const d
             const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
             return cudaMemcpy2DAsync(dC + j0 * m, 8 * m, C_host + j0 * ldc, 8 * ldc, 8 * m, cols, cudaMemcpyHostToDevice, hp->in);
         };
-        OZ_CUDA_CHECK(cudaEventRecord(hp->start, s));          // the workspace may still be in use on s
-        OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->in, hp->start, 0));
-        OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->out, hp->start, 0));
-        OZ_CUDA_CHECK(cudaMemcpy2DAsync(dA, 8 * m, A_host, 8 * lda, 8 * m, k, cudaMemcpyHostToDevice, hp->in));
-        if (!by_panel) OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB, 8 * k, B_host, 8 * ldb, 8 * k, n, cudaMemcpyHostToDevice, hp->in));
-        OZ_CUDA_CHECK(cudaEventRecord(hp->ab, hp->in));
-        // B runs one panel ahead of C, so that a panel's products are ready when its old C arrives
-        for (int p = 0; p <= np; ++p) {
-            if (by_panel && p < np) {
+        auto enqueue = [&]() -> oz_status_t {
+            OZ_CUDA_CHECK(cudaEventRecord(hp->start, s));          // the workspace may still be in use on s
+            OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->in, hp->start, 0));
+            OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->out, hp->start, 0));
+            OZ_CUDA_CHECK(cudaMemcpy2DAsync(dA, 8 * m, A_host, 8 * lda, 8 * m, k, cudaMemcpyHostToDevice, hp->in));
+            if (!by_panel) OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB, 8 * k, B_host, 8 * ldb, 8 * k, n, cudaMemcpyHostToDevice, hp->in));
+            OZ_CUDA_CHECK(cudaEventRecord(hp->ab, hp->in));
+            // B runs one panel ahead of C, so that a panel's products are ready when its old C arrives
+            for (int p = 0; p <= np; ++p) {
+                if (by_panel && p < np) {
+                    const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
+                    OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB + j0 * k, 8 * k, B_host + j0 * ldb, 8 * ldb, 8 * k, cols, cudaMemcpyHostToDevice, hp->in));
+                    OZ_CUDA_CHECK(cudaEventRecord(hp->b[p], hp->in));
+                }
+                if (beta != 0.0 && p > 0) {
+                    OZ_CUDA_CHECK(upload_c(p - 1));
+                    OZ_CUDA_CHECK(cudaEventRecord(hp->c[p - 1], hp->in));
+                }
+            }
+            OZ_CUDA_CHECK(cudaStreamWaitEvent(s, hp->ab, 0));
+            const oz_status_t product =
+                by_panel ? dgemm_panels(m, n, k, alpha, dA, dB, beta, dC, set, rt, s, ws, dev, plan, hp->b)
+                         : dgemm_impl(m, n, k, alpha, dA, m, dB, kk, beta, dC, m, set, route, s, ws, core, &plan);
+            if (product != OZ_OK) return product;
+            for (int p = 0; p < np; ++p) {
                 const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
-                OZ_CUDA_CHECK(cudaMemcpy2DAsync(dB + j0 * k, 8 * k, B_host + j0 * ldb, 8 * ldb, 8 * k, cols, cudaMemcpyHostToDevice, hp->in));
-                OZ_CUDA_CHECK(cudaEventRecord(hp->b[p], hp->in));
+                OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->out, hp->r[p], 0));
+                OZ_CUDA_CHECK(cudaMemcpy2DAsync(C_host + j0 * ldc, 8 * ldc, dC + j0 * m, 8 * m, 8 * m, cols,
+                                                cudaMemcpyDeviceToHost, hp->out));
             }
-            if (beta != 0.0 && p > 0) {
-                OZ_CUDA_CHECK(upload_c(p - 1));
-                OZ_CUDA_CHECK(cudaEventRecord(hp->c[p - 1], hp->in));
-            }
+            OZ_CUDA_CHECK(cudaEventRecord(hp->done, hp->out));
+            OZ_CUDA_CHECK(cudaStreamWaitEvent(s, hp->done, 0));
+            return OZ_OK;
+        };
+        st = enqueue();
+        if (st != OZ_OK) {
+            // the copies that are under way read the caller's buffers and write the workspace: whatever follows on the
+            // caller's stream comes after them (and a capture finds its fork joined)
+            if (cudaEventRecord(hp->ab, hp->in) == cudaSuccess) cudaStreamWaitEvent(s, hp->ab, 0);
+            if (cudaEventRecord(hp->done, hp->out) == cudaSuccess) cudaStreamWaitEvent(s, hp->done, 0);
         }
-        OZ_CUDA_CHECK(cudaStreamWaitEvent(s, hp->ab, 0));
-        if (by_panel) st = dgemm_panels(m, n, k, alpha, dA, dB, beta, dC, set, rt, s, ws, dev, plan, hp->b);
-        else st = dgemm_impl(m, n, k, alpha, dA, m, dB, kk, beta, dC, m, set, route, s, ws, core, &plan);
-        if (st != OZ_OK) return st;
-        for (int p = 0; p < np; ++p) {
-            const int64_t j0 = plan.col0[p], cols = plan.col0[p + 1] - j0;
-            OZ_CUDA_CHECK(cudaStreamWaitEvent(hp->out, hp->r[p], 0));
-            OZ_CUDA_CHECK(cudaMemcpy2DAsync(C_host + j0 * ldc, 8 * ldc, dC + j0 * m, 8 * m, 8 * m, cols,
-                                            cudaMemcpyDeviceToHost, hp->out));
-        }
-        OZ_CUDA_CHECK(cudaEventRecord(hp->done, hp->out));
-        OZ_CUDA_CHECK(cudaStreamWaitEvent(s, hp->done, 0));
-        return OZ_OK;
+        return st;
     }
     if (k > 0) {
         OZ_CUDA_CHECK(cudaMemcpy2DAsync(dA, 8 * m, A_host, 8 * lda, 8 * m, k, cudaMemcpyHostToDevice, s));

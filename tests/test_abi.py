@@ -112,3 +112,27 @@ def test_prepared_operand_sizes():
     assert oz.oz_workspace_bytes(m, n, k, oz.OZ_SET_S, 0) == a + b + r
     # ragged shapes are stored as whole tiles
     assert oz.oz_product_workspace_bytes(10007, 9973, oz.OZ_SET_S) == 24 * 10240 * 9984
+
+
+def test_refused_host_calls_are_refused_before_any_cuda_call():
+    """What oz_dgemm_host does not take is found on the host before a device is even looked up (so this runs without a
+    GPU; the addresses are never dereferenced): no copy is left running behind the caller's back."""
+    base = 0x7F0000000000
+
+    def host(m, n, k, alpha=1.0, beta=0.0, route=0, set_id=oz.OZ_SET_S):
+        return oz.oz_dgemm_host(m, n, k, alpha, base, max(m, 1), base, max(k, 1), beta, base, max(m, 1), set_id, route, 0)
+
+    for m, n, k in ((40, 30, 20), (1500, 1400, 64), (6000, 6000, 64), (40, 30, 0)):      # undivided and in panels
+        assert host(m, n, k, alpha=2.0, beta=1.0) == oz.OZ_ERR_UNSUPPORTED
+        assert host(m, n, k, beta=0.5) == oz.OZ_ERR_UNSUPPORTED
+    # accurate rule beyond the exact depth of its bound product
+    assert host(1500, 1400, 16385, route=oz.OZ_SCALE_ACCURATE) == oz.OZ_ERR_UNSUPPORTED
+    # row check off its scale rule, or with C in panels
+    assert host(40, 30, 20, route=oz.OZ_FALLBACK_FP64 | oz.OZ_SCALE_MAXEXP) == oz.OZ_ERR_UNSUPPORTED
+    assert host(6000, 6000, 64, route=oz.OZ_FALLBACK_FP64) == oz.OZ_ERR_UNSUPPORTED
+    # storage mode F beyond its one tile of columns, beyond its depth, with C in panels
+    assert host(1500, 1400, 64, route=oz.OZ_STORAGE_FUSED) == oz.OZ_ERR_UNSUPPORTED
+    assert host(1500, 100, 4098, route=oz.OZ_STORAGE_FUSED) == oz.OZ_ERR_UNSUPPORTED
+    assert host(200000, 100, 64, route=oz.OZ_STORAGE_FUSED) == oz.OZ_ERR_UNSUPPORTED
+    # nothing to do stays nothing to do
+    assert host(0, 30, 20, alpha=2.0) == oz.OZ_OK

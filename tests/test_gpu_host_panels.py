@@ -58,3 +58,27 @@ def test_host_routes_taken_undivided():
         want, st = gh.dgemm(A, B, "S", gh.route("fp8"))
         assert gh.sync_status() == st == 0
         assert (hC.numpy().T == want).all()
+
+
+def test_refused_call_leaves_nothing_behind():
+    """A host call that is refused enqueues no copy: the device call that follows at once in the same workspace has its
+    planes and residues to itself."""
+    import torch
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(8)
+    m, n, k, S = 1500, 1400, 64, oz.OZ_SET_S
+    rt, accurate = gh.route("fp8"), gh.route("fp8", "RN", "ACCURATE")
+    hA, hB, hC = (torch.full(shape, 3.0, dtype=torch.float64).pin_memory() for shape in ((k, m), (n, k), (n, m)))
+    A, B = np.asfortranarray(rng.standard_normal((m, 900))), np.asfortranarray(rng.standard_normal((900, n)))
+    gh.ensure_workspace(oz.oz_workspace_bytes(m, n, 900, S, rt) + 8 * (m * k + k * n + m * n) + 1024)
+    want, _ = gh.dgemm(A, B, "S", rt)
+    dA, dB, dC = gh.to_dev(A), gh.to_dev(B), torch.zeros((n, m), dtype=torch.float64, device="cuda")
+    for _ in range(4):
+        before = oz.oz_launch_count()
+        assert oz.oz_dgemm_host(m, n, k, 2.0, hA, m, hB, k, 1.0, hC, m, S, rt) == oz.OZ_ERR_UNSUPPORTED
+        assert oz.oz_dgemm_host(m, n, 16385, 1.0, hA, m, hB, 16385, 1.0, hC, m, S, accurate) == oz.OZ_ERR_UNSUPPORTED
+        assert oz.oz_launch_count() == before
+        oz.check(oz.oz_dgemm_ex(m, n, 900, 1.0, dA, m, dB, 900, 0.0, dC, m, S, rt), "oz_dgemm_ex")
+    assert gh.sync_status() == 0
+    assert (gh.from_dev(dC) == want).all() and bool((hC == 3.0).all())
