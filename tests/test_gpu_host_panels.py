@@ -82,3 +82,24 @@ def test_refused_call_leaves_nothing_behind():
         oz.check(oz.oz_dgemm_ex(m, n, 900, 1.0, dA, m, dB, 900, 0.0, dC, m, S, rt), "oz_dgemm_ex")
     assert gh.sync_status() == 0
     assert (gh.from_dev(dC) == want).all() and bool((hC == 3.0).all())
+
+
+@pytest.mark.parametrize("which", ["ABC", "B", "C"])
+def test_pageable_buffers_are_not_cut_up(which):
+    """Copies of pageable memory overlap nothing: such a call is the device call between its copies, kernel for kernel."""
+    import torch
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(12)
+    m, n, k, S, rt = 1500, 1401, 300, oz.OZ_SET_S, gh.route("fp8")
+    A, B, C0 = (np.asfortranarray(rng.standard_normal(shape)) for shape in ((m, k), (k, n), (m, n)))
+    gh.ensure_workspace(oz.oz_workspace_bytes(m, n, k, S, rt) + 8 * (m * k + k * n + m * n) + 1024)
+    host = {name: torch.from_numpy(np.ascontiguousarray(X.T)) for name, X in (("A", A), ("B", B), ("C", C0))}
+    host = {name: t if name in which else t.pin_memory() for name, t in host.items()}
+    before = oz.oz_launch_count()
+    want, st = gh.dgemm(A, B, "S", rt, -1.0, 1.0, C0)
+    undivided = oz.oz_launch_count() - before
+    oz.check(oz.oz_dgemm_host(m, n, k, -1.0, host["A"], m, host["B"], k, 1.0, host["C"], m, S, rt), "oz_dgemm_host")
+    assert gh.sync_status() == st == 0
+    assert oz.oz_launch_count() - before == 2 * undivided
+    assert (host["C"].numpy().T == want).all()
