@@ -79,3 +79,36 @@ def test_joint_deconstruction_shapes(m, n, k, set_name, sub):
     assert (got == gh.from_dev(dC)).all()
     if m * n <= 200000:
         assert (got == ozo.dgemm(A, B, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS)).all()
+
+
+@pytest.mark.parametrize("lines,k", [
+    (42001, 100),               # one piece of a line per row of a conversion tile
+    (33001, 130),               # two, the second one cut off by the row pitch
+    (703, 6001),                # 47 pieces a line: tiles start in the middle of lines, the last one is partly empty
+    (3, 33000),                 # fewer rows than resident tiles
+])
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("E", "int8"), ("A", "int8n")])
+def test_three_pass_deconstruction_of_columns(lines, k, set_name, sub):
+    """Columns too long or too many for the one-kernel form, planes in the documented layout: sampled lines are the
+    oracle's, and all bytes are those of the same columns deconstructed a few at a time."""
+    import torch
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(lines + k)
+    X = np.asfortranarray(rng.standard_normal((k, lines)))
+    X[:, lines // 2] = 0.0
+    X[k // 2, 1] = np.inf
+    rt = gh.route(sub)
+    got, shift, st = gh.deconstruct(1, X, set_name, rt)
+    assert st != 0 and shift[1] == -2 ** 31 and (got[:, 1] == 0).all()
+    pick = np.unique(np.array([0, 2 % lines, lines // 3, lines // 2, max(lines - 2, 0), lines - 1]))
+    pick = pick[pick != 1]
+    Y = np.asfortranarray(X[:, pick])
+    want_shift = ozo.shifts(1, Y, OSET[set_name], ozo.SCALE_CS, 0)
+    Q = ozo.quantise(1, Y, want_shift, ozo.QUANT_RN)
+    D = ozo.residues(Q, OSET[set_name])
+    assert (shift[pick] == want_shift).all()
+    assert (got[:, pick] == ozo.planes(D, OSET[set_name], OSUB[sub])).all()
+    step = max(1, min(lines, 2 ** 20 // k))
+    for a in range(0, lines, step):
+        part, part_shift, _ = gh.deconstruct(1, np.asfortranarray(X[:, a:a + step]), set_name, rt)
+        assert (shift[a:a + step] == part_shift).all() and (got[:, a:a + step] == part).all()
