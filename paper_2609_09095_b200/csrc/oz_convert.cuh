@@ -137,10 +137,12 @@ __device__ __forceinline__ float2 residue_pair(const Limbs<NP> &L, int q)
     return __ffma2_rn(quot, dup(-static_cast<float>(m)), v);
 }
 
+// One word of the table, which is written once, before a block barrier.  Free to move otherwise: the caller's address has
+// to depend on something that is read behind that barrier (elements from shared memory, or the table's own address).
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
 {
     uint32_t v;
-    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));      // the table is written once, before a block barrier
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
 }
 

@@ -136,6 +136,9 @@ fused_gemm_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constan
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_base_ptr;
+    // the elements of A come from global memory: the table's address is what keeps the look-ups behind the barrier
+    uint32_t table = lut_addr;
+    asm volatile("" : "+r"(table)::"memory");
 
     // planes of pass g: [first, first + count) in both operands' plane order (same counts on both sides)
     auto pass_first_plane = [&](int g) { return p.mod[g * F_GROUP].planeA0; };
@@ -346,10 +349,10 @@ fused_gemm_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constan
                     if (!ok) break;
                     uint8_t *out = ring_gen + stage * F_STAGE + (h * F_LINES + r) * 16 + kq * 4;
                     switch (g) {
-                    case 0: convert_pass<SET, LAYOUT_A, 0>(L, lut_addr, out); break;
-                    case 1: convert_pass<SET, LAYOUT_A, 1>(L, lut_addr, out); break;
-                    case 2: convert_pass<SET, LAYOUT_A, 2>(L, lut_addr, out); break;
-                    default: convert_pass<SET, LAYOUT_A, 3>(L, lut_addr, out); break;
+                    case 0: convert_pass<SET, LAYOUT_A, 0>(L, table, out); break;
+                    case 1: convert_pass<SET, LAYOUT_A, 1>(L, table, out); break;
+                    case 2: convert_pass<SET, LAYOUT_A, 2>(L, table, out); break;
+                    default: convert_pass<SET, LAYOUT_A, 3>(L, table, out); break;
                     }
                     // the tensor core reads shared memory through the asynchronous proxy
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
