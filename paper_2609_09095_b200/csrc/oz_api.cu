@@ -253,6 +253,9 @@ oz_status_t ensure_device_ready()
     if (st != OZ_OK) return st;
     st = upload_hosted_constants();
     if (st != OZ_OK) return st;
+    // A copy from pageable memory may return before it has arrived, and the first kernels may be on a stream that does not wait
+    // for the default one (they also read the tables before they wait for anything).
+    OZ_CUDA_CHECK(cudaStreamSynchronize(nullptr));
     g_ready[dev] = true;
     return OZ_OK;
 }
