@@ -131,8 +131,8 @@ typedef enum { OZ_SET_S = 0, OZ_SET_E = 1, OZ_SET_A = 2 } oz_modset_t;
  * which every row fails runs far below the emulated rate -- as the paper says, the fallback does not
  * accelerate.  OZ_ERR_RANGE is still reported (informational).  oz_query_fallback_rows() returns how
  * many rows were re-issued.  Needs OZ_SCALE_CS (the check is defined on its scan); not combined with
- * OZ_RECON_TENSOR; OZ_ERR_UNSUPPORTED from oz_dgemm_host and oz_dgemm_prepared; ignored by the stage
- * entry points.  Workspace: oz_workspace_bytes() with the same route (5 m + 768 bytes more). */
+ * OZ_RECON_TENSOR; OZ_ERR_UNSUPPORTED from oz_dgemm_prepared, and from oz_dgemm_host with 128 MiB of C or
+ * more; ignored by the stage entry points.  Workspace: oz_workspace_bytes() with the same route (5 m + 768 bytes more). */
 #define OZ_FALLBACK_FP64 0x8000u
 
 /* Storage mode F for tall-skinny products (Sec. "Storage Modes", mode F; "O4: pipelining"): the planes
@@ -143,8 +143,8 @@ typedef enum { OZ_SET_S = 0, OZ_SET_E = 1, OZ_SET_A = 2 } oz_modset_t;
  * result, bit for bit.  Applies when n <= 128, the substrate is FP8 or INT8 digits (merged schedule,
  * which the bit implies), and k is within the exact depth of one accumulator (k <= 4097 on set S,
  * 15420 on sets E and A for FP8; 262144 for INT8 digits); OZ_ERR_UNSUPPORTED otherwise, and with
- * OZ_SCALE_ACCURATE, OZ_RECON_TENSOR, OZ_FALLBACK_FP64, oz_dgemm_host and oz_dgemm_prepared.  Ignored by
- * the stage entry points. */
+ * OZ_SCALE_ACCURATE, OZ_RECON_TENSOR, OZ_FALLBACK_FP64, from oz_dgemm_prepared, and from oz_dgemm_host with
+ * 128 MiB of C or more.  Ignored by the stage entry points. */
 #define OZ_STORAGE_FUSED 0x10000u
 
 #define OZ_K_MAX 1048576
@@ -196,11 +196,17 @@ oz_status_t oz_dgemm_ex(int64_t m, int64_t n, int64_t k, double alpha, const dou
  * pageable memory do not overlap anything).  The operands are copied to staging areas inside the
  * registered workspace, which must hold oz_workspace_bytes() + 8 (m k + k n + m n) bytes, and C is
  * copied back; the call returns after enqueueing (the host buffers must stay valid until the stream
- * has drained).  When C is 128 MiB or more it travels in up to 16 column panels on two internal
- * streams: its upload overlaps the deconstruction and the residue GEMMs, and each panel is downloaded
- * while later ones are still uploaded and reconstructed.  `stream` waits for those internal streams,
- * so work enqueued on it afterwards, or a synchronisation of it, sees the finished C.  The internal
- * streams and events are created on a device's first such call (not inside a stream capture). */
+ * has drained).  From 8 MiB of traffic (B once, C once, or twice with beta = 1) the call is cut into up
+ * to 16 column panels on two internal copy streams.  With 512 columns or more, and not under
+ * OZ_SCALE_ACCURATE (whose shifts of A need all of B), the product itself runs panel by panel: a panel's columns
+ * of B and of the old C are uploaded, deconstructed, multiplied and downloaded while the next ones travel;
+ * otherwise C alone is uploaded, reconstructed and downloaded in panels.  With a pageable buffer, and on the two
+ * routes that take the undivided product only (OZ_FALLBACK_FP64, OZ_STORAGE_FUSED), panels start at
+ * 128 MiB of C and hold C alone -- where those two routes return OZ_ERR_UNSUPPORTED.  `stream` waits for the
+ * internal streams, so work enqueued on it afterwards, or a synchronisation of it, sees the finished C; also
+ * after an error, when what was enqueued before it still runs.  The copy streams and their events
+ * are created on a device's first call in panels: make it outside a stream capture.  (A captured call with less than 128 MiB
+ * of C that finds none takes the undivided product on `stream` instead.) */
 oz_status_t oz_dgemm_host(int64_t m, int64_t n, int64_t k, double alpha, const double *A_host,
                           int64_t lda, const double *B_host, int64_t ldb, double beta,
                           double *C_host, int64_t ldc, oz_modset_t set, uint32_t route,
@@ -313,8 +319,9 @@ oz_status_t oz_query_fallback_rows(void *stream, int64_t *rows);
  * oz_dgemm / oz_dgemm_ex / oz_dgemm_prepared record them on the call's stream: [0] before the
  * first kernel, [1] after the deconstruction of A, [2] once the deconstruction of B -- which runs
  * next to A's on an internal stream that forks from and joins the call's stream -- has finished
- * too, [3] after the residue GEMMs, [4] after the reconstruction.  The handles are copied; the
- * caller owns the events. */
+ * too, [3] after the residue GEMMs, [4] after the reconstruction.  oz_dgemm_host records them as well; where
+ * it runs the product panel by panel, [1] follows the deconstruction of A, and [2] to [4] are those of the last
+ * panel, so that [1] to [2] holds all earlier panels.  The handles are copied; the caller owns the events. */
 oz_status_t oz_set_stage_events(void *const *events);
 
 /* Number of kernels launched by the library on this process since load (for benchmarks). */

@@ -532,8 +532,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][2], stream));
         const int64_t ldr = round_up(m, 64);
-        st = launch_fused_gemm(m, n, k, A, lda, a.shift, b.planes, b.stride, b.pitch, set, rt, ws + L.R, ldr, n * ldr,
-                               stream);
+        st = launch_fused_gemm(m, n, k, A, lda, a.shift, b.planes, b.pitch, set, rt, ws + L.R, ldr, n * ldr, stream);
         if (st != OZ_OK) return st;
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][3], stream));
         st = launch_reconstruct(m, n, ws + L.R, ldr, n * ldr, a.shift, b.shift, set, alpha, beta, C, ldc, stream);

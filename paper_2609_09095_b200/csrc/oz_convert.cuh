@@ -1,6 +1,7 @@
-// Conversion of quantised FP64 elements into plane bytes (Algorithm 2: residues of every modulus from
-// the 16-bit limbs of the integer, digit split and plane codes by table look-up), shared by the
-// deconstruction kernels and by the product kernel that converts its A operand on the fly.
+// Conversion of FP64 elements into plane bytes (Algorithm 2): the quantised integer in four balanced FP32 limbs,
+// residues of every modulus from packed multiply-adds on them, digits by one more rounded division (odd squares) or
+// from a small table (powers of two and non-squares).  Shared by the deconstruction kernels and by the product
+// kernel that converts its A operand on the fly.
 // Internal to liboz_b200.so; every function is device-inline and lives in the including file's
 // anonymous namespace.
 #pragma once

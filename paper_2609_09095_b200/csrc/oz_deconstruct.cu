@@ -6,7 +6,8 @@
 //   scan_maxexp    largest floor(log2|x|) of every line, Inf/NaN detection
 //   scan_sumsq     CS rule only: exact integer sum of ceil(|x| 2^(9-E))^2 per line
 //   scan_finalize  shift[line] (sigma_i or tau_j of Eq. 1)
-//   convert        quantise, reduce modulo every modulus, look the plane bytes up, store
+//   convert        quantise, reduce modulo every modulus, split into digits, store the planes
+// Small operands take one kernel instead of the five, both operands of a product together where they fit.
 //
 // The scan is split over the inner dimension with integer atomics (max / or / add), so its
 // result does not depend on the order of the partial results: the shifts are bit-reproducible.
@@ -383,8 +384,6 @@ bound_plane_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int
 __global__ void accurate_finalize_kernel(ScanScratch s, int64_t lines, int L, int32_t *shift,
                                          unsigned int *status)
 {
-    dependency_release();
-    dependency_wait();
     dependency_release();
     dependency_wait();
     int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;

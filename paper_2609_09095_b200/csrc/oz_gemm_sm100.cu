@@ -540,24 +540,24 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 const ModInfo &mi = p.mod[it.mod];
                 // one stage: 128 bytes of K of plane pa of A and pb of B
                 auto load = [&](int pa, int pb, int kc) {
-                            if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) return false;
-                            uint32_t fb = full_bar + 8 * stage;
-                            uint32_t sa = tiles + stage * STAGE_BYTES;
-                            if (CG == 1) {
-                                mbar_expect_tx(fb, STAGE_BYTES);
-                                tma_load_3d(sa, &mapB, fb, kc * p.kc_x, it.tn * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
-                                tma_load_3d(sa + A_BYTES, &mapA, fb, kc * p.kc_x, it.tm * BLOCK_N, pa * p.plane_z + kc * p.kc_z);
-                            } else {
-                                // both CTAs' copies complete on the leader's barrier
-                                if (rank == 0) mbar_expect_tx(fb, 2 * STAGE_BYTES);
-                                const uint32_t fb_leader = map_to_cta(fb, 0);
-                                tma_load_3d_pair(sa, &mapB, fb_leader, kc * p.kc_x,
-                                                 it.tn * Tile<CG>::TILE_J + static_cast<int>(rank) * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
-                                tma_load_3d_pair(sa + A_BYTES, &mapA, fb_leader, kc * p.kc_x,
-                                                 it.tm * BLOCK_N + static_cast<int>(rank) * Tile<CG>::B_LINES, pa * p.plane_z + kc * p.kc_z);
-                            }
-                            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-                            return true;
+                    if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) return false;
+                    uint32_t fb = full_bar + 8 * stage;
+                    uint32_t sa = tiles + stage * STAGE_BYTES;
+                    if (CG == 1) {
+                        mbar_expect_tx(fb, STAGE_BYTES);
+                        tma_load_3d(sa, &mapB, fb, kc * p.kc_x, it.tn * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
+                        tma_load_3d(sa + A_BYTES, &mapA, fb, kc * p.kc_x, it.tm * BLOCK_N, pa * p.plane_z + kc * p.kc_z);
+                    } else {
+                        // both CTAs' copies complete on the leader's barrier
+                        if (rank == 0) mbar_expect_tx(fb, 2 * STAGE_BYTES);
+                        const uint32_t fb_leader = map_to_cta(fb, 0);
+                        tma_load_3d_pair(sa, &mapB, fb_leader, kc * p.kc_x,
+                                         it.tn * Tile<CG>::TILE_J + static_cast<int>(rank) * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
+                        tma_load_3d_pair(sa + A_BYTES, &mapA, fb_leader, kc * p.kc_x,
+                                         it.tm * BLOCK_N + static_cast<int>(rank) * Tile<CG>::B_LINES, pa * p.plane_z + kc * p.kc_z);
+                    }
+                    if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                    return true;
                 };
                 if (!DIRECT && p.pair_squares && mi.kind == 0) {
                     // the two planes of a chunk in two stages, side by side
@@ -1233,8 +1233,8 @@ bool fused_gemm_applies(int64_t m, int64_t n, int64_t k, int set, const Route &r
 // B's planes materialised in the layout of side 1 of the route; canonical residues in the public layout
 // R[mod][j][ldr], ldr a multiple of 64 and at least m rounded up to 64 (the last tile stores whole).
 oz_status_t launch_fused_gemm(int64_t m, int64_t n, int64_t k, const double *A, int64_t lda, const int32_t *shiftA,
-                              const uint8_t *PB, int64_t strideB, int64_t pitchB, int set, const Route &rt,
-                              void *R, int64_t ldr, int64_t mod_stride, cudaStream_t stream)
+                              const uint8_t *PB, int64_t pitchB, int set, const Route &rt, void *R, int64_t ldr,
+                              int64_t mod_stride, cudaStream_t stream)
 {
     if (!fused_gemm_applies(m, n, k, set, rt)) return OZ_ERR_UNSUPPORTED;
     if (ldr % F_LINES != 0 || ldr < round_up(m, F_LINES) || (reinterpret_cast<uintptr_t>(R) & 15u)) return OZ_ERR_INVALID_ARG;

@@ -182,8 +182,8 @@ struct PlaneGeom {
 inline PlaneGeom public_planes(int64_t plane_stride, int64_t row_pitch) { return {plane_stride, row_pitch, row_pitch, 128}; }
 inline PlaneGeom private_planes(int64_t lines, int64_t pitch) { return {lines * pitch, pitch, 128, 128 * lines}; }
 
-// `alone`: no other chain of kernels runs beside this one (see launch_if())
 // ---- stage launchers (host side of each .cu) ---------------------------------------------
+// `alone`: no other chain of kernels runs beside this one (see launch_if())
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
                                int32_t *shift, void *scratch, bool alone, cudaStream_t stream);
@@ -203,8 +203,6 @@ struct ResidueTiling {
 };
 ResidueTiling residue_tiling(int64_t m, int64_t n, int set);
 
-// loose: residues in [0, 2 m_i) (two-byte sets); tiled: R is the tile-ordered private array (ldr and
-// mod_stride are then ignored) and the planes are in the private layout
 // Both operands of a product in one launch, when the one-kernel form takes both (*taken says whether it did);
 // otherwise nothing is launched
 struct OperandJob {
@@ -240,6 +238,8 @@ int accurate_budget_log2(int set);
 // exponent-span check: threshold of the set against the product of the two operands' flatness codes
 unsigned int esc_threshold(int set);
 
+// loose: residues in [0, 2 m_i) (two-byte sets); tiled: R is the tile-ordered private array (ldr and
+// mod_stride are then ignored) and the planes are in the private layout
 oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA,
                                 int64_t strideA, int64_t pitchA, const uint8_t *PB,
                                 int64_t strideB, int64_t pitchB, int set, const Route &rt,
@@ -250,7 +250,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
 // schedule on digit planes, k within the exact depth of one accumulator); public residue layout
 bool fused_gemm_applies(int64_t m, int64_t n, int64_t k, int set, const Route &rt);
 oz_status_t launch_fused_gemm(int64_t m, int64_t n, int64_t k, const double *A, int64_t lda, const int32_t *shiftA,
-                              const uint8_t *PB, int64_t strideB, int64_t pitchB, int set, const Route &rt,
+                              const uint8_t *PB, int64_t pitchB, int set, const Route &rt,
                               void *R, int64_t ldr, int64_t mod_stride, cudaStream_t stream);
 
 // reconstruction from the tile-ordered array, columns [col0, col1) of the m x n output
@@ -287,9 +287,9 @@ oz_status_t launch_native_rows(int64_t m, int64_t n, int64_t k, const double *A,
 // ---- launching ---------------------------------------------------------------------------
 // The kernels of a call are launched as programmatic dependents of their predecessors on the stream: their blocks may
 // become resident, and set up what needs no global memory, while the predecessor's last blocks run.  In return every
-// kernel executes dependency_wait() before its first access to global memory and on every path (so
-// that its own completion implies its predecessor's), and lets its successor in with dependency_release() at
-// once.  256^3: 22.9 -> 19.0 us of GPU time a call together with the joint deconstruction of both operands.
+// kernel executes dependency_wait() on every path (so that its own completion implies its predecessor's) and before its
+// first access to global memory, but for the tables that ensure_device_ready() has put there before any launch, and
+// lets its successor in with dependency_release() at once.  256^3: 22.9 -> 19.0 us of GPU time a call together with the joint deconstruction of both operands.
 #ifdef __CUDACC__
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void dependency_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
