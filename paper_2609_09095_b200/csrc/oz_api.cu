@@ -580,6 +580,8 @@ oz_status_t dgemm_panels(int64_t m, int64_t n, int64_t k, double alpha, const do
 {
     const Layout L = make_layout(m, n, k, set, rt);
     oz_status_t st = ensure_device_ready();
+    // not used here, but a device's first whole-method call creates it for the later ones
+    if (st == OZ_OK) st = ensure_side_stream(dev);
     if (st != OZ_OK) return st;
     const OperandView a = operand_view(ws + L.offA, L.A), b = operand_view(ws + L.offB, L.B);
     const bool ev = g_stage_events_on[dev];
