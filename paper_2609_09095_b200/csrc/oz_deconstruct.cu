@@ -435,10 +435,15 @@ __device__ __forceinline__ void copy16(uint32_t dst, const double *src, int byte
 // A block takes tiles of 16 lines x 128 inner indices through shared memory (on side 0 that is the
 // transposition: loads run along the lines, plane stores along k) and a thread converts eight consecutive
 // elements of one line, so that half a warp stores 128 contiguous bytes of every plane.  The next tile's
-// elements are copied asynchronously while this one is converted.  Whole deconstruction of a 32768 x 4096
-// operand, integer limbs and a table for every modulus before -> now: native residues 1.77 -> 1.23 ms (side 0), 1.37 -> 1.06
-// (side 1); set S on FP8 1.76 -> 1.62 and 1.50 -> 1.52, where the 30 planes' scattered 128-byte writes (3.3 TB/s) bound it.
-template <int SET, int SIDE, int LAYOUT>
+// elements are copied asynchronously while this one is converted.  BY_LINE (side 1, planes kept line by line): the 16 rows
+// of a tile are consecutive 128-element pieces of a line, and of the next lines behind it, so that a tile stores 2 KiB at
+// a time in that layout too.
+// Bound: instruction issue (57 % of the slots busy at 8192 x 1024, set S) and, line by line on side 0, the planes' scattered
+// 128-byte writes.  Whole deconstruction of a 32768 x 4096 operand, integer limbs and a table for every modulus before -> now,
+// planes K chunk by K chunk: native residues 1.76 -> 1.19 ms (side 0), 1.37 -> 1.04 (side 1), set S on FP8 1.76 -> 1.39 and
+// 1.50 -> 1.28; planes line by line, set S: 1.76 -> 1.61 and 1.49 -> 1.23 (1.51 with 16 lines a tile).  Native residues take 16 lines a
+// tile in both layouts (1.04 and 1.05; 1.06 by lines).
+template <int SET, int SIDE, int LAYOUT, bool BY_LINE>
 __global__ void __launch_bounds__(kConvThreads, 3)
 convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
                const int32_t *__restrict__ shift, const uint32_t *__restrict__ lut_global,
@@ -459,30 +464,39 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
     // work items are numbered in 32 bits (checked on the host): cheap division
     const uint32_t nchunks = static_cast<uint32_t>((row_pitch + kChunk - 1) / kChunk);
     const uint32_t ltiles = static_cast<uint32_t>((lines + kTileLines - 1) / kTileLines);
-    const bool by_line = SIDE == 1 && geom.line_stride != kChunk;
-    const uint32_t items = by_line ? (static_cast<uint32_t>(lines) * nchunks + kTileLines - 1) / kTileLines : ltiles * nchunks;
+    const uint32_t items = BY_LINE ? (static_cast<uint32_t>(lines) * nchunks + kTileLines - 1) / kTileLines : ltiles * nchunks;
     const bool pairs = SIDE == 1 && (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
 
-    // line and first inner index of row `l` of a tile.  Side 0: neighbouring blocks take neighbouring lines; side 1:
-    // neighbouring inner indices; side 1 with planes kept line by line: the 16 rows are consecutive pieces of a line, and of
-    // the next lines behind it, so that a tile stores 2 KiB at a time there too (20000 columns of 2048, set S: 398 us in all,
-    // 470 with 16 lines a tile; 460 when a warp took four bytes a lane of 128 inner indices).
-    auto place = [&](uint32_t item, int l, int64_t &line, int64_t &k0) {
-        const uint32_t unit = by_line ? item * kTileLines + l : item;
-        const uint32_t q = unit / (SIDE == 0 ? ltiles : nchunks), rest = unit - q * (SIDE == 0 ? ltiles : nchunks);
-        line = by_line ? q : static_cast<int64_t>(SIDE == 0 ? rest : q) * kTileLines + l;
+    // first line and inner index of a tile (BY_LINE: of this warp's two rows).  Side 0: neighbouring blocks take
+    // neighbouring lines; side 1: neighbouring inner indices
+    auto place = [&](uint32_t item, int64_t &line0, int64_t &k0) {
+        if constexpr (BY_LINE) {
+            const uint32_t row = item * kTileLines + 2 * warp, q = row / nchunks;
+            line0 = q;
+            k0 = static_cast<int64_t>(row - q * nchunks) * kChunk;
+            return;
+        }
+        const uint32_t q = item / (SIDE == 0 ? ltiles : nchunks), rest = item - q * (SIDE == 0 ? ltiles : nchunks);
+        line0 = static_cast<int64_t>(SIDE == 0 ? rest : q) * kTileLines;
         k0 = static_cast<int64_t>(SIDE == 0 ? q : rest) * kChunk;
     };
+    // BY_LINE: to the row behind that one, the next piece of the line or the first of the next line
+    auto next_row = [&](int64_t &line, int64_t &k0) {
+        k0 += kChunk;
+        if (k0 >= row_pitch) {
+            k0 = 0;
+            ++line;
+        }
+    };
     auto request = [&](uint32_t item, int buf) {
-        int64_t line, k0;
-        // elements of a row: <= 0 where there is only padding
-        auto left_of = [&] { return static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk); };
+        int64_t line0, k0;
+        place(item, line0, k0);
+        int kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);        // <= 0: padding only
         const uint32_t base = tile_addr + buf * (kTileDoubles * 8);
         if (SIDE == 0) {
             // 16 lanes take the lines of one inner index, a warp two indices at a time
             const int l = lane & 15;
-            place(item, l, line, k0);
-            const int kleft = left_of();
+            const int64_t line = line0 + l;
             const bool live = line < lines && shift[line] != OZ_NONFINITE_SHIFT;
             const int kk0 = 2 * warp + (lane >> 4);
             const double *src = X + (live ? line : 0) + (k0 + kk0) * ldx;
@@ -496,8 +510,11 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int li = warp * 2 + h;
-                place(item, li, line, k0);
-                const int kleft = left_of();
+                if constexpr (BY_LINE) {
+                    if (h) next_row(line0, k0);
+                    kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);
+                }
+                const int64_t line = BY_LINE ? line0 : line0 + li;
                 const bool live = line < lines && shift[line] != OZ_NONFINITE_SHIFT;
                 const double *src = X + (live ? line : 0) * ldx + k0;
                 const uint32_t row = base + li * (kTilePitch * 8);
@@ -533,10 +550,13 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();                 // this tile (and, the first time, the table) is there
+        int64_t line0, k0;
+        place(item, line0, k0);
         const int li = warp * 2 + (lane >> 4);
-        int64_t line, k0;
-        place(item, li, line, k0);
-        const int64_t kb = k0 + (lane & 15) * 8;
+        if constexpr (BY_LINE) {
+            if (lane >> 4) next_row(line0, k0);
+        }
+        const int64_t line = BY_LINE ? line0 : line0 + li, kb = k0 + (lane & 15) * 8;
         if (line < lines && kb < row_pitch) {
             const int sigma_raw = shift[line];
             const int sigma = sigma_raw == OZ_NONFINITE_SHIFT ? 0 : sigma_raw;     // such a line is zero in the tile
@@ -867,15 +887,18 @@ oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t 
                            const PlaneGeom &geom, int tz, bool alone, cudaStream_t stream)
 {
     constexpr size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * sizeof(double) * kTileLines * kTilePitch;
-    static std::atomic<unsigned long long> ready{0};
-    OZ_CUDA_CHECK(allow_shared(convert_kernel<SET, SIDE, LAYOUT>, smem, ready));
+    constexpr bool kByLine = SIDE == 1 && LAYOUT != kLayoutNative;
+    static std::atomic<unsigned long long> ready[2] = {{0}, {0}};
+    const bool by_line = kByLine && geom.line_stride != kChunk;
+    const auto kernel = by_line ? convert_kernel<SET, SIDE, LAYOUT, kByLine> : convert_kernel<SET, SIDE, LAYOUT, false>;
+    OZ_CUDA_CHECK(allow_shared(kernel, smem, ready[by_line]));
     const int64_t nchunks = (geom.row_pitch + kChunk - 1) / kChunk;
     if (lines * nchunks >= 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;   // item numbers are 32-bit
     const int64_t need = ((lines + kTileLines - 1) / kTileLines) * nchunks;
     // persistent blocks: as many as are resident at once (each copies the table once)
     const int64_t cap = 3ll * sm_count();
     int grid = static_cast<int>(need < cap ? need : cap);
-    OZ_CUDA_CHECK(launch_if(alone, convert_kernel<SET, SIDE, LAYOUT>, dim3(grid), kConvThreads, smem, stream,
+    OZ_CUDA_CHECK(launch_if(alone, kernel, dim3(grid), kConvThreads, smem, stream,
                          X, ldx, lines, k, shift, lut, planes, geom, tz));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
