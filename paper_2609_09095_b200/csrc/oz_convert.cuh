@@ -53,7 +53,7 @@ __device__ __forceinline__ long long quantise(double x, int sigma, bool tz)
 // Every instruction works on a packed pair of elements: six for two residues, where 16-bit integer limbs
 // take seven for one.  What bounds the conversion is instruction issue (and the look-ups' shared-memory
 // wavefronts), so both the packed arithmetic and the digits of the odd squares, which need no table,
-// come straight off its time: 204 -> 125 thread-instructions per element on set S.
+// come straight off its time: 204 -> 146 thread-instructions per element of A on set S, 190 -> 137 of B.
 constexpr int kLimbBit1 = 16, kLimbBit2 = 31, kLimbBit3 = 45;
 // Largest |a'|, as 2^q, of an element whose product does not vanish: CS and MAXEXP stay below sqrt(M/2); the
 // accurate rule reaches sqrt(32) 2^(L/2) with L = floor(log2 of its budget) = 110, 112, 116.  (Elements

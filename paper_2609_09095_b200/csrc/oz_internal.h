@@ -174,8 +174,8 @@ void cs_bound_squared(int set, int64_t k, uint64_t *lo, uint64_t *hi);  // G^2 a
 //   public:   lines of row_pitch bytes (line_stride = row_pitch, chunk_stride = 128)
 //   private:  K chunk by K chunk, the 128-byte pieces of all lines one behind the other (line_stride = 128,
 //             chunk_stride = 128 lines; row_pitch = k rounded up to 128, so the size is that of the public layout).
-//             A 128-line TMA box is then 16 KiB of consecutive bytes, and so is what a conversion tile stores: with
-//             128-byte pieces a row pitch apart the plane writes stopped at 3.3 TB/s.
+//             A 128-line TMA box is then 16 KiB of consecutive bytes, and a conversion tile stores 2 KiB at a time instead
+//             of 128-byte pieces a row pitch apart (32768 x 4096, side 0, set S: 1.39 against 1.61 ms).
 struct PlaneGeom {
     int64_t plane_stride, row_pitch, line_stride, chunk_stride;
 };
