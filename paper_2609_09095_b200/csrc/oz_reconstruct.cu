@@ -15,6 +15,7 @@
 // test for the lift to [-M/2, M/2), and one round-to-nearest-even done in integer arithmetic.
 // A thread handles the consecutive rows whose residues share one 32-bit word per modulus (two
 // uint16, or four uint8 for the all-byte set).
+#include <cstring>
 #include <utility>
 
 #include "oz_internal.h"
@@ -23,10 +24,10 @@ namespace oz {
 namespace {
 
 struct ReconConst {
-    double V[kMaxR][3];        // V_i = V0 + V1 2^38 + V2 2^76
-    double Mc[3];              // M   = M0 + M1 2^38 + M2 2^76
+    double V[kMaxR][3];        // V_i = V0 + V1 + V2, the chunks in place: V1 and V2 are multiples of 2^cw and 2^(2cw)
+    double Mc[3];              // M   = M0 + M1 + M2 likewise
     double inv_M;              // 1/M (rounded)
-    double half_M_guard;       // (M/2) (1 - 2^-30): beyond it the lift is decided exactly
+    int half_M_guard;          // high word of (M/2) (1 - 2^-30): from it on the lift is decided exactly
     unsigned long long M_lo, M_hi;
 };
 
@@ -36,6 +37,10 @@ __constant__ ReconConst c_recon[kNumSets];
 // the 117.8-bit set A (residues < 2^8, 15 terms: sums < 2^52), so that three chunks cover M.
 __host__ __device__ constexpr int chunk_bits(int set) { return set == 2 ? 40 : 38; }
 __host__ __device__ constexpr double pow2d(int e) { double v = 1.0; for (int i = 0; i < e; ++i) v *= 2.0; return v; }
+// Resident blocks per SM.  The loads of a thread are independent, so this many keep memory busy; the registers they leave
+// (48, 64) hold everything.  16384 x 16384 update, set S, with 4 / 5 / 6 blocks: 2.18 / 2.17 / 2.17 ms; 6144 x 6144, set A, with
+// 3 / 4 / 5 blocks: 288 / 289 / 298 us.  Before the mapping and the arithmetic below: 2.35 ms and 327 us.
+template <int SET> constexpr int kReconBlocks = residue_bytes(SET) == 2 ? 5 : 4;
 constexpr double kRint = 6755399441055744.0;          // 1.5 * 2^52: (x + kRint) - kRint = rint(x)
 
 // x * 2^scale for a finite double x (exact unless the result leaves the normal range)
@@ -69,14 +74,14 @@ __device__ __forceinline__ void crt_sum(std::integer_sequence<int, I...>, const 
     (crt_term<SET, HALF, I>(c[I], S0, S1, S2), ...);
 }
 
-// Exact tail (rare path): the normalised chunks as a 128-bit integer, exact lift to
-// [-M/2, M/2), round-to-nearest-even conversion in integer arithmetic, power-of-two scale.
-__device__ __noinline__ double finish_exact(double T0, double T1, double T2, int shift_sum, int set)
+// Exact tail (rare path): the three chunks as a 128-bit integer, exact lift to [-M/2, M/2),
+// round-to-nearest-even conversion in integer arithmetic, power-of-two scale.
+__device__ __forceinline__ double finish_exact(double X0, double X1, double X2, int shift_sum, int set)
 {
     const ReconConst &K = c_recon[set];
-    const long long t0 = __double2ll_rn(T0), t1 = __double2ll_rn(T1), t2 = __double2ll_rn(T2);
-    // v = t0 + t1 2^cw + t2 2^(2cw) as a two's-complement (hi:lo) pair
     const int cw = chunk_bits(set);
+    const long long t0 = __double2ll_rn(X0), t1 = __double2ll_rn(X1 * (1.0 / pow2d(cw))), t2 = __double2ll_rn(X2 * (1.0 / pow2d(2 * cw)));
+    // v = t0 + t1 2^cw + t2 2^(2cw) as a two's-complement (hi:lo) pair
     unsigned long long lo = static_cast<unsigned long long>(t0) + (static_cast<unsigned long long>(t1) << cw);
     long long hi = (t0 >> 63) + (t1 >> (64 - cw)) + (lo < static_cast<unsigned long long>(t0) ? 1 : 0) +
                    static_cast<long long>(static_cast<unsigned long long>(t2) << (2 * cw - 64));
@@ -103,56 +108,50 @@ __device__ __noinline__ double finish_exact(double T0, double T1, double T2, int
     return neg ? -d : d;
 }
 
-template <int SET, int HALF>
-__device__ __forceinline__ double reconstruct_one(const uint32_t (&c)[kMaxR], int shift_sum)
+// alpha 2^-(sa + sb) c' where the fast path does not apply: NaN for a line with Inf/NaN, else by integers
+template <int SET>
+__device__ __noinline__ double row_value_exact(double X0, double X1, double X2, int sa, int sb, double alpha)
 {
-    const ReconConst &K = c_recon[SET];
-    double S0 = 0.0, S1 = 0.0, S2 = 0.0;
-    crt_sum<SET, HALF>(std::make_integer_sequence<int, set_r(SET)>{}, c, S0, S1, S2);
-    constexpr double kTwo38 = pow2d(chunk_bits(SET));          // 2^cw  (names kept from the 38-bit case)
-    constexpr double kTwoM38 = 1.0 / pow2d(chunk_bits(SET));   // 2^-cw
-    constexpr double kTwo76 = kTwo38 * kTwo38;                 // 2^(2cw)
-    double val = fma(S2, kTwo76, fma(S1, kTwo38, S0));
-    double kappa = (val * K.inv_M + kRint) - kRint;
-    double T0 = fma(-kappa, K.Mc[0], S0);              // exact: integers below 2^53
-    double T1 = fma(-kappa, K.Mc[1], S1);
-    double T2 = fma(-kappa, K.Mc[2], S2);
-    // carry-normalise so that the three chunks do not overlap: |T0|, |T1| <= 2^37
-    double c0 = (T0 * kTwoM38 + kRint) - kRint;
-    T0 = fma(-c0, kTwo38, T0);
-    T1 += c0;
-    double c1 = (T1 * kTwoM38 + kRint) - kRint;
-    T1 = fma(-c1, kTwo38, T1);
-    T2 += c1;
-    // c' = X2 + X1 + X0 exactly.  Fast path: two error-free additions give r = RN(s + t) and
-    // the exact residual rem of that last rounding; r is the correctly rounded value of c'
-    // unless c' lies within a hair of a rounding boundary (|rem| ~ half an ulp, or r a power
-    // of two) or within a hair of +-M/2 (where the symmetric lift could apply).  Those cases,
-    // a vanishing fraction of random data, take the exact integer path.
-    const double X2 = T2 * kTwo76, X1 = T1 * kTwo38;   // exact
-    const double s = X2 + X1;
-    const double err = X1 - (s - X2);                   // exact: s + err = X2 + X1
-    const double t = err + T0;
-    const double r = s + t;
-    const double rem = t - (r - s);                     // exact: r + rem = s + t
-    const long long rb = __double_as_longlong(r);
-    const int eb = static_cast<int>((rb >> 52) & 0x7FF);
-    if (eb == 0) return 0.0;                            // c' = 0 (r is an integer: never subnormal)
-    const double half_ulp = __longlong_as_double(static_cast<long long>(eb - 53) << 52);
-    const bool near_tie = fabs(rem) >= fma(-half_ulp, 9.313225746154785e-10, half_ulp);   // (1 - 2^-30)
-    const bool pow2 = (rb & 0xFFFFFFFFFFFFFll) == 0 && rem != 0.0;
-    const bool near_half_M = fabs(r) >= K.half_M_guard;
-    if (near_tie || pow2 || near_half_M) return finish_exact(T0, T1, T2, shift_sum, SET);
-    return scale_pow2(r, -shift_sum);
+    if (sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
+    return finish_exact(X0, X1, X2, sa + sb, SET) * alpha;
 }
 
-// one row of the thread's group: reconstruct, scale by alpha
-template <int SET, int H>
-__device__ __forceinline__ double row_value(const uint32_t (&w)[kMaxR], int sa, int sb, double alpha)
+// Column operand of row_scale(): shiftB with the mark of a column with Inf/NaN moved so far out that no sum with a row
+// shift (|sa| < 2^12, or INT32_MIN) wraps into the range of the fast path.
+__device__ __forceinline__ int column_shift(int sb) { return sb == OZ_NONFINITE_SHIFT ? 1 << 29 : sb; }
+
+// One row of the thread's group: value = fast alpha 2^-(sa + sb) c', returned as the rounded integer r and the power of
+// two to multiply it by (exact, and left to the caller so that an update of C is one fused multiply-add).
+// The chunks are not carry-normalised.  X2 + X1 = s + err by a fast two-sum, which is error-free because X2 is a multiple of
+// 2^(2cw) and so of ulp(X1) (|X1| < 2^(53+cw)); t = err + X0 loses at most 2^-52 of |err| + |X0|, and nothing below 2^53,
+// which |X0| < 2^52.1 alone does not reach: what it loses is below 2^-40 of half an ulp of s; s + t = r + rem exactly (s is a
+// multiple of 2^cw and so of ulp(t)).  Hence r is c' correctly rounded unless c' lies within 2^-29 of half an ulp from a
+// rounding boundary -- adding rem, enlarged by 2^-29, then moves r -- or so near to +-M/2 that the lift may apply.
+// 50 FP64 operations per output on set S where the carries and a test by exponents took 63.
+template <int SET, int HALF>
+__device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, int sb, int sb_mark, int alpha_sign, double alpha,
+                                          double &r, double &scale)
 {
-    const double nan = __longlong_as_double(0x7FF8000000000000ll);
-    double p = (sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT) ? nan : reconstruct_one<SET, H>(w, sa + sb);
-    return p * alpha;
+    const ReconConst &K = c_recon[SET];
+    double X0 = 0.0, X1 = 0.0, X2 = 0.0;
+    crt_sum<SET, HALF>(std::make_integer_sequence<int, set_r(SET)>{}, c, X0, X1, X2);
+    const double kappa = fma(X2 + X1, K.inv_M, kRint) - kRint;
+    X0 = fma(-kappa, K.Mc[0], X0);              // exact: integers below 2^53 (times 2^cw, 2^(2cw))
+    X1 = fma(-kappa, K.Mc[1], X1);
+    X2 = fma(-kappa, K.Mc[2], X2);
+    const double s = X2 + X1, err = X1 - (s - X2);
+    const double t = err + X0;
+    r = s + t;
+    const double rem = t - (r - s);
+    const int shift_sum = sa + sb_mark;
+    // 2^-shift_sum and r 2^-shift_sum are normal: r is zero or 1 <= |r| < 2^118
+    const bool easy = static_cast<unsigned>(shift_sum + 904) <= 1924u && fma(rem, 1.0 + 0x1p-29, r) == r &&
+                      (__double2hiint(r) & 0x7FFFFFFF) < K.half_M_guard;
+    scale = __hiloint2double(static_cast<int>(static_cast<uint32_t>(1023 - shift_sum) << 20) ^ alpha_sign, 0);
+    if (!easy) {
+        r = row_value_exact<SET>(X0, X1, X2, sa, sb, alpha);
+        scale = 1.0;
+    }
 }
 
 // scalar stores of up to two consecutive rows; `first` / `second`: which of them are written
@@ -182,28 +181,29 @@ __device__ __forceinline__ void reconstruct_rows(const uint32_t (&w)[kMaxR], int
 #pragma unroll
         for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + 2 * h);
     }
+    const int sb_mark = column_shift(sb), alpha_sign = alpha < 0.0 ? INT32_MIN : 0;
     {
-        double p0 = row_value<SET, 0>(w, sa[0], sb, alpha);
-        double p1 = nrows > 1 ? row_value<SET, 1>(w, sa[1], sb, alpha) : 0.0;
-        if (whole) *reinterpret_cast<double2 *>(out) = make_double2(old[0].x + p0, old[0].y + p1);
-        else store_pair(out, p0, p1, (keep & 1u) != 0, nrows > 1 && (keep & 2u) != 0, beta);
+        double r0, r1 = 0.0, f0, f1 = 1.0;
+        row_value<SET, 0>(w, sa[0], sb, sb_mark, alpha_sign, alpha, r0, f0);
+        if (nrows > 1) row_value<SET, 1>(w, sa[1], sb, sb_mark, alpha_sign, alpha, r1, f1);
+        if (whole) *reinterpret_cast<double2 *>(out) = make_double2(fma(r0, f0, old[0].x), fma(r1, f1, old[0].y));
+        else store_pair(out, r0 * f0, r1 * f1, (keep & 1u) != 0, nrows > 1 && (keep & 2u) != 0, beta);
     }
     if constexpr (ROWS == 4) {
         if (nrows > 2) {
-            double p2 = row_value<SET, 2>(w, sa[2], sb, alpha);
-            double p3 = nrows > 3 ? row_value<SET, 3>(w, sa[3], sb, alpha) : 0.0;
-            if (whole) *reinterpret_cast<double2 *>(out + 2) = make_double2(old[1].x + p2, old[1].y + p3);
-            else store_pair(out + 2, p2, p3, (keep & 4u) != 0, nrows > 3 && (keep & 8u) != 0, beta);
+            double r2, r3 = 0.0, f2, f3 = 1.0;
+            row_value<SET, 2>(w, sa[2], sb, sb_mark, alpha_sign, alpha, r2, f2);
+            if (nrows > 3) row_value<SET, 3>(w, sa[3], sb, sb_mark, alpha_sign, alpha, r3, f3);
+            if (whole) *reinterpret_cast<double2 *>(out + 2) = make_double2(fma(r2, f2, old[1].x), fma(r3, f3, old[1].y));
+            else store_pair(out + 2, r2 * f2, r3 * f3, (keep & 4u) != 0, nrows > 3 && (keep & 8u) != 0, beta);
         }
     }
 }
 
 // Each thread reconstructs ROWS consecutive rows of one column: the residues of those rows are one
 // 32-bit word per modulus (two uint16 for S and E, four uint8 for the all-byte set A).
-// Six blocks per SM (40 registers) for the two-byte sets: the kernel is bound by instruction issue
-// and gains from the extra warps; the four-row variant of set A would spill at that budget.
 template <int SET>
-__global__ void __launch_bounds__(256, residue_bytes(SET) == 2 ? 6 : 5)
+__global__ void __launch_bounds__(256, kReconBlocks<SET>)
 reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride, int64_t m,
                    int64_t n, const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
                    double alpha, double beta, double *__restrict__ C, int64_t ldc, int vecR, int vecC)
@@ -244,14 +244,13 @@ reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride,
 
 // Same reconstruction from the tile-ordered private array that the whole-method GEMM writes (see
 // ResidueTiling).  A thread takes one 32-bit word of a 32-column x 64-row block, i.e. ROWS consecutive
-// rows of one column.  The words of one column are dealt to consecutive threads, so that a warp
-// reads and writes 512 contiguous bytes of C (one or two whole columns of the block); its residue
-// loads are 16-byte pieces 512 bytes apart, and the warps of a thread block, which take neighbouring
-// columns, ask for whole 128-byte lines between them.
+// rows of one column.  A warp takes one 16-byte chunk of eight neighbouring columns: its residue loads are whole
+// 128-byte lines and its accesses to C eight pieces of 64 (128) contiguous bytes; the warps of a thread block, which
+// take the other chunks of the same columns, complete those to whole lines of C.
 // grid: x = (piece of the block, block within the tile, CTA rank of the pair), y = tile column, z = tile row
 // SKIP: rows flagged in `skip` are left untouched (they are re-issued on the native FP64 path).
 template <int SET, bool SKIP>
-__global__ void __launch_bounds__(256, residue_bytes(SET) == 2 ? 6 : 5)
+__global__ void __launch_bounds__(256, kReconBlocks<SET>)
 reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int tn0,
                          int64_t m, int64_t n, int64_t col0, int64_t col1,
                          const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
@@ -269,8 +268,9 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
     const uint32_t wi = (blockIdx.x / kPieces) & 15u;
     const uint32_t rank = blockIdx.x / (kPieces * 16);     // 0, or 0..1 with CTA pairs
     const uint32_t tn = static_cast<uint32_t>(tn0) + blockIdx.y, tm = blockIdx.z;
-    const uint32_t lane = piece * kCtaCols + threadIdx.x / kColWords;   // column of the block
-    const uint32_t wq = threadIdx.x % kColWords, c = wq >> 2, sub = wq & 3u;
+    constexpr int kChunks = kColWords / 4;                 // 16-byte chunks of one column: 8 or 4
+    const uint32_t warp = threadIdx.x >> 5, c = warp % kChunks, sub = threadIdx.x & 3u;
+    const uint32_t lane = piece * kCtaCols + warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u);   // column of the block
     const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * (16 / RB) + sub * ROWS;
     const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
     if (row >= m || j >= n || j < col0 || j >= col1) return;
@@ -303,6 +303,11 @@ oz_status_t upload_reconstruct_constants()
         for (int i = 0; i < set_r(set); ++i) M *= static_cast<unsigned>(modulus(set, i));
         const int cw = chunk_bits(set);
         const unsigned __int128 mask = (static_cast<unsigned __int128>(1) << cw) - 1;
+        auto chunks = [&](unsigned __int128 v, double (&out)[3]) {
+            out[0] = static_cast<double>(static_cast<unsigned long long>(v & mask));
+            out[1] = static_cast<double>(static_cast<unsigned long long>((v >> cw) & mask)) * pow2d(cw);
+            out[2] = static_cast<double>(static_cast<unsigned long long>(v >> (2 * cw))) * pow2d(2 * cw);
+        };
         ReconConst &K = host[set];
         for (int i = 0; i < kMaxR; ++i) K.V[i][0] = K.V[i][1] = K.V[i][2] = 0.0;
         for (int i = 0; i < set_r(set); ++i) {
@@ -312,15 +317,14 @@ oz_status_t upload_reconstruct_constants()
             for (unsigned c = 1; c < mi; ++c)
                 if ((static_cast<unsigned long long>(wm) * c) % mi == 1) { inv = c; break; }
             unsigned __int128 V = W * inv;          // < M, and V = 1 mod m_i, 0 mod the other moduli
-            K.V[i][0] = static_cast<double>(static_cast<unsigned long long>(V & mask));
-            K.V[i][1] = static_cast<double>(static_cast<unsigned long long>((V >> cw) & mask));
-            K.V[i][2] = static_cast<double>(static_cast<unsigned long long>(V >> (2 * cw)));
+            chunks(V, K.V[i]);
         }
-        K.Mc[0] = static_cast<double>(static_cast<unsigned long long>(M & mask));
-        K.Mc[1] = static_cast<double>(static_cast<unsigned long long>((M >> cw) & mask));
-        K.Mc[2] = static_cast<double>(static_cast<unsigned long long>(M >> (2 * cw)));
+        chunks(M, K.Mc);
         K.inv_M = 1.0 / static_cast<double>(M);
-        K.half_M_guard = 0.5 * static_cast<double>(M) * (1.0 - 9.313225746154785e-10);
+        const double guard = 0.5 * static_cast<double>(M) * (1.0 - 0x1p-30);
+        uint64_t guard_bits;
+        memcpy(&guard_bits, &guard, sizeof(guard));
+        K.half_M_guard = static_cast<int>(guard_bits >> 32);
         K.M_lo = static_cast<unsigned long long>(M);
         K.M_hi = static_cast<unsigned long long>(M >> 64);
     }

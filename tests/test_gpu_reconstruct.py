@@ -1,0 +1,41 @@
+"""Reconstruction at the edges of its fast path: scales whose power of two is no normal double, integers next to a
+rounding boundary, to a power of two and to +-M/2, marked lines.  The same values against every shift."""
+import numpy as np
+import pytest
+
+from oracle import oz_oracle as ozo
+
+pytestmark = pytest.mark.gpu
+
+OSET = {"S": ozo.SET_S, "E": ozo.SET_E, "A": ozo.SET_A}
+MARK = -(2 ** 31)
+
+
+@pytest.mark.parametrize("set_name", ["S", "E", "A"])
+@pytest.mark.parametrize("alpha,beta", [(1.0, 0.0), (-1.0, 1.0)])
+def test_scale_and_rounding_edges(set_name, alpha, beta):
+    import tests.gpu_helpers as gh
+    ms = ozo.modset(OSET[set_name])
+    M = int(np.prod([int(v) for v in ms], dtype=object))
+    xs = [0, 1, -1, 3, M // 2 - 1, -(M // 2), M // 2 - 2 ** 60, (M >> 1) - (M >> 22), -(M >> 1) + (M >> 31)]
+    for e in (53, 54, 60, 77, 81, 95, 106, 109):
+        tie_below, tie_above = 2 ** e - 2 ** max(e - 54, 0), 2 ** e + 2 ** max(e - 53, 0)
+        xs += [2 ** e, tie_below, tie_below + 1, tie_below - 1, -tie_above, tie_above + 1, -(tie_above - 1)]
+    # a rounding error just inside and just outside the guard of 2^-29 half units in the last place
+    xs += [2 ** 105 + 2 ** 52 - 2 ** 22, 2 ** 105 + 2 ** 52 - 2 ** 24, -(2 ** 105 + 2 ** 53 + 2 ** 52 + 2 ** 24)]
+    shifts = [-1200, -1010, -905, -904, -903, -100, 0, 57, 1019, 1020, 1021, 1022, 1100, 1180, MARK]
+    m, n = len(xs), len(shifts)
+    R = np.empty((len(ms), n, m), dtype=np.uint16)
+    for i, mm in enumerate(ms):
+        R[i] = np.array([x % mm for x in xs], dtype=np.uint16)
+    sA = np.zeros(m, dtype=np.int32)
+    sA[-1] = MARK                                    # a marked row against every column, the marked one among them
+    sB = np.array(shifts, dtype=np.int32)
+    C0 = np.asfortranarray(np.random.default_rng(7).standard_normal((m, n)))
+    CI = ozo.crt(R, OSET[set_name])
+    for ldr, rows in ((None, m), (None, m - 1)):     # pairs of rows whole, and a last row alone
+        Rr, CIr = np.ascontiguousarray(R[:, :, m - rows:]), CI[:, m - rows:]
+        got, _ = gh.reconstruct(Rr, sA[m - rows:], sB, set_name, alpha, beta, C0[m - rows:], ldr=ldr)
+        want = ozo.output(np.ascontiguousarray(CIr), sA[m - rows:], sB, alpha, beta, np.asfortranarray(C0[m - rows:]))
+        assert (np.isnan(got) == np.isnan(want)).all()
+        assert (got[~np.isnan(want)] == want[~np.isnan(want)]).all()
