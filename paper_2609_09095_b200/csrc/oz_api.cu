@@ -184,7 +184,8 @@ bool decode_route_for_set(int set, uint32_t route, Route *out)
 // of the interface.
 oz_status_t resolve_schedule(int set, int64_t k, int64_t n, bool automatic, Route *rt)
 {
-    if (rt->acc == 0)
+    rt->automatic = rt->acc == 0;
+    if (rt->automatic)
         rt->acc = (automatic && !rt->native() && k > 0) ? 1 : 2;
     return OZ_OK;
 }
@@ -484,6 +485,15 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     if (!ws || ws_bytes < L.total) return OZ_ERR_WORKSPACE;
     st = ensure_device_ready();
     if (st != OZ_OK) return st;
+    if (two_plane_applies(m, n, k, rt)) {      // fewer planes of A, more of B: within the workspace that the call has always needed
+        Route two = rt;
+        two.acc = 3;
+        const Layout T = make_layout(m, n, k, set, two);
+        if (T.total <= L.total) {
+            rt = two;
+            L = T;
+        }
+    }
     const OperandView a = operand_view(ws + L.offA, L.A), b = operand_view(ws + L.offB, L.B);
 
     // The two operands are deconstructed side by side: in one launch when both fit the one-kernel form, else B's

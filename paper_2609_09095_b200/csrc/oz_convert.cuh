@@ -13,16 +13,9 @@
 namespace oz {
 namespace {
 
-// Eq. 1 for one element, fast form: multiplying by the power of two 2^sigma is exact in FP64 (a
-// product that underflows is far below 1/2 and rounds to zero either way), and the hardware
-// conversion rounds to nearest-even or toward zero.  Valid while 2^sigma is a normal double.
-__device__ __forceinline__ long long quantise_fp(double x, double scale, bool tz)
-{
-    double y = x * scale;
-    return tz ? __double2ll_rz(y) : __double2ll_rn(y);
-}
-
-// Eq. 1 for one element, integer form (any sigma): a' = quant(x 2^sigma) as a 64-bit integer.
+// Eq. 1 for one element, integer form (any sigma): a' = quant(x 2^sigma) as a 64-bit integer.  While 2^sigma is a normal
+// double, split_limbs() multiplies by it instead: exact in FP64 (a product that underflows is far below 1/2 and rounds to
+// zero either way), and the hardware conversion rounds to nearest-even or toward zero.
 __device__ __forceinline__ long long quantise(double x, int sigma, bool tz)
 {
     unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
@@ -88,14 +81,45 @@ struct Limbs {
     uint32_t low[2 * NP];                    // bits 0..14 are those of a' (the power-of-two moduli)
 };
 
+// limbs of one quantised value
+__device__ __forceinline__ void limb_fields(long long a, float &f0, float &f1, float &f2, float &f3, uint32_t &low)
+{
+    constexpr unsigned long long kBias = (1ull << 15) + (1ull << 30) + (1ull << 44) + (1ull << 63);
+    const unsigned long long p = static_cast<unsigned long long>(a) + kBias;
+    const uint32_t lo = static_cast<uint32_t>(p), hi = static_cast<uint32_t>(p >> 32);
+    // a field OR 2^23's exponent is the float 2^23 + field
+    low = __byte_perm(lo, 0x4B000000u, 0x7610);
+    f0 = __uint_as_float(low);
+    f1 = __uint_as_float(((lo >> 16) & 0x7FFFu) | 0x4B000000u);
+    f2 = __uint_as_float((__funnelshift_r(lo, hi, 31) & 0x3FFFu) | 0x4B000000u);
+    f3 = __uint_as_float((hi >> 13) | 0x4B000000u);
+}
+
 // limbs of the quantised values of 2 NP elements
 template <int NP>
 __device__ __forceinline__ void split_limbs(const double (&x)[2 * NP], int sigma, bool tz, Limbs<NP> &L)
 {
-    // 2^sigma as a double when it is a normal number (always, except for lines of subnormals)
-    const bool fast = sigma >= -1000 && sigma <= 1000;
-    const double scale = __hiloint2double((1023 + (fast ? sigma : 0)) << 20, 0);
-    constexpr unsigned long long kBias = (1ull << 15) + (1ull << 30) + (1ull << 44) + (1ull << 63);
+    long long a[2 * NP];
+    if (sigma >= -1000 && sigma <= 1000) {       // 2^sigma is a normal number (always, except for lines of subnormals)
+        const double scale = __hiloint2double((1023 + sigma) << 20, 0);
+        if (!tz) {
+#pragma unroll
+            for (int e = 0; e < 2 * NP; ++e) a[e] = __double2ll_rn(x[e] * scale);
+        } else {
+#pragma unroll
+            for (int e = 0; e < 2 * NP; ++e) a[e] = __double2ll_rz(x[e] * scale);
+        }
+    } else {
+#pragma unroll 1
+        for (int e = 0; e < 2 * NP; ++e) {
+            double v = x[0];
+#pragma unroll
+            for (int f = 1; f < 2 * NP; ++f) v = e == f ? x[f] : v;
+            const long long w = quantise(v, sigma, tz);
+#pragma unroll
+            for (int f = 0; f < 2 * NP; ++f) a[f] = e == f ? w : a[f];
+        }
+    }
     constexpr float k23 = 8388608.0f;
     const float2 o0 = make_float2(-(k23 + 32768.0f), -(k23 + 32768.0f)), o1 = make_float2(-(k23 + 16384.0f), -(k23 + 16384.0f));
     const float2 o2 = make_float2(-(k23 + 8192.0f), -(k23 + 8192.0f)), o3 = make_float2(-(k23 + 262144.0f), -(k23 + 262144.0f));
@@ -103,18 +127,7 @@ __device__ __forceinline__ void split_limbs(const double (&x)[2 * NP], int sigma
     for (int q = 0; q < NP; ++q) {
         float f0[2], f1[2], f2[2], f3[2];
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const long long a = fast ? quantise_fp(x[2 * q + e], scale, tz) : quantise(x[2 * q + e], sigma, tz);
-            const unsigned long long p = static_cast<unsigned long long>(a) + kBias;
-            const uint32_t lo = static_cast<uint32_t>(p), hi = static_cast<uint32_t>(p >> 32);
-            // a field OR 2^23's exponent is the float 2^23 + field
-            const uint32_t u0 = __byte_perm(lo, 0x4B000000u, 0x7610);
-            L.low[2 * q + e] = u0;
-            f0[e] = __uint_as_float(u0);
-            f1[e] = __uint_as_float(((lo >> 16) & 0x7FFFu) | 0x4B000000u);
-            f2[e] = __uint_as_float((__funnelshift_r(lo, hi, 31) & 0x3FFFu) | 0x4B000000u);
-            f3[e] = __uint_as_float((hi >> 13) | 0x4B000000u);
-        }
+        for (int e = 0; e < 2; ++e) limb_fields(a[2 * q + e], f0[e], f1[e], f2[e], f3[e], L.low[2 * q + e]);
         L.l0[q] = __fadd2_rn(make_float2(f0[0], f0[1]), o0);
         L.l1[q] = __fadd2_rn(make_float2(f1[0], f1[1]), o1);
         L.l2[q] = __fadd2_rn(make_float2(f2[0], f2[1]), o2);
@@ -168,6 +181,27 @@ __device__ __forceinline__ void store_words(uint8_t *out, const uint32_t (&w)[N]
     else *reinterpret_cast<uint32_t *>(out) = w[0];
 }
 
+// Digits of four integer-valued numbers to base BASE, both rounded: d1 = rint(r / BASE), d0 = r - BASE d1
+template <int BASE, bool E4M3>
+__device__ __forceinline__ void digit_words(const float2 (&r)[2], uint32_t &w0, uint32_t &w1)
+{
+    float2 d0[2], d1[2], t1[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        t1[h] = __ffma2_rn(r[h], dup(inv_of(BASE)), dup(kRintF));
+        d1[h] = __fadd2_rn(t1[h], dup(-kRintF));
+        d0[h] = __ffma2_rn(d1[h], dup(-static_cast<float>(BASE)), r[h]);
+    }
+    if constexpr (E4M3) {
+        w0 = e4m3_pair(d0[0]) | (e4m3_pair(d0[1]) << 16);
+        w1 = e4m3_pair(d1[0]) | (e4m3_pair(d1[1]) << 16);
+    } else {
+        const float2 u0 = __fadd2_rn(d0[0], dup(kRintF)), u1 = __fadd2_rn(d0[1], dup(kRintF));
+        w0 = pack_low_bytes(__float_as_uint(u0.x), __float_as_uint(u0.y), __float_as_uint(u1.x), __float_as_uint(u1.y));
+        w1 = pack_low_bytes(__float_as_uint(t1[0].x), __float_as_uint(t1[0].y), __float_as_uint(t1[1].x), __float_as_uint(t1[1].y));
+    }
+}
+
 // One modulus (compile-time index I of set SET) for 2 NP consecutive inner-dimension elements: residues,
 // digits, and 1, 2 or 3 plane stores of 2 NP bytes.  Digits come from the table for the power-of-two and the
 // non-square moduli (Lemma 1's carry makes the latter irregular) and from one more rounded division for the
@@ -181,7 +215,7 @@ __device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut
     constexpr bool pow2 = (m & (m - 1)) == 0;
     constexpr int s = square_root(m);
     constexpr int NW = NP / 2;                       // plane words
-    constexpr bool e4m3 = LAYOUT == kLayoutDigits || LAYOUT == kLayoutMerged;      // else INT8 digits
+    constexpr bool e4m3 = LAYOUT == kLayoutDigits || LAYOUT == kLayoutMerged || LAYOUT == kLayoutTwo || LAYOUT == kLayoutFour;   // else INT8
     if constexpr (LAYOUT == kLayoutNative) {         // one plane: the centred residue itself
         uint32_t w[NW];
 #pragma unroll
@@ -196,27 +230,43 @@ __device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut
             }
         }
         store_words(out + plane * plane_stride, w);
+    } else if constexpr (two_plane_layout(LAYOUT)) {
+        // 6.3 instructions per element and modulus, and no shared memory (9 with the table, whose look-ups conflict)
+        constexpr bool four = s == 0 && (LAYOUT == kLayoutFour || LAYOUT == kLayoutFourI8);
+        constexpr int base = s ? s : 16;
+        uint32_t w[4][NW];
+#pragma unroll
+        for (int g = 0; g < NW; ++g) {
+            float2 r[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if constexpr (pow2) {        // the lowest limb carries the residue
+                    const float2 l = L.l0[2 * g + h];
+                    const float2 quot = __fadd2_rn(__ffma2_rn(l, dup(inv_of(m)), dup(kRintF)), dup(-kRintF));
+                    r[h] = __ffma2_rn(quot, dup(-static_cast<float>(m)), l);
+                } else {
+                    r[h] = residue_pair<SET, I>(L, 2 * g + h);
+                }
+            }
+            digit_words<base, e4m3>(r, w[0][g], w[1][g]);
+            if constexpr (four) {            // f = 16 e mod m, balanced
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float2 quot = __fadd2_rn(__ffma2_rn(r[h], dup(16.0f * inv_of(m)), dup(kRintF)), dup(-kRintF));
+                    r[h] = __ffma2_rn(quot, dup(-static_cast<float>(m)), __fmul2_rn(r[h], dup(16.0f)));
+                }
+                digit_words<base, e4m3>(r, w[2][g], w[3][g]);
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < (four ? 4 : 2); ++d) store_words(out + (plane + d) * plane_stride, w[d]);
     } else if constexpr (s != 0 && !pow2) {
-        // odd square: d1 = rint(r / s), d0 = r - s d1, both balanced and free of ties
+        // odd square: both digits balanced and free of ties
         uint32_t w0[NW], w1[NW];
 #pragma unroll
         for (int g = 0; g < NW; ++g) {
-            float2 d0[2], d1[2], t1[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float2 r = residue_pair<SET, I>(L, 2 * g + h);
-                t1[h] = __ffma2_rn(r, dup(inv_of(s)), dup(kRintF));
-                d1[h] = __fadd2_rn(t1[h], dup(-kRintF));
-                d0[h] = __ffma2_rn(d1[h], dup(-static_cast<float>(s)), r);
-            }
-            if constexpr (e4m3) {
-                w0[g] = e4m3_pair(d0[0]) | (e4m3_pair(d0[1]) << 16);
-                w1[g] = e4m3_pair(d1[0]) | (e4m3_pair(d1[1]) << 16);
-            } else {
-                const float2 u0 = __fadd2_rn(d0[0], dup(kRintF)), u1 = __fadd2_rn(d0[1], dup(kRintF));
-                w0[g] = pack_low_bytes(__float_as_uint(u0.x), __float_as_uint(u0.y), __float_as_uint(u1.x), __float_as_uint(u1.y));
-                w1[g] = pack_low_bytes(__float_as_uint(t1[0].x), __float_as_uint(t1[0].y), __float_as_uint(t1[1].x), __float_as_uint(t1[1].y));
-            }
+            const float2 r[2] = {residue_pair<SET, I>(L, 2 * g), residue_pair<SET, I>(L, 2 * g + 1)};
+            digit_words<s, e4m3>(r, w0[g], w1[g]);
         }
         store_words(out + plane * plane_stride, w0);
         store_words(out + (plane + 1) * plane_stride, w1);

@@ -26,7 +26,9 @@ namespace {
 constexpr int kConvThreads = 256;
 constexpr int kChunk = 128;            // inner-dimension elements of a conversion tile
 constexpr int kTileLines = 16;         // lines of a conversion tile: two per warp
-constexpr int kTilePitch = kChunk + 2; // doubles per tile row: an odd number of 16-byte chunks
+constexpr int kTileRow = (kChunk + 2) * 8;            // side 1: bytes of a tile row, an odd number of 16-byte chunks
+constexpr int kTileBytes = kTileLines * kTileRow;    // side 0 needs kTileLines * kChunk * 8 of them
+static_assert(kTileBytes % 128 == 0, "tile alignment");
 
 struct ScanScratch {
     unsigned long long *sumsq;  // [lines]  sum of squared magnitudes (accurate rule: maximum of the bound product)
@@ -418,11 +420,11 @@ __device__ __forceinline__ void load_table(uint32_t *lut, const uint32_t *__rest
         reinterpret_cast<uint4 *>(lut)[i] = reinterpret_cast<const uint4 *>(lut_global)[i];
 }
 
-// 16-byte chunk of a tile row that holds the element pair c: the eight lanes of a quarter warp, which read
+// Side 1: 16-byte chunk of a tile row that holds the element pair c: the eight lanes of a quarter warp, which read
 // chunks 4 l + e (l = 0..7), then hit eight different bank groups
 __device__ __forceinline__ int tile_chunk(int c) { return c ^ ((c >> 3) & 3); }
 
-// asynchronous copies of one (8 bytes) or two (16 bytes) elements; nothing is read and zeros are written when !live
+// asynchronous copies of one (8 bytes) or two (16 bytes) elements; nothing is read and zeros are written for bytes = 0
 __device__ __forceinline__ void copy8(uint32_t dst, const double *src, bool live)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(live ? 8 : 0) : "memory");
@@ -431,6 +433,10 @@ __device__ __forceinline__ void copy16(uint32_t dst, const double *src, int byte
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void copy16(uint32_t dst, const double *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 
 // A block takes tiles of 16 lines x 128 inner indices through shared memory (on side 0 that is the
 // transposition: loads run along the lines, plane stores along k) and a thread converts eight consecutive
@@ -438,11 +444,12 @@ __device__ __forceinline__ void copy16(uint32_t dst, const double *src, int byte
 // elements are copied asynchronously while this one is converted.  BY_LINE (side 1, planes kept line by line): the 16 rows
 // of a tile are consecutive 128-element pieces of a line, and of the next lines behind it, so that a tile stores 2 KiB at
 // a time in that layout too.
-// Bound: instruction issue (57 % of the slots busy at 8192 x 1024, set S) and, line by line on side 0, the planes' scattered
-// 128-byte writes.  Whole deconstruction of a 32768 x 4096 operand, integer limbs and a table for every modulus before -> now,
-// planes K chunk by K chunk: native residues 1.76 -> 1.19 ms (side 0), 1.37 -> 1.04 (side 1), set S on FP8 1.76 -> 1.39 and
-// 1.50 -> 1.28; planes line by line, set S: 1.76 -> 1.61 and 1.49 -> 1.23 (1.51 with 16 lines a tile).  Native residues take 16 lines a
-// tile in both layouts (1.04 and 1.05; 1.06 by lines).
+// Side 0 keeps a tile as [index in an octet][octet][line], 128 bytes a row, the 16-byte pieces of a row XORed with the octet's
+// number: two lines travel in one copy, and neither the copies nor the reads, eight at compile-time offsets from one
+// address, conflict.
+// Bound: instruction issue and the FP32 pipe (both 60 % busy), and, line by line on side 0, the planes' scattered
+// 128-byte writes.  What surrounds the arithmetic was half of the instructions: tiles are numbered without divisions, shifts are
+// loaded with the elements, and whole tiles are copied without a test.
 template <int SET, int SIDE, int LAYOUT, bool BY_LINE>
 __global__ void __launch_bounds__(kConvThreads, 3)
 convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
@@ -450,81 +457,116 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
                uint8_t *__restrict__ planes, const __grid_constant__ PlaneGeom geom, int tz)
 {
     const int64_t row_pitch = geom.row_pitch;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw);
-    double *tile = reinterpret_cast<double *>(smem_raw + lut_words_of(SET, LAYOUT) * 4);
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw + 2 * kTileBytes);
     const uint32_t lut_addr = static_cast<uint32_t>(__cvta_generic_to_shared(lut));
-    const uint32_t tile_addr = static_cast<uint32_t>(__cvta_generic_to_shared(tile));
-    constexpr int kTileDoubles = kTileLines * kTilePitch;
+    const uint32_t tile_addr = static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw));
     dependency_release();
     load_table<SET, LAYOUT>(lut, lut_global, threadIdx.x, kConvThreads);      // written once, before any call
     dependency_wait();
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // work items are numbered in 32 bits (checked on the host): cheap division
+    // work items are numbered in 32 bits (checked on the host)
     const uint32_t nchunks = static_cast<uint32_t>((row_pitch + kChunk - 1) / kChunk);
     const uint32_t ltiles = static_cast<uint32_t>((lines + kTileLines - 1) / kTileLines);
     const uint32_t items = BY_LINE ? (static_cast<uint32_t>(lines) * nchunks + kTileLines - 1) / kTileLines : ltiles * nchunks;
-    const bool pairs = SIDE == 1 && (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    const bool pairs = (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    const int li = warp * 2 + (lane >> 4), oct = lane & 15;        // this thread's line and octet of a tile
 
-    // first line and inner index of a tile (BY_LINE: of this warp's two rows).  Side 0: neighbouring blocks take
-    // neighbouring lines; side 1: neighbouring inner indices
-    auto place = [&](uint32_t item, int64_t &line0, int64_t &k0) {
+    // Position of a tile: slow index q (side 0: chunk, side 1: line tile) and fast index `rest`, so that neighbouring blocks
+    // take neighbouring lines (side 0) or neighbouring inner indices; BY_LINE: line and chunk of this warp's first row.  A step
+    // over the grid adds one constant to each, and one carry.
+    const uint32_t fast_count = SIDE == 0 ? ltiles : nchunks;
+    const uint32_t start = BY_LINE ? blockIdx.x * kTileLines + 2 * warp : blockIdx.x, step = BY_LINE ? gridDim.x * kTileLines : gridDim.x;
+    uint32_t q = start / fast_count, rest = start - q * fast_count;
+    const uint32_t dq = step / fast_count, dr = step - dq * fast_count;
+    auto advance = [&] {
+        q += dq;
+        rest += dr;
+        if (rest >= fast_count) {
+            rest -= fast_count;
+            ++q;
+        }
+    };
+    // this thread's line and the first inner index of the tile (BY_LINE: of the row)
+    auto place = [&](int64_t &line, int64_t &k0) {
         if constexpr (BY_LINE) {
-            const uint32_t row = item * kTileLines + 2 * warp, q = row / nchunks;
-            line0 = q;
-            k0 = static_cast<int64_t>(row - q * nchunks) * kChunk;
-            return;
-        }
-        const uint32_t q = item / (SIDE == 0 ? ltiles : nchunks), rest = item - q * (SIDE == 0 ? ltiles : nchunks);
-        line0 = static_cast<int64_t>(SIDE == 0 ? rest : q) * kTileLines;
-        k0 = static_cast<int64_t>(SIDE == 0 ? q : rest) * kChunk;
-    };
-    // BY_LINE: to the row behind that one, the next piece of the line or the first of the next line
-    auto next_row = [&](int64_t &line, int64_t &k0) {
-        k0 += kChunk;
-        if (k0 >= row_pitch) {
-            k0 = 0;
-            ++line;
+            line = q;
+            uint32_t chunk = rest;
+            if ((lane >> 4) && ++chunk == nchunks) {      // the row behind: next piece of the line, or the next line
+                chunk = 0;
+                ++line;
+            }
+            k0 = static_cast<int64_t>(chunk) * kChunk;
+        } else {
+            line = static_cast<int64_t>(SIDE == 0 ? rest : q) * kTileLines + li;
+            k0 = static_cast<int64_t>(SIDE == 0 ? q : rest) * kChunk;
         }
     };
-    auto request = [&](uint32_t item, int buf) {
-        int64_t line0, k0;
-        place(item, line0, k0);
-        int kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);        // <= 0: padding only
-        const uint32_t base = tile_addr + buf * (kTileDoubles * 8);
-        if (SIDE == 0) {
-            // 16 lanes take the lines of one inner index, a warp two indices at a time
-            const int l = lane & 15;
-            const int64_t line = line0 + l;
-            const bool live = line < lines && shift[line] != OZ_NONFINITE_SHIFT;
-            const int kk0 = 2 * warp + (lane >> 4);
-            const double *src = X + (live ? line : 0) + (k0 + kk0) * ldx;
+    // elements of a tile; rows beyond the lines and inner indices beyond k become zeros
+    auto request = [&](int buf) {
+        const uint32_t base = tile_addr + buf * kTileBytes;
+        if constexpr (SIDE == 0) {
+            const int64_t line0 = static_cast<int64_t>(rest) * kTileLines, k0 = static_cast<int64_t>(q) * kChunk;
+            if (pairs) {
+                // a thread copies lines 2c, 2c + 1 of inner indices kq + 32 u, octets kq / 8 + 4 u
+                const int c = threadIdx.x & 7, kq = threadIdx.x >> 3;
+                const uint32_t dst = base + ((kq & 7) * 16 + (kq >> 3)) * 128 + ((c ^ (kq >> 3)) << 4);
+                const double *src = X + line0 + 2 * c + (k0 + kq) * ldx;
+                if (line0 + kTileLines <= lines && k0 + kChunk <= k) {
 #pragma unroll
-            for (int u = 0; u < kChunk / 16; ++u) {
-                const int kk = kk0 + 16 * u;
-                const bool in = live && kk < kleft;
-                copy8(base + l * (kTilePitch * 8) + tile_chunk(warp + 8 * u) * 16 + (lane >> 4) * 8, in ? src + (16 * u) * ldx : X, in);
+                    for (int u = 0; u < 4; ++u) copy16((dst ^ ((u & 1) << 6)) + u * 512, src + 32 * u * ldx);
+                } else {
+                    const int64_t left = lines - (line0 + 2 * c);
+                    const int bytes = left >= 2 ? 16 : (left == 1 ? 8 : 0);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const bool in = bytes && k0 + kq + 32 * u < k;
+                        copy16((dst ^ ((u & 1) << 6)) + u * 512, in ? src + 32 * u * ldx : X, in ? bytes : 0);
+                    }
+                }
+            } else {
+                // line l of inner indices kq + 16 u, octets kq / 8 + 2 u
+                const int l = threadIdx.x & 15, kq = threadIdx.x >> 4;
+                const uint32_t dst = base + ((kq & 7) * 16 + (kq >> 3)) * 128 + (((l >> 1) ^ (kq >> 3)) << 4) + (l & 1) * 8;
+                const double *src = X + line0 + l + (k0 + kq) * ldx;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const bool in = line0 + l < lines && k0 + kq + 16 * u < k;
+                    copy8((dst ^ ((u & 3) << 5)) + u * 256, in ? src + 16 * u * ldx : X, in);
+                }
             }
         } else {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int li = warp * 2 + h;
+                int64_t line, k0;
                 if constexpr (BY_LINE) {
-                    if (h) next_row(line0, k0);
-                    kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);
+                    line = q;
+                    uint32_t chunk = rest;
+                    if (h && ++chunk == nchunks) {
+                        chunk = 0;
+                        ++line;
+                    }
+                    k0 = static_cast<int64_t>(chunk) * kChunk;
+                } else {
+                    line = static_cast<int64_t>(q) * kTileLines + warp * 2 + h;
+                    k0 = static_cast<int64_t>(rest) * kChunk;
                 }
-                const int64_t line = BY_LINE ? line0 : line0 + li;
-                const bool live = line < lines && shift[line] != OZ_NONFINITE_SHIFT;
+                const bool live = line < lines;
+                const int kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);        // <= 0: padding only
                 const double *src = X + (live ? line : 0) * ldx + k0;
-                const uint32_t row = base + li * (kTilePitch * 8);
+                const uint32_t row = base + (warp * 2 + h) * kTileRow;
                 if (pairs) {
 #pragma unroll
                     for (int u = 0; u < kChunk / 64; ++u) {
                         const int c = lane + 32 * u;
-                        const int left = live ? (kleft - 2 * c) * 8 : 0;
-                        const int bytes = left >= 16 ? 16 : (left > 0 ? left : 0);
-                        copy16(row + tile_chunk(c) * 16, bytes ? src + 2 * c : X, bytes);
+                        if (live && kleft == kChunk) {
+                            copy16(row + tile_chunk(c) * 16, src + 2 * c);
+                        } else {
+                            const int left = live ? (kleft - 2 * c) * 8 : 0;
+                            const int bytes = left >= 16 ? 16 : (left > 0 ? left : 0);
+                            copy16(row + tile_chunk(c) * 16, bytes ? src + 2 * c : X, bytes);
+                        }
                     }
                 } else {
 #pragma unroll
@@ -540,38 +582,52 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
     };
 
     int buf = 0;
-    if (blockIdx.x < items) request(blockIdx.x, 0);
+    int64_t line = 0, k0 = 0, next_line = 0, next_k0 = 0;
+    int sigma = 0, next_sigma = 0;
+    if (blockIdx.x < items) {
+        place(line, k0);
+        request(0);
+        sigma = line < lines ? shift[line] : 0;
+    }
     for (uint32_t item = blockIdx.x; item < items; item += gridDim.x, buf ^= 1) {
         const bool more = items - item > gridDim.x;
         if (more) {
-            request(item + gridDim.x, buf ^ 1);
+            advance();
+            place(next_line, next_k0);
+            request(buf ^ 1);
+            next_sigma = next_line < lines ? shift[next_line] : 0;
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();                 // this tile (and, the first time, the table) is there
-        int64_t line0, k0;
-        place(item, line0, k0);
-        const int li = warp * 2 + (lane >> 4);
-        if constexpr (BY_LINE) {
-            if (lane >> 4) next_row(line0, k0);
-        }
-        const int64_t line = BY_LINE ? line0 : line0 + li, kb = k0 + (lane & 15) * 8;
-        if (line < lines && kb < row_pitch) {
-            const int sigma_raw = shift[line];
-            const int sigma = sigma_raw == OZ_NONFINITE_SHIFT ? 0 : sigma_raw;     // such a line is zero in the tile
-            const double2 *row = reinterpret_cast<const double2 *>(tile + buf * kTileDoubles + li * kTilePitch);
+        if (line < lines && k0 + oct * 8 < row_pitch) {
             double x[8];
+            if constexpr (SIDE == 0) {
+                const double *src = reinterpret_cast<const double *>(smem_raw + buf * kTileBytes + oct * 128 + ((warp ^ (oct & 7)) << 4)) + (lane >> 4);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const double2 v = row[tile_chunk((lane & 15) * 4 + e)];
-                x[2 * e] = v.x;
-                x[2 * e + 1] = v.y;
+                for (int e = 0; e < 8; ++e) x[e] = src[e * 256];
+            } else {
+                const double2 *row = reinterpret_cast<const double2 *>(smem_raw + buf * kTileBytes + li * kTileRow);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const double2 v = row[tile_chunk(oct * 4 + e)];
+                    x[2 * e] = v.x;
+                    x[2 * e + 1] = v.y;
+                }
+            }
+            if (sigma == OZ_NONFINITE_SHIFT) {       // its planes are zeros
+                sigma = 0;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x[e] = 0.0;
             }
             convert8<SET, LAYOUT>(x, sigma, tz != 0, lut_addr,
-                                 planes + (k0 >> 7) * geom.chunk_stride + line * geom.line_stride + (kb & 127), geom.plane_stride);
+                                 planes + (k0 >> 7) * geom.chunk_stride + line * geom.line_stride + oct * 8, geom.plane_stride);
         }
         __syncthreads();                 // the tile may be overwritten
+        line = next_line;
+        k0 = next_k0;
+        sigma = next_sigma;
     }
 }
 
@@ -886,8 +942,8 @@ oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t 
                            const int32_t *shift, const uint32_t *lut, uint8_t *planes,
                            const PlaneGeom &geom, int tz, bool alone, cudaStream_t stream)
 {
-    constexpr size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * sizeof(double) * kTileLines * kTilePitch;
-    constexpr bool kByLine = SIDE == 1 && LAYOUT != kLayoutNative;
+    constexpr size_t smem = lut_words_of(SET, LAYOUT) * 4 + 2 * kTileBytes;
+    constexpr bool kByLine = SIDE == 1 && LAYOUT != kLayoutNative && !two_plane_layout(LAYOUT);
     static std::atomic<unsigned long long> ready[2] = {{0}, {0}};
     const bool by_line = kByLine && geom.line_stride != kChunk;
     const auto kernel = by_line ? convert_kernel<SET, SIDE, LAYOUT, kByLine> : convert_kernel<SET, SIDE, LAYOUT, false>;
@@ -1000,12 +1056,16 @@ oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const doub
     const uint32_t *lut = device_lut(set, rt.substrate);
 #define OZ_CONVERT(SET_, SIDE_, LAYOUT_)                                                                 \
     launch_convert<SET_, SIDE_, LAYOUT_>(X, ldx, lines, k, shift, lut, planes, geom, rt.quant, alone, stream)
-#define OZ_CONVERT_SET(SET_)                                                                             \
-    (side == 1 ? (layout == kLayoutMergedI8B ? OZ_CONVERT(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_CONVERT(SET_, 1, kLayoutDigitsI8)                    \
-                                             : OZ_CONVERT(SET_, 1, kLayoutDigits))                      \
-               : (layout == kLayoutMerged      ? OZ_CONVERT(SET_, 0, kLayoutMerged)                     \
-                  : layout == kLayoutMergedI8A ? OZ_CONVERT(SET_, 0, kLayoutMergedI8A) : layout == kLayoutDigitsI8 ? OZ_CONVERT(SET_, 0, kLayoutDigitsI8)                  \
-                                               : OZ_CONVERT(SET_, 0, kLayoutDigits)))
+#define OZ_CONVERT_SET(SET_)                                                                                          \
+    (layout == kLayoutDigits      ? (side == 0 ? OZ_CONVERT(SET_, 0, kLayoutDigits) : OZ_CONVERT(SET_, 1, kLayoutDigits))      \
+     : layout == kLayoutDigitsI8  ? (side == 0 ? OZ_CONVERT(SET_, 0, kLayoutDigitsI8) : OZ_CONVERT(SET_, 1, kLayoutDigitsI8))  \
+     : layout == kLayoutMerged    ? OZ_CONVERT(SET_, 0, kLayoutMerged)                                                   \
+     : layout == kLayoutMergedI8A ? OZ_CONVERT(SET_, 0, kLayoutMergedI8A)                                                \
+     : layout == kLayoutMergedI8B ? OZ_CONVERT(SET_, 1, kLayoutMergedI8B)                                                \
+     : layout == kLayoutTwo       ? OZ_CONVERT(SET_, 0, kLayoutTwo)                                                      \
+     : layout == kLayoutTwoI8     ? OZ_CONVERT(SET_, 0, kLayoutTwoI8)                                                    \
+     : layout == kLayoutFour      ? OZ_CONVERT(SET_, 1, kLayoutFour)                                                     \
+                                  : OZ_CONVERT(SET_, 1, kLayoutFourI8))
     const int layout = rt.layout(side);
     if (layout == kLayoutNative) return side == 0 ? OZ_CONVERT(2, 0, kLayoutNative) : OZ_CONVERT(2, 1, kLayoutNative);
     if (set == 0) return OZ_CONVERT_SET(0);
@@ -1027,12 +1087,16 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
         const FusedParams p = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, f.group);
         const int layout = rt.layout(side);
 #define OZ_FUSED(SET_, SIDE_, LAYOUT_) launch_fused<SET_, SIDE_, LAYOUT_>(p, f, alone, stream)
-#define OZ_FUSED_SET(SET_)                                                                      \
-    (side == 1 ? (layout == kLayoutMergedI8B ? OZ_FUSED(SET_, 1, kLayoutMergedI8B) : layout == kLayoutDigitsI8 ? OZ_FUSED(SET_, 1, kLayoutDigitsI8)             \
-                                             : OZ_FUSED(SET_, 1, kLayoutDigits))               \
-               : (layout == kLayoutMerged      ? OZ_FUSED(SET_, 0, kLayoutMerged)              \
-                  : layout == kLayoutMergedI8A ? OZ_FUSED(SET_, 0, kLayoutMergedI8A) : layout == kLayoutDigitsI8 ? OZ_FUSED(SET_, 0, kLayoutDigitsI8)           \
-                                               : OZ_FUSED(SET_, 0, kLayoutDigits)))
+#define OZ_FUSED_SET(SET_)                                                                                          \
+    (layout == kLayoutDigits      ? (side == 0 ? OZ_FUSED(SET_, 0, kLayoutDigits) : OZ_FUSED(SET_, 1, kLayoutDigits))      \
+     : layout == kLayoutDigitsI8  ? (side == 0 ? OZ_FUSED(SET_, 0, kLayoutDigitsI8) : OZ_FUSED(SET_, 1, kLayoutDigitsI8))  \
+     : layout == kLayoutMerged    ? OZ_FUSED(SET_, 0, kLayoutMerged)                                                   \
+     : layout == kLayoutMergedI8A ? OZ_FUSED(SET_, 0, kLayoutMergedI8A)                                                \
+     : layout == kLayoutMergedI8B ? OZ_FUSED(SET_, 1, kLayoutMergedI8B)                                                \
+     : layout == kLayoutTwo       ? OZ_FUSED(SET_, 0, kLayoutTwo)                                                      \
+     : layout == kLayoutTwoI8     ? OZ_FUSED(SET_, 0, kLayoutTwoI8)                                                    \
+     : layout == kLayoutFour      ? OZ_FUSED(SET_, 1, kLayoutFour)                                                     \
+                                  : OZ_FUSED(SET_, 1, kLayoutFourI8))
         if (layout == kLayoutNative) return side == 0 ? OZ_FUSED(2, 0, kLayoutNative) : OZ_FUSED(2, 1, kLayoutNative);
         if (set == 0) return OZ_FUSED_SET(0);
         if (set == 1) return OZ_FUSED_SET(1);
@@ -1075,6 +1139,8 @@ oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, in
     (layout == kLayoutMerged      ? launch_pair<SET_, kLayoutMerged, kLayoutDigits>(p, fa, fb, stream)      \
      : layout == kLayoutMergedI8A ? launch_pair<SET_, kLayoutMergedI8A, kLayoutMergedI8B>(p, fa, fb, stream) \
      : layout == kLayoutDigitsI8  ? launch_pair<SET_, kLayoutDigitsI8, kLayoutDigitsI8>(p, fa, fb, stream)  \
+     : layout == kLayoutTwo       ? launch_pair<SET_, kLayoutTwo, kLayoutFour>(p, fa, fb, stream)           \
+     : layout == kLayoutTwoI8     ? launch_pair<SET_, kLayoutTwoI8, kLayoutFourI8>(p, fa, fb, stream)       \
                                   : launch_pair<SET_, kLayoutDigits, kLayoutDigits>(p, fa, fb, stream))
     if (layout == kLayoutNative) return launch_pair<2, kLayoutNative, kLayoutNative>(p, fa, fb, stream);
     return set == 0 ? OZ_PAIR(0) : set == 1 ? OZ_PAIR(1) : OZ_PAIR(2);

@@ -82,6 +82,16 @@ struct Tile {
     static constexpr int STAGES = CG == 1 ? 4 : 6;               // 192 KiB ring either way
     static constexpr int TILE_J = BLOCK_M * CG;                  // columns of C per work item
 };
+// Two-plane schedule (SLIM, one tile of columns): a stage holds one of A's planes and the two tiles of B's planes that it
+// meets, one per accumulator.  SLIM is the number of lines of B that are loaded: with 64 a fourth stage fits.  The MMA
+// reads 128 lines all the same; those behind the 64 are whatever follows in the stage and end in columns that no one reads.
+template <int SLIM>
+struct SlimTile {
+    static constexpr int B_BYTES = SLIM * BLOCK_K;
+    static constexpr int STAGE_BYTES = 2 * B_BYTES + BLOCK_N * BLOCK_K;      // 64 or 48 KiB
+    static constexpr int STAGES = SLIM == 64 ? 4 : 3;                        // the same 192 KiB ring
+};
+static_assert(SlimTile<128>::STAGES * SlimTile<128>::STAGE_BYTES == 4 * 49152 && SlimTile<64>::STAGES * SlimTile<64>::STAGE_BYTES == 4 * 49152, "ring size");
 constexpr int TMEM_COLS = 512;                     // two accumulator slots of BLOCK_N columns
 constexpr int NUM_THREADS = 576;                   // 18 warps: 112 registers each fit the register file
 constexpr int FIRST_EPI_WARP = 2;                  // warp 0: producer, warp 1: MMA issuer
@@ -101,7 +111,7 @@ struct ModInfo {
     float w[3];           // weight of each job
     int reduce[3];        // reduce the accumulator modulo m before weighting (0: the exact FP32 range allows skipping it)
     int njobs;            // 2 (square), 3, 1 (native INT8 residues) or 2 (non-square, merged accumulators)
-    int kind;             // 0 square, 1 non-square separate, 2 native, 3 non-square merged
+    int kind;             // 0 square, 1 non-square separate, 2 native, 3 non-square merged, 4 / 5 non-square two-plane (SLIM)
     int planeA0, planeB0; // first stored plane of this modulus in A's and in B's plane arrays
     // Split-K inside the kernel: the K range of a job is cut into segments of whole chunks, each with
     // an accumulator of its own that is reduced before the next is added, so that every accumulator
@@ -387,6 +397,8 @@ __host__ __device__ constexpr uint32_t instr_desc()
            (static_cast<uint32_t>((BLOCK_M * CG) >> 4) << 24);
 }
 
+constexpr uint32_t kNegateB = 1u << 14;      // instruction descriptor: the second operand (planes of A) enters negated
+
 // work item -> (modulus, tile_m, tile_n): modulus-major so that one modulus' planes stay in L2;
 // inside a modulus, bands of 16 tile rows are swept column by column.
 struct Item { int mod, tm, tn; };
@@ -453,6 +465,23 @@ __device__ __forceinline__ void segment_range(const ModInfo &mi, int job, int se
     *kc1 = min(nk, *kc0 + len);
 }
 
+// Two-plane schedule: A's plane h = 0, 1 of a modulus and the planes of B that it is multiplied with, one for each
+// accumulator (first: -1 where the plane does not meet the first accumulator):
+//   square (kind 0):  d0 with e0 | e1,  d1 with - | e0:              d e = acc0 + s acc1
+//   kind 4:           d0 with e0 | e1,  d1 with f0 | f1:             d e = d0 e + d1 f,  f = 16 e mod m
+//   kind 5:           d0 with e0 | e1,  -16 d1 with -e0 | -e1:       planes of the merged layouts (kept operands)
+// with e = e0 + 16 e1, f = f0 + 16 f1:  d e = acc0 + 16 acc1 (mod m) for the non-squares.
+__device__ __forceinline__ void slim_stage(const ModInfo &mi, int h, int *first, int *second)
+{
+    if (mi.kind == 0) {
+        *first = h ? -1 : mi.planeB0;
+        *second = h ? mi.planeB0 : mi.planeB0 + 1;
+    } else {
+        *first = mi.planeB0 + (mi.kind == 4 ? 2 * h : 0);
+        *second = *first + 1;
+    }
+}
+
 // acc - m * rint(acc / m) for a pair of integer-valued floats below 2^24 (exact): rint through the
 // 1.5 * 2^23 constant, then one fused multiply-add
 __device__ __forceinline__ float2 mod_balanced2(float2 acc, float2 inv_m2, float2 neg_m2)
@@ -478,13 +507,18 @@ __device__ __forceinline__ float2 mod_balanced2(float2 acc, float2 inv_m2, float
 // BOUND: not a residue product but the magnitude-bound product of the accurate mode (Sec. 2 "The FP8
 //         variant", the "+1" pass): one plane per operand, one accumulator per tile, and instead of
 //         residues the epilogue reduces the row and column maxima of the tile into p.rowmax / p.colmax.
-template <int SUB, int CG, int RB, bool DIRECT, bool LOOSE, bool TILED, bool BOUND = false>
+// SLIM:    two-plane schedule of a product with one tile of columns (n <= 128), which reads A's planes from memory once
+//         and does little arithmetic with them: d = d0 + 16 d1 of a non-square modulus meets all of e (see kind 4, 5 in
+//         slim_stage()), so that dS is never read.  Both accumulators of a modulus fill in one K-loop, per K segment.
+template <int SUB, int CG, int RB, bool DIRECT, bool LOOSE, bool TILED, bool BOUND = false, int SLIM = 0>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ GemmParams p)
 {
-    constexpr int STAGES = Tile<CG>::STAGES;
-    constexpr int STAGE_BYTES = Tile<CG>::STAGE_BYTES;
+    static_assert(SLIM == 0 || (CG == 1 && !DIRECT && TILED && !BOUND), "two-plane schedule: whole-method digit products");
+    using Slim = SlimTile<SLIM ? SLIM : 128>;
+    constexpr int STAGES = SLIM ? Slim::STAGES : Tile<CG>::STAGES;
+    constexpr int STAGE_BYTES = SLIM ? Slim::STAGE_BYTES : Tile<CG>::STAGE_BYTES;
     // CTA pair: rank 0 leads (issues the MMAs, owns the `full` and `tmem-empty` barriers that both
     // CTAs signal); work items are dealt to pairs, so both CTAs walk the same item sequence.
     const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
@@ -559,6 +593,23 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                     return true;
                 };
+                if constexpr (SLIM != 0) {
+                    for (int kc = 0; ok && kc < p.nk; ++kc)
+                        for (int h = 0; ok && h < 2; ++h) {
+                            ok = mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status);
+                            if (!ok) break;
+                            const uint32_t fb = full_bar + 8 * stage, sa = tiles + stage * STAGE_BYTES;
+                            int first, second;
+                            slim_stage(mi, h, &first, &second);
+                            mbar_expect_tx(fb, first >= 0 ? STAGE_BYTES : STAGE_BYTES - Slim::B_BYTES);
+                            const int x = kc * p.kc_x, z = kc * p.kc_z;
+                            tma_load_3d(sa + 2 * Slim::B_BYTES, &mapA, fb, x, it.tm * BLOCK_N, (mi.planeA0 + h) * p.plane_z + z);
+                            if (first >= 0) tma_load_3d(sa, &mapB, fb, x, it.tn * BLOCK_M, first * p.plane_z + z);
+                            tma_load_3d(sa + Slim::B_BYTES, &mapB, fb, x, it.tn * BLOCK_M, second * p.plane_z + z);
+                            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                        }
+                    continue;
+                }
                 if (!DIRECT && p.pair_squares && mi.kind == 0) {
                     // the two planes of a chunk in two stages, side by side
                     for (int kc = 0; ok && kc < p.nk; ++kc)
@@ -592,6 +643,39 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             for (int64_t item = first_item; ok && item < p.total_items; item += item_step) {
                 Item it = decode_item(item, p);
                 const ModInfo &mi = p.mod[it.mod];
+                if constexpr (SLIM != 0) {
+                    // kind 5: A's second plane is -16 d1, which the tensor core negates
+                    const uint32_t idesc1 = mi.kind == 5 ? idesc | kNegateB : idesc;
+                    for (int seg = 0; ok && seg < mi.nseg_all; ++seg) {
+                        for (int h = 0; ok && h < 2; ++h)
+                            ok = mbar_wait(tempty_bar + 8 * h, ((slot_phase >> h) & 1u) ^ 1u, abort_flag, p.status);
+                        if (!ok) break;
+                        tc_fence_after();
+                        const int kc0 = seg * mi.seg_len_all, kc1 = min(p.nk, kc0 + mi.seg_len_all);
+                        for (int st = 0; st < 2 * (kc1 - kc0); ++st) {
+                            const int h = st & 1;
+                            ok = mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t sa = tiles + stage * STAGE_BYTES;
+                            const uint64_t e0 = smem_desc(sa), e1 = smem_desc(sa + Slim::B_BYTES), a = smem_desc(sa + 2 * Slim::B_BYTES);
+#pragma unroll
+                            for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
+                                const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
+                                const uint32_t accumulate = st > 0 || ks > 0 ? 1u : 0u, id = h ? idesc1 : idesc;
+                                if (mi.kind != 0 || h == 0) umma<SUB, CG>(tmem_base, e0 + o, a + o, id, accumulate);
+                                umma<SUB, CG>(tmem_base + BLOCK_N, e1 + o, a + o, id, accumulate);
+                            }
+                            umma_commit<CG>(empty_bar + 8 * stage);
+                            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                        }
+                        if (!ok) break;
+                        umma_commit<CG>(tfull_bar);
+                        umma_commit<CG>(tfull_bar + 8);
+                        slot_phase ^= 3u;
+                    }
+                    continue;
+                }
                 if (!DIRECT && p.pair_squares && mi.kind == 0) {
                     // d0 e0 into one slot, d1 e0 + d0 e1 into the other, from the four tiles of a chunk
                     for (int h = 0; ok && h < 2; ++h)
@@ -686,8 +770,11 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
 #pragma unroll
                 for (int c = 0; c < COLS_PER_WARP; ++c) comb[c] = 0u;
             }
-            for (int job = 0; ok && job < mi.njobs; ++job)
-            for (int seg = 0, nseg = job_segments(mi, job); ok && seg < nseg; ++seg) {
+            // SLIM: both jobs of a K segment before the next segment
+            const int outer = SLIM ? mi.nseg_all : mi.njobs;
+            for (int o = 0; ok && o < outer; ++o)
+            for (int i = 0, inner = SLIM ? 2 : job_segments(mi, o); ok && i < inner; ++i) {
+                const int job = SLIM ? i : o;
                 // every lane polls for itself; the outcome is made warp-uniform before anything that
                 // contains a warp barrier depends on it
                 ok = __all_sync(0xFFFFFFFFu, mbar_wait(tfull_bar + 8 * slot, (slot_phase >> slot) & 1u, abort_flag, p.status));
@@ -1001,12 +1088,12 @@ oz_status_t launch_fused_variant(const CUtensorMap &mapB, const GemmParams &p, c
     return OZ_OK;
 }
 
-template <int SUB, int CG, int RB, bool DIRECT = false, bool LOOSE = false, bool TILED = false, bool BOUND = false>
+template <int SUB, int CG, int RB, bool DIRECT = false, bool LOOSE = false, bool TILED = false, bool BOUND = false, int SLIM = 0>
 oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, const GemmParams &p, int sms,
                            cudaStream_t stream)
 {
     static_assert(!LOOSE || RB == 2, "a representative below 2m needs the two-byte element");
-    auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, LOOSE, TILED, BOUND>;
+    auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, LOOSE, TILED, BOUND, SLIM>;
     static std::atomic<unsigned long long> ready{0};
     OZ_CUDA_CHECK(allow_shared(kernel, SMEM_BYTES, ready));
     int64_t groups = sms / CG;                                    // CTAs, or CTA pairs
@@ -1064,7 +1151,7 @@ static int take_stall_flag()
 // Per-modulus constants of the epilogue and the accumulator schedule (jobs, weights, which
 // accumulators are reduced before they are weighted, K segments) for inner dimension k; p.r and p.nk
 // (chunks of BLOCK_K) are set by the caller.
-static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k)
+static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k, bool slim = false)
 {
     for (int i = 0; i < p.r; ++i) {
         const int mi = modulus(set, i), s = kSetTables.root[set][i];
@@ -1109,6 +1196,25 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k)
             mo.reduce[0] = (skip_all || (!split && 256 * kk + static_cast<int64_t>(s) * red <= lim)) ? 0 : 1;
             mo.reduce[1] = skip_all ? 0 : 1;
             mo.reduce[2] = 1;
+        } else if (slim) {
+            // d e = acc0 + 16 acc1.  Planes d0, d1 against e and f: terms 8 8 + 16 8 and 8 16 + 16 16.  Planes of the merged
+            // layouts, d0 and -16 d1 (Lemma 1: |d0| <= 14, |d1| <= 16 on the 9-bit tail, 8 and 8 on bytes): 14 14 + 256 14 and
+            // 14 16 + 256 16, or 8 8 + 128 8 in both, and K segments that keep these exact.
+            mo.njobs = 2;
+            mo.kind = rt.two_plane() ? 4 : 5;
+            mo.w[0] = 1.0f; mo.w[1] = 16.0f; mo.w[2] = 0.0f;
+            const int64_t t0 = mo.kind == 4 ? 192 : (mi > 256 ? 3780 : 1088), t1 = mo.kind == 4 ? 384 : (mi > 256 ? 4320 : 1088);
+            if (mo.kind == 5) {
+                const int seg_max = static_cast<int>((1 << 24) / t1 / BLOCK_K);
+                mo.nseg_all = (p.nk + seg_max - 1) / seg_max;
+                mo.seg_len_all = (p.nk + mo.nseg_all - 1) / mo.nseg_all;
+            }
+            const int64_t first = 16 * red * mo.nseg_all;     // the other accumulator's part once it is reduced
+            const bool one = mo.nseg_all == 1;
+            const bool skip_all = one && (t0 + 16 * t1) * kk <= lim;
+            mo.reduce[0] = (skip_all || (one && t0 * kk + first <= lim)) ? 0 : 1;
+            mo.reduce[1] = skip_all ? 0 : 1;
+            mo.reduce[2] = 1;
         } else if (rt.merged()) {
             // d e = -15 [d0 e0 - 16 d1 e1] + 16 dS eS; merged term <= 4095 (9-bit tail) or 1088 (bytes).
             // INT8 planes hold -d0 and 4*d1, so the accumulator is the NEGATIVE of the bracket (weight
@@ -1140,6 +1246,21 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k)
         }
         for (int j = 0; j < 3; ++j) mo.iw[j] = static_cast<int>(mo.w[j]);
     }
+}
+
+bool two_plane_applies(int64_t m, int64_t n, int64_t k, const Route &rt)
+{
+    return rt.automatic && rt.merged() && !rt.fused && n <= BLOCK_M && m >= n;
+}
+
+// Kept operands (planes of the merged layouts): a fifth less of A from memory for a sixth more products, and K segments on set S.
+// Taken up to 64 columns, and where the tiles cover the SMs or one segment holds k (10240 x 64 x 10240 a call, S: 554 -> 524 us,
+// 4000 x 64 x 4000 142 -> 124, 1500 x 16 x 6000 on E 97 -> 88; not 1000 x 32 x 12000 on S: 143 against 149, nor 100 columns:
+// 4000 x 100 x 4000 146 against 154).
+static bool slim_merged(int64_t m, int64_t n, int64_t k, int set, int sms)
+{
+    const int64_t tiles = set_r(set) * ((m + BLOCK_N - 1) / BLOCK_N);
+    return n <= 64 && (tiles >= sms || k <= (set == 0 ? 3840 : 15360));
 }
 
 ResidueTiling residue_tiling(int64_t m, int64_t n, int set)
@@ -1174,7 +1295,8 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     p.R = R; p.ldr = ldr; p.mod_stride = mod_stride;
     p.stall_producer = take_stall_flag();
     p.status = device_status_word();
-    fill_mod_info(p, set, rt, k);
+    const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(m, n, k, set, sm_count())));
+    fill_mod_info(p, set, rt, k, slim);
     // Squares in one K-loop: the products of a square read d0 and e0 twice, so job after job a K chunk costs six tiles;
     // with both accumulators open it costs four.  The drains of the two slots no longer hide behind each other's K-loop,
     // which costs less than the tiles at every size measured: 10240 x 64 x 10240 with a kept operator (DRAM) 680 -> 620 us a
@@ -1189,7 +1311,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
         const int chunks = static_cast<int>(pitchA / BLOCK_K);
         p.kc_x = 0; p.plane_z = chunks; p.kc_z = 1;
         maps = make_plane_map(&mapA, PA, m, BLOCK_K, BLOCK_K * m, planesA * chunks, BLOCK_N / cg) &&
-               make_plane_map(&mapB, PB, n, BLOCK_K, BLOCK_K * n, planesB * chunks, BLOCK_M);
+               make_plane_map(&mapB, PB, n, BLOCK_K, BLOCK_K * n, planesB * chunks, slim && n <= 64 ? 64 : BLOCK_M);
     } else {
         p.kc_x = BLOCK_K; p.plane_z = 1; p.kc_z = 0;
         maps = make_plane_map(&mapA, PA, m, pitchA, strideA, planesA, BLOCK_N / cg) &&
@@ -1207,6 +1329,13 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     // one accumulator per modulus of at most 128 * 128 * k <= 2^30: the direct drain with the exact division
     if (rt.native() && p.mod[0].nseg_all == 1 && k <= 65536)
         return tiled ? OZ_LAUNCH(1, 1, true, false, true) : OZ_LAUNCH(1, 1, true, false, false);
+    if (slim) {
+#define OZ_SLIM(SUB, RB) (n <= 64 ? launch_variant<SUB, 1, RB, false, RB == 2, true, false, 64>(mapA, mapB, p, sms, stream) \
+                                  : launch_variant<SUB, 1, RB, false, RB == 2, true, false, 128>(mapA, mapB, p, sms, stream))
+        if (rb == 1) return rt.substrate == 0 ? OZ_SLIM(0, 1) : OZ_SLIM(1, 1);
+        return rt.substrate == 0 ? OZ_SLIM(0, 2) : OZ_SLIM(1, 2);
+#undef OZ_SLIM
+    }
     if (rb == 1) return tiled ? OZ_LAUNCH_SUB(1, false, true) : OZ_LAUNCH_SUB(1, false, false);
     // the tile-ordered array is private to the whole-method calls, which also take the loose residues
     if (tiled) return OZ_LAUNCH_SUB(2, true, true);

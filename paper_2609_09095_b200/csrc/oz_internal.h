@@ -52,12 +52,18 @@ __host__ __device__ constexpr int square_root(int m)
 //                  not fit a byte: both operands carry 4*d1 in place of d1 and the A operand -d0
 //                  in place of d0, so that (-d0) e0 + (4 d1)(4 e1) = -(d0 e0 - 16 d1 e1)
 //   kLayoutDigitsI8  kLayoutDigits with INT8 instead of E4M3 bytes
+//   kLayoutTwo / kLayoutFour (and their INT8 forms)  the two-plane schedule of the whole-method calls with few columns:
+//                  A holds d0 and d1 of every modulus, B the digits e0, e1 of e and, for a non-square, f0, f1 of
+//                  f = 16 e mod m.  Digits to the base s (squares) or 16, each rounded to nearest: the schedule needs no
+//                  digit sums, so no carry of Lemma 1 and no table
 constexpr int kLayoutDigits = 0, kLayoutNative = 1, kLayoutMerged = 2, kLayoutMergedI8A = 3,
-              kLayoutMergedI8B = 4, kLayoutDigitsI8 = 5;
+              kLayoutMergedI8B = 4, kLayoutDigitsI8 = 5, kLayoutTwo = 6, kLayoutTwoI8 = 7, kLayoutFour = 8, kLayoutFourI8 = 9;
+constexpr int kNumLayouts = 10;
+__host__ __device__ constexpr bool two_plane_layout(int layout) { return layout >= kLayoutTwo; }
 
 __host__ __device__ constexpr int planes_of(int m, int layout = kLayoutDigits)
 {
-    return layout == kLayoutNative ? 1 : (square_root(m) ? 2 : 3);
+    return layout == kLayoutNative ? 1 : (square_root(m) || layout == kLayoutTwo || layout == kLayoutTwoI8) ? 2 : two_plane_layout(layout) ? 4 : 3;
 }
 
 __host__ __device__ constexpr int first_plane(int set, int i, int layout = kLayoutDigits)
@@ -76,7 +82,7 @@ __host__ __device__ constexpr int p_store(int set, int layout = kLayoutDigits)
 // set and search square roots).
 struct SetTables {
     int root[3][kMaxR];                         // square root of a square modulus, 0 otherwise
-    int first[3][6][kMaxR + 1];                 // first plane of modulus i per layout; [r]: the number of planes
+    int first[3][kNumLayouts][kMaxR + 1];               // first plane of modulus i per layout; [r]: the number of planes
 };
 constexpr SetTables make_set_tables()
 {
@@ -84,8 +90,8 @@ constexpr SetTables make_set_tables()
     for (int set = 0; set < 3; ++set)
         for (int i = 0; i < set_r(set); ++i) {
             t.root[set][i] = square_root(modulus(set, i));
-            for (int layout = 0; layout < 6; ++layout)
-                t.first[set][layout][i + 1] = t.first[set][layout][i] + (layout == kLayoutNative ? 1 : (t.root[set][i] ? 2 : 3));
+            for (int layout = 0; layout < kNumLayouts; ++layout)
+                t.first[set][layout][i + 1] = t.first[set][layout][i] + planes_of(modulus(set, i), layout);
         }
     return t;
 }
@@ -113,8 +119,11 @@ __host__ __device__ constexpr int lut_offset(int set, int i)
 __host__ __device__ constexpr int lut_words(int set) { return (lut_offset(set, set_r(set)) + 3) / 4 * 4; }
 static_assert(lut_words(0) <= kLutWords && lut_words(1) <= kLutWords && lut_words(2) <= kLutWords, "table size");
 
-// table words that a conversion into `layout` needs: native residues need none
-__host__ __device__ constexpr int lut_words_of(int set, int layout) { return layout == kLayoutNative ? 0 : lut_words(set); }
+// table words that a conversion into `layout` needs: native residues and the two-plane schedule need none
+__host__ __device__ constexpr int lut_words_of(int set, int layout)
+{
+    return layout == kLayoutNative || two_plane_layout(layout) ? 0 : lut_words(set);
+}
 
 // 2^e mod m
 __host__ __device__ constexpr uint32_t pow2_mod(int e, uint32_t m)
@@ -135,13 +144,16 @@ inline int64_t round_up(int64_t v, int64_t a) { return (v + a - 1) / a * a; }
 // ---- route decoding ----------------------------------------------------------------------
 struct Route {
     int substrate;  // 0 fp8, 1 int8 (two-limb digits), 2 int8 native (one residue plane, set A only)
-    int acc;        // 0 unspecified, 1 merged accumulators, 2 separate accumulators
+    int acc;        // 0 unspecified, 1 merged accumulators, 2 separate accumulators, 3 two-plane schedule (internal)
+    bool automatic; // the schedule was left to the library
     bool native() const { return substrate == 2; }
     bool merged() const { return acc == 1; }
+    bool two_plane() const { return acc == 3; }
     // plane layout of the operand on `side` (0: rows of A, 1: columns of B)
     int layout(int side) const
     {
         if (native()) return kLayoutNative;
+        if (two_plane()) return (side == 0 ? kLayoutTwo : kLayoutFour) + (substrate == 1 ? 1 : 0);
         if (!merged()) return substrate == 1 ? kLayoutDigitsI8 : kLayoutDigits;
         if (substrate == 1) return side == 0 ? kLayoutMergedI8A : kLayoutMergedI8B;
         return side == 0 ? kLayoutMerged : kLayoutDigits;
@@ -245,6 +257,9 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
                                 int64_t strideB, int64_t pitchB, int set, const Route &rt,
                                 void *R, int64_t ldr, int64_t mod_stride, bool loose, bool tiled,
                                 cudaStream_t stream);
+
+// Whether a whole-method call takes the two-plane schedule (planes private to the call, schedule left to the library)
+bool two_plane_applies(int64_t m, int64_t n, int64_t k, const Route &rt);
 
 // Storage mode F: residue products with A converted on the fly inside the kernel (n <= 128, merged
 // schedule on digit planes, k within the exact depth of one accumulator); public residue layout
