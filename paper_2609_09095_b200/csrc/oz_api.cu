@@ -244,14 +244,6 @@ oz_status_t ensure_device_ready()
     g_status_addr[dev] = static_cast<unsigned int *>(p);
     oz_status_t st = upload_reconstruct_constants();
     if (st != OZ_OK) return st;
-    unsigned char codes[33];
-    for (int d = 0; d <= 32; ++d) {
-        int code = 0;
-        e4m3_code(d, &code);            // odd digits above 16 are never produced
-        codes[d] = static_cast<unsigned char>(code);
-    }
-    st = upload_bound_codes(codes);
-    if (st != OZ_OK) return st;
     st = upload_hosted_constants();
     if (st != OZ_OK) return st;
     // A copy from pageable memory may return before it has arrived, and the first kernels may be on a stream that does not wait
@@ -510,16 +502,13 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         // Accurate mode: exponent scans, one magnitude plane per operand (kept in the first plane slot
         // of each operand, which the conversion overwrites afterwards), the bound product on the
         // tensor cores, the shifts from its row and column maxima, then the conversion as usual.
-        st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, true, stream);
-        if (st == OZ_OK) st = launch_scan(1, n, k, B, ldb, set, rt, b.shift, b.scratch, true, stream);
-        if (st == OZ_OK) st = launch_bound_plane(0, m, k, A, lda, a.scratch, a.planes, a.pitch, stream);
-        if (st == OZ_OK) st = launch_bound_plane(1, n, k, B, ldb, b.scratch, b.planes, b.pitch, stream);
+        const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
+        st = launch_scan(&ja, &jb, k, set, rt, true, stream);
+        if (st == OZ_OK) st = launch_bound_planes(ja, a.planes, jb, b.planes, k, a.pitch, stream);
         if (st == OZ_OK)
             st = launch_bound_gemm(m, n, k, a.planes, a.pitch, b.planes, b.pitch, bound_maxima(a.scratch, m),
                                    bound_maxima(b.scratch, n), stream);
-        const int budget = accurate_budget_log2(set);
-        if (st == OZ_OK) st = launch_accurate_finalize(m, a.scratch, budget, a.shift, stream);
-        if (st == OZ_OK) st = launch_accurate_finalize(n, b.scratch, budget, b.shift, stream);
+        if (st == OZ_OK) st = launch_accurate_finalize(ja, jb, accurate_budget_log2(set), stream);
         if (st == OZ_OK)
             st = launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, true, stream);
         if (ev && st == OZ_OK) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
@@ -536,7 +525,8 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
         if (st != OZ_OK) return st;
         OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-        st = launch_scan(0, m, k, A, lda, set, rt, a.shift, a.scratch, false, stream);
+        const ScanJob ja{m, A, lda, a.shift, a.scratch};
+        st = launch_scan(&ja, nullptr, k, set, rt, false, stream);
         if (st != OZ_OK) return st;
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
         OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
@@ -558,12 +548,20 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
         return product_impl(m, n, k, alpha, a, b, beta, C, ldc, set, rt, stream, ws + L.R, dev, plan);
     }
+    const bool scans = three_passes(0, m, k, set, rt) && three_passes(1, n, k, set, rt);
+    if (scans) {      // both operands in one launch per pass; the conversions then run side by side
+        const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
+        st = launch_scan(&ja, &jb, k, set, rt, true, stream);
+        if (st != OZ_OK) return st;
+    }
     OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
     OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
-    st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
+    st = scans ? launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, false, side)
+               : launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
     if (st != OZ_OK) return st;
     OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-    st = launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, false, stream);
+    st = scans ? launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, false, stream)
+               : launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, false, stream);
     if (st != OZ_OK) return st;
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
     OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));

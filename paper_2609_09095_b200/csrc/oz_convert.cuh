@@ -16,7 +16,7 @@ namespace {
 // Eq. 1 for one element, integer form (any sigma): a' = quant(x 2^sigma) as a 64-bit integer.  While 2^sigma is a normal
 // double, split_limbs() multiplies by it instead: exact in FP64 (a product that underflows is far below 1/2 and rounds to
 // zero either way), and the hardware conversion rounds to nearest-even or toward zero.
-__device__ __forceinline__ long long quantise(double x, int sigma, bool tz)
+__device__ __noinline__ long long quantise(double x, int sigma, bool tz)
 {
     unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
     int be = static_cast<int>((bits >> 52) & 0x7FF);
@@ -95,43 +95,35 @@ __device__ __forceinline__ void limb_fields(long long a, float &f0, float &f1, f
     f3 = __uint_as_float((hi >> 13) | 0x4B000000u);
 }
 
+template <int NP>
+__device__ __forceinline__ void limb_pair(long long a0, long long a1, int q, Limbs<NP> &L)
+{
+    constexpr float k23 = 8388608.0f;
+    float f0[2], f1[2], f2[2], f3[2];
+    limb_fields(a0, f0[0], f1[0], f2[0], f3[0], L.low[2 * q]);
+    limb_fields(a1, f0[1], f1[1], f2[1], f3[1], L.low[2 * q + 1]);
+    L.l0[q] = __fadd2_rn(make_float2(f0[0], f0[1]), make_float2(-(k23 + 32768.0f), -(k23 + 32768.0f)));
+    L.l1[q] = __fadd2_rn(make_float2(f1[0], f1[1]), make_float2(-(k23 + 16384.0f), -(k23 + 16384.0f)));
+    L.l2[q] = __fadd2_rn(make_float2(f2[0], f2[1]), make_float2(-(k23 + 8192.0f), -(k23 + 8192.0f)));
+    L.l3[q] = __fadd2_rn(make_float2(f3[0], f3[1]), make_float2(-(k23 + 262144.0f), -(k23 + 262144.0f)));
+}
+
 // limbs of the quantised values of 2 NP elements
 template <int NP>
 __device__ __forceinline__ void split_limbs(const double (&x)[2 * NP], int sigma, bool tz, Limbs<NP> &L)
 {
-    long long a[2 * NP];
     if (sigma >= -1000 && sigma <= 1000) {       // 2^sigma is a normal number (always, except for lines of subnormals)
         const double scale = __hiloint2double((1023 + sigma) << 20, 0);
         if (!tz) {
 #pragma unroll
-            for (int e = 0; e < 2 * NP; ++e) a[e] = __double2ll_rn(x[e] * scale);
+            for (int q = 0; q < NP; ++q) limb_pair(__double2ll_rn(x[2 * q] * scale), __double2ll_rn(x[2 * q + 1] * scale), q, L);
         } else {
 #pragma unroll
-            for (int e = 0; e < 2 * NP; ++e) a[e] = __double2ll_rz(x[e] * scale);
+            for (int q = 0; q < NP; ++q) limb_pair(__double2ll_rz(x[2 * q] * scale), __double2ll_rz(x[2 * q + 1] * scale), q, L);
         }
     } else {
-#pragma unroll 1
-        for (int e = 0; e < 2 * NP; ++e) {
-            double v = x[0];
 #pragma unroll
-            for (int f = 1; f < 2 * NP; ++f) v = e == f ? x[f] : v;
-            const long long w = quantise(v, sigma, tz);
-#pragma unroll
-            for (int f = 0; f < 2 * NP; ++f) a[f] = e == f ? w : a[f];
-        }
-    }
-    constexpr float k23 = 8388608.0f;
-    const float2 o0 = make_float2(-(k23 + 32768.0f), -(k23 + 32768.0f)), o1 = make_float2(-(k23 + 16384.0f), -(k23 + 16384.0f));
-    const float2 o2 = make_float2(-(k23 + 8192.0f), -(k23 + 8192.0f)), o3 = make_float2(-(k23 + 262144.0f), -(k23 + 262144.0f));
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        float f0[2], f1[2], f2[2], f3[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) limb_fields(a[2 * q + e], f0[e], f1[e], f2[e], f3[e], L.low[2 * q + e]);
-        L.l0[q] = __fadd2_rn(make_float2(f0[0], f0[1]), o0);
-        L.l1[q] = __fadd2_rn(make_float2(f1[0], f1[1]), o1);
-        L.l2[q] = __fadd2_rn(make_float2(f2[0], f2[1]), o2);
-        L.l3[q] = __fadd2_rn(make_float2(f3[0], f3[1]), o3);
+        for (int q = 0; q < NP; ++q) limb_pair(quantise(x[2 * q], sigma, tz), quantise(x[2 * q + 1], sigma, tz), q, L);
     }
 }
 

@@ -228,18 +228,24 @@ struct OperandJob {
 oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, int64_t k, int set, const Route &rt,
                                     bool *taken, cudaStream_t stream);
 
-// pieces of launch_deconstruct, and the steps of the accurate rule between them
-oz_status_t launch_scan(int side, int64_t lines, int64_t k, const double *X, int64_t ldx, int set,
-                        const Route &rt, int32_t *shift, void *scratch, bool alone, cudaStream_t stream);
+// pieces of launch_deconstruct, and the steps of the accurate rule between them.  The scans take side 0 (a), side 1 (b) or both.
+struct ScanJob {
+    int64_t lines;
+    const double *X;
+    int64_t ldx;
+    int32_t *shift;
+    void *scratch;
+};
+// whether launch_deconstruct() takes the scans and the conversion (else the one-kernel form)
+bool three_passes(int side, int64_t lines, int64_t k, int set, const Route &rt);
+oz_status_t launch_scan(const ScanJob *a, const ScanJob *b, int64_t k, int set, const Route &rt, bool alone, cudaStream_t stream);
 oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                   int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
                                   const int32_t *shift, bool alone, cudaStream_t stream);
-oz_status_t launch_bound_plane(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
-                               void *scratch, uint8_t *plane, int64_t pitch, cudaStream_t stream);
+oz_status_t launch_bound_planes(const ScanJob &a, uint8_t *planeA, const ScanJob &b, uint8_t *planeB, int64_t k, int64_t pitch,
+                                cudaStream_t stream);
 unsigned int *bound_maxima(void *scratch, int64_t lines);      // one word per line, word stride 2
-oz_status_t launch_accurate_finalize(int64_t lines, void *scratch, int budget_log2, int32_t *shift,
-                                     cudaStream_t stream);
-oz_status_t upload_bound_codes(const unsigned char *codes33);
+oz_status_t launch_accurate_finalize(const ScanJob &a, const ScanJob &b, int budget_log2, cudaStream_t stream);
 // the bound product on the tensor cores: rowmax[2 i] / colmax[2 j] receive (atomicMax) the bit pattern
 // of max_j / max_i of sum_k GA[i][k] GB[j][k], an integer-valued FP32 number; k <= kBoundKMax
 constexpr int64_t kBoundKMax = 16384;
