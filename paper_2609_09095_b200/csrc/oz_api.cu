@@ -397,7 +397,7 @@ oz_status_t product_impl(int64_t m, int64_t n, int64_t k, double alpha, const Op
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][2], stream));
     // the residues stay inside this call: tile-ordered, and the two-byte sets skip the canonicalisation
     oz_status_t st = launch_residue_gemm(m, n, k, a.planes, a.stride, a.pitch, b.planes, b.stride, b.pitch, set,
-                                         rt, R, 0, 0, residue_bytes(set) == 2, true, stream);
+                                         rt, R, 0, 0, true, stream);
     if (st != OZ_OK) return st;
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][3], stream));
     // the CRT recombination: exact FP64 chunk sums on the FP64 pipe, or (OZ_RECON_TENSOR) one small
@@ -993,7 +993,7 @@ oz_status_t oz_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA, 
     oz_status_t st = ensure_device_ready();
     if (st != OZ_OK) return st;
     return launch_residue_gemm(m, n, k, PA, strideA, pitchA, PB, strideB, pitchB, set, rt, R, ldr,
-                               mod_stride, false, false, static_cast<cudaStream_t>(stream));
+                               mod_stride, false, static_cast<cudaStream_t>(stream));
 }
 
 oz_status_t oz_reconstruct(int64_t m, int64_t n, const void *R, int64_t ldr, int64_t mod_stride,

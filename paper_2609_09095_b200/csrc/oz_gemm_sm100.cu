@@ -63,9 +63,11 @@ namespace oz {
 namespace {
 
 constexpr int BLOCK_M = 128;                       // MMA M: columns j of C (lines of B)
-constexpr int BLOCK_N = 256;                       // MMA N: rows i of C (lines of A)
+constexpr int BLOCK_N = 256;                       // MMA N: rows i of C (lines of A); NARROW_N where tiles are few
+constexpr int NARROW_N = 64;
 constexpr int BLOCK_K = 128;                       // bytes = elements (8-bit operands)
 constexpr int UMMA_K = 32;                         // 8-bit operands: 32 elements per instruction
+constexpr int RING_BYTES = 4 * 49152;              // the shared-memory ring: 192 KiB, whatever a stage holds
 constexpr int A_BYTES = BLOCK_M * BLOCK_K;         // 16 KiB: MMA operand a = 128 lines of B's planes per CTA
 
 // CG = 1: one CTA per tile of 128 columns x 256 rows of C.
@@ -74,37 +76,34 @@ constexpr int A_BYTES = BLOCK_M * BLOCK_K;         // 16 KiB: MMA operand a = 12
 //         of the 256 lines of A's planes (operand b), the tensor core reads both halves, and each
 //         CTA's TMEM holds the accumulators of its own 128 columns.  Per CTA this halves the
 //         shared-memory traffic of operand b and the TMA bytes per MMA.
-template <int CG>
+template <int CG, int BN = BLOCK_N>
 struct Tile {
-    static constexpr int B_LINES = BLOCK_N / CG;                 // lines of A's planes loaded per CTA
+    static constexpr int B_LINES = BN / CG;                     // lines of A's planes loaded per CTA
     static constexpr int B_BYTES = B_LINES * BLOCK_K;            // 32 KiB / 16 KiB
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;        // 48 KiB / 32 KiB
-    static constexpr int STAGES = CG == 1 ? 4 : 6;               // 192 KiB ring either way
+    static constexpr int STAGES = RING_BYTES / STAGE_BYTES;      // 4 / 6, narrow tiles 8 / 9
     static constexpr int TILE_J = BLOCK_M * CG;                  // columns of C per work item
 };
 // Two-plane schedule (SLIM, one tile of columns): a stage holds one of A's planes and the two tiles of B's planes that it
 // meets, one per accumulator.  SLIM is the number of lines of B that are loaded: with 64 a fourth stage fits.  The MMA
 // reads 128 lines all the same; those behind the 64 are whatever follows in the stage and end in columns that no one reads.
-template <int SLIM>
+template <int SLIM, int BN = BLOCK_N>
 struct SlimTile {
     static constexpr int B_BYTES = SLIM * BLOCK_K;
-    static constexpr int STAGE_BYTES = 2 * B_BYTES + BLOCK_N * BLOCK_K;      // 64 or 48 KiB
-    static constexpr int STAGES = SLIM == 64 ? 4 : 3;                        // the same 192 KiB ring
+    static constexpr int STAGE_BYTES = 2 * B_BYTES + BN * BLOCK_K;           // 64 or 48 KiB
+    static constexpr int STAGES = RING_BYTES / STAGE_BYTES;                  // 3 or 4, narrow tiles 4 or 8
 };
-static_assert(SlimTile<128>::STAGES * SlimTile<128>::STAGE_BYTES == 4 * 49152 && SlimTile<64>::STAGES * SlimTile<64>::STAGE_BYTES == 4 * 49152, "ring size");
 constexpr int TMEM_COLS = 512;                     // two accumulator slots of BLOCK_N columns
 constexpr int NUM_THREADS = 576;                   // 18 warps: 112 registers each fit the register file
 constexpr int FIRST_EPI_WARP = 2;                  // warp 0: producer, warp 1: MMA issuer
 constexpr int EPI_WARPS = 16;
-constexpr int COLS_PER_WARP = BLOCK_N / 4;         // four warps share a TMEM lane quarter
 #ifndef OZ_DRAIN_W
 #define OZ_DRAIN_W 16
 #endif
 constexpr int DRAIN_W = OZ_DRAIN_W;                // accumulator columns per tcgen05.ld of a drain: 64 running
                                                    // values + 16 loaded ones stay inside the 96 registers
 constexpr int XPOSE_BYTES = 16 * 128;                // per epilogue warp: 16 lines x 128 bytes
-constexpr size_t SMEM_BYTES = 4 * 49152 + EPI_WARPS * XPOSE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
-static_assert(Tile<1>::STAGES * Tile<1>::STAGE_BYTES == 4 * 49152 && Tile<2>::STAGES * Tile<2>::STAGE_BYTES == 4 * 49152, "ring size");
+constexpr size_t SMEM_BYTES = RING_BYTES + EPI_WARPS * XPOSE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 
 struct ModInfo {
     float m, inv_m;
@@ -388,12 +387,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr)
 }
 
 // instruction descriptor: D format, A/B formats, K-major both, N/8 at bit 17, M/16 at bit 24
-template <int SUB, int CG>
+template <int SUB, int CG, int BN = BLOCK_N>
 __host__ __device__ constexpr uint32_t instr_desc()
 {
     uint32_t cfmt = SUB == 0 ? 1u /*f32*/ : 2u /*s32*/;
     uint32_t abfmt = SUB == 0 ? 0u /*e4m3*/ : 1u /*s8*/;
-    return (cfmt << 4) | (abfmt << 7) | (abfmt << 10) | (static_cast<uint32_t>(BLOCK_N >> 3) << 17) |
+    return (cfmt << 4) | (abfmt << 7) | (abfmt << 10) | (static_cast<uint32_t>(BN >> 3) << 17) |
            (static_cast<uint32_t>((BLOCK_M * CG) >> 4) << 24);
 }
 
@@ -507,18 +506,22 @@ __device__ __forceinline__ float2 mod_balanced2(float2 acc, float2 inv_m2, float
 // BOUND: not a residue product but the magnitude-bound product of the accurate mode (Sec. 2 "The FP8
 //         variant", the "+1" pass): one plane per operand, one accumulator per tile, and instead of
 //         residues the epilogue reduces the row and column maxima of the tile into p.rowmax / p.colmax.
+// BN:      rows of C per tile: 256, or 64 for products with so few tiles that most SMs would be idle (narrow_tiles())
 // SLIM:    two-plane schedule of a product with one tile of columns (n <= 128), which reads A's planes from memory once
 //         and does little arithmetic with them: d = d0 + 16 d1 of a non-square modulus meets all of e (see kind 4, 5 in
 //         slim_stage()), so that dS is never read.  Both accumulators of a modulus fill in one K-loop, per K segment.
-template <int SUB, int CG, int RB, bool DIRECT, bool LOOSE, bool TILED, bool BOUND = false, int SLIM = 0>
+template <int SUB, int CG, int RB, bool DIRECT, bool LOOSE, bool TILED, bool BOUND = false, int SLIM = 0, int BN = BLOCK_N>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ GemmParams p)
 {
     static_assert(SLIM == 0 || (CG == 1 && !DIRECT && TILED && !BOUND), "two-plane schedule: whole-method digit products");
-    using Slim = SlimTile<SLIM ? SLIM : 128>;
-    constexpr int STAGES = SLIM ? Slim::STAGES : Tile<CG>::STAGES;
-    constexpr int STAGE_BYTES = SLIM ? Slim::STAGE_BYTES : Tile<CG>::STAGE_BYTES;
+    static_assert(BN == BLOCK_N || TILED, "narrow tiles: whole-method products");
+    using Slim = SlimTile<SLIM ? SLIM : 128, BN>;
+    constexpr int STAGES = SLIM ? Slim::STAGES : Tile<CG, BN>::STAGES;
+    constexpr int STAGE_BYTES = SLIM ? Slim::STAGE_BYTES : Tile<CG, BN>::STAGE_BYTES;
+    constexpr int COLS_PER_WARP = BN / 4;                // four warps share a TMEM lane quarter
+    static_assert(16 * STAGES + 48 <= 256, "barriers");
     // CTA pair: rank 0 leads (issues the MMAs, owns the `full` and `tmem-empty` barriers that both
     // CTAs signal); work items are dealt to pairs, so both CTAs walk the same item sequence.
     const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
@@ -527,13 +530,13 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t tiles = (raw + 1023u) & ~1023u;                     // 1024-byte aligned ring
-    const uint32_t bars = tiles + STAGES * STAGE_BYTES + EPI_WARPS * XPOSE_BYTES;
+    const uint32_t bars = tiles + RING_BYTES + EPI_WARPS * XPOSE_BYTES;
     const uint32_t full_bar = bars;                                   // STAGES x 8 bytes
     const uint32_t empty_bar = bars + 8 * STAGES;
     const uint32_t tfull_bar = bars + 16 * STAGES;                    // 2 x 8
     const uint32_t tempty_bar = tfull_bar + 16;                       // 2 x 8
     const uint32_t tmem_slot = tempty_bar + 16;                       // 4 bytes: TMEM base address
-    unsigned char *xpose_base = smem_raw + (tiles - raw) + STAGES * STAGE_BYTES;
+    unsigned char *xpose_base = smem_raw + (tiles - raw) + RING_BYTES;
     unsigned char *gen = xpose_base + EPI_WARPS * XPOSE_BYTES;
     volatile uint32_t *tmem_base_ptr = reinterpret_cast<volatile uint32_t *>(gen + 16 * STAGES + 32);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + 16 * STAGES + 40);
@@ -580,7 +583,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     if (CG == 1) {
                         mbar_expect_tx(fb, STAGE_BYTES);
                         tma_load_3d(sa, &mapB, fb, kc * p.kc_x, it.tn * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
-                        tma_load_3d(sa + A_BYTES, &mapA, fb, kc * p.kc_x, it.tm * BLOCK_N, pa * p.plane_z + kc * p.kc_z);
+                        tma_load_3d(sa + A_BYTES, &mapA, fb, kc * p.kc_x, it.tm * BN, pa * p.plane_z + kc * p.kc_z);
                     } else {
                         // both CTAs' copies complete on the leader's barrier
                         if (rank == 0) mbar_expect_tx(fb, 2 * STAGE_BYTES);
@@ -588,7 +591,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                         tma_load_3d_pair(sa, &mapB, fb_leader, kc * p.kc_x,
                                          it.tn * Tile<CG>::TILE_J + static_cast<int>(rank) * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
                         tma_load_3d_pair(sa + A_BYTES, &mapA, fb_leader, kc * p.kc_x,
-                                         it.tm * BLOCK_N + static_cast<int>(rank) * Tile<CG>::B_LINES, pa * p.plane_z + kc * p.kc_z);
+                                         it.tm * BN + static_cast<int>(rank) * Tile<CG, BN>::B_LINES, pa * p.plane_z + kc * p.kc_z);
                     }
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                     return true;
@@ -603,7 +606,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                             slim_stage(mi, h, &first, &second);
                             mbar_expect_tx(fb, first >= 0 ? STAGE_BYTES : STAGE_BYTES - Slim::B_BYTES);
                             const int x = kc * p.kc_x, z = kc * p.kc_z;
-                            tma_load_3d(sa + 2 * Slim::B_BYTES, &mapA, fb, x, it.tm * BLOCK_N, (mi.planeA0 + h) * p.plane_z + z);
+                            tma_load_3d(sa + 2 * Slim::B_BYTES, &mapA, fb, x, it.tm * BN, (mi.planeA0 + h) * p.plane_z + z);
                             if (first >= 0) tma_load_3d(sa, &mapB, fb, x, it.tn * BLOCK_M, first * p.plane_z + z);
                             tma_load_3d(sa + Slim::B_BYTES, &mapB, fb, x, it.tn * BLOCK_M, second * p.plane_z + z);
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -634,7 +637,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             }
         } else if (warp == 1 && lane == 0 && rank == 0) {
             // -------------------------------------------------------- MMA issuer (pair: leader CTA only)
-            constexpr uint32_t idesc = instr_desc<SUB, CG>();
+            constexpr uint32_t idesc = instr_desc<SUB, CG, BN>();
             int stage = 0;
             uint32_t phase = 0;
             int slot = 0;
@@ -786,9 +789,13 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                                        static_cast<uint32_t>(slot * BLOCK_N + part * COLS_PER_WARP);
                 if constexpr (DIRECT) {
                     // the only accumulator of this modulus lands in the combination registers as it is
-                    tmem_ld32_issue<0>(taddr, comb);
-                    tmem_ld32_issue<32>(taddr + 32, comb);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if constexpr (COLS_PER_WARP == 64) {
+                        tmem_ld32_issue<0>(taddr, comb);
+                        tmem_ld32_issue<32>(taddr + 32, comb);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    } else {
+                        tmem_ld16(taddr, comb);
+                    }
                 } else
 #pragma unroll
                 for (int c0 = 0; c0 < COLS_PER_WARP; c0 += DRAIN_W) {
@@ -851,7 +858,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             // this thread: column j of C, rows i0 .. i0+63 (contiguous in the residue array)
             const int64_t jw = static_cast<int64_t>(it.tn) * Tile<CG>::TILE_J + rank * BLOCK_M + q * 32;   // first column of the warp
             const int64_t j = jw + lane;
-            const int64_t i0 = static_cast<int64_t>(it.tm) * BLOCK_N + part * COLS_PER_WARP;
+            const int64_t i0 = static_cast<int64_t>(it.tm) * BN + part * COLS_PER_WARP;
             if (i0 >= p.m || jw >= p.n) continue;                                 // warp-uniform
             if constexpr (BOUND) {
                 // The accumulators are non-negative integers held exactly in FP32: their bit patterns
@@ -918,9 +925,11 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             if constexpr (TILED) {
                 // block (tile, CTA rank, warp), then modulus: the r residue blocks of one 32 x 64 patch of
                 // the output lie next to one another, which is how the reconstruction reads them
+                const int64_t tile = i0 / BLOCK_N;                   // the layout's tiles have 256 rows, its blocks 64
+                const int block = (static_cast<int>(i0 >> 6) & 3) * 4 + q, chunk0 = static_cast<int>(i0 & 63) * RB / 16;
                 unsigned char *blk = static_cast<unsigned char *>(p.R) +
-                    (((((static_cast<int64_t>(it.tm) * p.tiles_n + it.tn) * CG + rank) * EPI_WARPS + (part * 4 + q)) * p.r +
-                      it.mod) * static_cast<int64_t>(NCH * 512)) + lane * 16;
+                    ((((tile * p.tiles_n + it.tn) * CG + rank) * EPI_WARPS + block) * p.r + it.mod) * static_cast<int64_t>(64 * RB * 32) +
+                    chunk0 * 512 + lane * 16;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
                     uint4 val;
@@ -1088,12 +1097,12 @@ oz_status_t launch_fused_variant(const CUtensorMap &mapB, const GemmParams &p, c
     return OZ_OK;
 }
 
-template <int SUB, int CG, int RB, bool DIRECT = false, bool LOOSE = false, bool TILED = false, bool BOUND = false, int SLIM = 0>
+template <int SUB, int CG, int RB, bool DIRECT = false, bool LOOSE = false, bool TILED = false, bool BOUND = false, int SLIM = 0, int BN = BLOCK_N>
 oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, const GemmParams &p, int sms,
                            cudaStream_t stream)
 {
     static_assert(!LOOSE || RB == 2, "a representative below 2m needs the two-byte element");
-    auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, LOOSE, TILED, BOUND, SLIM>;
+    auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, LOOSE, TILED, BOUND, SLIM, BN>;
     static std::atomic<unsigned long long> ready{0};
     OZ_CUDA_CHECK(allow_shared(kernel, SMEM_BYTES, ready));
     int64_t groups = sms / CG;                                    // CTAs, or CTA pairs
@@ -1116,6 +1125,39 @@ oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, con
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
+}
+
+
+// Whole-method products (tile-ordered residues): the variants of one substrate, residue width and tile height
+template <int SUB, int RB, bool DIRECT, int BN>
+oz_status_t launch_tiled(const CUtensorMap &mapA, const CUtensorMap &mapB, const GemmParams &p, int cg, bool slim, int sms, cudaStream_t stream)
+{
+    constexpr bool LOOSE = RB == 2;
+    if constexpr (!DIRECT) {
+        if (slim)
+            return p.n <= 64 ? launch_variant<SUB, 1, RB, false, LOOSE, true, false, 64, BN>(mapA, mapB, p, sms, stream)
+                             : launch_variant<SUB, 1, RB, false, LOOSE, true, false, 128, BN>(mapA, mapB, p, sms, stream);
+    }
+    return cg == 2 ? launch_variant<SUB, 2, RB, DIRECT, LOOSE, true, false, 0, BN>(mapA, mapB, p, sms, stream)
+                   : launch_variant<SUB, 1, RB, DIRECT, LOOSE, true, false, 0, BN>(mapA, mapB, p, sms, stream);
+}
+
+template <int SUB, int RB, bool DIRECT>
+oz_status_t launch_tiled(const CUtensorMap &mapA, const CUtensorMap &mapB, const GemmParams &p, int cg, bool slim, bool narrow, int sms,
+                         cudaStream_t stream)
+{
+    return narrow ? launch_tiled<SUB, RB, DIRECT, NARROW_N>(mapA, mapB, p, cg, slim, sms, stream)
+                  : launch_tiled<SUB, RB, DIRECT, BLOCK_N>(mapA, mapB, p, cg, slim, sms, stream);
+}
+
+// Tiles of 64 rows instead of 256 where the rounds over the SMs then cost less.  A narrow tile is bound by its operands' way
+// from L2 to shared memory, of which it needs 5/8 per K chunk (20 of 32 KiB), not by its quarter of the products.
+bool narrow_tiles(int64_t m, int64_t tiles_n, int r, int cg, int sms)
+{
+    const int64_t groups = sms / cg;
+    const int64_t wide = (r * tiles_n * ((m + BLOCK_N - 1) / BLOCK_N) + groups - 1) / groups;
+    const int64_t narrow = (r * tiles_n * ((m + NARROW_N - 1) / NARROW_N) + groups - 1) / groups;
+    return 5 * narrow < 8 * wide;
 }
 
 }  // namespace
@@ -1278,13 +1320,16 @@ ResidueTiling residue_tiling(int64_t m, int64_t n, int set)
 oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA, int64_t strideA,
                                 int64_t pitchA, const uint8_t *PB, int64_t strideB, int64_t pitchB,
                                 int set, const Route &rt, void *R, int64_t ldr,
-                                int64_t mod_stride, bool loose, bool tiled, cudaStream_t stream)
+                                int64_t mod_stride, bool tiled, cudaStream_t stream)
 {
     const int cg = cta_group_choice(n);
     GemmParams p{};
     p.m = m; p.n = n; p.k = k;
-    p.tiles_m = static_cast<int>((m + BLOCK_N - 1) / BLOCK_N);             // 256 rows of C per tile
     p.tiles_n = static_cast<int>((n + BLOCK_M * cg - 1) / (BLOCK_M * cg)); // 128 (256) columns of C per tile
+    const int sms = sm_count();
+    const bool narrow = tiled && narrow_tiles(m, p.tiles_n, set_r(set), cg, sms);
+    const int rows = narrow ? NARROW_N : BLOCK_N;                          // rows of C per tile
+    p.tiles_m = static_cast<int>((m + rows - 1) / rows);
     const int rb = residue_bytes(set);
     p.vec_store = ((ldr * rb) % 16 == 0 && (mod_stride * rb) % 16 == 0 && (reinterpret_cast<uintptr_t>(R) & 15u) == 0) ? 1 : 0;
     p.nk = static_cast<int>((k + BLOCK_K - 1) / BLOCK_K);
@@ -1295,7 +1340,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     p.R = R; p.ldr = ldr; p.mod_stride = mod_stride;
     p.stall_producer = take_stall_flag();
     p.status = device_status_word();
-    const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(m, n, k, set, sm_count())));
+    const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(m, n, k, set, sms)));
     fill_mod_info(p, set, rt, k, slim);
     // Squares in one K-loop: the products of a square read d0 and e0 twice, so job after job a K chunk costs six tiles;
     // with both accumulators open it costs four.  The drains of the two slots no longer hide behind each other's K-loop,
@@ -1310,7 +1355,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     if (tiled) {       // private layout: one 128-byte column of lines per (plane, chunk); both operands have the same pitch
         const int chunks = static_cast<int>(pitchA / BLOCK_K);
         p.kc_x = 0; p.plane_z = chunks; p.kc_z = 1;
-        maps = make_plane_map(&mapA, PA, m, BLOCK_K, BLOCK_K * m, planesA * chunks, BLOCK_N / cg) &&
+        maps = make_plane_map(&mapA, PA, m, BLOCK_K, BLOCK_K * m, planesA * chunks, rows / cg) &&
                make_plane_map(&mapB, PB, n, BLOCK_K, BLOCK_K * n, planesB * chunks, slim && n <= 64 ? 64 : BLOCK_M);
     } else {
         p.kc_x = BLOCK_K; p.plane_z = 1; p.kc_z = 0;
@@ -1319,29 +1364,22 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     }
     if (!maps) return OZ_ERR_CUDA;
 
-    const int sms = sm_count();
-    // substrate 0: FP8 planes; otherwise INT8 planes (two-limb digits or native residues)
-#define OZ_LAUNCH(SUB, RB, DIRECT, LOOSE, TILED)                                                    \
-    (cg == 2 ? launch_variant<SUB, 2, RB, DIRECT, LOOSE, TILED>(mapA, mapB, p, sms, stream)        \
-             : launch_variant<SUB, 1, RB, DIRECT, LOOSE, TILED>(mapA, mapB, p, sms, stream))
-#define OZ_LAUNCH_SUB(RB, LOOSE, TILED)                                                             \
-    (rt.substrate == 0 ? OZ_LAUNCH(0, RB, false, LOOSE, TILED) : OZ_LAUNCH(1, RB, false, LOOSE, TILED))
     // one accumulator per modulus of at most 128 * 128 * k <= 2^30: the direct drain with the exact division
-    if (rt.native() && p.mod[0].nseg_all == 1 && k <= 65536)
-        return tiled ? OZ_LAUNCH(1, 1, true, false, true) : OZ_LAUNCH(1, 1, true, false, false);
-    if (slim) {
-#define OZ_SLIM(SUB, RB) (n <= 64 ? launch_variant<SUB, 1, RB, false, RB == 2, true, false, 64>(mapA, mapB, p, sms, stream) \
-                                  : launch_variant<SUB, 1, RB, false, RB == 2, true, false, 128>(mapA, mapB, p, sms, stream))
-        if (rb == 1) return rt.substrate == 0 ? OZ_SLIM(0, 1) : OZ_SLIM(1, 1);
-        return rt.substrate == 0 ? OZ_SLIM(0, 2) : OZ_SLIM(1, 2);
-#undef OZ_SLIM
+    const bool direct = rt.native() && p.mod[0].nseg_all == 1 && k <= 65536;
+    // substrate 0: FP8 planes; otherwise INT8 planes (two-limb digits or native residues)
+    if (tiled) {       // private to the whole-method calls, which also take the loose residues
+#define OZ_TILED(SUB, RB, DIRECT) launch_tiled<SUB, RB, DIRECT>(mapA, mapB, p, cg, slim, narrow, sms, stream)
+        if (direct) return OZ_TILED(1, 1, true);
+        if (rb == 1) return rt.substrate == 0 ? OZ_TILED(0, 1, false) : OZ_TILED(1, 1, false);
+        return rt.substrate == 0 ? OZ_TILED(0, 2, false) : OZ_TILED(1, 2, false);
+#undef OZ_TILED
     }
-    if (rb == 1) return tiled ? OZ_LAUNCH_SUB(1, false, true) : OZ_LAUNCH_SUB(1, false, false);
-    // the tile-ordered array is private to the whole-method calls, which also take the loose residues
-    if (tiled) return OZ_LAUNCH_SUB(2, true, true);
-    if (loose) return OZ_LAUNCH_SUB(2, true, false);
-    return OZ_LAUNCH_SUB(2, false, false);
-#undef OZ_LAUNCH_SUB
+#define OZ_LAUNCH(SUB, RB, DIRECT)                                                                  \
+    (cg == 2 ? launch_variant<SUB, 2, RB, DIRECT>(mapA, mapB, p, sms, stream)                      \
+             : launch_variant<SUB, 1, RB, DIRECT>(mapA, mapB, p, sms, stream))
+    if (direct) return OZ_LAUNCH(1, 1, true);
+    if (rb == 1) return rt.substrate == 0 ? OZ_LAUNCH(0, 1, false) : OZ_LAUNCH(1, 1, false);
+    return rt.substrate == 0 ? OZ_LAUNCH(0, 2, false) : OZ_LAUNCH(1, 2, false);
 #undef OZ_LAUNCH
 }
 

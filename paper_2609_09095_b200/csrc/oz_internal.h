@@ -256,12 +256,12 @@ int accurate_budget_log2(int set);
 // exponent-span check: threshold of the set against the product of the two operands' flatness codes
 unsigned int esc_threshold(int set);
 
-// loose: residues in [0, 2 m_i) (two-byte sets); tiled: R is the tile-ordered private array (ldr and
-// mod_stride are then ignored) and the planes are in the private layout
+// tiled: R is the tile-ordered private array (ldr and mod_stride are then ignored), with residues in [0, 2 m_i) for the
+// two-byte sets, and the planes are in the private layout
 oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA,
                                 int64_t strideA, int64_t pitchA, const uint8_t *PB,
                                 int64_t strideB, int64_t pitchB, int set, const Route &rt,
-                                void *R, int64_t ldr, int64_t mod_stride, bool loose, bool tiled,
+                                void *R, int64_t ldr, int64_t mod_stride, bool tiled,
                                 cudaStream_t stream);
 
 // Whether a whole-method call takes the two-plane schedule (planes private to the call, schedule left to the library)
