@@ -152,6 +152,22 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
     return v;
 }
 
+// The table in shared memory.  A look-up's byte offset comes out of FP32 arithmetic as the bit pattern of a denormal, exact while
+// those bits stay below 2^24.  Near: the table's address is part of that sum.  Far: in a cluster a block's shared addresses carry its
+// rank above bit 24, so the address is added to the offset as an integer.
+struct NearTable {
+    uint32_t addr;
+    __device__ __forceinline__ float base(uint32_t words) const { return __uint_as_float(addr + 4 * words); }
+    __device__ __forceinline__ uint32_t at(uint32_t bits) const { return lds_u32(bits); }
+    __device__ __forceinline__ uint32_t word(uint32_t i) const { return lds_u32(addr + 4 * i); }
+};
+struct FarTable {
+    uint32_t addr;
+    __device__ __forceinline__ float base(uint32_t words) const { return __uint_as_float(4 * words); }
+    __device__ __forceinline__ uint32_t at(uint32_t bits) const { return lds_u32(addr + bits); }
+    __device__ __forceinline__ uint32_t word(uint32_t i) const { return lds_u32(addr + 4 * i); }
+};
+
 // two E4M3 bytes (x in the low one); every digit is representable, so nothing is rounded
 __device__ __forceinline__ uint32_t e4m3_pair(float2 d)
 {
@@ -169,7 +185,8 @@ __device__ __forceinline__ uint32_t pack_low_bytes(uint32_t a, uint32_t b, uint3
 template <int N>
 __device__ __forceinline__ void store_words(uint8_t *out, const uint32_t (&w)[N])
 {
-    if constexpr (N == 2) *reinterpret_cast<uint2 *>(out) = make_uint2(w[0], w[1]);
+    if constexpr (N == 4) *reinterpret_cast<uint4 *>(out) = make_uint4(w[0], w[1], w[2], w[3]);
+    else if constexpr (N == 2) *reinterpret_cast<uint2 *>(out) = make_uint2(w[0], w[1]);
     else *reinterpret_cast<uint32_t *>(out) = w[0];
 }
 
@@ -197,9 +214,9 @@ __device__ __forceinline__ void digit_words(const float2 (&r)[2], uint32_t &w0, 
 // One modulus (compile-time index I of set SET) for 2 NP consecutive inner-dimension elements: residues,
 // digits, and 1, 2 or 3 plane stores of 2 NP bytes.  Digits come from the table for the power-of-two and the
 // non-square moduli (Lemma 1's carry makes the latter irregular) and from one more rounded division for the
-// odd squares.  lut: shared-memory address of the set's table.
-template <int SET, int LAYOUT, int I, int NP>
-__device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut, uint8_t *out, int64_t plane_stride)
+// odd squares.  lut: the set's table.
+template <int SET, int LAYOUT, int I, int NP, class Table>
+__device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, const Table &lut, uint8_t *out, int64_t plane_stride)
 {
     static_assert(NP % 2 == 0, "whole words");
     constexpr uint32_t m = modulus(SET, I);
@@ -223,7 +240,7 @@ __device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut
         }
         store_words(out + plane * plane_stride, w);
     } else if constexpr (two_plane_layout(LAYOUT)) {
-        // 6.3 instructions per element and modulus, and no shared memory (9 with the table, whose look-ups conflict)
+        // no table: 121 thread-instructions per element of A on set S where three planes take 127 and conflicting look-ups
         constexpr bool four = s == 0 && (LAYOUT == kLayoutFour || LAYOUT == kLayoutFourI8);
         constexpr int base = s ? s : 16;
         uint32_t w[4][NW];
@@ -272,16 +289,16 @@ __device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut
             if constexpr (pow2) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    t[e] = lds_u32(lut + 4 * lut_offset(SET, I) + ((L.low[4 * g + e] & (m - 1)) << 2));
+                    t[e] = lut.word(lut_offset(SET, I) + (L.low[4 * g + e] & (m - 1)));
             } else {
                 // byte offset 4 (r + bias) as the bits of a denormal: one multiply-add, no conversion
                 constexpr int bias = static_cast<int>(m / 2) + kLutGuard;
-                const float2 base = dup(__uint_as_float(lut + 4 * (lut_offset(SET, I) + bias)));
+                const float2 base = dup(lut.base(lut_offset(SET, I) + bias));
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float2 a = __ffma2_rn(residue_pair<SET, I>(L, 2 * g + h), dup(0x1p-147f), base);
-                    t[2 * h] = lds_u32(__float_as_uint(a.x));
-                    t[2 * h + 1] = lds_u32(__float_as_uint(a.y));
+                    t[2 * h] = lut.at(__float_as_uint(a.x));
+                    t[2 * h + 1] = lut.at(__float_as_uint(a.y));
                 }
             }
             const uint32_t t01 = __byte_perm(t[0], t[1], 0x5140), t23 = __byte_perm(t[2], t[3], 0x5140);
@@ -299,8 +316,8 @@ __device__ __forceinline__ void convert_modulus(const Limbs<NP> &L, uint32_t lut
     }
 }
 
-template <int SET, int LAYOUT, int NP, int... I>
-__device__ __forceinline__ void convert_all_moduli(std::integer_sequence<int, I...>, const Limbs<NP> &L, uint32_t lut,
+template <int SET, int LAYOUT, int NP, class Table, int... I>
+__device__ __forceinline__ void convert_all_moduli(std::integer_sequence<int, I...>, const Limbs<NP> &L, const Table &lut,
                                                    uint8_t *out, int64_t plane_stride)
 {
     (convert_modulus<SET, LAYOUT, I>(L, lut, out, plane_stride), ...);

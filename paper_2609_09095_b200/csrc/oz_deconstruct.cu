@@ -1,13 +1,14 @@
 // Deconstruction (Algorithm 2; scaling of Eq. 1): FP64 operand -> per-line shifts and K-major
 // 8-bit residue planes.
 //
-// Kernels, in launch order for one operand:
+// Kernels of the three-pass form, in launch order (the scans serve both operands of a product at once where both take it):
 //   scan_init      clears the per-line scratch (largest exponent, non-finite flag, sum of squares)
-//   scan_maxexp    largest floor(log2|x|) of every line, Inf/NaN detection
-//   scan_sumsq     CS rule only: exact integer sum of ceil(|x| 2^(9-E))^2 per line
+//   scan pass 0    largest floor(log2|x|) of every line, Inf/NaN detection
+//   scan pass 1    CS rule only: exact integer sum of ceil(|x| 2^(9-E))^2 per line
 //   scan_finalize  shift[line] (sigma_i or tau_j of Eq. 1)
 //   convert        quantise, reduce modulo every modulus, split into digits, store the planes
-// Small operands take one kernel instead of the five, both operands of a product together where they fit.
+// Small operands take one kernel instead of the five, both operands of a product together where they fit; lines that fit a
+// cluster's shared memory are read once by deconstruct_cluster_kernel.
 //
 // The scan is split over the inner dimension with integer atomics (max / or / add), so its
 // result does not depend on the order of the partial results: the shifts are bit-reproducible.
@@ -98,7 +99,7 @@ struct ScanSide {
 };
 
 // The scans take one operand or both operands of a product in one launch: blocks [0, a.blocks) serve side 0, the others
-// side 1 (2048^3 under the accurate rule: thirteen dependent launches before, nine now, 421 -> 370 us a call).
+// side 1 (2048^3 under the accurate rule: thirteen dependent launches before, nine now, 383 -> 345 us a call).
 __global__ void scan_init_kernel(ScanScratch sa, int64_t linesA, ScanScratch sb, int64_t linesB)
 {
     dependency_release();
@@ -389,8 +390,8 @@ __device__ __forceinline__ uint32_t bound_digit(double x, const BoundLine &b)
 // One byte per element: the E4M3 code of its magnitude digit, K-major like the residue planes
 // (out[line * pitch + kk]; bytes kk in [k, pitch) are zero), both operands in one launch.  A block takes 32 lines x 64 inner
 // indices of side 0, loaded along the lines, or 8 lines x 256 of side 1, one line a warp; the bytes go through shared memory
-// so that pieces of 64 and 256 bytes are stored.  Bound by DRAM: 2048 x 2048, both operands, 18 + 16 us with integer digits
-// from a table in constant memory, one element and barrier at a time -> 13 us.
+// so that pieces of 64 and 256 bytes are stored.  (18 + 16 us for two 2048 x 2048 operands when the digits were 64-bit shifts, their
+// codes came from constant memory at divergent addresses and a thread had four elements between two barriers.)
 struct BoundSide {
     const double *X;
     int64_t ldx, lines;
@@ -475,13 +476,13 @@ __global__ void accurate_finalize_kernel(const __grid_constant__ FinalizeSide a,
     shift[i] = ((L - clog) >> 1) + 4 - E;
 }
 
-// Eight consecutive inner-dimension elements of one line -> 8 bytes of every stored plane.
-template <int SET, int LAYOUT>
-__device__ __forceinline__ void convert8(const double (&x)[8], int sigma, bool tz, uint32_t lut, uint8_t *out,
-                                         int64_t plane_stride)
+// 2 NP consecutive inner-dimension elements of one line -> 2 NP bytes of every stored plane.
+template <int SET, int LAYOUT, int NP, class Table>
+__device__ __forceinline__ void convert(const double (&x)[2 * NP], int sigma, bool tz, const Table &lut, uint8_t *out,
+                                        int64_t plane_stride)
 {
-    Limbs<4> L;
-    split_limbs<4>(x, sigma, tz, L);
+    Limbs<NP> L;
+    split_limbs<NP>(x, sigma, tz, L);
     convert_all_moduli<SET, LAYOUT>(std::make_integer_sequence<int, set_r(SET)>{}, L, lut, out, plane_stride);
 }
 
@@ -494,8 +495,8 @@ __device__ __forceinline__ void load_table(uint32_t *lut, const uint32_t *__rest
 }
 
 // Side 1: 16-byte chunk of a tile row that holds the element pair c: the eight lanes of a quarter warp, which read
-// chunks 4 l + e (l = 0..7), then hit eight different bank groups
-__device__ __forceinline__ int tile_chunk(int c) { return c ^ ((c >> 3) & 3); }
+// chunks 4 l + e or 8 l + e (l = 0..7), then hit eight different bank groups
+__device__ __forceinline__ int tile_chunk(int c) { return c ^ ((c >> 3) & 7); }
 
 // asynchronous copies of one (8 bytes) or two (16 bytes) elements; nothing is read and zeros are written for bytes = 0
 __device__ __forceinline__ void copy8(uint32_t dst, const double *src, bool live)
@@ -511,18 +512,122 @@ __device__ __forceinline__ void copy16(uint32_t dst, const double *src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
+// The block's copies of a tile of 16 lines x 128 inner indices; what lies beyond the lines or beyond k becomes zeros.
+// Side 0 keeps a tile as [index in an octet][octet][line], 128 bytes a row, the 16-byte pieces of a row XORed with half the
+// octet's number: two lines travel in one copy, and neither the copies nor the reads, of one or two octets at compile-time
+// offsets from one address, conflict.
+__device__ __forceinline__ void request_side0(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k, bool pairs,
+                                              int64_t line0, int64_t k0, uint32_t base)
+{
+    if (pairs) {
+        // a thread copies lines 2c, 2c + 1 of inner indices kq + 32 u, octets kq / 8 + 4 u
+        const int c = threadIdx.x & 7, kq = threadIdx.x >> 3;
+        const uint32_t dst = base + ((kq & 7) * 16 + (kq >> 3)) * 128 + ((c ^ (kq >> 4)) << 4);
+        const double *src = X + line0 + 2 * c + (k0 + kq) * ldx;
+        if (line0 + kTileLines <= lines && k0 + kChunk <= k) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) copy16((dst ^ (u << 5)) + u * 512, src + 32 * u * ldx);
+        } else {
+            const int64_t left = lines - (line0 + 2 * c);
+            const int bytes = left >= 2 ? 16 : (left == 1 ? 8 : 0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = bytes && k0 + kq + 32 * u < k;
+                copy16((dst ^ (u << 5)) + u * 512, in ? src + 32 * u * ldx : X, in ? bytes : 0);
+            }
+        }
+    } else {
+        // line l of inner indices kq + 16 u, octets kq / 8 + 2 u
+        const int l = threadIdx.x & 15, kq = threadIdx.x >> 4;
+        const uint32_t dst = base + ((kq & 7) * 16 + (kq >> 3)) * 128 + ((l >> 1) << 4) + (l & 1) * 8;
+        const double *src = X + line0 + l + (k0 + kq) * ldx;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool in = line0 + l < lines && k0 + kq + 16 * u < k;
+            copy8((dst ^ (u << 4)) + u * 256, in ? src + 16 * u * ldx : X, in);
+        }
+    }
+}
+// side 1: a warp copies one row, 128 elements of a line
+__device__ __forceinline__ void request_row(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k, bool pairs,
+                                            int64_t line, int64_t k0, uint32_t row)
+{
+    const int lane = threadIdx.x & 31;
+    const bool live = line < lines;
+    const int kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);        // <= 0: padding only
+    const double *src = X + (live ? line : 0) * ldx + k0;
+    if (pairs) {
+#pragma unroll
+        for (int u = 0; u < kChunk / 64; ++u) {
+            const int c = lane + 32 * u;
+            if (live && kleft == kChunk) {
+                copy16(row + tile_chunk(c) * 16, src + 2 * c);
+            } else {
+                const int left = live ? (kleft - 2 * c) * 8 : 0;
+                const int bytes = left >= 16 ? 16 : (left > 0 ? left : 0);
+                copy16(row + tile_chunk(c) * 16, bytes ? src + 2 * c : X, bytes);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < kChunk / 32; ++u) {
+            const int kk = lane + 32 * u;
+            const bool in = live && kk < kleft;
+            copy8(row + tile_chunk(kk >> 1) * 16 + (kk & 1) * 8, in ? src + kk : X, in);
+        }
+    }
+}
+// this thread's eight elements of a tile: line 2 warp + lane / 16, octet lane % 16
+template <int SIDE>
+__device__ __forceinline__ void tile_octet(const unsigned char *tile, double (&x)[8])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, oct = lane & 15;
+    if constexpr (SIDE == 0) {
+        const double *src = reinterpret_cast<const double *>(tile + oct * 128 + ((warp ^ (oct >> 1)) << 4)) + (lane >> 4);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = src[e * 256];
+    } else {
+        const double2 *row = reinterpret_cast<const double2 *>(tile + (warp * 2 + (lane >> 4)) * kTileRow);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const double2 v = row[tile_chunk(oct * 4 + e)];
+            x[2 * e] = v.x;
+            x[2 * e + 1] = v.y;
+        }
+    }
+}
+
+// two consecutive octets of a tile: the same line, octets 2 j and 2 j + 1
+template <int SIDE>
+__device__ __forceinline__ void tile_octets(const unsigned char *tile, int j, double (&x)[16])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if constexpr (SIDE == 0) {
+        const double *src = reinterpret_cast<const double *>(tile + j * 256 + ((warp ^ j) << 4)) + (lane >> 4);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = src[(e & 7) * 256 + (e >> 3) * 16];
+    } else {
+        const double2 *row = reinterpret_cast<const double2 *>(tile + (warp * 2 + (lane >> 4)) * kTileRow);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const double2 v = row[tile_chunk(j * 8 + e)];
+            x[2 * e] = v.x;
+            x[2 * e + 1] = v.y;
+        }
+    }
+}
+
 // A block takes tiles of 16 lines x 128 inner indices through shared memory (on side 0 that is the
 // transposition: loads run along the lines, plane stores along k) and a thread converts eight consecutive
 // elements of one line, so that half a warp stores 128 contiguous bytes of every plane.  The next tile's
 // elements are copied asynchronously while this one is converted.  BY_LINE (side 1, planes kept line by line): the 16 rows
 // of a tile are consecutive 128-element pieces of a line, and of the next lines behind it, so that a tile stores 2 KiB at
 // a time in that layout too.
-// Side 0 keeps a tile as [index in an octet][octet][line], 128 bytes a row, the 16-byte pieces of a row XORed with the octet's
-// number: two lines travel in one copy, and neither the copies nor the reads, eight at compile-time offsets from one
-// address, conflict.
-// Bound: instruction issue and the FP32 pipe (both 60 % busy), and, line by line on side 0, the planes' scattered
-// 128-byte writes.  What surrounds the arithmetic was half of the instructions: tiles are numbered without divisions, shifts are
-// loaded with the elements, and whole tiles are copied without a test.
+// Bound: with digit planes DRAM (32768 x 1024, set S on FP8, side 0: 251 us, 243 with the arithmetic left out: 38 bytes an element at
+// 5.1 TB/s), on native residues instruction issue and the FP32 pipe (60 % busy each; 184 us against 131), and, line by line
+// on side 0, the planes' scattered 128-byte writes.  What surrounds the arithmetic was a third of the instructions: tiles are
+// numbered without divisions, shifts are loaded with the elements, whole tiles are copied without a test.  147 -> 127
+// thread-instructions per element of A on set S, 125 -> 105 on native residues (205 -> 184 us).
 template <int SET, int SIDE, int LAYOUT, bool BY_LINE>
 __global__ void __launch_bounds__(kConvThreads, conv_blocks(LAYOUT))
 convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t k,
@@ -544,7 +649,7 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
     const uint32_t ltiles = static_cast<uint32_t>((lines + kTileLines - 1) / kTileLines);
     const uint32_t items = BY_LINE ? (static_cast<uint32_t>(lines) * nchunks + kTileLines - 1) / kTileLines : ltiles * nchunks;
     const bool pairs = (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
-    const int li = warp * 2 + (lane >> 4), oct = lane & 15;        // this thread's line and octet of a tile
+    const int li = warp * 2 + (lane >> 4), oct = lane & 15;        // this thread's line and octet of a tile (see tile_octet)
 
     // Position of a tile: slow index q (side 0: chunk, side 1: line tile) and fast index `rest`, so that neighbouring blocks
     // take neighbouring lines (side 0) or neighbouring inner indices; BY_LINE: line and chunk of this warp's first row.  A step
@@ -580,35 +685,7 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
     auto request = [&](int buf) {
         const uint32_t base = tile_addr + buf * kTileBytes;
         if constexpr (SIDE == 0) {
-            const int64_t line0 = static_cast<int64_t>(rest) * kTileLines, k0 = static_cast<int64_t>(q) * kChunk;
-            if (pairs) {
-                // a thread copies lines 2c, 2c + 1 of inner indices kq + 32 u, octets kq / 8 + 4 u
-                const int c = threadIdx.x & 7, kq = threadIdx.x >> 3;
-                const uint32_t dst = base + ((kq & 7) * 16 + (kq >> 3)) * 128 + ((c ^ (kq >> 3)) << 4);
-                const double *src = X + line0 + 2 * c + (k0 + kq) * ldx;
-                if (line0 + kTileLines <= lines && k0 + kChunk <= k) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) copy16((dst ^ ((u & 1) << 6)) + u * 512, src + 32 * u * ldx);
-                } else {
-                    const int64_t left = lines - (line0 + 2 * c);
-                    const int bytes = left >= 2 ? 16 : (left == 1 ? 8 : 0);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const bool in = bytes && k0 + kq + 32 * u < k;
-                        copy16((dst ^ ((u & 1) << 6)) + u * 512, in ? src + 32 * u * ldx : X, in ? bytes : 0);
-                    }
-                }
-            } else {
-                // line l of inner indices kq + 16 u, octets kq / 8 + 2 u
-                const int l = threadIdx.x & 15, kq = threadIdx.x >> 4;
-                const uint32_t dst = base + ((kq & 7) * 16 + (kq >> 3)) * 128 + (((l >> 1) ^ (kq >> 3)) << 4) + (l & 1) * 8;
-                const double *src = X + line0 + l + (k0 + kq) * ldx;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const bool in = line0 + l < lines && k0 + kq + 16 * u < k;
-                    copy8((dst ^ ((u & 3) << 5)) + u * 256, in ? src + 16 * u * ldx : X, in);
-                }
-            }
+            request_side0(X, ldx, lines, k, pairs, static_cast<int64_t>(rest) * kTileLines, static_cast<int64_t>(q) * kChunk, base);
         } else {
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -625,30 +702,7 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
                     line = static_cast<int64_t>(q) * kTileLines + warp * 2 + h;
                     k0 = static_cast<int64_t>(rest) * kChunk;
                 }
-                const bool live = line < lines;
-                const int kleft = static_cast<int>(k - k0 < kChunk ? k - k0 : kChunk);        // <= 0: padding only
-                const double *src = X + (live ? line : 0) * ldx + k0;
-                const uint32_t row = base + (warp * 2 + h) * kTileRow;
-                if (pairs) {
-#pragma unroll
-                    for (int u = 0; u < kChunk / 64; ++u) {
-                        const int c = lane + 32 * u;
-                        if (live && kleft == kChunk) {
-                            copy16(row + tile_chunk(c) * 16, src + 2 * c);
-                        } else {
-                            const int left = live ? (kleft - 2 * c) * 8 : 0;
-                            const int bytes = left >= 16 ? 16 : (left > 0 ? left : 0);
-                            copy16(row + tile_chunk(c) * 16, bytes ? src + 2 * c : X, bytes);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int u = 0; u < kChunk / 32; ++u) {
-                        const int kk = lane + 32 * u;
-                        const bool in = live && kk < kleft;
-                        copy8(row + tile_chunk(kk >> 1) * 16 + (kk & 1) * 8, in ? src + kk : X, in);
-                    }
-                }
+                request_row(X, ldx, lines, k, pairs, line, k0, base + (warp * 2 + h) * kTileRow);
             }
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -676,25 +730,13 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
         __syncthreads();                 // this tile (and, the first time, the table) is there
         if (line < lines && k0 + oct * 8 < row_pitch) {
             double x[8];
-            if constexpr (SIDE == 0) {
-                const double *src = reinterpret_cast<const double *>(smem_raw + buf * kTileBytes + oct * 128 + ((warp ^ (oct & 7)) << 4)) + (lane >> 4);
-#pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] = src[e * 256];
-            } else {
-                const double2 *row = reinterpret_cast<const double2 *>(smem_raw + buf * kTileBytes + li * kTileRow);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const double2 v = row[tile_chunk(oct * 4 + e)];
-                    x[2 * e] = v.x;
-                    x[2 * e + 1] = v.y;
-                }
-            }
+            tile_octet<SIDE>(smem_raw + buf * kTileBytes, x);
             if (sigma == OZ_NONFINITE_SHIFT) {       // its planes are zeros
                 sigma = 0;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) x[e] = 0.0;
             }
-            convert8<SET, LAYOUT>(x, sigma, tz != 0, lut_addr,
+            convert<SET, LAYOUT, 4>(x, sigma, tz != 0, NearTable{lut_addr},
                                  planes + (k0 >> 7) * geom.chunk_stride + line * geom.line_stride + oct * 8, geom.plane_stride);
         }
         __syncthreads();                 // the tile may be overwritten
@@ -911,7 +953,7 @@ __device__ __forceinline__ void deconstruct_lines(const FusedParams &p, int bloc
                 for (int e = 0; e < 8; ++e) x[e] = (!dead && kb + e < k) ? src[e] : 0.0;
                 if (dead) sigma = 0;
             }
-            convert8<SET, LAYOUT>(x, sigma, p.tz != 0, lut_addr,
+            convert<SET, LAYOUT, 4>(x, sigma, p.tz != 0, NearTable{lut_addr},
                                   p.planes + (kb >> 7) * p.geom.chunk_stride + (line0 + l) * p.geom.line_stride + (kb & 127),
                                   p.geom.plane_stride);
             l += line_step;
@@ -1040,6 +1082,269 @@ FusedParams fused_params(int side, int64_t lines, int64_t k, const double *X, in
     p.shift = shift;
     p.status = device_status_word();
     return p;
+}
+
+// ---- whole deconstruction by clusters ---------------------------------------------------------
+// Operands above the one-kernel form: a cluster of up to five blocks holds 16 whole lines in its shared memory, `tiles` tiles of
+// 128 inner indices a block, so that the operand is read once where scans and conversion read it three times (24 -> 8 bytes an
+// element).  A half-warp owns a line in every block; its partial results (largest high word, then the norm sums)
+// travel to the other blocks of the cluster through distributed shared memory, one cluster barrier each.  Blocks stay
+// resident and walk the strips of 16 lines; a tile's place is refilled with the next strip as soon as it has been converted, so
+// that loads run beside the arithmetic.  Same functions and integer sums as the other forms: the same bits.
+// Bound: DRAM, 8 bytes read and all planes written at the rate that such a mix reaches (5.2 to 5.5 TB/s: what the conversion takes
+// when its arithmetic is left out).
+struct ClusterParams {
+    FusedParams f;               // group, pitch: not used
+    int tiles;
+};
+constexpr int kClusterMax = 8;
+struct ClusterExchange {         // per line and block of the cluster
+    unsigned long long sumsq[kTileLines][kClusterMax];
+    unsigned int l1[kTileLines][kClusterMax];
+    unsigned int key[2][kTileLines][kClusterMax];      // strips in turn: without norm sums, one barrier a strip is all there is
+};
+// Largest exponents as keys that order like them: the high word of |x|, or 1100 + e of a subnormal, 0 for zeros only
+constexpr unsigned int kFirstNormal = 0x00100000u, kFirstNonfinite = 0x7FF00000u;
+__device__ __forceinline__ int key_exponent(unsigned int key)
+{
+    return key >= kFirstNormal ? static_cast<int>(key >> 20) - 1023 : (key ? static_cast<int>(key) - 1100 : INT32_MIN);
+}
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t cluster_blocks()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ uint32_t remote(const void *p, uint32_t rank)
+{
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ void store_remote(uint32_t addr, unsigned int v) { asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
+__device__ __forceinline__ void store_remote(uint32_t addr, unsigned long long v) { asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory"); }
+__device__ __forceinline__ void cluster_barrier()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int SET, int SIDE, int LAYOUT>
+__global__ void __launch_bounds__(kConvThreads, 2)
+deconstruct_cluster_kernel(const __grid_constant__ ClusterParams cp)
+{
+    const FusedParams &p = cp.f;
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int T = cp.tiles;
+    ClusterExchange &ex = *reinterpret_cast<ClusterExchange *>(smem_raw + T * kTileBytes);
+    uint32_t *lut = reinterpret_cast<uint32_t *>(smem_raw + T * kTileBytes + sizeof(ClusterExchange));
+    const uint32_t lut_addr = static_cast<uint32_t>(__cvta_generic_to_shared(lut));
+    const uint32_t tile_addr = static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw));
+    dependency_release();
+    load_table<SET, LAYOUT>(lut, p.lut_global, threadIdx.x, kConvThreads);      // written once, before any call
+    dependency_wait();
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int li = warp * 2 + (lane >> 4), oct = lane & 15;
+    const unsigned int half = lane < 16 ? 0xFFFFu : 0xFFFF0000u;
+    const uint32_t rank = cluster_rank(), C = cluster_blocks();
+    const bool pairs = (p.ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15u) == 0;
+    const int64_t nchunks = (p.geom.row_pitch + kChunk - 1) / kChunk, strips = (p.lines + kTileLines - 1) / kTileLines;
+    const int64_t chunk0 = static_cast<int64_t>(rank) * T;
+    const int nt = static_cast<int>(nchunks - chunk0 < T ? (nchunks - chunk0 > 0 ? nchunks - chunk0 : 0) : T);
+    auto request = [&](int64_t strip, int t) {
+        const uint32_t base = tile_addr + t * kTileBytes;
+        const int64_t line0 = strip * kTileLines, k0 = (chunk0 + t) * kChunk;
+        if constexpr (SIDE == 0) {
+            request_side0(p.X, p.ldx, p.lines, p.k, pairs, line0, k0, base);
+        } else {
+            request_row(p.X, p.ldx, p.lines, p.k, pairs, line0 + warp * 2, k0, base + warp * 2 * kTileRow);
+            request_row(p.X, p.ldx, p.lines, p.k, pairs, line0 + warp * 2 + 1, k0, base + (warp * 2 + 1) * kTileRow);
+        }
+    };
+    const int64_t first = blockIdx.x / C, step = gridDim.x / C;
+    cluster_barrier();                   // every block of the cluster has started: its shared memory may be written
+    int turn = 0;
+    if (first < strips)
+        for (int t = 0; t < nt; ++t) request(first, t);
+    for (int64_t strip = first; strip < strips; strip += step, turn ^= 1) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();                 // the strip (and, the first time, the table) is there
+        const int64_t line = strip * kTileLines + li;
+        // ---- largest exponent
+        unsigned int key = 0u;
+        for (int t = 0; t < nt; ++t) {
+            double x[8];
+            tile_octet<SIDE>(smem_raw + t * kTileBytes, x);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) key = max(key, static_cast<unsigned int>(__double2hiint(x[e])) & 0x7FFFFFFFu);
+        }
+        key = __reduce_max_sync(half, key);
+        if (__any_sync(0xFFFFFFFFu, key < kFirstNormal)) {        // zeros and subnormals only: exponents from the whole words
+            unsigned int small = 0u;
+            for (int t = 0; t < nt; ++t) {
+                double x[8];
+                tile_octet<SIDE>(smem_raw + t * kTileBytes, x);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    int ex1;
+                    if (classify(x[e], &ex1) == 1 && ex1 < -1022) small = max(small, static_cast<unsigned int>(ex1 + 1100));
+                }
+            }
+            small = __reduce_max_sync(half, small);
+            if (key < kFirstNormal) key = small;
+        }
+        if (static_cast<uint32_t>(oct) < C) store_remote(remote(&ex.key[turn][li][rank], oct), key);
+        cluster_barrier();
+        key = __reduce_max_sync(half, static_cast<uint32_t>(oct) < C ? ex.key[turn][li][oct] : 0u);
+        const int E = key_exponent(key);
+        const bool bad = key >= kFirstNonfinite;
+        // ---- norm sums
+        unsigned long long S = 0ull;
+        unsigned int l1 = 0u;
+        if (p.rule == 1) {
+            if (!bad && E != INT32_MIN) {        // uniform over the half-warp
+                const bool fast_scale = 9 - E >= -1000 && 9 - E <= 1000;
+                const double scale9 = __hiloint2double((1023 + (fast_scale ? 9 - E : 0)) << 20, 0);
+                for (int t = 0; t < nt; ++t) {
+                    double x[8];
+                    tile_octet<SIDE>(smem_raw + t * kTileBytes, x);
+                    unsigned int part = 0u;           // eight terms of at most 2^20
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        unsigned int abar;
+                        if (fast_scale) {
+                            abar = __double2uint_ru(fabs(x[e]) * scale9);
+                            if (abar == 0u && x[e] != 0.0) abar = 1u;
+                        } else {
+                            abar = scaled_magnitude(x[e], E);
+                        }
+                        part += abar * abar;
+                        l1 += abar;
+                    }
+                    S += part;
+                }
+            }
+            __syncwarp();
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
+            l1 = __reduce_add_sync(half, l1);
+            if (static_cast<uint32_t>(oct) < C) {
+                store_remote(remote(&ex.sumsq[li][rank], oct), S);
+                store_remote(remote(&ex.l1[li][rank], oct), l1);
+            }
+            cluster_barrier();
+            S = static_cast<uint32_t>(oct) < C ? ex.sumsq[li][oct] : 0ull;
+            l1 = __reduce_add_sync(half, static_cast<uint32_t>(oct) < C ? ex.l1[li][oct] : 0u);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) S += __shfl_xor_sync(0xFFFFFFFFu, S, o);
+        }
+        // ---- the shift (same arithmetic as scan_finalize_kernel)
+        int sigma = 0;
+        if (oct == 0 && line < p.lines) {
+            if (bad) sigma = OZ_NONFINITE_SHIFT;
+            else if (E != INT32_MIN) sigma = p.rule == 0 ? p.tbits - 1 - E : norm_exponent(S, p.g2lo, p.g2hi) + 9 - E;
+            if (rank == 0) {
+                p.shift[line] = sigma;
+                if (bad) {
+                    atomicOr(p.status, 1u << OZ_ERR_NONFINITE_INPUT);
+                } else if (E != INT32_MIN && p.rule == 1) {
+                    atomicMin(p.status + 1 + p.side, line_flatness(l1, S, p.k));
+                    p.status[3] = p.esc_threshold;
+                }
+            }
+        }
+        sigma = __shfl_sync(0xFFFFFFFFu, sigma, lane & 16);
+        // ---- conversion, tile by tile, each followed by the copy of the next strip's
+        const bool more = strip + step < strips;
+        for (int t = 0; t < nt; t += 2) {        // a thread takes 16 elements: the half-warps' halves take two tiles at once
+            const int tt = t + (oct >> 3);
+            const int64_t chunk = chunk0 + tt;
+            const int k_in = (oct & 7) * 16;                 // first of this thread's indices in the tile
+            if (tt < nt && line < p.lines && chunk * kChunk + k_in < p.geom.row_pitch) {
+                double x[16];
+                tile_octets<SIDE>(smem_raw + tt * kTileBytes, oct & 7, x);
+                int sig = sigma;
+                if (sig == OZ_NONFINITE_SHIFT) {       // its planes are zeros
+                    sig = 0;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) x[e] = 0.0;
+                }
+                convert<SET, LAYOUT, 8>(x, sig, p.tz != 0, FarTable{lut_addr},
+                                        p.planes + chunk * p.geom.chunk_stride + line * p.geom.line_stride + k_in, p.geom.plane_stride);
+            }
+            if (more) {
+                __syncthreads();             // these tiles have been read
+                request(strip + step, t);
+                if (t + 1 < nt) request(strip + step, t + 1);
+            }
+        }
+    }
+    cluster_barrier();                   // no block leaves while another may still write to it
+}
+
+// Blocks of a cluster and tiles of a block for lines of `chunks` tiles, two blocks on an SM; blocks = 0: three passes.
+// Clusters of one or two blocks (k up to 1280 or 1536) win at every size measured up to 800 MB: deconstruction of 6912 x 6912 x
+// 1024, set E, 202 -> 155 us, whole call 100000 x 64 x 1000 on INT8 digits 1824 -> 1537 us.  Longer lines spread a cluster's
+// reads over the whole operand (side 0: 128 bytes from each of k columns), and one table and one block less per SM hide
+// less: up to five blocks and 256 MiB still win (6144 x 6144 x 3072 native 350 -> 335 us, 20000 x 16 x 3000 890 -> 847 us a
+// call), beyond that three passes do (4096^3, set S: 331 us against 402; 60000 x 200 x 2500 native 2000 us a call against 2300;
+// 131072 x 128 x 4096 5.4 ms against 8.0).
+struct ClusterShape { int blocks, tiles; size_t smem; };
+ClusterShape cluster_shape(int set, int layout, int64_t lines, int64_t k, int64_t chunks)
+{
+    const size_t fixed = lut_words_of(set, layout) * 4 + sizeof(ClusterExchange);
+    const int most = static_cast<int>((226 * 1024 / 2 - 1024 - fixed) / kTileBytes);
+    const int64_t blocks = (chunks + most - 1) / most, bytes = 8 * lines * k;
+    if (blocks > 5 || bytes > (blocks <= 2 ? 1ll << 30 : 1ll << 28)) return {0, 0, 0};
+    const int tiles = static_cast<int>((chunks + blocks - 1) / blocks);
+    return {static_cast<int>(blocks), tiles, fixed + static_cast<size_t>(tiles) * kTileBytes};
+}
+
+template <int SET, int SIDE, int LAYOUT>
+oz_status_t launch_cluster(const ClusterParams &p, const ClusterShape &shape, bool alone, cudaStream_t stream)
+{
+    const auto kernel = deconstruct_cluster_kernel<SET, SIDE, LAYOUT>;
+    static std::atomic<unsigned long long> ready{0};
+    OZ_CUDA_CHECK(allow_shared(kernel, kMaxShared, ready));
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kConvThreads);
+    cfg.dynamicSmemBytes = shape.smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(shape.blocks);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // clusters that are resident at once, asked once per shape
+    static std::atomic<int> resident[kClusterMax + 1][8];
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3(static_cast<unsigned>(shape.blocks));
+    int clusters = resident[shape.blocks][shape.tiles].load(std::memory_order_relaxed);
+    if (!clusters) {
+        OZ_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg));
+        if (clusters < 1) clusters = 1;
+        resident[shape.blocks][shape.tiles].store(clusters, std::memory_order_relaxed);
+    }
+    const int64_t strips = (p.f.lines + kTileLines - 1) / kTileLines;
+    // as many as share the strips evenly
+    const int64_t rounds = (strips + clusters - 1) / clusters, used = (strips + rounds - 1) / rounds;
+    cfg.gridDim = dim3(static_cast<unsigned>(used * shape.blocks));
+    cfg.numAttrs = alone ? 2 : 1;
+    OZ_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, p));
+    count_launch();
+    OZ_CUDA_CHECK(cudaGetLastError());
+    return OZ_OK;
 }
 
 template <int SET, int SIDE, int LAYOUT>
@@ -1185,7 +1490,21 @@ static FusedShape lone_shape(int side, int64_t lines, int64_t k, int set, const 
     return f;
 }
 
-bool three_passes(int side, int64_t lines, int64_t k, int set, const Route &rt) { return lone_shape(side, lines, k, set, rt).group <= 0; }
+// The cluster form: planes in the private layout of the whole-method schedules, lines that fit a cluster.  Not under the row
+// check, which reads the scan results.
+static ClusterShape by_clusters(int side, int64_t lines, int64_t k, int set, const Route &rt, const PlaneGeom &geom)
+{
+    const int layout = rt.layout(side);
+    const bool built = layout == kLayoutNative || (side == 0 ? layout != kLayoutDigits && layout != kLayoutDigitsI8
+                                                             : layout == kLayoutDigits || layout == kLayoutMergedI8B);
+    if (rt.fallback || !built || geom.line_stride != kChunk || k < 1) return {0, 0, 0};
+    return cluster_shape(set, layout, lines, k, (geom.row_pitch + kChunk - 1) / kChunk);
+}
+
+bool three_passes(int side, int64_t lines, int64_t k, int set, const Route &rt)
+{
+    return lone_shape(side, lines, k, set, rt).group <= 0 && by_clusters(side, lines, k, set, rt, private_planes(lines, round_up(k, kChunk))).blocks == 0;
+}
 
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
@@ -1213,6 +1532,27 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
         return OZ_FUSED_SET(2);
 #undef OZ_FUSED_SET
 #undef OZ_FUSED
+    }
+    const ClusterShape c = by_clusters(side, lines, k, set, rt, geom);
+    if (c.blocks) {
+        ClusterParams p;
+        p.f = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, 0);
+        p.tiles = c.tiles;
+        const int layout = rt.layout(side);
+#define OZ_CLUSTER(SET_, SIDE_, LAYOUT_) launch_cluster<SET_, SIDE_, LAYOUT_>(p, c, alone, stream)
+#define OZ_CLUSTER_SET(SET_)                                                                                    \
+    (layout == kLayoutMerged      ? OZ_CLUSTER(SET_, 0, kLayoutMerged)                                         \
+     : layout == kLayoutMergedI8A ? OZ_CLUSTER(SET_, 0, kLayoutMergedI8A)                                      \
+     : layout == kLayoutMergedI8B ? OZ_CLUSTER(SET_, 1, kLayoutMergedI8B)                                      \
+     : layout == kLayoutTwo       ? OZ_CLUSTER(SET_, 0, kLayoutTwo)                                            \
+     : layout == kLayoutTwoI8     ? OZ_CLUSTER(SET_, 0, kLayoutTwoI8)                                          \
+                                  : OZ_CLUSTER(SET_, 1, kLayoutDigits))
+        if (layout == kLayoutNative) return side == 0 ? OZ_CLUSTER(2, 0, kLayoutNative) : OZ_CLUSTER(2, 1, kLayoutNative);
+        if (set == 0) return OZ_CLUSTER_SET(0);
+        if (set == 1) return OZ_CLUSTER_SET(1);
+        return OZ_CLUSTER_SET(2);
+#undef OZ_CLUSTER_SET
+#undef OZ_CLUSTER
     }
     const ScanJob job{lines, X, ldx, shift, scratch};
     oz_status_t st = launch_scan(side == 0 ? &job : nullptr, side == 1 ? &job : nullptr, k, set, rt, alone, stream);

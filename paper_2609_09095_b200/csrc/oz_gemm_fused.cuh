@@ -84,7 +84,7 @@ __device__ __forceinline__ void convert_pass_moduli(std::integer_sequence<int, S
                                                     uint8_t *out)
 {
     constexpr int first = first_plane(SET, F_GROUP * G, LAYOUT);
-    (convert_modulus<SET, LAYOUT, F_GROUP * G + S>(L, lut, out - first * F_A_PLANE, F_A_PLANE), ...);
+    (convert_modulus<SET, LAYOUT, F_GROUP * G + S>(L, NearTable{lut}, out - first * F_A_PLANE, F_A_PLANE), ...);
 }
 
 template <int SET, int LAYOUT, int G>
