@@ -541,30 +541,28 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         return OZ_OK;
     }
     bool both = false;
-    st = launch_deconstruct_pair({m, A, lda, a.planes, private_planes(m, a.pitch), a.shift},
-                                 {n, B, ldb, b.planes, private_planes(n, b.pitch), b.shift}, k, set, rt, &both, stream);
+    st = launch_deconstruct_pair({m, A, lda, a.planes, private_planes(m, a.pitch), a.shift, a.scratch},
+                                 {n, B, ldb, b.planes, private_planes(n, b.pitch), b.shift, b.scratch}, k, set, rt, &both, stream);
     if (st != OZ_OK) return st;
-    if (both) {
-        if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
-        return product_impl(m, n, k, alpha, a, b, beta, C, ldc, set, rt, stream, ws + L.R, dev, plan);
-    }
-    const bool scans = three_passes(0, m, k, set, rt) && three_passes(1, n, k, set, rt);
-    if (scans) {      // both operands in one launch per pass; the conversions then run side by side
-        const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
-        st = launch_scan(&ja, &jb, k, set, rt, true, stream);
+    if (!both) {
+        const bool scans = three_passes(0, m, k, set, rt) && three_passes(1, n, k, set, rt);
+        if (scans) {      // both operands in one launch per pass; the conversions then run side by side
+            const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
+            st = launch_scan(&ja, &jb, k, set, rt, true, stream);
+            if (st != OZ_OK) return st;
+        }
+        OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
+        OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
+        st = scans ? launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, false, side)
+                   : launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
+        if (st != OZ_OK) return st;
+        OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
+        st = scans ? launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, false, stream)
+                   : launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, false, stream);
         if (st != OZ_OK) return st;
     }
-    OZ_CUDA_CHECK(cudaEventRecord(g_fork[dev], stream));
-    OZ_CUDA_CHECK(cudaStreamWaitEvent(side, g_fork[dev], 0));
-    st = scans ? launch_convert_planes(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, false, side)
-               : launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
-    if (st != OZ_OK) return st;
-    OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-    st = scans ? launch_convert_planes(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, false, stream)
-               : launch_deconstruct(0, m, k, A, lda, set, rt, a.planes, private_planes(m, a.pitch), a.shift, a.scratch, false, stream);
-    if (st != OZ_OK) return st;
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
-    OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
+    if (!both) OZ_CUDA_CHECK(cudaStreamWaitEvent(stream, g_join[dev], 0));
     if (!rt.fallback) return product_impl(m, n, k, alpha, a, b, beta, C, ldc, set, rt, stream, ws + L.R, dev, plan);
     // Algorithm 1, last line / Algorithm 3, "ESC range check": the rows that fail the check are left
     // out of the reconstruction and re-issued on the native FP64 path from the caller's old C

@@ -767,7 +767,17 @@ struct FusedParams {
     PlaneGeom geom;
     int32_t *shift;
     unsigned int *status;
+    ScanScratch scan;          // where the lines' scan results go as well, for the row check; null: nowhere
 };
+
+// a line's scan results, as the scan kernels leave them
+__device__ __forceinline__ void keep_scan(const ScanScratch &s, int64_t line, unsigned long long sumsq, int emax, bool bad, unsigned int l1)
+{
+    if (!s.emax) return;
+    s.sumsq[line] = sumsq;
+    s.emax[line] = emax;
+    s.nonfinite[line] = bad ? kNonfiniteBit : static_cast<int>(l1);
+}
 
 // position of inner index kk in a line's buffer: one spare double behind every eight, so that threads that read
 // eight consecutive elements each (stride 9) touch all banks
@@ -933,6 +943,7 @@ __device__ __forceinline__ void deconstruct_lines(const FusedParams &p, int bloc
             const int sh = line_shift(p, res[tid]);
             res[tid].shift = sh;
             p.shift[line0 + tid] = sh;
+            keep_scan(p.scan, line0 + tid, res[tid].sumsq, res[tid].exponent(), res[tid].bad(), res[tid].l1);
         }
         __syncthreads();
         // ---- conversion: a thread takes eight consecutive inner indices of one line; a step over the block adds a constant to
@@ -1063,9 +1074,10 @@ oz_status_t launch_pair(const PairParams &p, const FusedShape &fa, const FusedSh
 
 // parameters of the one-kernel form for one operand
 FusedParams fused_params(int side, int64_t lines, int64_t k, const double *X, int64_t ldx, int set, const Route &rt,
-                         uint8_t *planes, const PlaneGeom &geom, int32_t *shift, int group)
+                         uint8_t *planes, const PlaneGeom &geom, int32_t *shift, void *scratch, int group)
 {
     FusedParams p{};
+    if (rt.fallback) p.scan = carve_scratch(scratch, lines);      // the row check reads the scan results
     p.X = X; p.ldx = ldx; p.lines = lines; p.k = k;
     p.group = group;
     p.pitch = fused_pitch(static_cast<int>(k));
@@ -1253,6 +1265,7 @@ deconstruct_cluster_kernel(const __grid_constant__ ClusterParams cp)
             else if (E != INT32_MIN) sigma = p.rule == 0 ? p.tbits - 1 - E : norm_exponent(S, p.g2lo, p.g2hi) + 9 - E;
             if (rank == 0) {
                 p.shift[line] = sigma;
+                keep_scan(p.scan, line, S, E, bad, l1);
                 if (bad) {
                     atomicOr(p.status, 1u << OZ_ERR_NONFINITE_INPUT);
                 } else if (E != INT32_MIN && p.rule == 1) {
@@ -1483,21 +1496,19 @@ oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const doub
 // the one-kernel form's shape for an operand by itself, group = 0: three passes
 static FusedShape lone_shape(int side, int64_t lines, int64_t k, int set, const Route &rt)
 {
-    if (rt.fallback) return FusedShape{0, 0, 0, 0};      // the row check reads the scan results of the three-pass form
     const int sms = sm_count();
     FusedShape f = fused_shape(set, rt.layout(side), side, lines, k, false, 2ll * sms);
     if (f.group <= 0) f = fused_shape(set, rt.layout(side), side, lines, k, true, sms);
     return f;
 }
 
-// The cluster form: planes in the private layout of the whole-method schedules, lines that fit a cluster.  Not under the row
-// check, which reads the scan results.
+// The cluster form: planes in the private layout of the whole-method schedules, lines that fit a cluster
 static ClusterShape by_clusters(int side, int64_t lines, int64_t k, int set, const Route &rt, const PlaneGeom &geom)
 {
     const int layout = rt.layout(side);
     const bool built = layout == kLayoutNative || (side == 0 ? layout != kLayoutDigits && layout != kLayoutDigitsI8
                                                              : layout == kLayoutDigits || layout == kLayoutMergedI8B);
-    if (rt.fallback || !built || geom.line_stride != kChunk || k < 1) return {0, 0, 0};
+    if (!built || geom.line_stride != kChunk || k < 1) return {0, 0, 0};
     return cluster_shape(set, layout, lines, k, (geom.row_pitch + kChunk - 1) / kChunk);
 }
 
@@ -1513,7 +1524,7 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
     if (rt.rule == 2) return OZ_ERR_UNSUPPORTED;      // the accurate rule needs both operands
     const FusedShape f = lone_shape(side, lines, k, set, rt);
     if (f.group > 0) {
-        const FusedParams p = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, f.group);
+        const FusedParams p = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, scratch, f.group);
         const int layout = rt.layout(side);
 #define OZ_FUSED(SET_, SIDE_, LAYOUT_) launch_fused<SET_, SIDE_, LAYOUT_>(p, f, alone, stream)
 #define OZ_FUSED_SET(SET_)                                                                                          \
@@ -1536,7 +1547,7 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
     const ClusterShape c = by_clusters(side, lines, k, set, rt, geom);
     if (c.blocks) {
         ClusterParams p;
-        p.f = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, 0);
+        p.f = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, scratch, 0);
         p.tiles = c.tiles;
         const int layout = rt.layout(side);
 #define OZ_CLUSTER(SET_, SIDE_, LAYOUT_) launch_cluster<SET_, SIDE_, LAYOUT_>(p, c, alone, stream)
@@ -1564,7 +1575,7 @@ oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, in
                                     bool *taken, cudaStream_t stream)
 {
     *taken = false;
-    if (rt.rule == 2 || rt.fallback) return OZ_OK;      // shifts from both operands; the row check's scan results
+    if (rt.rule == 2) return OZ_OK;      // shifts from both operands
     const int sms = sm_count();
     // The resident blocks are shared out by the operands' sizes.  Taken when both operands then finish in one round
     // (1009 x 983 x 1021: 77.0 -> 68.8 us a call; 1300 x 300 x 1400, one large block per SM: 81.5 -> 70.8); with more rounds the
@@ -1581,8 +1592,8 @@ oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, in
     }
     if (!one_round) return OZ_OK;
     PairParams p;
-    p.a = fused_params(0, a.lines, k, a.X, a.ldx, set, rt, a.planes, a.geom, a.shift, fa.group);
-    p.b = fused_params(1, b.lines, k, b.X, b.ldx, set, rt, b.planes, b.geom, b.shift, fb.group);
+    p.a = fused_params(0, a.lines, k, a.X, a.ldx, set, rt, a.planes, a.geom, a.shift, a.scratch, fa.group);
+    p.b = fused_params(1, b.lines, k, b.X, b.ldx, set, rt, b.planes, b.geom, b.shift, b.scratch, fb.group);
     p.blocksA = fa.grid;
     *taken = true;
     const int layout = rt.layout(0);
@@ -1599,7 +1610,7 @@ oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, in
 }
 
 // flags, ordered list and number of the rows that go to the native FP64 path, from the scan results
-// that the three-pass deconstruction of both operands left in their scratch blocks
+// that the deconstruction of both operands left in their scratch blocks
 oz_status_t launch_esc_rows(void *scratchA, int64_t m, void *scratchB, int64_t n, int64_t k, int set,
                             unsigned char *flag, int *list, unsigned int *count, cudaStream_t stream)
 {

@@ -224,6 +224,7 @@ struct OperandJob {
     uint8_t *planes;
     PlaneGeom geom;
     int32_t *shift;
+    void *scratch;
 };
 oz_status_t launch_deconstruct_pair(const OperandJob &a, const OperandJob &b, int64_t k, int set, const Route &rt,
                                     bool *taken, cudaStream_t stream);
@@ -296,7 +297,7 @@ oz_status_t launch_reconstruct_hosted(int64_t m, int64_t n, const void *R, const
                                       cudaStream_t stream);
 
 // Out-of-range rows (Algorithm 1, last line; Algorithm 3, "ESC range check"): flags, ascending list and
-// number of the rows that go to the native FP64 path, from the scan results that the three-pass
+// number of the rows that go to the native FP64 path, from the scan results that the
 // deconstruction left in the two scratch blocks; and the native path itself
 oz_status_t launch_esc_rows(void *scratchA, int64_t m, void *scratchB, int64_t n, int64_t k, int set,
                             unsigned char *flag, int *list, unsigned int *count, cudaStream_t stream);

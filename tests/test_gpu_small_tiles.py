@@ -26,7 +26,7 @@ def test_few_tiles(set_name, sub, m, n, k):
 @pytest.mark.parametrize("m,n,k", [(16, 16, 128), (33, 17, 129), (15, 40, 7), (50, 260, 384), (201, 99, 250)])
 @pytest.mark.parametrize("pad,offset", [(0, 0), (1, 0), (2, 1), (3, 1)])
 def test_three_pass_conversion_on_views(m, n, k, pad, offset):
-    """The row check takes the scans and the tile conversion at every size.  Operands inside a larger block: leading dimensions
+    """The accurate rule takes the scans and the tile conversion at every size.  Operands inside a larger block: leading dimensions
     of either parity, a first element on a 16-byte boundary or not, and NaN around them that must not be read as data."""
     import torch
     import paper_2609_09095_b200 as oz
@@ -36,8 +36,8 @@ def test_three_pass_conversion_on_views(m, n, k, pad, offset):
     if m > 15:
         A[3, :] = 0.0
         A[7, k // 2] = np.nan
-    rt = gh.route("fp8", fallback=True)
-    want, flags = ozo.dgemm_fallback(A, B, ozo.SET_S)
+    rt = gh.route("fp8", rule="ACCURATE")
+    want = ozo.dgemm(A, B, ozo.SET_S, ozo.QUANT_RN, ozo.SCALE_ACCURATE)
     gh.ensure_workspace(oz.oz_workspace_bytes(m, n, k, oz.OZ_SET_S, rt))
 
     def inside(X):
