@@ -103,8 +103,9 @@ typedef enum { OZ_SET_S = 0, OZ_SET_E = 1, OZ_SET_A = 2 } oz_modset_t;
  * that is reduced modulo m_i before the segments are added (split-K inside the kernel; the residues
  * are the same).
  * SEPARATE: the three accumulators of Eq. 8.  With neither bit, oz_dgemm / oz_dgemm_ex /
- * oz_dgemm_host pick MERGED on the digit substrates (their planes are internal), and the stage entry
- * points use SEPARATE.  Planes written with MERGED must be multiplied with MERGED.  Not defined for
+ * oz_dgemm_host pick MERGED on the digit substrates (their planes are internal), or, with n <= 128 and m >= n,
+ * two digit planes of A per modulus against the digits of e and of 16 e (same residues, no more workspace), and the
+ * stage entry points use SEPARATE.  Planes written with MERGED must be multiplied with MERGED.  Not defined for
  * OZ_SUB_INT8_NATIVE (one plane per modulus). */
 #define OZ_ACC_MERGED   0x1000u
 #define OZ_ACC_SEPARATE 0x2000u
