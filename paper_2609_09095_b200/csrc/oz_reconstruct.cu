@@ -108,17 +108,22 @@ __device__ __forceinline__ double finish_exact(double X0, double X1, double X2, 
     return neg ? -d : d;
 }
 
-// alpha 2^-(sa + sb) c' where the fast path does not apply: NaN for a line with Inf/NaN, else by integers
+// alpha 2^-(sa + sb) c' where the fast path does not apply: NaN for a line with Inf/NaN, else by integers.  The sum of the shifts
+// is taken in 64 bits; beyond 2^20 the result is zero or infinite whatever c' is.
 template <int SET>
 __device__ __noinline__ double row_value_exact(double X0, double X1, double X2, int sa, int sb, double alpha)
 {
     if (sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
-    return finish_exact(X0, X1, X2, sa + sb, SET) * alpha;
+    const long long sum = static_cast<long long>(sa) + sb;
+    return finish_exact(X0, X1, X2, static_cast<int>(min(max(sum, -(1ll << 20)), 1ll << 20)), SET) * alpha;
 }
 
-// Column operand of row_scale(): shiftB with the mark of a column with Inf/NaN moved so far out that no sum with a row
-// shift (|sa| < 2^12, or INT32_MIN) wraps into the range of the fast path.
-__device__ __forceinline__ int column_shift(int sb) { return sb == OZ_NONFINITE_SHIFT ? 1 << 29 : sb; }
+// Whether a shift may enter the 32-bit sums of the fast path: |shift| <= 2^30, which the mark of a line with Inf/NaN exceeds
+constexpr int kShiftLimit = 1 << 30;
+__device__ __forceinline__ bool ordinary_shift(int s)
+{
+    return static_cast<uint32_t>(s) + static_cast<uint32_t>(kShiftLimit) <= 2u * static_cast<uint32_t>(kShiftLimit);
+}
 
 // One row of the thread's group: value = fast alpha 2^-(sa + sb) c', returned as the rounded integer r and the power of
 // two to multiply it by (exact, and left to the caller so that an update of C is one fused multiply-add).
@@ -129,7 +134,7 @@ __device__ __forceinline__ int column_shift(int sb) { return sb == OZ_NONFINITE_
 // rounding boundary -- adding rem, enlarged by 2^-29, then moves r -- or so near to +-M/2 that the lift may apply.
 // 50 FP64 operations per output on set S where the carries and a test by exponents took 63.
 template <int SET, int HALF>
-__device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, int sb, int sb_mark, int alpha_sign, double alpha,
+__device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, int sb, bool fast_column, int alpha_sign, double alpha,
                                           double &r, double &scale)
 {
     const ReconConst &K = c_recon[SET];
@@ -143,11 +148,11 @@ __device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, in
     const double t = err + X0;
     r = s + t;
     const double rem = t - (r - s);
-    const int shift_sum = sa + sb_mark;
+    const uint32_t shift_sum = static_cast<uint32_t>(sa) + static_cast<uint32_t>(sb);
     // 2^-shift_sum and r 2^-shift_sum are normal: r is zero or 1 <= |r| < 2^118
-    const bool easy = static_cast<unsigned>(shift_sum + 904) <= 1924u && fma(rem, 1.0 + 0x1p-29, r) == r &&
+    const bool easy = fast_column && ordinary_shift(sa) && shift_sum + 904u <= 1924u && fma(rem, 1.0 + 0x1p-29, r) == r &&
                       (__double2hiint(r) & 0x7FFFFFFF) < K.half_M_guard;
-    scale = __hiloint2double(static_cast<int>(static_cast<uint32_t>(1023 - shift_sum) << 20) ^ alpha_sign, 0);
+    scale = __hiloint2double(static_cast<int>((1023u - shift_sum) << 20) ^ alpha_sign, 0);
     if (!easy) {
         r = row_value_exact<SET>(X0, X1, X2, sa, sb, alpha);
         scale = 1.0;
@@ -181,19 +186,20 @@ __device__ __forceinline__ void reconstruct_rows(const uint32_t (&w)[kMaxR], int
 #pragma unroll
         for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + 2 * h);
     }
-    const int sb_mark = column_shift(sb), alpha_sign = alpha < 0.0 ? INT32_MIN : 0;
+    const bool fast_column = ordinary_shift(sb);
+    const int alpha_sign = alpha < 0.0 ? INT32_MIN : 0;
     {
         double r0, r1 = 0.0, f0, f1 = 1.0;
-        row_value<SET, 0>(w, sa[0], sb, sb_mark, alpha_sign, alpha, r0, f0);
-        if (nrows > 1) row_value<SET, 1>(w, sa[1], sb, sb_mark, alpha_sign, alpha, r1, f1);
+        row_value<SET, 0>(w, sa[0], sb, fast_column, alpha_sign, alpha, r0, f0);
+        if (nrows > 1) row_value<SET, 1>(w, sa[1], sb, fast_column, alpha_sign, alpha, r1, f1);
         if (whole) *reinterpret_cast<double2 *>(out) = make_double2(fma(r0, f0, old[0].x), fma(r1, f1, old[0].y));
         else store_pair(out, r0 * f0, r1 * f1, (keep & 1u) != 0, nrows > 1 && (keep & 2u) != 0, beta);
     }
     if constexpr (ROWS == 4) {
         if (nrows > 2) {
             double r2, r3 = 0.0, f2, f3 = 1.0;
-            row_value<SET, 2>(w, sa[2], sb, sb_mark, alpha_sign, alpha, r2, f2);
-            if (nrows > 3) row_value<SET, 3>(w, sa[3], sb, sb_mark, alpha_sign, alpha, r3, f3);
+            row_value<SET, 2>(w, sa[2], sb, fast_column, alpha_sign, alpha, r2, f2);
+            if (nrows > 3) row_value<SET, 3>(w, sa[3], sb, fast_column, alpha_sign, alpha, r3, f3);
             if (whole) *reinterpret_cast<double2 *>(out + 2) = make_double2(fma(r2, f2, old[1].x), fma(r3, f3, old[1].y));
             else store_pair(out + 2, r2 * f2, r3 * f3, (keep & 4u) != 0, nrows > 3 && (keep & 8u) != 0, beta);
         }

@@ -39,3 +39,28 @@ def test_scale_and_rounding_edges(set_name, alpha, beta):
         want = ozo.output(np.ascontiguousarray(CIr), sA[m - rows:], sB, alpha, beta, np.asfortranarray(C0[m - rows:]))
         assert (np.isnan(got) == np.isnan(want)).all()
         assert (got[~np.isnan(want)] == want[~np.isnan(want)]).all()
+
+
+@pytest.mark.parametrize("set_name", ["S", "E", "A"])
+def test_marks_and_far_shifts(set_name):
+    """A marked line gives NaN whatever the shift of its partner, and shifts whose sum leaves 32 bits give zero or infinity
+    like any other sum that far out."""
+    import tests.gpu_helpers as gh
+    ms = ozo.modset(OSET[set_name])
+    top = 2 ** 31 - 1
+    sA = np.array([MARK, -(2 ** 29) - 904, -(2 ** 29), -(2 ** 29) + 57, -(2 ** 29) + 1020, 2 ** 29 + 57, 2 ** 30, 2 ** 30 + 1, -(2 ** 30) - 1,
+                   top, top - 56, -top, -top + 57, 0, 57], dtype=np.int32)
+    sB = np.array([MARK, 0, 57, top, top - 904, top - 2 ** 29, -top, -top + 57, -top + 1020, -(2 ** 30) - 5, 2 ** 29, 3 - 2 ** 29], dtype=np.int32)
+    m, n = len(sA), len(sB)
+    xs = np.array([[(-1) ** (i + j) * (3 + i + 16 * j) for i in range(m)] for j in range(n)], dtype=object)
+    R = np.array([[[x % int(mm) for x in row] for row in xs] for mm in ms], dtype=np.uint16)
+    got, _ = gh.reconstruct(R, sA, sB, set_name)
+    for i in range(m):
+        for j in range(n):
+            s = int(sA[i]) + int(sB[j])
+            if MARK in (int(sA[i]), int(sB[j])):
+                assert np.isnan(got[i, j]), (int(sA[i]), int(sB[j]))
+            else:
+                sign = -1.0 if xs[j][i] < 0 else 1.0
+                want = sign * np.inf if s < -2000 else 0.0 if s > 2000 else float(xs[j][i]) * 2.0 ** -s if s < 1000 else np.ldexp(float(xs[j][i]), -s)
+                assert got[i, j] == want, (int(sA[i]), int(sB[j]))
