@@ -253,6 +253,9 @@ reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride,
 // rows of one column.  A warp takes one 16-byte chunk of eight neighbouring columns: its residue loads are whole
 // 128-byte lines and its accesses to C eight pieces of 64 (128) contiguous bytes; the warps of a thread block, which
 // take the other chunks of the same columns, complete those to whole lines of C.
+// Where C takes single elements only (odd ldc, or C on an odd multiple of 8), an access in eight pieces leaves 16 or more partly
+// written sectors; a warp then takes consecutive words of one column, 512 contiguous bytes of C, and its residue loads touch eight
+// lines (7625 x 2449 x 512, set S: 1208 -> 711 us a call; 8371 x 10544 x 256: 3556 -> 1900).
 // grid: x = (piece of the block, block within the tile, CTA rank of the pair), y = tile column, z = tile row
 // SKIP: rows flagged in `skip` are left untouched (they are re-issued on the native FP64 path).
 template <int SET, bool SKIP>
@@ -275,8 +278,9 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
     const uint32_t rank = blockIdx.x / (kPieces * 16);     // 0, or 0..1 with CTA pairs
     const uint32_t tn = static_cast<uint32_t>(tn0) + blockIdx.y, tm = blockIdx.z;
     constexpr int kChunks = kColWords / 4;                 // 16-byte chunks of one column: 8 or 4
-    const uint32_t warp = threadIdx.x >> 5, c = warp % kChunks, sub = threadIdx.x & 3u;
-    const uint32_t lane = piece * kCtaCols + warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u);   // column of the block
+    const uint32_t warp = threadIdx.x >> 5, sub = threadIdx.x & 3u;
+    const uint32_t c = vecC ? warp % kChunks : (threadIdx.x >> 2) % kChunks;
+    const uint32_t lane = piece * kCtaCols + (vecC ? warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u) : threadIdx.x / kColWords);   // column of the block
     const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * (16 / RB) + sub * ROWS;
     const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
     if (row >= m || j >= n || j < col0 || j >= col1) return;
