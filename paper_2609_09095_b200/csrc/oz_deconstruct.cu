@@ -260,22 +260,35 @@ __global__ void scan_finalize_kernel(const __grid_constant__ FinalizeSide a, con
     const int side = i < a.lines ? 0 : 1;
     if (side) i -= a.lines;
     const ScanScratch s = side ? b.s : a.s;
-    const int tbits = side ? b.tbits : a.tbits;
     int32_t *shift = side ? b.shift : a.shift;
-    if (i >= (side ? b.lines : a.lines)) return;
-    if (s.nonfinite[i] < 0) {
-        shift[i] = OZ_NONFINITE_SHIFT;
-        atomicOr(status, 1u << OZ_ERR_NONFINITE_INPUT);
-        return;
+    unsigned int flatness = 0xFFFFFFFFu;
+    bool bad = false;
+    if (i < (side ? b.lines : a.lines)) {
+        const int E = s.emax[i];
+        bad = s.nonfinite[i] < 0;
+        if (bad) {
+            shift[i] = OZ_NONFINITE_SHIFT;
+        } else if (E == INT32_MIN) {
+            shift[i] = 0;
+        } else if (rule == 0) {
+            shift[i] = (side ? b.tbits : a.tbits) - 1 - E;
+        } else {
+            shift[i] = norm_exponent(s.sumsq[i], g2lo, g2hi) + 9 - E;
+            flatness = line_flatness(static_cast<unsigned int>(s.nonfinite[i]), s.sumsq[i], k);
+        }
     }
-    int E = s.emax[i];
-    if (E == INT32_MIN) { shift[i] = 0; return; }
-    if (rule == 0) { shift[i] = tbits - 1 - E; return; }
-    shift[i] = norm_exponent(s.sumsq[i], g2lo, g2hi) + 9 - E;
     // Exponent-span check (Algorithm 1, "ESC check"): the smallest flatness of each operand's lines is kept in
-    // the device status block and judged against the set's threshold when the status is queried.
-    atomicMin(status + 1 + side, line_flatness(static_cast<unsigned int>(s.nonfinite[i]), s.sumsq[i], k));
-    status[3] = esc_threshold;
+    // the device status block and judged against the set's threshold when the status is queried.  One update a warp and side: a
+    // warp may hold lines of both, and its lanes would queue up at the two words (8000 lines: 8.6 us, 4.4 with one update).
+    const unsigned int qa = __reduce_min_sync(0xFFFFFFFFu, side ? 0xFFFFFFFFu : flatness);
+    const unsigned int qb = __reduce_min_sync(0xFFFFFFFFu, side ? flatness : 0xFFFFFFFFu);
+    bad = __any_sync(0xFFFFFFFFu, bad);
+    if ((threadIdx.x & 31) == 0) {
+        if (bad) atomicOr(status, 1u << OZ_ERR_NONFINITE_INPUT);
+        if (qa != 0xFFFFFFFFu) atomicMin(status + 1, qa);
+        if (qb != 0xFFFFFFFFu) atomicMin(status + 2, qb);
+        if (min(qa, qb) != 0xFFFFFFFFu) status[3] = esc_threshold;
+    }
 }
 
 // ---- out-of-range rows (Algorithm 1, last line; Algorithm 3, "ESC range check; re-issue out-of-range
