@@ -1334,6 +1334,41 @@ ClusterShape cluster_shape(int set, int layout, int64_t lines, int64_t k, int64_
     return {static_cast<int>(blocks), tiles, fixed + static_cast<size_t>(tiles) * kTileBytes};
 }
 
+// Clusters of this many blocks that are resident at once on the current device, asked once per device.  One kernel stands for all:
+// each has 127 or 128 registers, 256 threads and no more than half of a multiprocessor's shared memory, so two blocks a
+// multiprocessor.  (A cluster stays inside a group of multiprocessors, which three and more do not fill: 148, 93, 71 and 56 clusters of
+// two to five blocks on 148 multiprocessors.)
+cudaError_t resident_clusters(int blocks, int *clusters)
+{
+    static std::atomic<int> known[64][kClusterMax + 1];
+    int dev = 0;
+    cudaError_t rc = cudaGetDevice(&dev);
+    if (rc != cudaSuccess) return rc;
+    std::atomic<int> &here = known[dev & 63][blocks];
+    *clusters = here.load(std::memory_order_relaxed);
+    if (*clusters) return cudaSuccess;
+    const auto kernel = deconstruct_cluster_kernel<2, 0, kLayoutNative>;
+    constexpr size_t half = kMaxShared / 2 - 1024;
+    static std::atomic<unsigned long long> ready{0};
+    if ((rc = allow_shared(kernel, kMaxShared, ready)) != cudaSuccess) return rc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(kConvThreads);
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+    cfg.dynamicSmemBytes = half;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(blocks);
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    rc = cudaOccupancyMaxActiveClusters(clusters, kernel, &cfg);
+    if (rc != cudaSuccess) return rc;
+    if (*clusters < 1) *clusters = 1;
+    here.store(*clusters, std::memory_order_relaxed);
+    return cudaSuccess;
+}
+
 template <int SET, int SIDE, int LAYOUT>
 oz_status_t launch_cluster(const ClusterParams &p, const ClusterShape &shape, bool alone, cudaStream_t stream)
 {
@@ -1352,16 +1387,8 @@ oz_status_t launch_cluster(const ClusterParams &p, const ClusterShape &shape, bo
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    // clusters that are resident at once, asked once per shape
-    static std::atomic<int> resident[kClusterMax + 1][8];
-    cfg.numAttrs = 1;
-    cfg.gridDim = dim3(static_cast<unsigned>(shape.blocks));
-    int clusters = resident[shape.blocks][shape.tiles].load(std::memory_order_relaxed);
-    if (!clusters) {
-        OZ_CUDA_CHECK(cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg));
-        if (clusters < 1) clusters = 1;
-        resident[shape.blocks][shape.tiles].store(clusters, std::memory_order_relaxed);
-    }
+    int clusters = 1;
+    OZ_CUDA_CHECK(resident_clusters(shape.blocks, &clusters));
     const int64_t strips = (p.f.lines + kTileLines - 1) / kTileLines;
     // as many as share the strips evenly
     const int64_t rounds = (strips + clusters - 1) / clusters, used = (strips + rounds - 1) / rounds;
