@@ -1316,24 +1316,6 @@ deconstruct_cluster_kernel(const __grid_constant__ ClusterParams cp)
     cluster_barrier();                   // no block leaves while another may still write to it
 }
 
-// Blocks of a cluster and tiles of a block for lines of `chunks` tiles, two blocks on an SM; blocks = 0: three passes.
-// Clusters of one or two blocks (k up to 1280 or 1536) win at every size measured up to 800 MB: deconstruction of 6912 x 6912 x
-// 1024, set E, 202 -> 155 us, whole call 100000 x 64 x 1000 on INT8 digits 1824 -> 1537 us.  Longer lines spread a cluster's
-// reads over the whole operand (side 0: 128 bytes from each of k columns), and one table and one block less per SM hide
-// less: up to five blocks and 256 MiB still win (6144 x 6144 x 3072 native 350 -> 335 us, 20000 x 16 x 3000 890 -> 847 us a
-// call), beyond that three passes do (4096^3, set S: 331 us against 402; 60000 x 200 x 2500 native 2000 us a call against 2300;
-// 131072 x 128 x 4096 5.4 ms against 8.0).
-struct ClusterShape { int blocks, tiles; size_t smem; };
-ClusterShape cluster_shape(int set, int layout, int64_t lines, int64_t k, int64_t chunks)
-{
-    const size_t fixed = lut_words_of(set, layout) * 4 + sizeof(ClusterExchange);
-    const int most = static_cast<int>((226 * 1024 / 2 - 1024 - fixed) / kTileBytes);
-    const int64_t blocks = (chunks + most - 1) / most, bytes = 8 * lines * k;
-    if (blocks > 5 || bytes > (blocks <= 2 ? 1ll << 30 : 1ll << 28)) return {0, 0, 0};
-    const int tiles = static_cast<int>((chunks + blocks - 1) / blocks);
-    return {static_cast<int>(blocks), tiles, fixed + static_cast<size_t>(tiles) * kTileBytes};
-}
-
 // Clusters of this many blocks that are resident at once on the current device, asked once per device.  One kernel stands for all:
 // each has 127 or 128 registers, 256 threads and no more than half of a multiprocessor's shared memory, so two blocks a
 // multiprocessor.  (A cluster stays inside a group of multiprocessors, which three and more do not fill: 148, 93, 71 and 56 clusters of
@@ -1367,6 +1349,35 @@ cudaError_t resident_clusters(int blocks, int *clusters)
     if (*clusters < 1) *clusters = 1;
     here.store(*clusters, std::memory_order_relaxed);
     return cudaSuccess;
+}
+
+// Blocks of a cluster and tiles of a block for lines of `chunks` tiles, two blocks on an SM; blocks = 0: three passes.
+// Clusters of one block win at every size measured up to 800 MB.  Larger ones are weighed against the three passes, which
+// read operands of this size from L2 and fill their last wave better: in units of what the passes take for a million elements, a strip
+// costs a cluster 0.44 a tile and 0.2 (rounds of resident clusters), and either form its start.  That is the time of every
+// layout measured, 384 to 3700 inner indices and 4.5 to 40 million elements, within 6 percent (rms).  Clusters of three and more
+// have to win by 8 percent: what they leave of the machine to the other operand's kernels is not in the sum.  3000 x 2500 x 1700, set S, 580 us with
+// clusters of three on both sides, 541 without; 2100^3 474 and 443; 6144 x 6144 x 3072 native 1836 with clusters of four, 1860
+// without.  Above 256 MiB a cluster of three or more spreads its reads over too much memory (side 0: 128 bytes from each of k
+// columns; 60000 x 200 x 2500 native 2000 us a call against 2300), and so does any cluster above 1 GiB; beyond five blocks one table
+// and one block less per SM hide too little (4096^3, set S: 331 us against 402).
+struct ClusterShape { int blocks, tiles; size_t smem; };
+ClusterShape cluster_shape(int set, int layout, int side, int64_t lines, int64_t k, int64_t chunks)
+{
+    const size_t fixed = lut_words_of(set, layout) * 4 + sizeof(ClusterExchange);
+    const int most = static_cast<int>((226 * 1024 / 2 - 1024 - fixed) / kTileBytes);
+    const int64_t blocks = (chunks + most - 1) / most, bytes = 8 * lines * k;
+    if (blocks > 5 || bytes > (blocks <= 2 ? 1ll << 30 : 1ll << 28)) return {0, 0, 0};
+    const int tiles = static_cast<int>((chunks + blocks - 1) / blocks);
+    if (blocks > 1) {
+        int clusters = 1;
+        if (resident_clusters(static_cast<int>(blocks), &clusters) != cudaSuccess) return {0, 0, 0};
+        const int64_t strips = (lines + kTileLines - 1) / kTileLines, rounds = (strips + clusters - 1) / clusters;
+        const double by_clusters = static_cast<double>(rounds) * (0.44 * tiles + 0.2) + 0.6;
+        const double by_passes = 1e-6 * static_cast<double>(lines * k) + (side == 0 ? 1.4 : 0.6);
+        if (by_clusters >= (blocks == 2 ? 1.0 : 0.92) * by_passes) return {0, 0, 0};
+    }
+    return {static_cast<int>(blocks), tiles, fixed + static_cast<size_t>(tiles) * kTileBytes};
 }
 
 template <int SET, int SIDE, int LAYOUT>
@@ -1549,7 +1560,7 @@ static ClusterShape by_clusters(int side, int64_t lines, int64_t k, int set, con
     const bool built = layout == kLayoutNative || (side == 0 ? layout != kLayoutDigits && layout != kLayoutDigitsI8
                                                              : layout == kLayoutDigits || layout == kLayoutMergedI8B);
     if (!built || geom.line_stride != kChunk || k < 1) return {0, 0, 0};
-    return cluster_shape(set, layout, lines, k, (geom.row_pitch + kChunk - 1) / kChunk);
+    return cluster_shape(set, layout, side, lines, k, (geom.row_pitch + kChunk - 1) / kChunk);
 }
 
 bool three_passes(int side, int64_t lines, int64_t k, int set, const Route &rt)
