@@ -112,7 +112,7 @@ __device__ __forceinline__ void limb_pair(long long a0, long long a1, int q, Lim
 template <int NP>
 __device__ __forceinline__ void split_limbs(const double (&x)[2 * NP], int sigma, bool tz, Limbs<NP> &L)
 {
-    if (sigma >= -1000 && sigma <= 1000) {       // 2^sigma is a normal number (always, except for lines of subnormals)
+    if (sigma >= -1000 && sigma <= 1000) {       // 2^sigma is a normal number: always, except for lines of (nearly) subnormals; no sigma is below -979
         const double scale = __hiloint2double((1023 + sigma) << 20, 0);
         if (!tz) {
 #pragma unroll
@@ -121,6 +121,18 @@ __device__ __forceinline__ void split_limbs(const double (&x)[2 * NP], int sigma
 #pragma unroll
             for (int q = 0; q < NP; ++q) limb_pair(__double2ll_rz(x[2 * q] * scale), __double2ll_rz(x[2 * q + 1] * scale), q, L);
         }
+    } else if constexpr (NP == 2) {
+        // Four elements a thread (the product kernel, whose tiles wait for their slowest row): sigma > 1000, the line holds numbers
+        // below 2^-880 only, which 2^1000 lifts into the normal range without rounding.  (3000 x 100 x 1500 in storage mode F with three
+        // such rows, set E: 385 us a call with the integer form, 354 with two multiplications; with eight or sixteen elements a thread
+        // they cost the other lines registers that spill.)
+        const double scale = __hiloint2double((1023 + sigma - 1000) << 20, 0);
+        auto lifted = [&](double v) {
+            const double y = v * 0x1p1000 * scale;
+            return tz ? __double2ll_rz(y) : __double2ll_rn(y);
+        };
+#pragma unroll
+        for (int q = 0; q < NP; ++q) limb_pair(lifted(x[2 * q]), lifted(x[2 * q + 1]), q, L);
     } else {
 #pragma unroll
         for (int q = 0; q < NP; ++q) limb_pair(quantise(x[2 * q], sigma, tz), quantise(x[2 * q + 1], sigma, tz), q, L);

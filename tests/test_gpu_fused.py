@@ -61,6 +61,24 @@ def test_fused_mode_special_lines():
     assert (np.isnan(got) == np.isnan(want)).all() and (got[~np.isnan(want)] == want[~np.isnan(want)]).all()
 
 
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("E", "int8"), ("A", "fp8")])
+@pytest.mark.parametrize("quant,rule", [("RN", "CS"), ("TZ", "CS"), ("TZ", "MAXEXP")])
+def test_fused_mode_scales_beyond_one_double(set_name, sub, quant, rule):
+    """Rows on either side of the scale 2^1000, where one multiplication becomes two, down to single subnormals."""
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(23)
+    m, n, k = 200, 40, 333
+    A, B = rng.standard_normal((m, k)), np.asfortranarray(rng.standard_normal((k, n)))
+    A[:170] *= np.exp2(-920.0 - np.arange(170))[:, None]
+    A[150, 1] = 1e-200
+    A[160:164] = 0.0
+    A[160, 7] = A[161, 0] = A[162, k - 1] = 5e-324
+    A = np.asfortranarray(A)
+    got, st = gh.dgemm(A, B, set_name, _fused(sub, quant, rule))
+    assert st == 0
+    assert (got == ozo.dgemm(A, B, OSET[set_name], getattr(ozo, "QUANT_" + quant), getattr(ozo, "SCALE_" + rule))).all()
+
+
 def test_fused_mode_limits():
     import torch
     import paper_2609_09095_b200 as oz
