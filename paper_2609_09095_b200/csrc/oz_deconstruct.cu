@@ -387,8 +387,9 @@ __device__ __forceinline__ BoundLine bound_line(const ScanScratch &s, int64_t li
     BoundLine b;
     b.E = live ? s.emax[line] : INT32_MIN;
     b.dead = !live || b.E == INT32_MIN || s.nonfinite[line] < 0;
-    b.fast = 4 - b.E >= -1000 && 4 - b.E <= 1000;         // 2^(4-E) as a double
-    b.scale = __hiloint2double((1023 + (b.fast && !b.dead ? 4 - b.E : 0)) << 20, 0);
+    const int up = b.dead ? 0 : 4 - b.E;                  // (no sum with the mark of a line of zeros)
+    b.fast = up >= -1000 && up <= 1000;                   // 2^(4-E) as a double
+    b.scale = __hiloint2double((1023 + (b.fast ? up : 0)) << 20, 0);
     return b;
 }
 __device__ __forceinline__ uint32_t bound_digit(double x, const BoundLine &b)
