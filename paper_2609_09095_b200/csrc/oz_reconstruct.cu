@@ -108,14 +108,15 @@ __device__ __forceinline__ double finish_exact(double X0, double X1, double X2, 
     return neg ? -d : d;
 }
 
-// alpha 2^-(sa + sb) c' where the fast path does not apply: NaN for a line with Inf/NaN, else by integers.  The sum of the shifts
-// is taken in 64 bits; beyond 2^20 the result is zero or infinite whatever c' is.
+// alpha 2^-(sa + sb) c' where the fast path does not apply: NaN for a line with Inf/NaN; else from r, where that is c' correctly
+// rounded and only the scale is out of reach, or by integers.  The sum of the shifts is taken in 64 bits; beyond 2^20 the result is
+// zero or infinite whatever c' is.
 template <int SET>
-__device__ __noinline__ double row_value_exact(double X0, double X1, double X2, int sa, int sb, double alpha)
+__device__ __noinline__ double row_value_exact(double X0, double X1, double X2, double r, bool rounded, int sa, int sb, double alpha)
 {
     if (sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
-    const long long sum = static_cast<long long>(sa) + sb;
-    return finish_exact(X0, X1, X2, static_cast<int>(min(max(sum, -(1ll << 20)), 1ll << 20)), SET) * alpha;
+    const int sum = static_cast<int>(min(max(static_cast<long long>(sa) + sb, -(1ll << 20)), 1ll << 20));
+    return (rounded ? scale_pow2(r, -sum) : finish_exact(X0, X1, X2, sum, SET)) * alpha;
 }
 
 // Whether a shift may enter the 32-bit sums of the fast path: |shift| <= 2^30, which the mark of a line with Inf/NaN exceeds
@@ -150,11 +151,11 @@ __device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, in
     const double rem = t - (r - s);
     const uint32_t shift_sum = static_cast<uint32_t>(sa) + static_cast<uint32_t>(sb);
     // 2^-shift_sum and r 2^-shift_sum are normal: r is zero or 1 <= |r| < 2^118
-    const bool easy = fast_column && ordinary_shift(sa) && shift_sum + 904u <= 1924u && fma(rem, 1.0 + 0x1p-29, r) == r &&
-                      (__double2hiint(r) & 0x7FFFFFFF) < K.half_M_guard;
+    const bool in_range = fast_column && ordinary_shift(sa) && shift_sum + 904u <= 1924u;
+    const bool rounded = fma(rem, 1.0 + 0x1p-29, r) == r && (__double2hiint(r) & 0x7FFFFFFF) < K.half_M_guard;
     scale = __hiloint2double(static_cast<int>((1023u - shift_sum) << 20) ^ alpha_sign, 0);
-    if (!easy) {
-        r = row_value_exact<SET>(X0, X1, X2, sa, sb, alpha);
+    if (!(in_range && rounded)) {
+        r = row_value_exact<SET>(X0, X1, X2, r, rounded, sa, sb, alpha);
         scale = 1.0;
     }
 }
