@@ -477,7 +477,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
     if (!ws || ws_bytes < L.total) return OZ_ERR_WORKSPACE;
     st = ensure_device_ready();
     if (st != OZ_OK) return st;
-    if (two_plane_applies(m, n, k, rt)) {      // fewer planes of A, more of B: within the workspace that the call has always needed
+    if (two_plane_applies(m, n, rt)) {      // fewer planes of A, more of B: within the workspace that the call has always needed
         Route two = rt;
         two.acc = 3;
         const Layout T = make_layout(m, n, k, set, two);
@@ -545,9 +545,9 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
                                  {n, B, ldb, b.planes, private_planes(n, b.pitch), b.shift, b.scratch}, k, set, rt, &both, stream);
     if (st != OZ_OK) return st;
     if (!both) {
-        const bool scans = three_passes(0, m, k, set, rt) && three_passes(1, n, k, set, rt);
+        const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
+        const bool scans = three_passes(0, ja, k, set, rt) && three_passes(1, jb, k, set, rt);
         if (scans) {      // both operands in one launch per pass; the conversions then run side by side
-            const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
             st = launch_scan(&ja, &jb, k, set, rt, true, stream);
             if (st != OZ_OK) return st;
         }

@@ -31,7 +31,8 @@ constexpr int kTileRow = (kChunk + 2) * 8;            // side 1: bytes of a tile
 constexpr int kTileBytes = kTileLines * kTileRow;    // side 0 needs kTileLines * kChunk * 8 of them
 static_assert(kTileBytes % 128 == 0, "tile alignment");
 
-// resident blocks per SM: four where no table takes shared memory and 64 registers are enough
+// resident blocks per SM: four where no table takes shared memory and 64 registers are enough (three against four: 131072 x 128 x 4096 on
+// INT8 digits 7645 and 7326 us a call, native planes of 32768 x 1024 337 and 324 us on side 0, 281 and 273 on side 1)
 __host__ __device__ constexpr int conv_blocks(int layout) { return layout == kLayoutNative || two_plane_layout(layout) ? 4 : 3; }
 
 struct ScanScratch {
@@ -512,6 +513,12 @@ __device__ __forceinline__ void load_table(uint32_t *lut, const uint32_t *__rest
 // chunks 4 l + e or 8 l + e (l = 0..7), then hit eight different bank groups
 __device__ __forceinline__ int tile_chunk(int c) { return c ^ ((c >> 3) & 7); }
 
+// Whether an operand's elements may travel two at a time: 16-byte aligned columns
+__host__ __device__ inline bool element_pairs(const double *X, int64_t ldx)
+{
+    return (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+}
+
 // asynchronous copies of one (8 bytes) or two (16 bytes) elements; nothing is read and zeros are written for bytes = 0
 __device__ __forceinline__ void copy8(uint32_t dst, const double *src, bool live)
 {
@@ -662,7 +669,7 @@ convert_kernel(const double *__restrict__ X, int64_t ldx, int64_t lines, int64_t
     const uint32_t nchunks = static_cast<uint32_t>((row_pitch + kChunk - 1) / kChunk);
     const uint32_t ltiles = static_cast<uint32_t>((lines + kTileLines - 1) / kTileLines);
     const uint32_t items = BY_LINE ? (static_cast<uint32_t>(lines) * nchunks + kTileLines - 1) / kTileLines : ltiles * nchunks;
-    const bool pairs = (ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    const bool pairs = element_pairs(X, ldx);
     const int li = warp * 2 + (lane >> 4), oct = lane & 15;        // this thread's line and octet of a tile (see tile_octet)
 
     // Position of a tile: slow index q (side 0: chunk, side 1: line tile) and fast index `rest`, so that neighbouring blocks
@@ -1019,8 +1026,9 @@ deconstruct_pair_kernel(const __grid_constant__ PairParams p)
 
 // Lines per thread-block pass of the fused kernel and its launch shape; group = 0: not applicable
 // (the lines are too long for shared memory).
-// Largest operand of the one-kernel form.  Above, the three-pass kernels win (2500 x 2500 x 1024: equal; 1500^3: 171
-// against 165 us a call; 4000 x 1000 x 1000: 217 against 229).
+// Largest operand of the one-kernel form; above, clusters or three passes.  A call with the limit at 2 M, 4 M and 8 M elements: 3000 x 300 x
+// 1200, set S, 125, 116 and 126 us; 4000 x 1000 x 1000 230, 225 and 225; 2500 x 2500 x 1024 308, 308 and 298; 2300 x 2300 x 2000 467, 467 and
+// 478 (native 255, 255 and 270); only a tall operand of few rounds would go on winning (5000 x 200 x 1000 137, 138 and 119).
 constexpr int64_t kFusedMaxElems = 1ll << 22;
 struct FusedShape { int group, threads, grid; size_t smem; };
 
@@ -1117,8 +1125,10 @@ FusedParams fused_params(int side, int64_t lines, int64_t k, const double *X, in
 // travel to the other blocks of the cluster through distributed shared memory, one cluster barrier each.  Blocks stay
 // resident and walk the strips of 16 lines; a tile's place is refilled with the next strip as soon as it has been converted, so
 // that loads run beside the arithmetic.  Same functions and integer sums as the other forms: the same bits.
-// Bound: DRAM, 8 bytes read and all planes written at the rate that such a mix reaches (5.2 to 5.5 TB/s: what the conversion takes
-// when its arithmetic is left out).
+// Bound: the phases of a strip, one behind the other, with 16 warps an SM to cover them.  8192 x 1024, set S on FP8: 89 us a side, 3.6 TB/s of
+// the bytes it cannot do without where their traffic alone runs at 5.2 to 5.5; issue slots 41 % busy, no pipe above 31 %, the waits
+// spread over dependent arithmetic, table look-ups, global loads and barriers.  6144 x 3072 native, clusters of four: 157 us, 2.8 TB/s, issue 46 %, FP32
+// pipe 44 %.
 struct ClusterParams {
     FusedParams f;               // group, pitch: not used
     int tiles;
@@ -1181,7 +1191,7 @@ deconstruct_cluster_kernel(const __grid_constant__ ClusterParams cp)
     const int li = warp * 2 + (lane >> 4), oct = lane & 15;
     const unsigned int half = lane < 16 ? 0xFFFFu : 0xFFFF0000u;
     const uint32_t rank = cluster_rank(), C = cluster_blocks();
-    const bool pairs = (p.ldx & 1) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15u) == 0;
+    const bool pairs = element_pairs(p.X, p.ldx);
     const int64_t nchunks = (p.geom.row_pitch + kChunk - 1) / kChunk, strips = (p.lines + kTileLines - 1) / kTileLines;
     const int64_t chunk0 = static_cast<int64_t>(rank) * T;
     const int nt = static_cast<int>(nchunks - chunk0 < T ? (nchunks - chunk0 > 0 ? nchunks - chunk0 : 0) : T);
@@ -1361,22 +1371,24 @@ cudaError_t resident_clusters(int blocks, int *clusters)
 // clusters of three on both sides, 541 without; 2100^3 474 and 443; 6144 x 6144 x 3072 native 1836 with clusters of four, 1860
 // without.  Above 256 MiB a cluster of three or more spreads its reads over too much memory (side 0: 128 bytes from each of k
 // columns; 60000 x 200 x 2500 native 2000 us a call against 2300), and so does any cluster above 1 GiB; beyond five blocks one table
-// and one block less per SM hide too little (4096^3, set S: 331 us against 402).
+// and one block less per SM hide too little (4096^3, set S: 331 us against 402).  Operands that are copied element by element (an odd
+// leading dimension, or off the 16-byte boundary) cost a cluster a fifth more on side 0 and a twentieth on side 1, the passes
+// nothing (median over the same sizes; 40113 x 135 x 1071 by clusters 1024 us a call, by passes 913), also in clusters of one.
 struct ClusterShape { int blocks, tiles; size_t smem; };
-ClusterShape cluster_shape(int set, int layout, int side, int64_t lines, int64_t k, int64_t chunks)
+ClusterShape cluster_shape(int set, int layout, int side, int64_t lines, int64_t k, int64_t chunks, bool pairs)
 {
     const size_t fixed = lut_words_of(set, layout) * 4 + sizeof(ClusterExchange);
     const int most = static_cast<int>((226 * 1024 / 2 - 1024 - fixed) / kTileBytes);
     const int64_t blocks = (chunks + most - 1) / most, bytes = 8 * lines * k;
     if (blocks > 5 || bytes > (blocks <= 2 ? 1ll << 30 : 1ll << 28)) return {0, 0, 0};
     const int tiles = static_cast<int>((chunks + blocks - 1) / blocks);
-    if (blocks > 1) {
+    if (blocks > 1 || !pairs) {
         int clusters = 1;
         if (resident_clusters(static_cast<int>(blocks), &clusters) != cudaSuccess) return {0, 0, 0};
         const int64_t strips = (lines + kTileLines - 1) / kTileLines, rounds = (strips + clusters - 1) / clusters;
-        const double by_clusters = static_cast<double>(rounds) * (0.44 * tiles + 0.2) + 0.6;
+        const double by_clusters = (static_cast<double>(rounds) * (0.44 * tiles + 0.2) + 0.6) * (pairs ? 1.0 : side == 0 ? 1.2 : 1.05);
         const double by_passes = 1e-6 * static_cast<double>(lines * k) + (side == 0 ? 1.4 : 0.6);
-        if (by_clusters >= (blocks == 2 ? 1.0 : 0.92) * by_passes) return {0, 0, 0};
+        if (by_clusters >= (blocks <= 2 ? 1.0 : 0.92) * by_passes) return {0, 0, 0};
     }
     return {static_cast<int>(blocks), tiles, fixed + static_cast<size_t>(tiles) * kTileBytes};
 }
@@ -1554,19 +1566,23 @@ static FusedShape lone_shape(int side, int64_t lines, int64_t k, int set, const 
     return f;
 }
 
-// The cluster form: planes in the private layout of the whole-method schedules, lines that fit a cluster
-static ClusterShape by_clusters(int side, int64_t lines, int64_t k, int set, const Route &rt, const PlaneGeom &geom)
+// The cluster form: planes in the private layout, lines that fit a cluster, and the layouts of the schedules that calls take by
+// default (merged, native, A of the two-plane schedule; B's digits on FP8 are those of either schedule).  INT8 calls with
+// OZ_ACC_SEPARATE therefore take three passes on both operands and FP8 calls with it on A; so does B of the two-plane schedule, whose 128
+// lines at most exceed 4 M elements from k = 32768 on, beyond any cluster.
+static ClusterShape by_clusters(int side, int64_t lines, int64_t k, int set, const Route &rt, const PlaneGeom &geom, const double *X, int64_t ldx)
 {
     const int layout = rt.layout(side);
     const bool built = layout == kLayoutNative || (side == 0 ? layout != kLayoutDigits && layout != kLayoutDigitsI8
                                                              : layout == kLayoutDigits || layout == kLayoutMergedI8B);
     if (!built || geom.line_stride != kChunk || k < 1) return {0, 0, 0};
-    return cluster_shape(set, layout, side, lines, k, (geom.row_pitch + kChunk - 1) / kChunk);
+    return cluster_shape(set, layout, side, lines, k, (geom.row_pitch + kChunk - 1) / kChunk, element_pairs(X, ldx));
 }
 
-bool three_passes(int side, int64_t lines, int64_t k, int set, const Route &rt)
+bool three_passes(int side, const ScanJob &j, int64_t k, int set, const Route &rt)
 {
-    return lone_shape(side, lines, k, set, rt).group <= 0 && by_clusters(side, lines, k, set, rt, private_planes(lines, round_up(k, kChunk))).blocks == 0;
+    return lone_shape(side, j.lines, k, set, rt).group <= 0 &&
+           by_clusters(side, j.lines, k, set, rt, private_planes(j.lines, round_up(k, kChunk)), j.X, j.ldx).blocks == 0;
 }
 
 oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
@@ -1596,7 +1612,7 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
 #undef OZ_FUSED_SET
 #undef OZ_FUSED
     }
-    const ClusterShape c = by_clusters(side, lines, k, set, rt, geom);
+    const ClusterShape c = by_clusters(side, lines, k, set, rt, geom, X, ldx);
     if (c.blocks) {
         ClusterParams p;
         p.f = fused_params(side, lines, k, X, ldx, set, rt, planes, geom, shift, scratch, 0);

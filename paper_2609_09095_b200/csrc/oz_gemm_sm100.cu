@@ -1151,7 +1151,9 @@ oz_status_t launch_tiled(const CUtensorMap &mapA, const CUtensorMap &mapB, const
 }
 
 // Tiles of 64 rows instead of 256 where the rounds over the SMs then cost less.  A narrow tile is bound by its operands' way
-// from L2 to shared memory, of which it needs 5/8 per K chunk (20 of 32 KiB), not by its quarter of the products.
+// from L2 to shared memory, not by its quarter of the products: per K chunk it needs 5/8 of a wide one's bytes in CTA pairs and with
+// 128 lines of B in the two-plane schedule (20 of 32, 40 of 64 KiB), half in the other forms (24 of 48).  5/8 serves them all: with
+// 4/8 and 6/8 products of 200 to 9000 rows and 16 to 300 columns stayed within 3 percent either way (1300 x 128 x 300: 23.2, 22.6 and 22.6 us).
 bool narrow_tiles(int64_t m, int64_t tiles_n, int r, int cg, int sms)
 {
     const int64_t groups = sms / cg;
@@ -1290,15 +1292,15 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k, bo
     }
 }
 
-bool two_plane_applies(int64_t m, int64_t n, int64_t k, const Route &rt)
+bool two_plane_applies(int64_t m, int64_t n, const Route &rt)
 {
     return rt.automatic && rt.merged() && !rt.fused && n <= BLOCK_M && m >= n;
 }
 
 // Kept operands (planes of the merged layouts): a fifth less of A from memory for a sixth more products, and K segments on set S.
-// Taken up to 64 columns, and where the tiles cover the SMs or one segment holds k (10240 x 64 x 10240 a call, S: 554 -> 524 us,
-// 4000 x 64 x 4000 142 -> 124, 1500 x 16 x 6000 on E 97 -> 88; not 1000 x 32 x 12000 on S: 143 against 149, nor 100 columns:
-// 4000 x 100 x 4000 146 against 154).
+// Taken up to 64 columns, and where the tiles cover the SMs or one segment holds k (the call with three planes and with two, S:
+// 10240 x 64 x 10240 558 -> 541 us, 10240 x 16 x 10240 558 -> 523; 6000 x 32 x 3000 on A 158 -> 139; 4000 x 64 x 4000 the same; 1500 x 16 x 6000
+// on E 95 -> 97; not 1000 x 32 x 12000 on S: 138 -> 146, nor 100 columns: 4000 x 100 x 4000 119 -> 118).
 static bool slim_merged(int64_t m, int64_t n, int64_t k, int set, int sms)
 {
     const int64_t tiles = set_r(set) * ((m + BLOCK_N - 1) / BLOCK_N);

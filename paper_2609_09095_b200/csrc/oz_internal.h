@@ -237,8 +237,8 @@ struct ScanJob {
     int32_t *shift;
     void *scratch;
 };
-// whether launch_deconstruct() takes the scans and the conversion (else the one-kernel form)
-bool three_passes(int side, int64_t lines, int64_t k, int set, const Route &rt);
+// whether launch_deconstruct() takes the scans and the conversion into private planes (else the one-kernel or the cluster form)
+bool three_passes(int side, const ScanJob &job, int64_t k, int set, const Route &rt);
 oz_status_t launch_scan(const ScanJob *a, const ScanJob *b, int64_t k, int set, const Route &rt, bool alone, cudaStream_t stream);
 oz_status_t launch_convert_planes(int side, int64_t lines, int64_t k, const double *X, int64_t ldx,
                                   int set, const Route &rt, uint8_t *planes, const PlaneGeom &geom,
@@ -266,7 +266,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
                                 cudaStream_t stream);
 
 // Whether a whole-method call takes the two-plane schedule (planes private to the call, schedule left to the library)
-bool two_plane_applies(int64_t m, int64_t n, int64_t k, const Route &rt);
+bool two_plane_applies(int64_t m, int64_t n, const Route &rt);
 
 // Storage mode F: residue products with A converted on the fly inside the kernel (n <= 128, merged
 // schedule on digit planes, k within the exact depth of one accumulator); public residue layout

@@ -54,10 +54,11 @@ def _same(got, want):
 
 @pytest.mark.parametrize("set_name,sub", ROUTES)
 @pytest.mark.parametrize("lines,k,pad,offset", [
-    (7010, 597, 0, 0),          # one block
-    (4699, 1191, 1, 0),         # two; an odd leading dimension on one side or the other
+    (9470, 597, 0, 0),          # one block
+    (4699, 1191, 0, 0),         # two, odd leading dimensions on both sides
+    (4700, 1190, 0, 1),         # two, off the 16-byte boundary
     (2970, 1893, 2, 0),         # three
-    (2266, 2441, 1, 1),         # four, off the 16-byte boundary
+    (2266, 2442, 0, 0),         # four
     (1785, 3150, 3, 0),         # five
 ])
 @pytest.mark.parametrize("side", [0, 1])
