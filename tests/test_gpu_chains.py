@@ -25,7 +25,10 @@ def test_calls_back_to_back_in_one_workspace():
             (256, 256, 256, "S", "fp8", "CS", 0),                        # joint deconstruction, early reconstruction
             (1500, 1490, 1500, "S", "fp8", "CS", 0),                     # two streams, one-kernel form of each operand
             (200, 300, 260, "A", "int8n", "MAXEXP", 0),
-            (3000, 2500, 1700, "E", "int8", "CS", 0),                    # three-pass deconstruction
+            (3000, 2500, 1700, "E", "int8", "CS", 0),                    # three passes over both: joint scans, then two streams
+            (1000, 900, 5003, "S", "fp8", "CS", 0),                      # the same with lines too long for a cluster
+            (4700, 4500, 1190, "E", "int8", "CS", 0),                    # both by clusters, on two streams
+            (4700, 64, 1190, "S", "fp8", "CS", oz.OZ_FALLBACK_FP64),     # A by clusters, with the row check behind it
             (64, 33, 700, "S", "int8", "CS", 0),
             (700, 650, 500, "S", "fp8", "ACCURATE", 0),
             (2000, 100, 900, "S", "fp8", "CS", oz.OZ_STORAGE_FUSED),

@@ -10,13 +10,15 @@ from oracle import oz_oracle as ozo
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("m,n,k,set_name,sub,mode", [
-    (256, 256, 256, "S", "fp8", None),            # one-kernel deconstruction
-    (300, 2200, 2100, "A", "int8n", None),        # three-pass deconstruction of B
-    (300, 100, 500, "S", "fp8", "fused"),         # storage mode F: A converted inside the product kernel
-    (200, 150, 300, "A", "fp8", "fallback"),      # native FP64 path: the number of re-issued rows varies per replay
+@pytest.mark.parametrize("m,n,k,set_name,sub,mode,launches", [
+    (256, 256, 256, "S", "fp8", None, 3),            # one-kernel deconstruction
+    (300, 2200, 2100, "A", "int8n", None, 8),        # three-pass deconstruction of B
+    (100, 4700, 1190, "S", "fp8", None, 4),          # deconstruction of B by clusters
+    (1000, 900, 5003, "S", "fp8", None, 8),          # three passes over both: joint scans, then a fork for the conversions
+    (300, 100, 500, "S", "fp8", "fused", 7),         # storage mode F: A converted inside the product kernel
+    (200, 150, 300, "A", "fp8", "fallback", 5),      # native FP64 path: the number of re-issued rows varies per replay
 ])
-def test_dgemm_replayed_from_a_cuda_graph(m, n, k, set_name, sub, mode):
+def test_dgemm_replayed_from_a_cuda_graph(m, n, k, set_name, sub, mode, launches):
     import torch
     import paper_2609_09095_b200 as oz
     import tests.gpu_helpers as gh
@@ -32,7 +34,9 @@ def test_dgemm_replayed_from_a_cuda_graph(m, n, k, set_name, sub, mode):
     side = torch.cuda.Stream()
     with torch.cuda.stream(side):
         # plain call first: internal stream and events are created outside the capture
+        before = oz.oz_launch_count()
         oz.check(oz.oz_dgemm(m, n, k, dA, m, dB, k, dC, m, sid, rt, side), "oz_dgemm")
+        assert oz.oz_launch_count() - before == launches
         side.synchronize()
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph, stream=side):
@@ -55,5 +59,5 @@ def test_dgemm_replayed_from_a_cuda_graph(m, n, k, set_name, sub, mode):
             want, flag = ozo.dgemm_fallback(A, B, oset)
             assert oz.oz_query_fallback_rows() == int(flag.sum())
         else:
-            want = ozo.dgemm(A, B, oset)
-        assert (gh.from_dev(dC) == want).all()
+            want = ozo.dgemm(np.asfortranarray(A[:300]), B, oset)
+        assert (gh.from_dev(dC)[:300] == want).all()
