@@ -456,7 +456,7 @@ def main():
         achieved = lowp_flops / (gemm_ms * 1e-3) / 1e12
         roof_nominal = 4500.0 / (passes + 1)               # P_low/(3r+1), or P_low/(r+1) native INT8, at B200's dense 8-bit rate
         hbm = peaks["hbm_gbs"]
-        dec_bytes = 24 * (m * k + k * n) + (p_store_a * m + p_store * n) * k   # two scan passes + convert read; planes written
+        dec_bytes = 8 * (m * k + k * n) + (p_store_a * m + p_store * n) * k    # operands read once, planes written, whatever form is taken
         rb = oz.oz_residue_elem_bytes(modset)                 # bytes per stored residue
         rec_bytes = (rb * r + 8 + (8 if cfg.beta else 0)) * m * n
         plane_bytes = float((p_store_a * m + p_store * n) * k)
@@ -495,7 +495,7 @@ def main():
             "stages": {
                 "deconstruct_A_ms": float(stage_ms[0]), "deconstruct_join_ms": float(stage_ms[1]),
                 "residue_gemm_ms": gemm_ms, "reconstruct_ms": float(stage_ms[3]),
-                "deconstruct_GBps": dec_bytes / ((stage_ms[0] + stage_ms[1]) * 1e-3) / 1e9,
+                "deconstruct_bytes": dec_bytes, "deconstruct_GBps": dec_bytes / ((stage_ms[0] + stage_ms[1]) * 1e-3) / 1e9,
                 "reconstruct_GBps": rec_bytes / (stage_ms[3] * 1e-3) / 1e9,
                 "reconstruct_bytes": rec_bytes,
                 "call_ms_median": float(np.median(step_totals)), "call_ms_best": float(step_totals.min()),
