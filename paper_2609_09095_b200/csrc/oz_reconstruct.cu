@@ -39,8 +39,9 @@ __host__ __device__ constexpr int chunk_bits(int set) { return set == 2 ? 40 : 3
 __host__ __device__ constexpr double pow2d(int e) { double v = 1.0; for (int i = 0; i < e; ++i) v *= 2.0; return v; }
 // Resident blocks per SM.  The loads of a thread are independent, so this many keep memory busy; the registers they leave
 // (48, 64) hold everything.  16384 x 16384 update, set S, with 4 / 5 / 6 blocks: 2.18 / 2.17 / 2.17 ms; 6144 x 6144, set A, with
-// 3 / 4 / 5 blocks: 288 / 289 / 298 us.  Before the mapping and the arithmetic below: 2.35 ms and 327 us.
-template <int SET> constexpr int kReconBlocks = residue_bytes(SET) == 2 ? 5 : 4;
+// 3 / 4 / 5 blocks: 288 / 289 / 298 us.  Before the mapping and the arithmetic below: 2.35 ms and 327 us.  One more where C takes
+// single elements only, since its old values are then waited for in turn.
+template <int SET, bool VEC = true> constexpr int kReconBlocks = (residue_bytes(SET) == 2 ? 5 : 4) + (VEC ? 0 : 1);
 constexpr double kRint = 6755399441055744.0;          // 1.5 * 2^52: (x + kRint) - kRint = rint(x)
 
 // x * 2^scale for a finite double x (exact unless the result leaves the normal range)
@@ -108,22 +109,35 @@ __device__ __forceinline__ double finish_exact(double X0, double X1, double X2, 
     return neg ? -d : d;
 }
 
-// alpha 2^-(sa + sb) c' where the fast path does not apply: NaN for a line with Inf/NaN; else from r, where that is c' correctly
+// The three chunks summed: r is c' correctly rounded if the result is true (see row_value())
+template <int SET>
+__device__ __forceinline__ bool round_chunks(double X0, double X1, double X2, double &r)
+{
+    const double s = X2 + X1, err = X1 - (s - X2);
+    const double t = err + X0;
+    r = s + t;
+    const double rem = t - (r - s);
+    return fma(rem, 1.0 + 0x1p-29, r) == r && (__double2hiint(r) & 0x7FFFFFFF) < c_recon[SET].half_M_guard;
+}
+
+// alpha 2^-(sa + sb) c' (alpha = 1 or -1, as a sign bit: in a register pair of its own it spilled) where the fast path does not apply: NaN for a line with Inf/NaN; else from r, where that is c' correctly
 // rounded and only the scale is out of reach, or by integers.  The sum of the shifts is taken in 64 bits; beyond 2^20 the result is
 // zero or infinite whatever c' is.
 template <int SET>
-__device__ __noinline__ double row_value_exact(double X0, double X1, double X2, double r, bool rounded, int sa, int sb, double alpha)
+__device__ __noinline__ double row_value_exact(double X0, double X1, double X2, int sa, int sb, int alpha_sign)
 {
+    const double alpha = __hiloint2double(0x3FF00000 ^ alpha_sign, 0);
     if (sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
     const int sum = static_cast<int>(min(max(static_cast<long long>(sa) + sb, -(1ll << 20)), 1ll << 20));
-    return (rounded ? scale_pow2(r, -sum) : finish_exact(X0, X1, X2, sum, SET)) * alpha;
+    double r;
+    return (round_chunks<SET>(X0, X1, X2, r) ? scale_pow2(r, -sum) : finish_exact(X0, X1, X2, sum, SET)) * alpha;
 }
 
-// Whether a shift may enter the 32-bit sums of the fast path: |shift| <= 2^30, which the mark of a line with Inf/NaN exceeds
-constexpr int kShiftLimit = 1 << 30;
-__device__ __forceinline__ bool ordinary_shift(int s)
+// Whether a row's shift may enter the 32-bit sums of the fast path: |sa| <= 2^30, which the mark of a row with Inf/NaN exceeds.  No sum
+// with a column's shift, whatever that is and the mark of a column among them, then wraps into the range of row_value().
+__device__ __forceinline__ bool ordinary_row(int sa)
 {
-    return static_cast<uint32_t>(s) + static_cast<uint32_t>(kShiftLimit) <= 2u * static_cast<uint32_t>(kShiftLimit);
+    return static_cast<uint32_t>(sa) + (1u << 30) <= 1u << 31;
 }
 
 // One row of the thread's group: value = fast alpha 2^-(sa + sb) c', returned as the rounded integer r and the power of
@@ -135,7 +149,7 @@ __device__ __forceinline__ bool ordinary_shift(int s)
 // rounding boundary -- adding rem, enlarged by 2^-29, then moves r -- or so near to +-M/2 that the lift may apply.
 // 50 FP64 operations per output on set S where the carries and a test by exponents took 63.
 template <int SET, int HALF>
-__device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, int sb, bool fast_column, int alpha_sign, double alpha,
+__device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, int sb, int alpha_sign,
                                           double &r, double &scale)
 {
     const ReconConst &K = c_recon[SET];
@@ -145,17 +159,12 @@ __device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, in
     X0 = fma(-kappa, K.Mc[0], X0);              // exact: integers below 2^53 (times 2^cw, 2^(2cw))
     X1 = fma(-kappa, K.Mc[1], X1);
     X2 = fma(-kappa, K.Mc[2], X2);
-    const double s = X2 + X1, err = X1 - (s - X2);
-    const double t = err + X0;
-    r = s + t;
-    const double rem = t - (r - s);
+    const bool rounded = round_chunks<SET>(X0, X1, X2, r);
     const uint32_t shift_sum = static_cast<uint32_t>(sa) + static_cast<uint32_t>(sb);
-    // 2^-shift_sum and r 2^-shift_sum are normal: r is zero or 1 <= |r| < 2^118
-    const bool in_range = fast_column && ordinary_shift(sa) && shift_sum + 904u <= 1924u;
-    const bool rounded = fma(rem, 1.0 + 0x1p-29, r) == r && (__double2hiint(r) & 0x7FFFFFFF) < K.half_M_guard;
     scale = __hiloint2double(static_cast<int>((1023u - shift_sum) << 20) ^ alpha_sign, 0);
-    if (!(in_range && rounded)) {
-        r = row_value_exact<SET>(X0, X1, X2, r, rounded, sa, sb, alpha);
+    // in range: 2^-shift_sum and r 2^-shift_sum are normal; r is zero or 1 <= |r| < 2^118
+    if (!(ordinary_row(sa) && shift_sum + 904u <= 1924u && rounded)) {
+        r = row_value_exact<SET>(X0, X1, X2, sa, sb, alpha_sign);
         scale = 1.0;
     }
 }
@@ -187,20 +196,19 @@ __device__ __forceinline__ void reconstruct_rows(const uint32_t (&w)[kMaxR], int
 #pragma unroll
         for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + 2 * h);
     }
-    const bool fast_column = ordinary_shift(sb);
     const int alpha_sign = alpha < 0.0 ? INT32_MIN : 0;
     {
         double r0, r1 = 0.0, f0, f1 = 1.0;
-        row_value<SET, 0>(w, sa[0], sb, fast_column, alpha_sign, alpha, r0, f0);
-        if (nrows > 1) row_value<SET, 1>(w, sa[1], sb, fast_column, alpha_sign, alpha, r1, f1);
+        row_value<SET, 0>(w, sa[0], sb, alpha_sign, r0, f0);
+        if (nrows > 1) row_value<SET, 1>(w, sa[1], sb, alpha_sign, r1, f1);
         if (whole) *reinterpret_cast<double2 *>(out) = make_double2(fma(r0, f0, old[0].x), fma(r1, f1, old[0].y));
         else store_pair(out, r0 * f0, r1 * f1, (keep & 1u) != 0, nrows > 1 && (keep & 2u) != 0, beta);
     }
     if constexpr (ROWS == 4) {
         if (nrows > 2) {
             double r2, r3 = 0.0, f2, f3 = 1.0;
-            row_value<SET, 2>(w, sa[2], sb, fast_column, alpha_sign, alpha, r2, f2);
-            if (nrows > 3) row_value<SET, 3>(w, sa[3], sb, fast_column, alpha_sign, alpha, r3, f3);
+            row_value<SET, 2>(w, sa[2], sb, alpha_sign, r2, f2);
+            if (nrows > 3) row_value<SET, 3>(w, sa[3], sb, alpha_sign, r3, f3);
             if (whole) *reinterpret_cast<double2 *>(out + 2) = make_double2(fma(r2, f2, old[1].x), fma(r3, f3, old[1].y));
             else store_pair(out + 2, r2 * f2, r3 * f3, (keep & 4u) != 0, nrows > 3 && (keep & 8u) != 0, beta);
         }
@@ -254,17 +262,18 @@ reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride,
 // rows of one column.  A warp takes one 16-byte chunk of eight neighbouring columns: its residue loads are whole
 // 128-byte lines and its accesses to C eight pieces of 64 (128) contiguous bytes; the warps of a thread block, which
 // take the other chunks of the same columns, complete those to whole lines of C.
-// Where C takes single elements only (odd ldc, or C on an odd multiple of 8), an access in eight pieces leaves 16 or more partly
-// written sectors; a warp then takes consecutive words of one column, 512 contiguous bytes of C, and its residue loads touch eight
-// lines (7625 x 2449 x 512, set S: 1208 -> 711 us a call; 8371 x 10544 x 256: 3556 -> 1900).
+// VEC: C takes pairs of elements (even ldc, C on a multiple of 16 bytes).  Otherwise an update of C (beta = 1), whose loads and stores of
+// single elements in eight pieces each cost more the more there are, gives a warp consecutive words of one column: 512 contiguous
+// bytes of C for residue loads that touch eight lines.  1009 x 983 x 256, set S: 39 us a call against 52; 4501 x 4400 x 128: 400 against
+// 732; plain stores are faster in pieces (34 us against 36, 334 against 352).
 // grid: x = (piece of the block, block within the tile, CTA rank of the pair), y = tile column, z = tile row
 // SKIP: rows flagged in `skip` are left untouched (they are re-issued on the native FP64 path).
-template <int SET, bool SKIP>
-__global__ void __launch_bounds__(256, kReconBlocks<SET>)
+template <int SET, bool SKIP, bool VEC>
+__global__ void __launch_bounds__(256, kReconBlocks<SET, VEC>)
 reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int tn0,
                          int64_t m, int64_t n, int64_t col0, int64_t col1,
                          const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
-                         double alpha, double beta, double *__restrict__ C, int64_t ldc, int vecC,
+                         double alpha, double beta, double *__restrict__ C, int64_t ldc,
                          const unsigned char *__restrict__ skip)
 {
     dependency_release();
@@ -280,8 +289,9 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
     const uint32_t tn = static_cast<uint32_t>(tn0) + blockIdx.y, tm = blockIdx.z;
     constexpr int kChunks = kColWords / 4;                 // 16-byte chunks of one column: 8 or 4
     const uint32_t warp = threadIdx.x >> 5, sub = threadIdx.x & 3u;
-    const uint32_t c = vecC ? warp % kChunks : (threadIdx.x >> 2) % kChunks;
-    const uint32_t lane = piece * kCtaCols + (vecC ? warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u) : threadIdx.x / kColWords);   // column of the block
+    const bool spread = VEC || beta == 0.0;
+    const uint32_t c = spread ? warp % kChunks : (threadIdx.x >> 2) % kChunks;
+    const uint32_t lane = piece * kCtaCols + (spread ? warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u) : threadIdx.x / kColWords);   // column of the block
     const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * (16 / RB) + sub * ROWS;
     const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
     if (row >= m || j >= n || j < col0 || j >= col1) return;
@@ -301,7 +311,7 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
     uint32_t w[kMaxR];
 #pragma unroll
     for (int i = 0; i < r; ++i) w[i] = *reinterpret_cast<const uint32_t *>(base + i * (kBlockWords * 4));
-    reconstruct_rows<SET>(w, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, vecC != 0, keep);
+    reconstruct_rows<SET>(w, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, VEC, keep);
 }
 
 }  // namespace
@@ -381,13 +391,15 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     // Blocks that become resident beside the GEMM's keep the multiprocessor's memory split at the GEMM's (28 KiB of L1) for
     // the whole kernel: worth the overlapped launch up to a million outputs only (16384 x 16384: 11.4 -> 11.9 ms a call)
     const bool early = m * n <= (1ll << 20);
+#define OZ_RECON_KERNEL(SET_, SKIP_) (vecC ? reconstruct_tiled_kernel<SET_, SKIP_, true> : reconstruct_tiled_kernel<SET_, SKIP_, false>)
 #define OZ_RECON_TILED(SET_)                                                                                         \
-    OZ_CUDA_CHECK(launch_if(early, skip ? reconstruct_tiled_kernel<SET_, true> : reconstruct_tiled_kernel<SET_, false>, grid, 256, 0, \
-                         stream, R, t.cg, t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, vecC, skip))
+    OZ_CUDA_CHECK(launch_if(early, skip ? OZ_RECON_KERNEL(SET_, true) : OZ_RECON_KERNEL(SET_, false), grid, 256, 0, stream, R, t.cg, \
+                         t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, skip))
     if (set == 2) OZ_RECON_TILED(2);
     else if (set == 0) OZ_RECON_TILED(0);
     else OZ_RECON_TILED(1);
 #undef OZ_RECON_TILED
+#undef OZ_RECON_KERNEL
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
