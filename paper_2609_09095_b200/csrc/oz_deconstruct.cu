@@ -1372,8 +1372,8 @@ cudaError_t resident_clusters(int blocks, int *clusters)
 // without.  Above 256 MiB a cluster of three or more spreads its reads over too much memory (side 0: 128 bytes from each of k
 // columns; 60000 x 200 x 2500 native 2000 us a call against 2300), and so does any cluster above 1 GiB; beyond five blocks one table
 // and one block less per SM hide too little (4096^3, set S: 331 us against 402).  Operands that are copied element by element (an odd
-// leading dimension, or off the 16-byte boundary) cost a cluster a fifth more on side 0 and a twentieth on side 1, the passes
-// nothing (median over the same sizes; 40113 x 135 x 1071 by clusters 1024 us a call, by passes 913), also in clusters of one.
+// leading dimension, or off the 16-byte boundary) cost the passes nothing more and a cluster of two a tenth on side 0, larger ones a fifth, and a
+// twentieth on side 1 (medians over the same sizes; 40113 x 135 x 1071 by clusters 1024 us a call, by passes 913).
 struct ClusterShape { int blocks, tiles; size_t smem; };
 ClusterShape cluster_shape(int set, int layout, int side, int64_t lines, int64_t k, int64_t chunks, bool pairs)
 {
@@ -1382,13 +1382,13 @@ ClusterShape cluster_shape(int set, int layout, int side, int64_t lines, int64_t
     const int64_t blocks = (chunks + most - 1) / most, bytes = 8 * lines * k;
     if (blocks > 5 || bytes > (blocks <= 2 ? 1ll << 30 : 1ll << 28)) return {0, 0, 0};
     const int tiles = static_cast<int>((chunks + blocks - 1) / blocks);
-    if (blocks > 1 || !pairs) {
+    if (blocks > 1) {
         int clusters = 1;
         if (resident_clusters(static_cast<int>(blocks), &clusters) != cudaSuccess) return {0, 0, 0};
         const int64_t strips = (lines + kTileLines - 1) / kTileLines, rounds = (strips + clusters - 1) / clusters;
-        const double by_clusters = (static_cast<double>(rounds) * (0.44 * tiles + 0.2) + 0.6) * (pairs ? 1.0 : side == 0 ? 1.2 : 1.05);
+        const double by_clusters = (static_cast<double>(rounds) * (0.44 * tiles + 0.2) + 0.6) * (pairs ? 1.0 : side == 1 ? 1.05 : blocks == 2 ? 1.1 : 1.2);
         const double by_passes = 1e-6 * static_cast<double>(lines * k) + (side == 0 ? 1.4 : 0.6);
-        if (by_clusters >= (blocks <= 2 ? 1.0 : 0.92) * by_passes) return {0, 0, 0};
+        if (by_clusters >= (blocks == 2 ? 1.0 : 0.92) * by_passes) return {0, 0, 0};
     }
     return {static_cast<int>(blocks), tiles, fixed + static_cast<size_t>(tiles) * kTileBytes};
 }
