@@ -39,9 +39,10 @@ __host__ __device__ constexpr int chunk_bits(int set) { return set == 2 ? 40 : 3
 __host__ __device__ constexpr double pow2d(int e) { double v = 1.0; for (int i = 0; i < e; ++i) v *= 2.0; return v; }
 // Resident blocks per SM.  The loads of a thread are independent, so this many keep memory busy; the registers they leave
 // (48, 64) hold everything.  16384 x 16384 update, set S, with 4 / 5 / 6 blocks: 2.18 / 2.17 / 2.17 ms; 6144 x 6144, set A, with
-// 3 / 4 / 5 blocks: 288 / 289 / 298 us.  Before the mapping and the arithmetic below: 2.35 ms and 327 us.  One more where C takes
-// single elements only, since its old values are then waited for in turn.
-template <int SET, bool VEC = true> constexpr int kReconBlocks = (residue_bytes(SET) == 2 ? 5 : 4) + (VEC ? 0 : 1);
+// 3 / 4 / 5 blocks: 288 / 289 / 298 us.  Before the mapping and the arithmetic below: 2.35 ms and 327 us.  One more where single elements
+// of C are updated, since their old values are waited for in turn; not for plain stores, whose blocks of 40 registers would fit beside a
+// GEMM's and become resident with it (499 x 366 x 2755 under the accurate rule 94 -> 102 us a call).
+template <int SET, bool SINGLE_UPDATES = false> constexpr int kReconBlocks = (residue_bytes(SET) == 2 ? 5 : 4) + (SINGLE_UPDATES ? 1 : 0);
 constexpr double kRint = 6755399441055744.0;          // 1.5 * 2^52: (x + kRint) - kRint = rint(x)
 
 // x * 2^scale for a finite double x (exact unless the result leaves the normal range)
@@ -262,14 +263,15 @@ reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride,
 // rows of one column.  A warp takes one 16-byte chunk of eight neighbouring columns: its residue loads are whole
 // 128-byte lines and its accesses to C eight pieces of 64 (128) contiguous bytes; the warps of a thread block, which
 // take the other chunks of the same columns, complete those to whole lines of C.
-// VEC: C takes pairs of elements (even ldc, C on a multiple of 16 bytes).  Otherwise an update of C (beta = 1), whose loads and stores of
-// single elements in eight pieces each cost more the more there are, gives a warp consecutive words of one column: 512 contiguous
-// bytes of C for residue loads that touch eight lines.  1009 x 983 x 256, set S: 39 us a call against 52; 4501 x 4400 x 128: 400 against
-// 732; plain stores are faster in pieces (34 us against 36, 334 against 352).
+// ACCESS: how C is taken, in pairs of elements (even ldc, C on a multiple of 16 bytes), or singly, stored or updated.  Updates of single
+// elements, whose loads and stores in eight pieces each cost more the more there are, give a warp consecutive words of one column: 512
+// contiguous bytes of C for residue loads that touch eight lines.  1009 x 983 x 256, set S: 39 us a call against 52; 4501 x 4400 x 128: 400
+// against 732; plain stores are faster in pieces (34 us against 36, 334 against 352).
 // grid: x = (piece of the block, block within the tile, CTA rank of the pair), y = tile column, z = tile row
 // SKIP: rows flagged in `skip` are left untouched (they are re-issued on the native FP64 path).
-template <int SET, bool SKIP, bool VEC>
-__global__ void __launch_bounds__(256, kReconBlocks<SET, VEC>)
+enum { kPairs, kSingleStores, kSingleUpdates };
+template <int SET, bool SKIP, int ACCESS>
+__global__ void __launch_bounds__(256, kReconBlocks<SET, ACCESS == kSingleUpdates>)
 reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int tn0,
                          int64_t m, int64_t n, int64_t col0, int64_t col1,
                          const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
@@ -289,7 +291,7 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
     const uint32_t tn = static_cast<uint32_t>(tn0) + blockIdx.y, tm = blockIdx.z;
     constexpr int kChunks = kColWords / 4;                 // 16-byte chunks of one column: 8 or 4
     const uint32_t warp = threadIdx.x >> 5, sub = threadIdx.x & 3u;
-    const bool spread = VEC || beta == 0.0;
+    constexpr bool spread = ACCESS != kSingleUpdates;
     const uint32_t c = spread ? warp % kChunks : (threadIdx.x >> 2) % kChunks;
     const uint32_t lane = piece * kCtaCols + (spread ? warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u) : threadIdx.x / kColWords);   // column of the block
     const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * (16 / RB) + sub * ROWS;
@@ -311,7 +313,7 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
     uint32_t w[kMaxR];
 #pragma unroll
     for (int i = 0; i < r; ++i) w[i] = *reinterpret_cast<const uint32_t *>(base + i * (kBlockWords * 4));
-    reconstruct_rows<SET>(w, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, VEC, keep);
+    reconstruct_rows<SET>(w, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, ACCESS == kPairs, keep);
 }
 
 }  // namespace
@@ -391,7 +393,10 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     // Blocks that become resident beside the GEMM's keep the multiprocessor's memory split at the GEMM's (28 KiB of L1) for
     // the whole kernel: worth the overlapped launch up to a million outputs only (16384 x 16384: 11.4 -> 11.9 ms a call)
     const bool early = m * n <= (1ll << 20);
-#define OZ_RECON_KERNEL(SET_, SKIP_) (vecC ? reconstruct_tiled_kernel<SET_, SKIP_, true> : reconstruct_tiled_kernel<SET_, SKIP_, false>)
+#define OZ_RECON_KERNEL(SET_, SKIP_)                                                    \
+    (vecC          ? reconstruct_tiled_kernel<SET_, SKIP_, kPairs>                      \
+     : beta == 0.0 ? reconstruct_tiled_kernel<SET_, SKIP_, kSingleStores>               \
+                   : reconstruct_tiled_kernel<SET_, SKIP_, kSingleUpdates>)
 #define OZ_RECON_TILED(SET_)                                                                                         \
     OZ_CUDA_CHECK(launch_if(early, skip ? OZ_RECON_KERNEL(SET_, true) : OZ_RECON_KERNEL(SET_, false), grid, 256, 0, stream, R, t.cg, \
                          t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, skip))
