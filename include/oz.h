@@ -114,7 +114,7 @@ typedef enum { OZ_SET_S = 0, OZ_SET_E = 1, OZ_SET_A = 2 } oz_modset_t;
  * (Algorithm 3, the "[INT8-TENSOR + SIMT]" branch: about r multiply-accumulates per output as one
  * small unsigned 8-bit product, then carry, lift and the single rounding in integer arithmetic).
  * Same results bit for bit.  The default form evaluates the same weighted sum in exact FP64 chunks;
- * on B200, whose FP64 pipe is as wide as its integer pipe, that form is about 1.8 times faster, so
+ * on B200, whose FP64 pipe is as wide as its integer pipe, that form is about twice as fast, so
  * this bit is for comparison and for parts with a narrow FP64 pipe.  Ignored by the stage entry points. */
 #define OZ_RECON_TENSOR 0x4000u
 
@@ -286,7 +286,8 @@ oz_status_t oz_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA,
 
 /* Reconstruction (Algorithm 3; Eq. 4-5 and the final step of Sec. 2 (iv)): the integer
  * c'_ij in [-M/2, M/2) congruent to the residues, times 2^-(shiftA[i]+shiftB[j]), rounded once;
- * C = alpha P (beta = 0) or C = C + alpha P (beta = 1).  The CRT is evaluated exactly.  R has the
+ * C = alpha P (beta = 0) or C = C + alpha P (beta = 1).  The CRT is evaluated exactly.  A shift may be any
+ * 32-bit number; OZ_NONFINITE_SHIFT on either side gives NaN whatever the other shift is.  R has the
  * layout and element type that oz_residue_gemm writes for `set`; an entry may be any representative
  * of its residue class below 2 m_i that fits the element type, not only the canonical one (adding
  * m_i to c_i changes the CRT sum by a multiple of M). */
