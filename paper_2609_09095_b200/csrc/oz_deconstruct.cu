@@ -1363,7 +1363,8 @@ cudaError_t resident_clusters(int blocks, int *clusters)
 }
 
 // Blocks of a cluster and tiles of a block for lines of `chunks` tiles, two blocks on an SM; blocks = 0: three passes.
-// Clusters of one block win at every size measured up to 800 MB.  Larger ones are weighed against the three passes, which
+// Clusters of one block win at every size measured up to 800 MB, and of two in the two-plane layouts, which need no table (90316 x 26 x 803 on A
+// 1181 us a call against 1254 in three passes, 41247 x 22 x 901 517 against 540).  Larger ones are weighed against the three passes, which
 // read operands of this size from L2 and fill their last wave better: in units of what the passes take for a million elements, a strip
 // costs a cluster 0.44 a tile and 0.2 (rounds of resident clusters), and either form its start.  That is the time of every
 // layout measured, 384 to 3700 inner indices and 4.5 to 40 million elements, within 6 percent (rms).  Clusters of three and more
@@ -1382,7 +1383,7 @@ ClusterShape cluster_shape(int set, int layout, int side, int64_t lines, int64_t
     const int64_t blocks = (chunks + most - 1) / most, bytes = 8 * lines * k;
     if (blocks > 5 || bytes > (blocks <= 2 ? 1ll << 30 : 1ll << 28)) return {0, 0, 0};
     const int tiles = static_cast<int>((chunks + blocks - 1) / blocks);
-    if (blocks > 1) {
+    if (blocks > (two_plane_layout(layout) ? 2 : 1)) {
         int clusters = 1;
         if (resident_clusters(static_cast<int>(blocks), &clusters) != cudaSuccess) return {0, 0, 0};
         const int64_t strips = (lines + kTileLines - 1) / kTileLines, rounds = (strips + clusters - 1) / clusters;
