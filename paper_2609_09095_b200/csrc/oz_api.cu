@@ -242,9 +242,7 @@ oz_status_t ensure_device_ready()
     g_lut_addr[dev] = static_cast<const uint32_t *>(p);
     OZ_CUDA_CHECK(cudaGetSymbolAddress(&p, g_status));
     g_status_addr[dev] = static_cast<unsigned int *>(p);
-    oz_status_t st = upload_reconstruct_constants();
-    if (st != OZ_OK) return st;
-    st = upload_hosted_constants();
+    oz_status_t st = upload_hosted_constants();
     if (st != OZ_OK) return st;
     // A copy from pageable memory may return before it has arrived, and the first kernels may be on a stream that does not wait
     // for the default one (they also read the tables before they wait for anything).

@@ -126,6 +126,11 @@ struct ModInfo {
     // native INT8 residues, one accumulator of at most 2^30 in magnitude (k <= 65536): exact division
     uint32_t magic39;     // ceil(2^39 / m): floor(u / m) = (u * magic39) >> 39 exactly for u < 2^31 + 256, m in (128, 256]
     uint32_t bias30;      // the multiple of m just above 2^30
+    // private residue array
+    int store_form;       // kStoredByte, kStoredTen or kStoredPair
+    int store_start;      // the byte of a patch where this modulus' residues begin
+    float centre;         // (m + 1) / 2 (FP32 epilogue)
+    int reserved;         // whole 16-byte pieces: a size of 108 cost the public native variant spills
 };
 
 struct GemmParams {
@@ -136,6 +141,7 @@ struct GemmParams {
     int pair_squares;               // squares: both jobs in one K-loop
     int stall_producer;             // test hook: the producer issues no copy, so every wait runs out
     int r;
+    int patch_bytes;                // private residue array: bytes of a 32 x 64 patch
     int64_t total_items;
     void *R;                        // residues: uint16 (RB = 2) or uint8 (RB = 1, byte moduli)
     int64_t ldr, mod_stride;
@@ -493,16 +499,15 @@ __device__ __forceinline__ float2 mod_balanced2(float2 acc, float2 inv_m2, float
 // RB: bytes of one stored residue (2: uint16, 1: uint8 for the all-byte modulus set)
 // DIRECT: native INT8 residues -- one accumulator per modulus, loaded straight into the registers
 //         that otherwise hold the running combination of several accumulators
-// LOOSE: the stored residue is some representative in [0, 2 m_i) instead of the canonical one in
-//         [0, m_i) (two-byte residues only).  The reconstruction is indifferent to it -- the CRT
-//         weight of m_i is a multiple of M -- and the epilogue saves the canonicalisation; used for
-//         the residues that stay inside the whole-method calls.
 // TILED: the residue array is the private, tile-ordered one of the whole-method calls (see
-//         residue_tiling() below): the 32 columns x 64 rows that an epilogue warp owns form one
-//         contiguous block, [16-byte chunk][lane], so that every store instruction of a warp writes
+//         ResidueTiling): the 32 columns x 64 rows that an epilogue warp owns form one
+//         contiguous patch, [16-byte chunk][lane], so that every store instruction of a warp writes
 //         512 consecutive bytes straight from registers -- no transposition through shared memory,
 //         which the tensor pipe and the TMA writes need for themselves.  The reconstruction reads
 //         the same order.  Without it the public layout R[mod][j][ldr] is written.
+//         Sets S and E store 8, 10 or 16 bits a residue (stored_form()): 1.2 instead of 0.5 byte permutations a value, but five
+//         16-byte stores a thread and modulus instead of eight.  The FP32 epilogue starts its combination at -centre and adds the
+//         centre to the balanced result, which leaves a representative in [0, m + 1] without a comparison.
 // BOUND: not a residue product but the magnitude-bound product of the accurate mode (Sec. 2 "The FP8
 //         variant", the "+1" pass): one plane per operand, one accumulator per tile, and instead of
 //         residues the epilogue reduces the row and column maxima of the tile into p.rowmax / p.colmax.
@@ -510,13 +515,14 @@ __device__ __forceinline__ float2 mod_balanced2(float2 acc, float2 inv_m2, float
 // SLIM:    two-plane schedule of a product with one tile of columns (n <= 128), which reads A's planes from memory once
 //         and does little arithmetic with them: d = d0 + 16 d1 of a non-square modulus meets all of e (see kind 4, 5 in
 //         slim_stage()), so that dS is never read.  Both accumulators of a modulus fill in one K-loop, per K segment.
-template <int SUB, int CG, int RB, bool DIRECT, bool LOOSE, bool TILED, bool BOUND = false, int SLIM = 0, int BN = BLOCK_N>
+template <int SUB, int CG, int RB, bool DIRECT, bool TILED, bool BOUND = false, int SLIM = 0, int BN = BLOCK_N>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                     const __grid_constant__ GemmParams p)
 {
     static_assert(SLIM == 0 || (CG == 1 && !DIRECT && TILED && !BOUND), "two-plane schedule: whole-method digit products");
     static_assert(BN == BLOCK_N || TILED, "narrow tiles: whole-method products");
+    constexpr bool PACKED = TILED && RB == 2 && !BOUND;  // sets S and E in the private array
     using Slim = SlimTile<SLIM ? SLIM : 128, BN>;
     constexpr int STAGES = SLIM ? Slim::STAGES : Tile<CG, BN>::STAGES;
     constexpr int STAGE_BYTES = SLIM ? Slim::STAGE_BYTES : Tile<CG, BN>::STAGE_BYTES;
@@ -764,14 +770,15 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             Item it = decode_item(item, p);
             const ModInfo &mi = p.mod[it.mod];
             const float mm = mi.m, inv_m = mi.inv_m;
-            const float loose_offset = mm + 8388608.0f;          // exact: m < 2^11
+            const float centre_big = mi.centre + 8388608.0f;     // exact: m < 2^11
             const float2 inv_m2 = make_float2(inv_m, inv_m), neg_m2 = make_float2(-mm, -mm);
             const uint32_t im = mi.mi, imagic = mi.magic, ibias = mi.bias;
             // running combination per element: FP32 (FP8 route) or INT32 (INT8 routes), as raw bits
             uint32_t comb[COLS_PER_WARP];
             if constexpr (!DIRECT) {
+                const uint32_t start = PACKED && SUB == 0 ? __float_as_uint(-mi.centre) : 0u;
 #pragma unroll
-                for (int c = 0; c < COLS_PER_WARP; ++c) comb[c] = 0u;
+                for (int c = 0; c < COLS_PER_WARP; ++c) comb[c] = start;
             }
             // SLIM: both jobs of a K segment before the next segment.  (The bound is read where it is compared: in a register of its
             // own it costs the public FP8 variants 144 bytes of spills instead of 48, 4096 x 4096 x 1024: 516 us against 485.)
@@ -881,8 +888,8 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     float t = __uint_as_float(cv);
                     float quot = fmaf(t, inv_m, 12582912.0f) - 12582912.0f;
                     float res = fmaf(-quot, mm, t);                      // |res| <= ~m/2
-                    if constexpr (LOOSE) {
-                        return __float_as_uint(res + loose_offset);      // res + m in (0, 2m), low mantissa bits
+                    if constexpr (PACKED) {
+                        return __float_as_uint(res + centre_big);        // in the low mantissa bits
                     } else {
                         res = res < 0.0f ? res + mm : res;               // canonical [0, m)
                         return __float_as_uint(res + 8388608.0f);        // integer in the low mantissa bits
@@ -893,14 +900,14 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 } else {
                     uint32_t u = cv + ibias;
                     uint32_t r = u - __umulhi(u, imagic) * im;           // in [0, 2m)
-                    return LOOSE ? r : min(r, r - im);                   // canonical [0, m) unless LOOSE
+                    return min(r, r - im);                               // canonical [0, m)
                 }
             };
-            // same for two values at once; the loose FP32 form is done with packed pairs
+            // same for two values at once; the balanced FP32 form is done with packed pairs
             auto final_bits2 = [&](uint32_t c0v, uint32_t c1v, uint32_t &b0, uint32_t &b1) {
-                if constexpr (SUB == 0 && LOOSE) {
+                if constexpr (SUB == 0 && PACKED) {
                     const float2 res = mod_balanced2(make_float2(__uint_as_float(c0v), __uint_as_float(c1v)), inv_m2, neg_m2);
-                    const float2 out = __fadd2_rn(res, make_float2(loose_offset, loose_offset));
+                    const float2 out = __fadd2_rn(res, make_float2(centre_big, centre_big));
                     b0 = __float_as_uint(out.x);
                     b1 = __float_as_uint(out.y);
                 } else {
@@ -908,11 +915,11 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     b1 = final_bits(c1v);
                 }
             };
-            // four consecutive rows starting at combination value c -> one (RB = 1) or two (RB = 2) words
-            auto pack4 = [&](int c, uint32_t &w0, uint32_t &w1) {
+            // rows a, a + 1, b and b + 1 of the thread's run -> one (RB = 1) or two (RB = 2) words
+            auto pack_rows = [&](int a, int b, uint32_t &w0, uint32_t &w1) {
                 uint32_t b0, b1, b2, b3;
-                final_bits2(comb[c], comb[c + 1], b0, b1);
-                final_bits2(comb[c + 2], comb[c + 3], b2, b3);
+                final_bits2(comb[a], comb[a + 1], b0, b1);
+                final_bits2(comb[b], comb[b + 1], b2, b3);
                 if constexpr (RB == 2) {
                     w0 = __byte_perm(b0, b1, 0x5410);
                     w1 = __byte_perm(b2, b3, 0x5410);
@@ -923,37 +930,62 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             };
             constexpr int NCH = COLS_PER_WARP * RB / 16;     // 16-byte chunks of a thread's run of rows
             if constexpr (TILED) {
-                // block (tile, CTA rank, warp), then modulus: the r residue blocks of one 32 x 64 patch of
-                // the output lie next to one another, which is how the reconstruction reads them
-                const int64_t tile = i0 / BLOCK_N;                   // the layout's tiles have 256 rows, its blocks 64
-                const int block = (static_cast<int>(i0 >> 6) & 3) * 4 + q, chunk0 = static_cast<int>(i0 & 63) * RB / 16;
-                unsigned char *blk = static_cast<unsigned char *>(p.R) +
-                    ((((tile * p.tiles_n + it.tn) * CG + rank) * EPI_WARPS + block) * p.r + it.mod) * static_cast<int64_t>(64 * RB * 32) +
-                    chunk0 * 512 + lane * 16;
+                // patch (tile, CTA rank, warp), then modulus: the residues of one 32 x 64 patch of the output lie next to one
+                // another, which is how the reconstruction reads them
+                const int64_t tile = i0 / BLOCK_N;                   // the layout's tiles have 256 rows, its patches 64
+                const int patch = (static_cast<int>(i0 >> 6) & 3) * 4 + q, chunk0 = static_cast<int>(i0 & 63) / 16;
+                unsigned char *base = static_cast<unsigned char *>(p.R) +
+                    (((tile * p.tiles_n + it.tn) * CG + rank) * EPI_WARPS + patch) * static_cast<int64_t>(p.patch_bytes) + mi.store_start + lane * 16;
+                if constexpr (PACKED) {
+                    if (mi.store_form == kStoredPair) {
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    uint4 val;
-                    if constexpr (RB == 2) {
-                        pack4(8 * c, val.x, val.y);
-                        pack4(8 * c + 4, val.z, val.w);
+                        for (int c = 0; c < COLS_PER_WARP / 8; ++c) {
+                            uint4 val;
+                            pack_rows(8 * c, 8 * c + 2, val.x, val.y);
+                            pack_rows(8 * c + 4, 8 * c + 6, val.z, val.w);
+                            *reinterpret_cast<uint4 *>(base + (2 * chunk0 + c) * 512) = val;
+                        }
                     } else {
-                        uint32_t unused;
-                        pack4(16 * c, val.x, unused);
-                        pack4(16 * c + 4, val.y, unused);
-                        pack4(16 * c + 8, val.z, unused);
-                        pack4(16 * c + 12, val.w, unused);
+                        uint32_t high[COLS_PER_WARP / 16];           // bits 8 and 9 of sixteen rows
+#pragma unroll
+                        for (int g = 0; g < COLS_PER_WARP / 16; ++g) {
+                            uint32_t lo[4], hi[4];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                uint32_t w0, w1;
+                                pack_rows(16 * g + 2 * h, 16 * g + 2 * h + 8, w0, w1);
+                                lo[h] = __byte_perm(w0, w1, 0x6420);
+                                hi[h] = __byte_perm(w0, w1, 0x7531) & 0x03030303u;   // 1024 is 0 modulo 1024
+                            }
+                            *reinterpret_cast<uint4 *>(base + (chunk0 + g) * 512) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                            high[g] = (hi[0] + 4u * hi[1]) + 16u * (hi[2] + 4u * hi[3]);
+                        }
+                        if (mi.store_form == kStoredTen) {
+                            if constexpr (COLS_PER_WARP == 64) *reinterpret_cast<uint4 *>(base + 2048) = make_uint4(high[0], high[1], high[2], high[3]);
+                            else *reinterpret_cast<uint32_t *>(base + 2048 + 4 * chunk0) = high[0];
+                        }
                     }
-                    *reinterpret_cast<uint4 *>(blk + c * 512) = val;
+                } else {
+#pragma unroll
+                    for (int c = 0; c < COLS_PER_WARP / 16; ++c) {
+                        uint4 val;
+                        uint32_t unused;
+                        pack_rows(16 * c, 16 * c + 8, val.x, unused);
+                        pack_rows(16 * c + 2, 16 * c + 10, val.y, unused);
+                        pack_rows(16 * c + 4, 16 * c + 12, val.z, unused);
+                        pack_rows(16 * c + 6, 16 * c + 14, val.w, unused);
+                        *reinterpret_cast<uint4 *>(base + (chunk0 + c) * 512) = val;
+                    }
                 }
             } else {
             // residues packed 4 / RB to a word in row order
             uint32_t packed[COLS_PER_WARP * RB / 4];
 #pragma unroll
             for (int c = 0; c < COLS_PER_WARP; c += 4) {
-                if constexpr (RB == 2) pack4(c, packed[c >> 1], packed[(c >> 1) + 1]);
+                if constexpr (RB == 2) pack_rows(c, c + 2, packed[c >> 1], packed[(c >> 1) + 1]);
                 else {
                     uint32_t unused;
-                    pack4(c, packed[c >> 2], unused);
+                    pack_rows(c, c + 2, packed[c >> 2], unused);
                 }
             }
             unsigned char *rbase = static_cast<unsigned char *>(p.R) + it.mod * p.mod_stride * RB;
@@ -1097,12 +1129,11 @@ oz_status_t launch_fused_variant(const CUtensorMap &mapB, const GemmParams &p, c
     return OZ_OK;
 }
 
-template <int SUB, int CG, int RB, bool DIRECT = false, bool LOOSE = false, bool TILED = false, bool BOUND = false, int SLIM = 0, int BN = BLOCK_N>
+template <int SUB, int CG, int RB, bool DIRECT = false, bool TILED = false, bool BOUND = false, int SLIM = 0, int BN = BLOCK_N>
 oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, const GemmParams &p, int sms,
                            cudaStream_t stream)
 {
-    static_assert(!LOOSE || RB == 2, "a representative below 2m needs the two-byte element");
-    auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, LOOSE, TILED, BOUND, SLIM, BN>;
+    auto kernel = residue_gemm_kernel<SUB, CG, RB, DIRECT, TILED, BOUND, SLIM, BN>;
     static std::atomic<unsigned long long> ready{0};
     OZ_CUDA_CHECK(allow_shared(kernel, SMEM_BYTES, ready));
     int64_t groups = sms / CG;                                    // CTAs, or CTA pairs
@@ -1132,14 +1163,13 @@ oz_status_t launch_variant(const CUtensorMap &mapA, const CUtensorMap &mapB, con
 template <int SUB, int RB, bool DIRECT, int BN>
 oz_status_t launch_tiled(const CUtensorMap &mapA, const CUtensorMap &mapB, const GemmParams &p, int cg, bool slim, int sms, cudaStream_t stream)
 {
-    constexpr bool LOOSE = RB == 2;
     if constexpr (!DIRECT) {
         if (slim)
-            return p.n <= 64 ? launch_variant<SUB, 1, RB, false, LOOSE, true, false, 64, BN>(mapA, mapB, p, sms, stream)
-                             : launch_variant<SUB, 1, RB, false, LOOSE, true, false, 128, BN>(mapA, mapB, p, sms, stream);
+            return p.n <= 64 ? launch_variant<SUB, 1, RB, false, true, false, 64, BN>(mapA, mapB, p, sms, stream)
+                             : launch_variant<SUB, 1, RB, false, true, false, 128, BN>(mapA, mapB, p, sms, stream);
     }
-    return cg == 2 ? launch_variant<SUB, 2, RB, DIRECT, LOOSE, true, false, 0, BN>(mapA, mapB, p, sms, stream)
-                   : launch_variant<SUB, 1, RB, DIRECT, LOOSE, true, false, 0, BN>(mapA, mapB, p, sms, stream);
+    return cg == 2 ? launch_variant<SUB, 2, RB, DIRECT, true, false, 0, BN>(mapA, mapB, p, sms, stream)
+                   : launch_variant<SUB, 1, RB, DIRECT, true, false, 0, BN>(mapA, mapB, p, sms, stream);
 }
 
 template <int SUB, int RB, bool DIRECT>
@@ -1205,9 +1235,9 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k, bo
         // squares), |d1| <= 16, |d0+d1| <= 22 (Lemma 1), a reduced accumulator by (m+1)/2 <= 545
         // (FP32 path, balanced) or m-1 <= 1088 (integer path, canonical).  A job's accumulator may
         // be weighted without reducing it first while the worst-case sum stays inside the exact
-        // range: 2^24 for the FP32 epilogue, 2^31 (minus headroom for the bias) for the integer one.
+        // range: 2^24 for the FP32 epilogue (minus the centre), 2^31 (minus headroom for the bias) for the integer one.
         const bool integer = rt.substrate != 0;
-        const int64_t lim = integer ? (1ll << 31) - 8192 : (1ll << 24) - 1, kk = k > 0 ? k : 1;
+        const int64_t lim = integer ? (1ll << 31) - 8192 : (1ll << 24) - 546, kk = k > 0 ? k : 1;
         const int64_t red = integer ? 1088 : 545;
         ModInfo &mo = p.mod[i];
         mo.mi = static_cast<uint32_t>(mi);
@@ -1215,6 +1245,9 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k, bo
         mo.bias = static_cast<uint32_t>((((1ull << 31) + mi - 1) / mi) * mi);
         mo.magic39 = mi > 128 ? static_cast<uint32_t>(((1ull << 39) + mi - 1) / mi) : 0u;
         mo.bias30 = static_cast<uint32_t>((((1ull << 30) + mi - 1) / mi) * mi);
+        mo.store_form = stored_form(set, i);
+        mo.store_start = stored_start(set, i);
+        mo.centre = static_cast<float>((mi + 1) / 2);
         mo.planeA0 = kSetTables.first[set][rt.layout(0)][i];
         mo.planeB0 = kSetTables.first[set][rt.layout(1)][i];
         mo.nseg = 1;
@@ -1340,6 +1373,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     p.total_items = static_cast<int64_t>(p.r) * p.tiles_m * p.tiles_n;
     if (p.total_items >= 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;        // item numbers are 32-bit in the kernel
     p.R = R; p.ldr = ldr; p.mod_stride = mod_stride;
+    p.patch_bytes = patch_bytes(set);
     p.stall_producer = take_stall_flag();
     p.status = device_status_word();
     const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(m, n, k, set, sms)));
@@ -1369,7 +1403,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     // one accumulator per modulus of at most 128 * 128 * k <= 2^30: the direct drain with the exact division
     const bool direct = rt.native() && p.mod[0].nseg_all == 1 && k <= 65536;
     // substrate 0: FP8 planes; otherwise INT8 planes (two-limb digits or native residues)
-    if (tiled) {       // private to the whole-method calls, which also take the loose residues
+    if (tiled) {
 #define OZ_TILED(SUB, RB, DIRECT) launch_tiled<SUB, RB, DIRECT>(mapA, mapB, p, cg, slim, narrow, sms, stream)
         if (direct) return OZ_TILED(1, 1, true);
         if (rb == 1) return rt.substrate == 0 ? OZ_TILED(0, 1, false) : OZ_TILED(1, 1, false);
@@ -1472,8 +1506,8 @@ oz_status_t launch_bound_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *GA
         !make_plane_map(&mapB, GB, n, pitchB, n * pitchB, 1, BLOCK_M))
         return OZ_ERR_CUDA;
     const int sms = sm_count();
-    return cg == 2 ? launch_variant<0, 2, 2, true, false, false, true>(mapA, mapB, p, sms, stream)
-                   : launch_variant<0, 1, 2, true, false, false, true>(mapA, mapB, p, sms, stream);
+    return cg == 2 ? launch_variant<0, 2, 2, true, false, true>(mapA, mapB, p, sms, stream)
+                   : launch_variant<0, 1, 2, true, false, true>(mapA, mapB, p, sms, stream);
 }
 
 }  // namespace oz

@@ -33,6 +33,26 @@ __host__ __device__ constexpr int modulus(int set, int i)
 // bytes of one stored residue in [0, m): the moduli of set A fit a byte
 __host__ __device__ constexpr int residue_bytes(int set) { return set == 2 ? 1 : 2; }
 
+// How the private residue array of the whole-method calls stores a residue of modulus i: some representative in [0, m + 1], modulo 2^10
+// or 2^8 where m is that, in one byte, in ten bits (moduli up to 1024) or in two bytes.  (Set A: canonical.)
+enum { kStoredByte, kStoredTen, kStoredPair };
+__host__ __device__ constexpr int stored_form(int set, int i)
+{
+    return modulus(set, i) <= 256 ? kStoredByte : modulus(set, i) <= 1024 ? kStoredTen : kStoredPair;
+}
+// bytes of one modulus' residues of a 32 x 64 patch of the output (see ResidueTiling), of those before it, and of a whole patch
+__host__ __device__ constexpr int stored_bytes(int set, int i)
+{
+    return stored_form(set, i) == kStoredByte ? 2048 : stored_form(set, i) == kStoredTen ? 2560 : 4096;
+}
+__host__ __device__ constexpr int stored_start(int set, int i)
+{
+    int o = 0;
+    for (int j = 0; j < i; ++j) o += stored_bytes(set, j);
+    return o;
+}
+__host__ __device__ constexpr int patch_bytes(int set) { return stored_start(set, set_r(set)); }
+
 // square root of a square modulus, 0 otherwise
 __host__ __device__ constexpr int square_root(int m)
 {
@@ -201,12 +221,15 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
                                int32_t *shift, void *scratch, bool alone, cudaStream_t stream);
 
 // Tile-ordered private residue array of the whole-method calls.  The output is cut into tiles of
-// 256 rows x tile_cols columns (128, or 256 when CTA pairs are used); a tile is 16 blocks (32 with
-// pairs: rank-major) of 32 columns x 64 rows, one per epilogue warp, block w = quarter + 4 * part
-// covering columns 32 * quarter .. +31 (of the rank's 128) and rows 64 * part .. +63; a block is
-// stored as [16-byte chunk c][column], chunk c holding 16 / residue_bytes consecutive rows.
-// Order in memory: tile row, tile column, CTA rank, block, modulus -- the r residue blocks of one
-// 32 x 64 patch of the output are consecutive (4 KiB each, 2 KiB for byte residues).
+// 256 rows x tile_cols columns (128, or 256 when CTA pairs are used); a tile is 16 patches (32 with
+// pairs: rank-major) of 32 columns x 64 rows, one per epilogue warp, patch w = quarter + 4 * part
+// covering columns 32 * quarter .. +31 (of the rank's 128) and rows 64 * part .. +63.
+// Order in memory: tile row, tile column, CTA rank, patch, modulus -- the residues of one patch are consecutive, modulus
+// after modulus (stored_start()).  Those of a modulus are stored as [16-byte chunk c][column], chunk c holding 16
+// consecutive rows (two-byte form: 8), word s of it rows 2 s, 2 s + 1, 2 s + 8 and 2 s + 9 -- the rows of one thread of the
+// reconstruction, four of which then access 64 contiguous bytes of C (row_of()).  Ten-bit form: the low bytes like that, then 16 bytes
+// a column with the high bits, word c for the rows of chunk c: bits 2 s and 2 s + 1 of its byte e belong to byte e of word s.
+// Set S takes 15.75 bytes an output, where two bytes a residue take 24; E 15.25 instead of 26; A 15.
 struct ResidueTiling {
     int cg;              // 1: tiles of 128 columns, 2: CTA pairs, tiles of 256 columns
     int tile_cols;
@@ -257,8 +280,7 @@ int accurate_budget_log2(int set);
 // exponent-span check: threshold of the set against the product of the two operands' flatness codes
 unsigned int esc_threshold(int set);
 
-// tiled: R is the tile-ordered private array (ldr and mod_stride are then ignored), with residues in [0, 2 m_i) for the
-// two-byte sets, and the planes are in the private layout
+// tiled: R is the tile-ordered private array (ldr and mod_stride are then ignored), and the planes are in the private layout
 oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *PA,
                                 int64_t strideA, int64_t pitchA, const uint8_t *PB,
                                 int64_t strideB, int64_t pitchB, int set, const Route &rt,
@@ -287,7 +309,6 @@ oz_status_t launch_reconstruct(int64_t m, int64_t n, const void *R, int64_t ldr,
                                cudaStream_t stream);
 
 // uploads the reconstruction constants of every set to the current device
-oz_status_t upload_reconstruct_constants();
 oz_status_t upload_hosted_constants();
 
 // reconstruction from the tile-ordered array with the CRT recombination on the INT8 tensor pipe

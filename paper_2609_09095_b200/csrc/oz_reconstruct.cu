@@ -3,19 +3,18 @@
 //
 // The paper's SIMT branch walks Garner's mixed-radix digits (r(r-1)/2 multiply-reduce steps).
 // CRT fixes c' uniquely, so any exact evaluation gives the same integer; this kernel uses the
-// weighted form
-//     c' = sum_i c_i V_i  -  kappa M,     V_i = ((M/m_i)^-1 mod m_i) (M/m_i) mod M,
-// with every V_i and M cut into three 38-bit chunks (40-bit for the all-byte set).  A stored
-// residue is below 2 m_i < 2^11.1 (the whole-method calls keep a representative in (0, 2 m_i); 2^8
-// for the byte set), so each of the three chunk sums is an integer below 2^53 -- at most 2^52.8 --
-// and is formed EXACTLY by FP64 fused multiply-adds (r MACs per chunk).  kappa = round(S/M) comes from a floating estimate; the
-// carry-normalised chunks are then summed with error-free additions, which give the correctly
-// rounded FP64 value directly unless c' lies within a hair of a rounding boundary, of a power of
-// two or of +-M/2 -- those rare outputs take an exact path: the 128-bit integer, an exact range
-// test for the lift to [-M/2, M/2), and one round-to-nearest-even done in integer arithmetic.
-// A thread handles the consecutive rows whose residues share one 32-bit word per modulus (two
-// uint16, or four uint8 for the all-byte set).
-#include <cstring>
+// weighted form over groups of moduli.  With P_g the product of the two or three moduli of group g,
+//     c' = sum_g u_g N_g  -  kappa M,     N_g = M / P_g,     u_g = sum_{i in g} c_i a_i,
+// where a_i is 0 modulo the other moduli of its group and (N_g)^-1 modulo m_i, balanced: u_g is a 32-bit integer that two or
+// three integer multiply-adds form from the stored residues, and one conversion serves the whole group.  Every N_g and M is cut
+// into a high and a middle part of at most 21 signed bits and the rest: the sums of the first two are integers below 2^53
+// (group_bounds()) and formed EXACTLY by FP64 fused multiply-adds, that of the third is off by less than kRestError.
+// kappa = round(S/M) comes from a floating estimate; error-free additions then give the correctly rounded FP64 value unless
+// c' lies within kRestError of a rounding boundary, is so small that this error counts, or lies near +-M/2 -- those rare
+// outputs take an exact path: the 128-bit integer, an exact range test for the lift to [-M/2, M/2), and one
+// round-to-nearest-even done in integer arithmetic.  A term for every modulus, three parts of 38 or 40 bits each, took 36 (S) to 45 (A)
+// FP64 multiply-adds and 12 to 15 conversions an output where this takes 18 and 6 (A: 15 and 5).
+// A thread handles four rows of a column, two where the outputs are few.
 #include <utility>
 
 #include "oz_internal.h"
@@ -23,26 +22,172 @@
 namespace oz {
 namespace {
 
-struct ReconConst {
-    double V[kMaxR][3];        // V_i = V0 + V1 + V2, the chunks in place: V1 and V2 are multiples of 2^cw and 2^(2cw)
-    double Mc[3];              // M   = M0 + M1 + M2 likewise
-    double inv_M;              // 1/M (rounded)
-    int half_M_guard;          // high word of (M/2) (1 - 2^-30): from it on the lift is decided exactly
-    unsigned long long M_lo, M_hi;
-};
+// ---- groups of moduli -----------------------------------------------------------------------------
+constexpr int kMaxGroups = 6;
+__host__ __device__ constexpr int set_groups(int set) { return set == 2 ? 5 : 6; }
+// Moduli of a group (indices, -1: none): those that keep the sum of the bounds of |u_g| small, so that the rest's error is small.
+__host__ __device__ constexpr int group_member(int set, int g, int e)
+{
+    constexpr int S[6][3] = {{5, 9, -1}, {3, 4, -1}, {7, 10, -1}, {1, 2, -1}, {0, 6, -1}, {8, 11, -1}};
+    constexpr int E[6][3] = {{7, 11, 12}, {5, 8, -1}, {4, 9, -1}, {0, 6, -1}, {1, 3, -1}, {2, 10, -1}};
+    constexpr int A[6][3] = {{1, 9, 11}, {6, 7, 12}, {0, 3, 4}, {2, 5, 8}, {10, 13, 14}, {-1, -1, -1}};
+    return set == 0 ? S[g][e] : set == 1 ? E[g][e] : A[g][e];
+}
+// places of the middle and of the high part
+__host__ __device__ constexpr int mid_bit(int set) { return set == 0 ? 52 : set == 1 ? 55 : 54; }
+__host__ __device__ constexpr int high_bit(int set) { return mid_bit(set) + 21; }
 
-__constant__ ReconConst c_recon[kNumSets];
-
-// Chunk width: 38 bits for S and E (stored residues < 2^11.1, 13 terms: sums < 2^52.8); 40 bits for
-// the 117.8-bit set A (residues < 2^8, 15 terms: sums < 2^52), so that three chunks cover M.
-__host__ __device__ constexpr int chunk_bits(int set) { return set == 2 ? 40 : 38; }
+struct Wide { uint64_t lo, hi; };                 // 128-bit constants at compile time
+__host__ __device__ constexpr Wide wide_mul(Wide w, uint64_t m)      // m below 2^31, no overflow
+{
+    const uint64_t p0 = (w.lo & 0xFFFFFFFFull) * m, p1 = (w.lo >> 32) * m + (p0 >> 32);
+    return {(p0 & 0xFFFFFFFFull) | (p1 << 32), w.hi * m + (p1 >> 32)};
+}
+__host__ __device__ constexpr uint64_t group_product(int set, int g)
+{
+    uint64_t p = 1;
+    for (int e = 0; e < 3; ++e)
+        if (group_member(set, g, e) >= 0) p *= static_cast<uint64_t>(modulus(set, group_member(set, g, e)));
+    return p;
+}
+__host__ __device__ constexpr bool in_group(int set, int g, int i)
+{
+    return group_member(set, g, 0) == i || group_member(set, g, 1) == i || group_member(set, g, 2) == i;
+}
+// N_g; g = -1: M
+__host__ __device__ constexpr Wide group_weight(int set, int g)
+{
+    Wide w{1, 0};
+    for (int i = 0; i < set_r(set); ++i)
+        if (g < 0 || !in_group(set, g, i)) w = wide_mul(w, static_cast<uint64_t>(modulus(set, i)));
+    return w;
+}
+// N = high 2^high_bit + mid 2^mid_bit + rest, the last two balanced
+struct Parts { int64_t high, mid, rest; };
+__host__ __device__ constexpr Parts split_parts(int set, Wide w)
+{
+    const int b = mid_bit(set), c = high_bit(set) - b;
+    Parts p{};
+    p.rest = static_cast<int64_t>(w.lo & ((1ull << b) - 1));
+    uint64_t up = (w.lo >> b) | (w.hi << (64 - b));
+    if (p.rest >> (b - 1)) { p.rest -= 1ll << b; ++up; }
+    p.mid = static_cast<int64_t>(up & ((1ull << c) - 1));
+    up >>= c;
+    if (p.mid >> (c - 1)) { p.mid -= 1ll << c; ++up; }
+    p.high = static_cast<int64_t>(up);
+    return p;
+}
+// a_i of member e of group g
+__host__ __device__ constexpr int64_t member_weight(int set, int g, int e)
+{
+    const int i = group_member(set, g, e);
+    if (i < 0) return 0;
+    const uint64_t m = static_cast<uint64_t>(modulus(set, i)), P = group_product(set, g);
+    uint64_t other = 1;                              // M / m_i modulo m_i
+    for (int j = 0; j < set_r(set); ++j)
+        if (j != i) other = other * static_cast<uint64_t>(modulus(set, j)) % m;
+    uint64_t inv = 1;
+    while (other * inv % m != 1) ++inv;
+    const uint64_t a = P / m * inv % P;
+    return 2 * a > P ? static_cast<int64_t>(a) - static_cast<int64_t>(P) : static_cast<int64_t>(a);
+}
+// Largest number that stands for a residue: all that a form can hold; two bytes, as everything in the public layout of sets S and E: below 2 m,
+// but for the groups of three, whose sums would leave 32 bits: there the public layout's numbers are reduced first.
+__host__ __device__ constexpr bool reduced_first(int set, int i)
+{
+    bool three = false;
+    for (int g = 0; g < set_groups(set); ++g) three = three || (in_group(set, g, i) && group_member(set, g, 2) >= 0);
+    return set != 2 && three;
+}
+__host__ __device__ constexpr int64_t largest_number(int set, int i)
+{
+    const int64_t form = stored_form(set, i) == kStoredByte ? 255 : stored_form(set, i) == kStoredTen ? 1023 : 0, twice = 2 * modulus(set, i) - 1;
+    return set == 2 || reduced_first(set, i) || form > twice ? form : twice;
+}
+__host__ __device__ constexpr int64_t abs64(int64_t x) { return x < 0 ? -x : x; }
+// bound of |u_g|: the terms of one sign
+__host__ __device__ constexpr int64_t group_reach(int set, int g)
+{
+    int64_t pos = 0, neg = 0;
+    for (int e = 0; e < 3; ++e) {
+        if (group_member(set, g, e) < 0) continue;
+        const int64_t t = largest_number(set, group_member(set, g, e)) * member_weight(set, g, e);
+        if (t > 0) pos += t;
+        else neg -= t;
+    }
+    return pos > neg ? pos : neg;
+}
 __host__ __device__ constexpr double pow2d(int e) { double v = 1.0; for (int i = 0; i < e; ++i) v *= 2.0; return v; }
-// Resident blocks per SM.  The loads of a thread are independent, so this many keep memory busy; the registers they leave
-// (48, 64) hold everything.  16384 x 16384 update, set S, with 4 / 5 / 6 blocks: 2.18 / 2.17 / 2.17 ms; 6144 x 6144, set A, with
-// 3 / 4 / 5 blocks: 288 / 289 / 298 us.  Before the mapping and the arithmetic below: 2.35 ms and 327 us.  One more where single elements
-// of C are updated, since their old values are waited for in turn; not for plain stores, whose blocks of 40 registers would fit beside a
-// GEMM's and become resident with it (499 x 366 x 2755 under the accurate rule 94 -> 102 us a call).
-template <int SET, bool SINGLE_UPDATES = false> constexpr int kReconBlocks = (residue_bytes(SET) == 2 ? 5 : 4) + (SINGLE_UPDATES ? 1 : 0);
+struct Bounds { double high, mid, rest, kappa; bool words; };
+// of the three sums in units of their places, with kappa M taken off (which makes the high one small); every u_g in 32 bits
+__host__ __device__ constexpr Bounds group_bounds(int set)
+{
+    Bounds b{0.0, 0.0, 0.0, 1.0, true};
+    for (int g = 0; g < set_groups(set); ++g) {
+        const Parts p = split_parts(set, group_weight(set, g));
+        const double u = static_cast<double>(group_reach(set, g));
+        b.high += u * static_cast<double>(abs64(p.high));
+        b.mid += u * static_cast<double>(abs64(p.mid));
+        b.rest += u * static_cast<double>(abs64(p.rest));
+        b.kappa += u / static_cast<double>(group_product(set, g));
+        if (u >= 2147483648.0 || abs64(p.high) >= (1ll << 21)) b.words = false;
+    }
+    const Parts m = split_parts(set, group_weight(set, -1));
+    b.mid += b.kappa * static_cast<double>(abs64(m.mid));
+    b.rest += b.kappa * static_cast<double>(abs64(m.rest));
+    return b;
+}
+// Bound, as a power of two, of what the rest's multiply-adds (one a group and one of kappa M) and the last addition to it lose
+__host__ __device__ constexpr int rest_error_log2(int set)
+{
+    const double e = group_bounds(set).rest * (set_groups(set) + 3) / pow2d(53);
+    int l = 0;
+    while (pow2d(l) < e) ++l;
+    return l;
+}
+template <int SET> constexpr int kRestErrorLog2 = rest_error_log2(SET);
+template <int SET> constexpr bool kExact = group_bounds(SET).words && group_bounds(SET).high < 9007199254740992.0 &&
+                                           group_bounds(SET).mid < 9007199254740992.0 && mid_bit(SET) > kRestErrorLog2<SET> + 4;
+static_assert(kExact<0> && kExact<1> && kExact<2>, "the high and middle sums are exact, every group's integer fits 32 bits");
+
+// High words of doubles: below the first, the rest's error may reach a quarter of an ulp; from the second on (M / 2 but for its last bits),
+// the lift is decided exactly.
+__host__ __device__ constexpr uint32_t small_word(int set) { return static_cast<uint32_t>(1023 + rest_error_log2(set) + 56) << 20; }
+__host__ __device__ constexpr uint32_t half_M_word(int set)
+{
+    Wide w = group_weight(set, -1);
+    int bits = 128;
+    while (!(w.hi >> 63)) { w.hi = (w.hi << 1) | (w.lo >> 63); w.lo <<= 1; --bits; }
+    return (static_cast<uint32_t>(1023 + bits - 2) << 20 | static_cast<uint32_t>((w.hi >> 43) & 0xFFFFFu)) - 1u;
+}
+__host__ __device__ constexpr double inverse_M(int set)
+{
+    const Wide w = group_weight(set, -1);
+    return 1.0 / (static_cast<double>(w.hi) * pow2d(64) + static_cast<double>(w.lo));
+}
+
+// ---- kernels ----------------------------------------------------------------------------------------
+// Constants that do not fit an instruction's immediate operand (the high and middle parts do: 21 significant bits)
+struct ReconConst { double rest[kMaxGroups], M_rest, inv_M; };
+template <int SET>
+constexpr ReconConst recon_constants()
+{
+    ReconConst c{};
+    for (int g = 0; g < set_groups(SET); ++g) c.rest[g] = static_cast<double>(split_parts(SET, group_weight(SET, g)).rest);
+    c.M_rest = static_cast<double>(split_parts(SET, group_weight(SET, -1)).rest);
+    c.inv_M = inverse_M(SET);
+    return c;
+}
+__constant__ ReconConst c_recon[kNumSets] = {recon_constants<0>(), recon_constants<1>(), recon_constants<2>()};
+
+// Threads of a block of the private layout's kernel: one warp for each chunk of sixteen rows and, of two rows a thread, each half of it; eight columns.  1024
+// threads on an SM: numbers, sums and old values of C take 64 registers.  16384 x 16384 update, set S, in blocks of 256 threads 1709 us, of 128
+// 1611 us, the same with 896 threads on an SM (72 registers), 1893 with 1152 (56, spills).
+__host__ __device__ constexpr int tiled_threads(int rows) { return rows == 4 ? 128 : 256; }
+// Up to this many outputs two rows a thread (from 1200 x 1200 on four are faster): 512 x 512 on set S 23.7 us a call, with four rows 25.7; 700 x 700 x 300 29.3 and 30.6.
+constexpr int64_t kFewOutputs = 700000;
+// Public layout: blocks of 128 threads, nine an SM with two rows a thread (56 registers).  6000 x 6000 update, set E, with 8 / 9 / 10: 288 / 274 / 281 us
+constexpr int kPublicThreads = 128;
 constexpr double kRint = 6755399441055744.0;          // 1.5 * 2^52: (x + kRint) - kRint = rint(x)
 
 // x * 2^scale for a finite double x (exact unless the result leaves the normal range)
@@ -55,45 +200,216 @@ __device__ __forceinline__ double scale_pow2(double x, int scale)
     return scalbn(x, scale);        // zero, or a result outside the normal range
 }
 
-// w packs the residues of consecutive rows (two uint16 or four uint8); HALF selects the row
-template <int SET, int HALF, int I>
-__device__ __forceinline__ void crt_term(uint32_t w, double &S0, double &S1, double &S2)
+// The numbers of a thread's rows: lo the low bytes, hi the bits above them in the same bytes (ten-bit form); two-byte form: lo the first
+// two rows, hi the others
+struct Numbers { uint32_t lo[kMaxR], hi[kMaxR]; };
+
+template <uint32_t SELECT>
+__device__ __forceinline__ uint32_t permute(uint32_t a, uint32_t b)
 {
-    const ReconConst &K = c_recon[SET];
-    constexpr int BITS = 8 * residue_bytes(SET);
-    const uint32_t c = (w >> (BITS * HALF)) & ((1u << BITS) - 1u);
-    // exact; the hardware conversion keeps this off the FP64 pipe, which bounds the kernel
-    double cd = __uint2double_rn(c);
-    S0 = fma(cd, K.V[I][0], S0);
-    S1 = fma(cd, K.V[I][1], S1);
-    S2 = fma(cd, K.V[I][2], S2);
+    uint32_t v;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(v) : "r"(a), "r"(b), "n"(SELECT));
+    return v;
 }
 
-template <int SET, int HALF, int... I>
-__device__ __forceinline__ void crt_sum(std::integer_sequence<int, I...>, const uint32_t (&c)[kMaxR],
-                                        double &S0, double &S1, double &S2)
+// number of modulus I in row H of the thread
+template <int SET, bool PRIVATE, int H, int I>
+__device__ __forceinline__ uint32_t number(const Numbers &w)
 {
-    (crt_term<SET, HALF, I>(c[I], S0, S1, S2), ...);
+    constexpr int form = PRIVATE || residue_bytes(SET) == 1 ? stored_form(SET, I) : static_cast<int>(kStoredPair);
+    if constexpr (form == kStoredByte) {
+        return permute<0x4440u + H>(w.lo[I], 0u);
+    } else if constexpr (form == kStoredTen) {
+        return permute<0xCC40u + 0x1111u * H>(w.lo[I], w.hi[I]);              // above the two bytes: the sign of one below 4
+    } else {
+        const uint32_t c = permute<(H & 1) ? 0x4432u : 0x4410u>(H < 2 ? w.lo[I] : w.hi[I], 0u);
+        return !PRIVATE && reduced_first(SET, I) ? min(c, c - static_cast<uint32_t>(modulus(SET, I))) : c;
+    }
 }
 
-// Exact tail (rare path): the three chunks as a 128-bit integer, exact lift to [-M/2, M/2),
+template <int SET, bool PRIVATE, int H, int G>
+__device__ __forceinline__ int group_value(const Numbers &w)
+{
+    constexpr int i0 = group_member(SET, G, 0), i1 = group_member(SET, G, 1), i2 = group_member(SET, G, 2);
+    constexpr uint32_t a0 = static_cast<uint32_t>(member_weight(SET, G, 0)), a1 = static_cast<uint32_t>(member_weight(SET, G, 1)),
+                       a2 = static_cast<uint32_t>(member_weight(SET, G, 2));
+    uint32_t u = number<SET, PRIVATE, H, i0>(w) * a0;
+    u = number<SET, PRIVATE, H, i1>(w) * a1 + u;
+    if constexpr (i2 >= 0) u = number<SET, PRIVATE, H, i2>(w) * a2 + u;
+    return static_cast<int>(u);
+}
+
+template <int SET, bool PRIVATE, int H, int G>
+__device__ __forceinline__ void crt_term(const Numbers &w, double &X0, double &X1, double &X2)
+{
+    constexpr Parts p = split_parts(SET, group_weight(SET, G));
+    constexpr double high = static_cast<double>(p.high) * pow2d(high_bit(SET)), mid = static_cast<double>(p.mid) * pow2d(mid_bit(SET));
+    const double d = __int2double_rn(group_value<SET, PRIVATE, H, G>(w)), rest = c_recon[SET].rest[G];
+    X0 = G == 0 ? d * rest : fma(d, rest, X0);
+    X1 = G == 0 ? d * mid : fma(d, mid, X1);
+    X2 = G == 0 ? d * high : fma(d, high, X2);
+}
+
+template <int SET, bool PRIVATE, int H, int... G>
+__device__ __forceinline__ void crt_sum(std::integer_sequence<int, G...>, const Numbers &w, double &X0, double &X1, double &X2)
+{
+    (crt_term<SET, PRIVATE, H, G>(w, X0, X1, X2), ...);
+}
+
+template <int SET, bool PRIVATE, int H, int... G>
+__device__ __forceinline__ void group_values(std::integer_sequence<int, G...>, const Numbers &w, int (&u)[kMaxGroups])
+{
+    ((u[G] = group_value<SET, PRIVATE, H, G>(w)), ...);
+}
+
+template <int SET, int... G>
+__device__ __forceinline__ unsigned __int128 exact_sum(std::integer_sequence<int, G...>, const int (&u)[kMaxGroups])
+{
+    unsigned __int128 v = 0;
+    auto term = [&](int ug, Wide N) {
+        v += static_cast<unsigned __int128>(static_cast<__int128>(ug)) * ((static_cast<unsigned __int128>(N.hi) << 64) | N.lo);
+    };
+    (term(u[G], group_weight(SET, G)), ...);
+    return v;
+}
+
+// The numbers of a thread from the public layout: ROWS consecutive rows of a column
+template <int SET>
+struct PublicLoader {
+    static constexpr bool kPrivate = false;
+    const unsigned char *base;
+    int64_t stride;                  // bytes from modulus to modulus
+    int nrows;
+    bool words;                      // one 32-bit load covers the rows
+    __device__ __forceinline__ void load(Numbers &w) const
+    {
+        constexpr int RB = residue_bytes(SET), ROWS = 4 / RB;
+#pragma unroll
+        for (int i = 0; i < set_r(SET); ++i) {
+            w.hi[i] = 0u;
+            const unsigned char *src = base + i * stride;
+            if (words) {
+                w.lo[i] = *reinterpret_cast<const uint32_t *>(src);    // ldr is a multiple of ROWS: in bounds
+            } else {
+                uint32_t v = 0;
+#pragma unroll
+                for (int h = 0; h < ROWS; ++h) {
+                    if (h < nrows) {
+                        uint32_t e = RB == 2 ? reinterpret_cast<const uint16_t *>(src)[h] : src[h];
+                        v |= e << (8 * RB * h);
+                    }
+                }
+                w.lo[i] = v;
+            }
+        }
+    }
+};
+
+// From a patch of the private array: chunk c, column, word of the chunk; of two rows a thread, the half of the word
+template <int SET, int ROWS>
+struct PatchLoader {
+    static constexpr bool kPrivate = true;
+    const unsigned char *patch;
+    uint32_t c, column, word, half;
+    template <int I>
+    __device__ __forceinline__ void load_modulus(Numbers &w) const
+    {
+        constexpr int form = stored_form(SET, I);
+        const unsigned char *src = patch + stored_start(SET, I);           // a compile-time offset from one address
+        w.hi[I] = 0u;
+        if constexpr (form == kStoredPair) {
+            w.lo[I] = *reinterpret_cast<const uint32_t *>(src + ((2 * c + (ROWS == 2 ? half : 0u)) * 32 + column) * 16 + word * 4);
+            if constexpr (ROWS == 4) w.hi[I] = *reinterpret_cast<const uint32_t *>(src + ((2 * c + 1) * 32 + column) * 16 + word * 4);
+        } else {
+            w.lo[I] = *reinterpret_cast<const uint32_t *>(src + (c * 32 + column) * 16 + word * 4);
+            if constexpr (form == kStoredTen) w.hi[I] = *reinterpret_cast<const uint32_t *>(src + 2048 + column * 16 + c * 4);
+        }
+    }
+    template <int I>
+    __device__ __forceinline__ void own_rows(Numbers &w) const
+    {
+        const uint32_t skip = ROWS == 2 ? 16 * half : 0u;
+        if constexpr (stored_form(SET, I) == kStoredTen) w.hi[I] = (w.hi[I] >> (2 * word + skip)) & 0x03030303u;        // the thread's bits
+        if constexpr (stored_form(SET, I) != kStoredPair && ROWS == 2) w.lo[I] >>= skip;
+    }
+    template <int... I>
+    __device__ __forceinline__ void load_all(std::integer_sequence<int, I...>, Numbers &w) const
+    {
+        (load_modulus<I>(w), ...);
+        (own_rows<I>(w), ...);
+    }
+    __device__ __forceinline__ void load(Numbers &w) const { load_all(std::make_integer_sequence<int, set_r(SET)>{}, w); }
+};
+
+// u_g where every residue is zero and stands there as 0 or as m
+template <int SET>
+__host__ __device__ constexpr int64_t group_of_moduli(int g)
+{
+    int64_t u = 0;
+    for (int e = 0; e < 3; ++e)
+        if (group_member(SET, g, e) >= 0) u += modulus(SET, group_member(SET, g, e)) % 1024 * member_weight(SET, g, e);
+    return u;
+}
+template <int SET, bool MODULI>
+__device__ __forceinline__ bool no_residue(const int (&u)[kMaxGroups])
+{
+    bool zero = u[0] == (MODULI ? static_cast<int>(group_of_moduli<SET>(0)) : 0);
+    zero = zero && u[1] == (MODULI ? static_cast<int>(group_of_moduli<SET>(1)) : 0) && u[2] == (MODULI ? static_cast<int>(group_of_moduli<SET>(2)) : 0) &&
+           u[3] == (MODULI ? static_cast<int>(group_of_moduli<SET>(3)) : 0) && u[4] == (MODULI ? static_cast<int>(group_of_moduli<SET>(4)) : 0);
+    if constexpr (set_groups(SET) == 6) zero = zero && u[5] == (MODULI ? static_cast<int>(group_of_moduli<SET>(5)) : 0);
+    return zero;
+}
+
+// alpha 2^-(sa + sb) c' (alpha = 1 or -1, as a sign bit) where only the scale is out of reach: r is c' correctly rounded.  NaN for a line with
+// Inf/NaN.  The sum of the shifts is taken in 64 bits; beyond 2^20 the result is zero or infinite whatever c' is.
+__device__ __forceinline__ bool marked(int sa, int sb) { return sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT; }
+__device__ __forceinline__ int far_sum(int sa, int sb)
+{
+    return static_cast<int>(min(max(static_cast<long long>(sa) + sb, -(1ll << 20)), 1ll << 20));
+}
+__device__ __noinline__ double row_value_far(double r, int sa, int sb, int alpha_sign)
+{
+    const double alpha = __hiloint2double(0x3FF00000 ^ alpha_sign, 0);
+    if (marked(sa, sb)) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
+    return scale_pow2(r, -far_sum(sa, sb)) * alpha;
+}
+
+// The same where c' itself has to be formed: the sum modulo 2^128 (|c'| is below 2^118), exact lift to [-M/2, M/2),
 // round-to-nearest-even conversion in integer arithmetic, power-of-two scale.
-__device__ __forceinline__ double finish_exact(double X0, double X1, double X2, int shift_sum, int set)
+// `from` reads the numbers once more: held until here they would cost the common case a third of its registers.
+template <int SET, class Loader>
+__device__ __noinline__ double row_value_exact(Loader from, int h, int sa, int sb, int alpha_sign)
 {
-    const ReconConst &K = c_recon[set];
-    const int cw = chunk_bits(set);
-    const long long t0 = __double2ll_rn(X0), t1 = __double2ll_rn(X1 * (1.0 / pow2d(cw))), t2 = __double2ll_rn(X2 * (1.0 / pow2d(2 * cw)));
-    // v = t0 + t1 2^cw + t2 2^(2cw) as a two's-complement (hi:lo) pair
-    unsigned long long lo = static_cast<unsigned long long>(t0) + (static_cast<unsigned long long>(t1) << cw);
-    long long hi = (t0 >> 63) + (t1 >> (64 - cw)) + (lo < static_cast<unsigned long long>(t0) ? 1 : 0) +
-                   static_cast<long long>(static_cast<unsigned long long>(t2) << (2 * cw - 64));
-    const __int128 M = static_cast<__int128>((static_cast<unsigned __int128>(K.M_hi) << 64) | K.M_lo);
+    const double alpha = __hiloint2double(0x3FF00000 ^ alpha_sign, 0);
+    if (marked(sa, sb)) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
+    Numbers w;
+    from.load(w);
+    // row h in the place of the first one
+#pragma unroll
+    for (int i = 0; i < set_r(SET); ++i) {
+        if (Loader::kPrivate ? stored_form(SET, i) == kStoredPair : residue_bytes(SET) == 2) {
+            w.lo[i] = (h < 2 ? w.lo[i] : w.hi[i]) >> (16 * (h & 1));
+        } else {
+            w.lo[i] >>= 8 * h;
+            w.hi[i] >>= 8 * h;
+        }
+    }
+    int u[kMaxGroups] = {};
+    group_values<SET, Loader::kPrivate, 0>(std::make_integer_sequence<int, set_groups(SET)>{}, w, u);
+    if (no_residue<SET, false>(u) || no_residue<SET, true>(u)) return 0.0 * alpha;       // structural zeros of a product
+    constexpr Wide Mw = group_weight(SET, -1);
+    const __int128 M = static_cast<__int128>((static_cast<unsigned __int128>(Mw.hi) << 64) | Mw.lo);
     const __int128 Mh = M >> 1;     // M is even for every set (each holds a power of two)
-    __int128 v = static_cast<__int128>((static_cast<unsigned __int128>(static_cast<unsigned long long>(hi)) << 64) | lo);
+    double share = 0.0;             // S / M
+#pragma unroll
+    for (int g = 0; g < set_groups(SET); ++g) share += static_cast<double>(u[g]) / static_cast<double>(group_product(SET, g));
+    const __int128 kappa = static_cast<__int128>(__double2int_rn(share));
+    __int128 v = static_cast<__int128>(exact_sum<SET>(std::make_integer_sequence<int, set_groups(SET)>{}, u) -
+                                       static_cast<unsigned __int128>(M) * static_cast<unsigned __int128>(kappa));
     if (v >= Mh) v -= M;
     else if (v < -Mh) v += M;
-    lo = static_cast<unsigned long long>(v);
-    hi = static_cast<long long>(v >> 64);
+    unsigned long long lo = static_cast<unsigned long long>(v);
+    long long hi = static_cast<long long>(v >> 64);
     const bool neg = hi < 0;
     if (neg) {
         lo = 0ull - lo;
@@ -101,74 +417,43 @@ __device__ __forceinline__ double finish_exact(double X0, double X1, double X2, 
     }
     // nearest double, ties to even: top 64 bits with a sticky bit far below the rounding position
     const unsigned long long uhi = static_cast<unsigned long long>(hi);
-    const int lz = __clzll(static_cast<long long>(uhi | 1ull));          // uhi < 2^49: lz in [15, 63]
+    const int lz = __clzll(static_cast<long long>(uhi | 1ull));          // uhi < 2^54: lz in [10, 63]
     const unsigned long long top = (uhi << lz) | (lo >> (64 - lz));
     const unsigned long long rest = lo << lz;
-    unsigned long long mant = uhi ? (top | (rest ? 1ull : 0ull)) : lo;
-    int scale = (uhi ? 64 - lz : 0) - shift_sum;
-    double d = scale_pow2(__ull2double_rn(mant), scale);
-    return neg ? -d : d;
+    const unsigned long long mant = uhi ? (top | (rest ? 1ull : 0ull)) : lo;
+    const double d = scale_pow2(__ull2double_rn(mant), (uhi ? 64 - lz : 0) - far_sum(sa, sb));
+    return (neg ? -d : d) * alpha;
 }
 
-// The three chunks summed: r is c' correctly rounded if the result is true (see row_value())
-template <int SET>
-__device__ __forceinline__ bool round_chunks(double X0, double X1, double X2, double &r)
+// One row: r, and whether it is c' correctly rounded.
+// X2 + X1 = s + err by a fast two-sum, which is error-free because X2 is a multiple of 2^high_bit and so of ulp(X1)
+// (|X1| < 2^(53 + mid_bit)); t = err + X0, where X0 is off by its multiply-adds' roundings; s + t = r + rem exactly (s is a multiple of
+// 2^mid_bit and so of ulp(t)).  All that is lost is below 2^kRestErrorLog2, so r is c' correctly rounded where rem enlarged by that much
+// does not move it and |r| is in the range of range_word(): from 2^56 times that error on, so that the other side is no nearer, a power of two
+// included, and below M / 2.
+template <int SET, bool PRIVATE, int H>
+__device__ __forceinline__ bool row_value(const Numbers &w, double &r)
 {
+    constexpr Parts M = split_parts(SET, group_weight(SET, -1));
+    constexpr double M1 = static_cast<double>(M.mid) * pow2d(mid_bit(SET)), M2 = static_cast<double>(M.high) * pow2d(high_bit(SET));
+    double X0 = 0.0, X1 = 0.0, X2 = 0.0;
+    crt_sum<SET, PRIVATE, H>(std::make_integer_sequence<int, set_groups(SET)>{}, w, X0, X1, X2);
+    const double minus_kappa = kRint - fma(X2 + X1, c_recon[SET].inv_M, kRint);
+    X0 = fma(minus_kappa, c_recon[SET].M_rest, X0);
+    X1 = fma(minus_kappa, M1, X1);              // exact: integers below 2^53 in units of their places
+    X2 = fma(minus_kappa, M2, X2);
     const double s = X2 + X1, err = X1 - (s - X2);
     const double t = err + X0;
     r = s + t;
     const double rem = t - (r - s);
-    return fma(rem, 1.0 + 0x1p-29, r) == r && (__double2hiint(r) & 0x7FFFFFFF) < c_recon[SET].half_M_guard;
+    constexpr int kErrorWord = (1023 + kRestErrorLog2<SET>) << 20;
+    const double more = rem + __hiloint2double((__double2hiint(rem) & INT32_MIN) | kErrorWord, 0);
+    return r + more == r;
 }
-
-// alpha 2^-(sa + sb) c' (alpha = 1 or -1, as a sign bit: in a register pair of its own it spilled) where the fast path does not apply: NaN for a line with Inf/NaN; else from r, where that is c' correctly
-// rounded and only the scale is out of reach, or by integers.  The sum of the shifts is taken in 64 bits; beyond 2^20 the result is
-// zero or infinite whatever c' is.
+// below kRangeSpan for |r| in that range (the sign shifted out)
+template <int SET> constexpr uint32_t kRangeSpan = 2u * (half_M_word(SET) - small_word(SET));
 template <int SET>
-__device__ __noinline__ double row_value_exact(double X0, double X1, double X2, int sa, int sb, int alpha_sign)
-{
-    const double alpha = __hiloint2double(0x3FF00000 ^ alpha_sign, 0);
-    if (sb == OZ_NONFINITE_SHIFT || sa == OZ_NONFINITE_SHIFT) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
-    const int sum = static_cast<int>(min(max(static_cast<long long>(sa) + sb, -(1ll << 20)), 1ll << 20));
-    double r;
-    return (round_chunks<SET>(X0, X1, X2, r) ? scale_pow2(r, -sum) : finish_exact(X0, X1, X2, sum, SET)) * alpha;
-}
-
-// Whether a row's shift may enter the 32-bit sums of the fast path: |sa| <= 2^30, which the mark of a row with Inf/NaN exceeds.  No sum
-// with a column's shift, whatever that is and the mark of a column among them, then wraps into the range of row_value().
-__device__ __forceinline__ bool ordinary_row(int sa)
-{
-    return static_cast<uint32_t>(sa) + (1u << 30) <= 1u << 31;
-}
-
-// One row of the thread's group: value = fast alpha 2^-(sa + sb) c', returned as the rounded integer r and the power of
-// two to multiply it by (exact, and left to the caller so that an update of C is one fused multiply-add).
-// The chunks are not carry-normalised.  X2 + X1 = s + err by a fast two-sum, which is error-free because X2 is a multiple of
-// 2^(2cw) and so of ulp(X1) (|X1| < 2^(53+cw)); t = err + X0 loses at most 2^-52 of |err| + |X0|, and nothing below 2^53,
-// which |X0| < 2^52.1 alone does not reach: what it loses is below 2^-40 of half an ulp of s; s + t = r + rem exactly (s is a
-// multiple of 2^cw and so of ulp(t)).  Hence r is c' correctly rounded unless c' lies within 2^-29 of half an ulp from a
-// rounding boundary -- adding rem, enlarged by 2^-29, then moves r -- or so near to +-M/2 that the lift may apply.
-// 50 FP64 operations per output on set S where the carries and a test by exponents took 63.
-template <int SET, int HALF>
-__device__ __forceinline__ void row_value(const uint32_t (&c)[kMaxR], int sa, int sb, int alpha_sign,
-                                          double &r, double &scale)
-{
-    const ReconConst &K = c_recon[SET];
-    double X0 = 0.0, X1 = 0.0, X2 = 0.0;
-    crt_sum<SET, HALF>(std::make_integer_sequence<int, set_r(SET)>{}, c, X0, X1, X2);
-    const double kappa = fma(X2 + X1, K.inv_M, kRint) - kRint;
-    X0 = fma(-kappa, K.Mc[0], X0);              // exact: integers below 2^53 (times 2^cw, 2^(2cw))
-    X1 = fma(-kappa, K.Mc[1], X1);
-    X2 = fma(-kappa, K.Mc[2], X2);
-    const bool rounded = round_chunks<SET>(X0, X1, X2, r);
-    const uint32_t shift_sum = static_cast<uint32_t>(sa) + static_cast<uint32_t>(sb);
-    scale = __hiloint2double(static_cast<int>((1023u - shift_sum) << 20) ^ alpha_sign, 0);
-    // in range: 2^-shift_sum and r 2^-shift_sum are normal; r is zero or 1 <= |r| < 2^118
-    if (!(ordinary_row(sa) && shift_sum + 904u <= 1924u && rounded)) {
-        r = row_value_exact<SET>(X0, X1, X2, sa, sb, alpha_sign);
-        scale = 1.0;
-    }
-}
+__device__ __forceinline__ uint32_t range_word(double r) { return 2u * static_cast<uint32_t>(__double2hiint(r)) - 2u * small_word(SET); }
 
 // scalar stores of up to two consecutive rows; `first` / `second`: which of them are written
 __device__ __forceinline__ void store_pair(double *out, double p0, double p1, bool first, bool second, double beta)
@@ -177,183 +462,157 @@ __device__ __forceinline__ void store_pair(double *out, double p0, double p1, bo
     if (second) out[1] = beta != 0.0 ? out[1] + p1 : p1;
 }
 
-// the ROWS consecutive rows of column j whose residues are packed in w[]: reconstruct, update C.
+// ROWS rows of a column, row_of(0) .. from `row` on: reconstruct, update C with fast alpha 2^-(sa + sb) c'.
 // For beta = 1 the old values of C are requested before the arithmetic starts, so that their latency
-// hides behind it.  `keep`: bit h set = row h is written (rows that go to the native FP64 path are not).
-template <int SET>
-__device__ __forceinline__ void reconstruct_rows(const uint32_t (&w)[kMaxR], int64_t row, int nrows, int sb,
+// hides behind it.  nrows: rows of C from `row` on.  `keep`: bit h set = the thread's row h is written (rows that go to the native FP64 path are not).
+// The tests of a thread's rows are taken together: one branch a thread, which almost none takes.
+template <bool PRIVATE> __device__ __forceinline__ constexpr int row_of(int h) { return (h & 1) + (PRIVATE ? 8 : 2) * (h >> 1); }
+template <int SET, int ROWS, class Loader, int... H>
+__device__ __forceinline__ void reconstruct_rows(std::integer_sequence<int, H...>, const Loader &from, int64_t row, int nrows, int sb,
                                                  const int32_t *__restrict__ shiftA, double alpha, double beta,
-                                                 double *out, bool vecC, uint32_t keep = 0xFu)
+                                                 double *out, bool vecC, uint32_t keep)
 {
-    constexpr int ROWS = 4 / residue_bytes(SET);
+    constexpr bool PRIVATE = Loader::kPrivate;
+    // all residue loads are issued before any arithmetic: independent requests in flight per
+    // thread, kept packed so that they fit the register budget
+    Numbers w;
+    from.load(w);
     int sa[ROWS];
 #pragma unroll
-    for (int h = 0; h < ROWS; ++h) sa[h] = h < nrows ? shiftA[row + h] : 0;
-    const bool whole = vecC && nrows == ROWS && (keep & ((1u << ROWS) - 1u)) == ((1u << ROWS) - 1u);
+    for (int h = 0; h < ROWS; ++h) sa[h] = row_of<PRIVATE>(h) < nrows ? shiftA[row + row_of<PRIVATE>(h)] : 0;
+    const bool whole = vecC && nrows > row_of<PRIVATE>(ROWS - 1) && (keep & ((1u << ROWS) - 1u)) == ((1u << ROWS) - 1u);
     double2 old[ROWS / 2];
 #pragma unroll
     for (int h = 0; h < ROWS / 2; ++h) old[h] = make_double2(0.0, 0.0);
     if (whole && beta != 0.0) {
 #pragma unroll
-        for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + 2 * h);
+        for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + row_of<PRIVATE>(2 * h));
     }
     const int alpha_sign = alpha < 0.0 ? INT32_MIN : 0;
-    {
-        double r0, r1 = 0.0, f0, f1 = 1.0;
-        row_value<SET, 0>(w, sa[0], sb, alpha_sign, r0, f0);
-        if (nrows > 1) row_value<SET, 1>(w, sa[1], sb, alpha_sign, r1, f1);
-        if (whole) *reinterpret_cast<double2 *>(out) = make_double2(fma(r0, f0, old[0].x), fma(r1, f1, old[0].y));
-        else store_pair(out, r0 * f0, r1 * f1, (keep & 1u) != 0, nrows > 1 && (keep & 2u) != 0, beta);
+    double r[ROWS];
+    bool rounded[ROWS];
+    ((rounded[H] = row_value<SET, PRIVATE, H>(w, r[H])), ...);
+    // 2^-(sa + sb) and r 2^-(sa + sb) are normal for sums in [-904, 1020] (1 <= |r| < 2^118); the sum is taken in 32 bits, which a shift of
+    // at most 2^30, unlike the mark of a row with Inf/NaN, cannot wrap into that range whatever the column's is, its mark among them
+    uint32_t scale[ROWS], far = 0u, wide = 0u, range = 0u;
+    bool all = true;
+    const uint32_t scale0 = (1023u + 904u) << 20 ^ static_cast<uint32_t>(alpha_sign);
+#pragma unroll
+    for (int h = 0; h < ROWS; ++h) {
+        const uint32_t sum = static_cast<uint32_t>(sa[h]) + static_cast<uint32_t>(sb) + 904u;
+        far = max(far, sum);
+        wide |= static_cast<uint32_t>(sa[h]) + (1u << 30);
+        range = max(range, range_word<SET>(r[h]));
+        scale[h] = scale0 - (sum << 20);                 // high word of alpha 2^-(sa + sb)
+        all = all && rounded[h];
     }
-    if constexpr (ROWS == 4) {
-        if (nrows > 2) {
-            double r2, r3 = 0.0, f2, f3 = 1.0;
-            row_value<SET, 2>(w, sa[2], sb, alpha_sign, r2, f2);
-            if (nrows > 3) row_value<SET, 3>(w, sa[3], sb, alpha_sign, r3, f3);
-            if (whole) *reinterpret_cast<double2 *>(out + 2) = make_double2(fma(r2, f2, old[1].x), fma(r3, f3, old[1].y));
-            else store_pair(out + 2, r2 * f2, r3 * f3, (keep & 4u) != 0, nrows > 3 && (keep & 8u) != 0, beta);
-        }
+    if (!(all && far <= 1924u && wide < 1u << 31 && range < kRangeSpan<SET>)) {
+        auto fix = [&](auto index) {
+            constexpr int h = decltype(index)::value;
+            const bool good = rounded[h] && range_word<SET>(r[h]) < kRangeSpan<SET>;
+            const bool near = static_cast<uint32_t>(sa[h]) + static_cast<uint32_t>(sb) + 904u <= 1924u && static_cast<uint32_t>(sa[h]) + (1u << 30) < 1u << 31;
+            if (good && near) return;
+            if (good) {
+                r[h] = row_value_far(r[h], sa[h], sb, alpha_sign);
+            } else if (row_of<PRIVATE>(h) < nrows) {
+                r[h] = row_value_exact<SET>(from, h, sa[h], sb, alpha_sign);
+            }
+            scale[h] = 0x3FF00000u;
+        };
+        (fix(std::integral_constant<int, H>{}), ...);
+    }
+#pragma unroll
+    for (int p = 0; p < ROWS / 2; ++p) {
+        const int first = row_of<PRIVATE>(2 * p);
+        const double f0 = __hiloint2double(static_cast<int>(scale[2 * p]), 0), f1 = __hiloint2double(static_cast<int>(scale[2 * p + 1]), 0);
+        if (whole) *reinterpret_cast<double2 *>(out + first) = make_double2(fma(r[2 * p], f0, old[p].x), fma(r[2 * p + 1], f1, old[p].y));
+        else store_pair(out + first, r[2 * p] * f0, r[2 * p + 1] * f1, nrows > first && (keep >> (2 * p) & 1u), nrows > first + 1 && (keep >> (2 * p + 1) & 1u), beta);
     }
 }
 
 // Each thread reconstructs ROWS consecutive rows of one column: the residues of those rows are one
 // 32-bit word per modulus (two uint16 for S and E, four uint8 for the all-byte set A).
 template <int SET>
-__global__ void __launch_bounds__(256, kReconBlocks<SET>)
+__global__ void __launch_bounds__(kPublicThreads, residue_bytes(SET) == 2 ? 9 : 8)
 reconstruct_kernel(const void *__restrict__ Rv, int64_t ldr, int64_t mod_stride, int64_t m,
                    int64_t n, const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
                    double alpha, double beta, double *__restrict__ C, int64_t ldc, int vecR, int vecC)
 {
     dependency_release();
     dependency_wait();
-    constexpr int RB = residue_bytes(SET), ROWS = 4 / RB, r = set_r(SET);
+    constexpr int RB = residue_bytes(SET), ROWS = 4 / RB;
     // grid.x covers the row groups of a column, grid.y (and .z beyond 65535) the columns: no division
-    const int64_t row = (blockIdx.x * 256ll + threadIdx.x) * ROWS;
+    const int64_t row = (blockIdx.x * static_cast<int64_t>(kPublicThreads) + threadIdx.x) * ROWS;
     if (row >= m) return;
     const int64_t j = blockIdx.y + 65535ll * blockIdx.z;
     if (j >= n) return;
     const int nrows = m - row < ROWS ? static_cast<int>(m - row) : ROWS;
 
-    // all residue loads are issued before any arithmetic: r independent requests in flight per
-    // thread, kept packed so that they fit the register budget
-    uint32_t w[kMaxR];
-    const unsigned char *base = static_cast<const unsigned char *>(Rv) + (j * ldr + row) * RB;
-#pragma unroll
-    for (int i = 0; i < r; ++i) {
-        const unsigned char *src = base + i * mod_stride * RB;
-        if (vecR) {
-            w[i] = *reinterpret_cast<const uint32_t *>(src);       // ldr is a multiple of ROWS: in bounds
-        } else {
-            uint32_t v = 0;
-#pragma unroll
-            for (int h = 0; h < ROWS; ++h) {
-                if (h < nrows) {
-                    uint32_t e = RB == 2 ? reinterpret_cast<const uint16_t *>(src)[h] : src[h];
-                    v |= e << (8 * RB * h);
-                }
-            }
-            w[i] = v;
-        }
-    }
-    reconstruct_rows<SET>(w, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, vecC != 0);
+    const PublicLoader<SET> from{static_cast<const unsigned char *>(Rv) + (j * ldr + row) * RB, mod_stride * RB, nrows, vecR != 0};
+    reconstruct_rows<SET, ROWS>(std::make_integer_sequence<int, ROWS>{}, from, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, vecC != 0, 0xFu);
 }
 
 // Same reconstruction from the tile-ordered private array that the whole-method GEMM writes (see
-// ResidueTiling).  A thread takes one 32-bit word of a 32-column x 64-row block, i.e. ROWS consecutive
-// rows of one column.  A warp takes one 16-byte chunk of eight neighbouring columns: its residue loads are whole
-// 128-byte lines and its accesses to C eight pieces of 64 (128) contiguous bytes; the warps of a thread block, which
+// ResidueTiling).  A thread takes four rows of one column: one 32-bit word of low bytes per modulus, and a word of high bits that the
+// four threads of a 16-byte chunk share.  A warp takes one chunk of eight neighbouring columns: its loads of low bytes are whole
+// 128-byte lines and its accesses to C eight pieces of 64 contiguous bytes; its next ones and the warps of a thread block, which
 // take the other chunks of the same columns, complete those to whole lines of C.
 // ACCESS: how C is taken, in pairs of elements (even ldc, C on a multiple of 16 bytes), or singly, stored or updated.  Updates of single
 // elements, whose loads and stores in eight pieces each cost more the more there are, give a warp consecutive words of one column: 512
 // contiguous bytes of C for residue loads that touch eight lines.  1009 x 983 x 256, set S: 39 us a call against 52; 4501 x 4400 x 128: 400
 // against 732; plain stores are faster in pieces (34 us against 36, 334 against 352).
-// grid: x = (piece of the block, block within the tile, CTA rank of the pair), y = tile column, z = tile row
+// The loads wait for DRAM as long as the arithmetic takes, so the first block of a patch asks for the patch that is `ahead` of it, in the order of the
+// blocks, to be brought into L2: 16384 x 16384 update, set S, 1803 -> 1725 us (old values of C too: 1760; only those: 1922), 8192 x 8192 on set A
+// 401 -> 363 us.  (Patches in a ring of shared memory, two ahead, two blocks of 512 threads an SM: 2920 us.)
+// grid: x = (piece of the patch, patch within the tile, CTA rank of the pair), y = tile column, z = tile row
 // SKIP: rows flagged in `skip` are left untouched (they are re-issued on the native FP64 path).
 enum { kPairs, kSingleStores, kSingleUpdates };
-template <int SET, bool SKIP, int ACCESS>
-__global__ void __launch_bounds__(256, kReconBlocks<SET, ACCESS == kSingleUpdates>)
+// ROWS: four, or two where the outputs are few and a thread's chain of arithmetic counts (launch_reconstruct_tiled())
+template <int SET, bool SKIP, int ACCESS, int ROWS>
+__global__ void __launch_bounds__(tiled_threads(ROWS), 1024 / tiled_threads(ROWS))
 reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int tn0,
                          int64_t m, int64_t n, int64_t col0, int64_t col1,
                          const int32_t *__restrict__ shiftA, const int32_t *__restrict__ shiftB,
                          double alpha, double beta, double *__restrict__ C, int64_t ldc,
-                         const unsigned char *__restrict__ skip)
+                         const unsigned char *__restrict__ skip, uint32_t ahead)
 {
     dependency_release();
     dependency_wait();
-    constexpr int RB = residue_bytes(SET), ROWS = 4 / RB, r = set_r(SET);
-    constexpr int kBlockWords = 64 * 32 * RB / 4;          // words of one 32 x 64 block: 1024 or 512
-    constexpr int kColWords = 64 / ROWS;                   // words of one column of the block: 32 or 16
-    constexpr int kCtaCols = 256 / kColWords;              // columns per thread block: 8 or 16
-    constexpr int kPieces = 32 / kCtaCols;                 // thread blocks per residue block: 4 or 2
+    constexpr int kColThreads = 64 / ROWS;                 // threads to a column of the patch
+    constexpr int kPieces = 32 * kColThreads / tiled_threads(ROWS);        // thread blocks per patch: 4
     const uint32_t piece = blockIdx.x % kPieces;
     const uint32_t wi = (blockIdx.x / kPieces) & 15u;
     const uint32_t rank = blockIdx.x / (kPieces * 16);     // 0, or 0..1 with CTA pairs
     const uint32_t tn = static_cast<uint32_t>(tn0) + blockIdx.y, tm = blockIdx.z;
-    constexpr int kChunks = kColWords / 4;                 // 16-byte chunks of one column: 8 or 4
     const uint32_t warp = threadIdx.x >> 5, sub = threadIdx.x & 3u;
     constexpr bool spread = ACCESS != kSingleUpdates;
-    const uint32_t c = spread ? warp % kChunks : (threadIdx.x >> 2) % kChunks;
-    const uint32_t lane = piece * kCtaCols + (spread ? warp / kChunks * 8 + ((threadIdx.x >> 2) & 7u) : threadIdx.x / kColWords);   // column of the block
-    const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * (16 / RB) + sub * ROWS;
+    const uint32_t c = spread ? warp & 3u : (threadIdx.x >> 2) & 3u;               // four chunks of sixteen rows
+    const uint32_t half = ROWS == 4 ? 0u : spread ? warp >> 2 : (threadIdx.x >> 4) & 1u;
+    const uint32_t lane = piece * 8 + (spread ? (threadIdx.x >> 2) & 7u : threadIdx.x / kColThreads);      // column of the patch
+    const uint32_t patch = ((tm * static_cast<uint32_t>(tiles_n) + tn) * static_cast<uint32_t>(cg) + rank) * 16 + wi;
+    if (ahead != 0 && threadIdx.x == 0 && piece == 0) {
+        const uint32_t next = patch + ahead;
+        if (next < static_cast<uint32_t>(tiles_n) * gridDim.z * static_cast<uint32_t>(cg) * 16)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
+                         ::"l"(static_cast<const unsigned char *>(Rv) + next * static_cast<int64_t>(patch_bytes(SET))), "r"(patch_bytes(SET)) : "memory");
+    }
+    const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * 16 + half * 8 + sub * 2;
     const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
     if (row >= m || j >= n || j < col0 || j >= col1) return;
-    const int nrows = m - row < ROWS ? static_cast<int>(m - row) : ROWS;
+    const int nrows = m - row < 16 ? static_cast<int>(m - row) : 16;
     uint32_t keep = 0xFu;
     if constexpr (SKIP) {
         keep = 0u;
 #pragma unroll
         for (int h = 0; h < ROWS; ++h)
-            if (h < nrows && !skip[row + h]) keep |= 1u << h;
+            if (row_of<true>(h) < nrows && !skip[row + row_of<true>(h)]) keep |= 1u << h;
         if (!keep) return;
     }
-    const int64_t wb = ((static_cast<int64_t>(tm) * tiles_n + tn) * cg + rank) * 16 + wi;
-    // the r blocks of this patch are consecutive: modulus i at a compile-time offset
-    const unsigned char *base = static_cast<const unsigned char *>(Rv) +
-                                ((wb * r) * kBlockWords + c * 128 + lane * 4 + sub) * 4;
-    uint32_t w[kMaxR];
-#pragma unroll
-    for (int i = 0; i < r; ++i) w[i] = *reinterpret_cast<const uint32_t *>(base + i * (kBlockWords * 4));
-    reconstruct_rows<SET>(w, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, ACCESS == kPairs, keep);
+    const PatchLoader<SET, ROWS> from{static_cast<const unsigned char *>(Rv) + patch * static_cast<int64_t>(patch_bytes(SET)), c, lane, sub, half};
+    reconstruct_rows<SET, ROWS>(std::make_integer_sequence<int, ROWS>{}, from, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, ACCESS == kPairs, keep);
 }
 
 }  // namespace
-
-oz_status_t upload_reconstruct_constants()
-{
-    static ReconConst host[kNumSets];
-    for (int set = 0; set < kNumSets; ++set) {
-        unsigned __int128 M = 1;
-        for (int i = 0; i < set_r(set); ++i) M *= static_cast<unsigned>(modulus(set, i));
-        const int cw = chunk_bits(set);
-        const unsigned __int128 mask = (static_cast<unsigned __int128>(1) << cw) - 1;
-        auto chunks = [&](unsigned __int128 v, double (&out)[3]) {
-            out[0] = static_cast<double>(static_cast<unsigned long long>(v & mask));
-            out[1] = static_cast<double>(static_cast<unsigned long long>((v >> cw) & mask)) * pow2d(cw);
-            out[2] = static_cast<double>(static_cast<unsigned long long>(v >> (2 * cw))) * pow2d(2 * cw);
-        };
-        ReconConst &K = host[set];
-        for (int i = 0; i < kMaxR; ++i) K.V[i][0] = K.V[i][1] = K.V[i][2] = 0.0;
-        for (int i = 0; i < set_r(set); ++i) {
-            unsigned mi = static_cast<unsigned>(modulus(set, i));
-            unsigned __int128 W = M / mi;
-            unsigned wm = static_cast<unsigned>(W % mi), inv = 0;
-            for (unsigned c = 1; c < mi; ++c)
-                if ((static_cast<unsigned long long>(wm) * c) % mi == 1) { inv = c; break; }
-            unsigned __int128 V = W * inv;          // < M, and V = 1 mod m_i, 0 mod the other moduli
-            chunks(V, K.V[i]);
-        }
-        chunks(M, K.Mc);
-        K.inv_M = 1.0 / static_cast<double>(M);
-        const double guard = 0.5 * static_cast<double>(M) * (1.0 - 0x1p-30);
-        uint64_t guard_bits;
-        memcpy(&guard_bits, &guard, sizeof(guard));
-        K.half_M_guard = static_cast<int>(guard_bits >> 32);
-        K.M_lo = static_cast<unsigned long long>(M);
-        K.M_hi = static_cast<unsigned long long>(M >> 64);
-    }
-    OZ_CUDA_CHECK(cudaMemcpyToSymbol(c_recon, host, sizeof(host)));
-    return OZ_OK;
-}
 
 oz_status_t launch_reconstruct(int64_t m, int64_t n, const void *R, int64_t ldr,
                                int64_t mod_stride, const int32_t *shiftA, const int32_t *shiftB,
@@ -364,13 +623,13 @@ oz_status_t launch_reconstruct(int64_t m, int64_t n, const void *R, int64_t ldr,
     const int rows = 4 / residue_bytes(set);
     int vecR = (ldr % rows == 0 && mod_stride % rows == 0 && (reinterpret_cast<uintptr_t>(R) & 3u) == 0) ? 1 : 0;
     int vecC = ((ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0) ? 1 : 0;
-    int64_t bx = ((m + rows - 1) / rows + 255) / 256;
+    int64_t bx = ((m + rows - 1) / rows + kPublicThreads - 1) / kPublicThreads;
     if (bx > 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;
     if (n > 65535ll * 65535ll) return OZ_ERR_UNSUPPORTED;
     dim3 grid(static_cast<unsigned>(bx), static_cast<unsigned>(n < 65535 ? n : 65535),
               static_cast<unsigned>((n + 65534) / 65535));
     auto kernel = set == 2 ? reconstruct_kernel<2> : set == 0 ? reconstruct_kernel<0> : reconstruct_kernel<1>;
-    OZ_CUDA_CHECK(launch(kernel, grid, 256, 0, stream, R, ldr, mod_stride, m, n, shiftA, shiftB, alpha, beta, C, ldc, vecR, vecC));
+    OZ_CUDA_CHECK(launch(kernel, grid, kPublicThreads, 0, stream, R, ldr, mod_stride, m, n, shiftA, shiftB, alpha, beta, C, ldc, vecR, vecC));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;
@@ -385,7 +644,9 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     const ResidueTiling t = residue_tiling(m, n, set);
     const int tn0 = static_cast<int>(col0 / t.tile_cols);
     const int ntn = static_cast<int>((col1 + t.tile_cols - 1) / t.tile_cols) - tn0;
-    const int pieces = 64 * 32 * residue_bytes(set) / 4 / 256;
+    // there the threads of four rows do not fill the chip
+    const bool few = m * n <= kFewOutputs;
+    constexpr int pieces = 4;              // thread blocks per patch
     if (t.tiles_m > 65535 || ntn > 65535) return OZ_ERR_UNSUPPORTED;
     const int vecC = ((ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0) ? 1 : 0;
     const dim3 grid(static_cast<unsigned>(pieces * 16 * t.cg), static_cast<unsigned>(ntn),
@@ -393,13 +654,18 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     // Blocks that become resident beside the GEMM's keep the multiprocessor's memory split at the GEMM's (28 KiB of L1) for
     // the whole kernel: worth the overlapped launch up to a million outputs only (16384 x 16384: 11.4 -> 11.9 ms a call)
     const bool early = m * n <= (1ll << 20);
-#define OZ_RECON_KERNEL(SET_, SKIP_)                                                    \
-    (vecC          ? reconstruct_tiled_kernel<SET_, SKIP_, kPairs>                      \
-     : beta == 0.0 ? reconstruct_tiled_kernel<SET_, SKIP_, kSingleStores>               \
-                   : reconstruct_tiled_kernel<SET_, SKIP_, kSingleUpdates>)
+    // one round of resident blocks ahead; not for a panel, whose blocks do not walk the array from end to end
+    const int64_t patches = static_cast<int64_t>(t.tiles_m) * t.tiles_n * t.cg * 16;
+    if (patches > 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;       // as the residue GEMM
+    const uint32_t ahead = ntn == t.tiles_n ? static_cast<uint32_t>(1024 / tiled_threads(few ? 2 : 4) * sm_count() / pieces) : 0u;
+#define OZ_RECON_KERNEL(SET_, SKIP_, ROWS_)                                             \
+    (vecC          ? reconstruct_tiled_kernel<SET_, SKIP_, kPairs, ROWS_>               \
+     : beta == 0.0 ? reconstruct_tiled_kernel<SET_, SKIP_, kSingleStores, ROWS_>        \
+                   : reconstruct_tiled_kernel<SET_, SKIP_, kSingleUpdates, ROWS_>)
 #define OZ_RECON_TILED(SET_)                                                                                         \
-    OZ_CUDA_CHECK(launch_if(early, skip ? OZ_RECON_KERNEL(SET_, true) : OZ_RECON_KERNEL(SET_, false), grid, 256, 0, stream, R, t.cg, \
-                         t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, skip))
+    OZ_CUDA_CHECK(launch_if(early, few ? (skip ? OZ_RECON_KERNEL(SET_, true, 2) : OZ_RECON_KERNEL(SET_, false, 2))   \
+                                       : (skip ? OZ_RECON_KERNEL(SET_, true, 4) : OZ_RECON_KERNEL(SET_, false, 4)), grid, tiled_threads(few ? 2 : 4), 0, stream, R, t.cg, \
+                         t.tiles_n, tn0, m, n, col0, col1, shiftA, shiftB, alpha, beta, C, ldc, skip, ahead))
     if (set == 2) OZ_RECON_TILED(2);
     else if (set == 0) OZ_RECON_TILED(0);
     else OZ_RECON_TILED(1);

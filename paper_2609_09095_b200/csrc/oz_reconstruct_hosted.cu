@@ -17,8 +17,8 @@
 // even, through the 64 leading bits and a sticky bit).  No FP64 arithmetic except the update of C.
 //
 // The residues come in the tile-ordered private layout of the whole-method calls (ResidueTiling): a
-// thread block of 128 threads takes 128 consecutive words of a 32 x 64 patch, i.e. ROWS = 2 (uint16
-// residues) or 4 (uint8) outputs per thread, ROWS small products per step.
+// thread block of 128 threads takes ROWS = 2 (sets S and E) or 4 rows of 128 neighbouring pieces of columns of a 32 x 64 patch,
+// ROWS outputs per thread, ROWS small products per step.
 //
 // Every wait is bounded; on expiry the block records OZ_ERR_TIMEOUT, frees its TMEM and returns.
 #include "oz_internal.h"
@@ -201,6 +201,24 @@ __device__ __forceinline__ double finish_from_sums(const uint32_t (&P)[16], int 
     return neg ? -d : d;
 }
 
+// The residues of modulus i in two rows (sets S and E; row even) or four of a column of the patch (see ResidueTiling) as the numbers that are
+// stored: two 16-bit halves, or four bytes
+template <int SET>
+__device__ __forceinline__ uint32_t stored_rows(const unsigned char *patch, int i, uint32_t column, uint32_t row)
+{
+    const unsigned char *src = patch + stored_start(SET, i);
+    const int form = stored_form(SET, i);
+    const uint32_t word = (row & 7u) >> 1, half = (row >> 2) & 2u;                // word of the chunk; its lower or upper two bytes
+    const unsigned char *low = src + ((row >> 4) * 32 + column) * 16 + word * 4;
+    if (residue_bytes(SET) == 1) return *reinterpret_cast<const uint32_t *>(low);
+    if (form == kStoredPair) return *reinterpret_cast<const uint32_t *>(src + ((row >> 3) * 32 + column) * 16 + (row & 7u) * 2);
+    const uint32_t two = *reinterpret_cast<const uint16_t *>(low + half);
+    uint32_t high = 0u;
+    if (form == kStoredTen)
+        high = (*reinterpret_cast<const uint32_t *>(src + 2048 + column * 16 + (row >> 4) * 4) >> (2 * word + 8 * half)) & 0x0303u;
+    return __byte_perm(two, high, 0x5140);
+}
+
 template <int SET>
 __global__ void __launch_bounds__(128)
 reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int tn0, int ntn, int tiles_m,
@@ -252,30 +270,32 @@ reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int 
         const uint32_t tm = static_cast<uint32_t>(tile / ntn);
         const uint32_t w_idx = piece * 128u + t;
         const uint32_t lane = (w_idx >> 2) & 31u, sub = w_idx & 3u;
-        const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + piece * (16 / RB) + sub * ROWS;
+        // the thread's rows: row, row + 1 and, of set A, row + 8, row + 9
+        const uint32_t row0 = piece * (16 / RB) + sub * 2;
+        const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + row0;
+        auto row_of = [](int h) { return (h & 1) + 8 * (h >> 1); };
         const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
         const bool valid = row < m && j < n && j >= col0 && j < col1;
         const int64_t wb = ((static_cast<int64_t>(tm) * tiles_n + tn) * cg + rank) * 16 + wi;
-        const unsigned char *base = static_cast<const unsigned char *>(Rv) + ((wb * r) * kBlockWords + w_idx) * 4;
+        const unsigned char *patch = static_cast<const unsigned char *>(Rv) + wb * patch_bytes(SET);
         uint32_t w[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-            w[i] = (i < r && valid) ? *reinterpret_cast<const uint32_t *>(base + i * (kBlockWords * 4)) : 0u;
+        for (int i = 0; i < 16; ++i) w[i] = (i < r && valid) ? stored_rows<SET>(patch, i, lane, row0) : 0u;
         // old values of C and the shifts travel while the tensor core works
-        const int nrows = valid ? (m - row < ROWS ? static_cast<int>(m - row) : ROWS) : 0;
-        const bool whole = vecC != 0 && nrows == ROWS;
+        const int64_t left = valid ? m - row : 0;
+        const bool whole = vecC != 0 && left > row_of(ROWS - 1);
         double *out = C + row + j * ldc;
         double2 old[ROWS / 2];
 #pragma unroll
         for (int h = 0; h < ROWS / 2; ++h) old[h] = make_double2(0.0, 0.0);
         if (whole && beta != 0.0) {
 #pragma unroll
-            for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + 2 * h);
+            for (int h = 0; h < ROWS / 2; ++h) old[h] = *reinterpret_cast<const double2 *>(out + 8 * h);
         }
         const int sb = valid ? shiftB[j] : 0;
         int sa[ROWS];
 #pragma unroll
-        for (int h = 0; h < ROWS; ++h) sa[h] = h < nrows ? shiftA[row + h] : 0;
+        for (int h = 0; h < ROWS; ++h) sa[h] = row_of(h) < left ? shiftA[row + row_of(h)] : 0;
 
         // ---- this thread's ROWS outputs as rows t of the ROWS operand tiles
 #pragma unroll
@@ -341,11 +361,11 @@ reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int 
         if (whole) {
 #pragma unroll
             for (int h = 0; h < ROWS / 2; ++h)
-                *reinterpret_cast<double2 *>(out + 2 * h) = make_double2(old[h].x + val[2 * h], old[h].y + val[2 * h + 1]);
+                *reinterpret_cast<double2 *>(out + 8 * h) = make_double2(old[h].x + val[2 * h], old[h].y + val[2 * h + 1]);
         } else {
 #pragma unroll
             for (int h = 0; h < ROWS; ++h)
-                if (h < nrows) out[h] = beta != 0.0 ? out[h] + val[h] : val[h];
+                if (row_of(h) < left) out[row_of(h)] = beta != 0.0 ? out[row_of(h)] + val[h] : val[h];
         }
         // the next step's products overwrite the accumulators: every thread has read its rows
     }
@@ -386,7 +406,7 @@ oz_status_t upload_hosted_constants()
                     else if (byte) return OZ_ERR_UNSUPPORTED;     // would need a seventeenth position
                 }
             }
-            cmax_sum += rb == 2 ? 2 * mi : mi;             // two-byte sets store a representative below 2 m_i
+            cmax_sum += stored_form(set, i) == kStoredByte ? 255 : stored_form(set, i) == kStoredTen ? 1023 : 2 * mi;
         }
         for (int i = 0; i < 4; ++i) {
             K.M[i] = static_cast<uint32_t>(M >> (32 * i));

@@ -64,3 +64,36 @@ def test_marks_and_far_shifts(set_name):
                 sign = -1.0 if xs[j][i] < 0 else 1.0
                 want = sign * np.inf if s < -2000 else 0.0 if s > 2000 else float(xs[j][i]) * 2.0 ** -s if s < 1000 else np.ldexp(float(xs[j][i]), -s)
                 assert got[i, j] == want, (int(sA[i]), int(sB[j]))
+
+
+@pytest.mark.parametrize("set_name,sub,recon", [("S", "fp8", None), ("S", "int8", None), ("E", "fp8", None), ("E", "int8", None), ("A", "fp8", None),
+                                                ("A", "int8", None), ("A", "int8n", None), ("S", "fp8", "tensor"), ("E", "int8", "tensor")])
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (63, 31, 5), (64, 32, 40), (65, 33, 64), (80, 129, 17), (257, 65, 96), (1200, 1090, 33)])
+def test_stored_forms_and_small_results(set_name, sub, recon, m, n, k):
+    """Residues of every stored form through edges of patches (32 columns x 64 rows, chunks of sixteen) and more patches than the blocks of a round:
+    outputs that are zero, that cancel almost to nothing, whose integers span the range of a row, and ordinary ones."""
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m * 7 + n * 3 + k)
+    A = rng.standard_normal((m, k))
+    B = rng.standard_normal((k, n))
+    A[::5, : k // 2] = 0.0                            # rows and columns that share no index: products that are zero
+    B[k // 2:, ::3] = 0.0
+    A[::7] = np.round(A[::7] * 4.0)                   # integers, many results equal or zero
+    if k > 1:
+        A[1::11, 1] = A[1::11, 0]                     # cancels to 2^-40 of the terms
+        B[1, 1::6] = -B[0, 1::6] * (1.0 + 2.0 ** -40)
+        A[1::11, 2:] = 0.0
+    B[:, 2::13] *= 2.0 ** rng.integers(-70, 1, size=B[:, 2::13].shape).astype(np.float64)
+    for alpha, beta, pad in ((1.0, 0.0, 0), (-1.0, 1.0, 0), (-1.0, 1.0, 1), (-1.0, 0.0, 1)):
+        C0 = np.asfortranarray(rng.standard_normal((m, n)))
+        rt = gh.route(sub, recon=recon)
+        gh.ensure_workspace(oz.oz_workspace_bytes(m, n, k, gh.SETS[set_name], rt))
+        Af, Bf = np.asfortranarray(A), np.asfortranarray(B)
+        Cp = np.asfortranarray(np.vstack([C0, np.full((pad + m % 2, n), 3.0)]))       # even and odd leading dimensions
+        dC = gh.to_dev(Cp)
+        oz.check(oz.oz_dgemm_ex(m, n, k, alpha, gh.to_dev(Af), m, gh.to_dev(Bf), k, beta, dC, Cp.shape[0], gh.SETS[set_name], rt), "oz_dgemm_ex")
+        assert gh.sync_status() == 0
+        got = gh.from_dev(dC)
+        want = ozo.dgemm(Af, Bf, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS, alpha=alpha, beta=beta, C0=C0)
+        assert (got[:m] == want).all() and (got[m:] == 3.0).all()
