@@ -11,22 +11,25 @@
 // emulated rows.  C(i,j) = alpha P (beta = 0) or C(i,j) + alpha P (beta = 1) from the caller's old
 // C: the reconstruction leaves the re-issued rows untouched.
 //
-// Work distribution: the re-issued rows come as an ascending list whose length only the device knows.  Resident
-// blocks (two per SM) walk tiles of S x S outputs, S = 32 (2 x 2 a thread) or 16 (one a thread), chosen from the
-// length by small_tiles().  1024 / S inner indices are staged in shared memory at a time and the next ones
-// are requested before the arithmetic.  Bound: the FP64 pipe, ten instructions per multiply-add, 0.88 of it
-// when every row is re-issued (3000 x 3000 x 1500: 8.56 ms; 8.53 with 64 x 64 tiles in one pass over the grid).  With few
-// rows those tiles left most SMs idle; now 60 of 2003 rows x 1999 x 1501 take 0.20 instead of 0.71 ms, 85 of
-// 3000 rows x 3000 x 3000 0.60 instead of 1.39, 3 of 300 rows x 300 x 3000 0.13 instead of 1.35.
+// Work distribution: the re-issued rows come as an ascending list whose length only the device knows.  Two resident
+// blocks an SM walk tiles of 32 x 32 outputs (2 x 2 a thread), or each half of a block by itself tiles of 8 x 16 (one a thread), chosen
+// from the length by small_tiles().  The next inner indices are on their way while a stage is worked on, of small tiles two stages of 64 (the gathered
+// rows come from as many DRAM pages: with 32 indices a stage 10 of 2500 rows x 900 x 2500 took 614 us a call instead of 399).  Bound: the FP64 pipe, ten
+// instructions of two cycles per multiply-add and warp.  Against tiles of 16 x 16 that a whole block took, in whole rounds: 3 of 300 rows x 300 x 3000
+// 247 -> 139 us a call, 700 rows x 40 x 2000 160 -> 112, 60 of 2003 x 1999 x 1501 495 -> 463.
 #include "oz_internal.h"
 
 namespace oz {
 namespace {
 
 constexpr int kFbThreads = 256, kFbBlocksPerSm = 2;
-constexpr int kFbStage = 1024;                   // elements of each operand per stage
-constexpr int kFbStageDoubles = 64 * (16 + 2);   // one staged operand: the larger of (1024 / S) (S + 2)
-static_assert(32 * (32 + 2) <= kFbStageDoubles, "stage size");
+constexpr int kLargeStage = 32, kSmallStage = 64;       // inner indices per stage
+constexpr int kLarge = 32;                       // rows and columns of a large tile
+constexpr int kSmallRows = 8, kSmallCols = 16;   // of a small one
+constexpr int kLargeRow = kLarge + 2;            // doubles per staged index of a large tile: rows stay 16-byte aligned
+constexpr int kSmallLine = kSmallStage + 2;         // doubles per staged line of a small tile: two indices in one load, no bank conflicts
+constexpr int kSmallDoubles = 3 * (kSmallRows + kSmallCols) * kSmallLine;       // three stages of a half block
+constexpr int kFbSharedDoubles = 2 * kLargeStage * kLargeRow > 2 * kSmallDoubles ? 2 * kLargeStage * kLargeRow : 2 * kSmallDoubles;
 
 struct NativeParams {
     int64_t m, n, k, lda, ldb, ldc;
@@ -38,22 +41,30 @@ struct NativeParams {
     double *C;
 };
 
-// A round of 32 x 32 tiles over the resident blocks takes 0.20 us per inner index whether one or both blocks of an
-// SM have a tile (the chains of dependent additions bound it), a round of 16 x 16 tiles 0.066 us: the smaller tiles
-// win while their rounds are fewer than three times those of the larger.
-__device__ __forceinline__ bool small_tiles(int64_t rows, int64_t n, int64_t slots)
+// one multiply-add of an entry: acc + a b with the rounding errors of both operations collected in comp
+__device__ __forceinline__ void native_step(double a, double b, double &acc, double &comp)
 {
-    const int64_t tiles32 = ((rows + 31) / 32) * ((n + 31) / 32), tiles16 = ((rows + 15) / 16) * ((n + 15) / 16);
-    return (tiles16 + slots - 1) / slots < 3 * ((tiles32 + slots - 1) / slots);
+    const double q = __dmul_rn(a, b);
+    const double qe = __fma_rn(a, b, -q);
+    const double s = __dadd_rn(acc, q);
+    const double bb = __dsub_rn(s, acc);
+    const double se = __dadd_rn(__dsub_rn(acc, __dsub_rn(s, bb)), __dsub_rn(q, bb));
+    comp = __dadd_rn(comp, __dadd_rn(qe, se));
+    acc = s;
 }
 
-template <int S>
-__device__ __forceinline__ void native_tiles(const NativeParams &p, int64_t rows, double *As, double *Bs, int64_t *row_of)
+__device__ __forceinline__ void native_store(const NativeParams &p, int64_t row, int64_t j, double acc, double comp)
 {
-    constexpr int T = S / 16;                    // outputs of a thread per direction
-    constexpr int K = kFbStage / S;              // inner indices per stage
-    constexpr int kUnroll = T == 1 ? 16 : 8;      // keeps several inner indices' chains in flight
-    constexpr int P = S + 2;                     // doubles per staged index: rows stay 16-byte aligned
+    const double v = p.shiftB[j] == OZ_NONFINITE_SHIFT ? __longlong_as_double(0x7FF8000000000000ll) : __dadd_rn(acc, comp);
+    double *out = p.C + row + j * p.ldc;
+    const double x = __dmul_rn(p.alpha, v);
+    *out = p.beta != 0.0 ? __dadd_rn(*out, x) : x;
+}
+
+__device__ __forceinline__ void native_large(const NativeParams &p, int64_t rows, double *shared, int64_t *row_of)
+{
+    constexpr int S = kLarge, T = 2, K = kLargeStage, P = kLargeRow;
+    double *As = shared, *Bs = shared + K * P;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int64_t tcols = (p.n + S - 1) / S, tiles = tcols * ((rows + S - 1) / S);
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -93,53 +104,108 @@ __device__ __forceinline__ void native_tiles(const NativeParams &p, int64_t rows
             }
             __syncthreads();
             if (k0 + K < p.k) request(k0 + K);
-#pragma unroll kUnroll
+#pragma unroll 8
             for (int kk = 0; kk < kn; ++kk) {
-                double a[T], b[T];
-                if constexpr (T == 1) {
-                    a[0] = As[kk * P + ty];
-                    b[0] = Bs[kk * P + tx];
-                } else {
-#pragma unroll
-                    for (int h = 0; h < T; h += 2) {
-                        const double2 a2 = *reinterpret_cast<const double2 *>(As + kk * P + ty * T + h);
-                        const double2 b2 = *reinterpret_cast<const double2 *>(Bs + kk * P + tx * T + h);
-                        a[h] = a2.x; a[h + 1] = a2.y;
-                        b[h] = b2.x; b[h + 1] = b2.y;
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < T; ++r)
-#pragma unroll
-                    for (int c = 0; c < T; ++c) {
-                        const double q = __dmul_rn(a[r], b[c]);
-                        const double qe = __fma_rn(a[r], b[c], -q);
-                        const double s = __dadd_rn(acc[r][c], q);
-                        const double bb = __dsub_rn(s, acc[r][c]);
-                        const double se = __dadd_rn(__dsub_rn(acc[r][c], __dsub_rn(s, bb)), __dsub_rn(q, bb));
-                        comp[r][c] = __dadd_rn(comp[r][c], __dadd_rn(qe, se));
-                        acc[r][c] = s;
-                    }
+                const double2 a = *reinterpret_cast<const double2 *>(As + kk * P + ty * T);
+                const double2 b = *reinterpret_cast<const double2 *>(Bs + kk * P + tx * T);
+                native_step(a.x, b.x, acc[0][0], comp[0][0]);
+                native_step(a.x, b.y, acc[0][1], comp[0][1]);
+                native_step(a.y, b.x, acc[1][0], comp[1][0]);
+                native_step(a.y, b.y, acc[1][1], comp[1][1]);
             }
         }
-
-        const double nan = __longlong_as_double(0x7FF8000000000000ll);
 #pragma unroll
         for (int c = 0; c < T; ++c) {
             const int64_t j = c0 + tx * T + c;
             if (j >= p.n) continue;
-            const bool bad = p.shiftB[j] == OZ_NONFINITE_SHIFT;
 #pragma unroll
-            for (int r = 0; r < T; ++r) {
-                const int64_t row = row_of[ty * T + r];
-                if (row < 0) continue;
-                const double v = bad ? nan : __dadd_rn(acc[r][c], comp[r][c]);
-                double *out = p.C + row + j * p.ldc;
-                const double x = __dmul_rn(p.alpha, v);
-                *out = p.beta != 0.0 ? __dadd_rn(*out, x) : x;
-            }
+            for (int r = 0; r < T; ++r)
+                if (row_of[ty * T + r] >= 0) native_store(p, row_of[ty * T + r], j, acc[r][c], comp[r][c]);
         }
     }
+}
+
+extern __shared__ __align__(16) double fb_shared[];
+
+// half: this half of the block's number; it keeps its own barrier and shared memory.  (Out of line: inlined it costs the large tiles 2 percent.)
+__device__ __noinline__ void native_small(const NativeParams &p, int64_t rows, int half)
+{
+    double *shared = fb_shared + half * kSmallDoubles;
+    constexpr int K = kSmallStage, L = kSmallLine, kStage = (kSmallRows + kSmallCols) * L;
+    const int tid = threadIdx.x & 127, tx = tid & 15, ty = tid >> 4;
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(shared));
+    const int64_t tcols = (p.n + kSmallCols - 1) / kSmallCols, tiles = tcols * ((rows + kSmallRows - 1) / kSmallRows);
+    auto sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(half + 1) : "memory"); };
+    const int nk = static_cast<int>((p.k + K - 1) / K);
+    for (int64_t t = blockIdx.x + static_cast<int64_t>(half) * gridDim.x; t < tiles; t += 2 * gridDim.x) {      // few tiles: one to an SM
+        const int64_t r0 = t / tcols * kSmallRows, c0 = (t - t / tcols * tcols) * kSmallCols;
+        // Copies: a thread takes four indices of one row of A (consecutive threads consecutive rows) and one index of eight columns of B.  Rows and columns
+        // behind the last one repeat it and are not stored; indices behind k are not read.
+        const int ar = tid & 7, ak = tid >> 3, bk = tid & 63, bc = tid >> 6;
+        const double *a_next = p.A + p.list[r0 + ar < rows ? r0 + ar : rows - 1] + ak * p.lda;
+        const double *b_next = p.B + bk;
+        int64_t b_off[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) b_off[u] = (c0 + bc + 2 * u < p.n ? c0 + bc + 2 * u : p.n - 1) * p.ldb;
+        const uint32_t a_dst = base + static_cast<uint32_t>(ar * L + ak) * 8, b_dst = base + static_cast<uint32_t>((kSmallRows + bc) * L + bk) * 8;
+        auto copy = [](uint32_t dst, const double *src, bool in) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
+        };
+        auto request = [&](int stage, int left) {       // left: indices from this stage's first one to k
+            const uint32_t off = static_cast<uint32_t>(stage * kStage) * 8;
+            if (left >= K) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) copy(a_dst + off + 128 * u, a_next + 16 * u * p.lda, true);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) copy(b_dst + off + 2 * L * 8 * u, b_next + b_off[u], true);
+            } else {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) copy(a_dst + off + 128 * u, ak + 16 * u < left ? a_next + 16 * u * p.lda : p.A, ak + 16 * u < left);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) copy(b_dst + off + 2 * L * 8 * u, bk < left ? b_next + b_off[u] : p.B, bk < left);
+            }
+            a_next += K * p.lda;
+            b_next += K;
+        };
+        double acc = 0.0, comp = 0.0;
+        const int k = static_cast<int>(p.k);
+        request(0, k);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (nk > 1) request(1, k - K);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        int stage = 0;
+        for (int i = 0; i < nk; ++i) {
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            sync();                              // this stage is there, and the one before it has been read
+            if (i + 2 < nk) request(stage == 0 ? 2 : stage - 1, k - (i + 2) * K);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            const double *As = shared + stage * kStage + ty * L, *Bs = shared + stage * kStage + (kSmallRows + tx) * L;
+            const int kn = k - i * K < K ? k - i * K : K;
+            if (kn == K) {
+#pragma unroll 8
+                for (int kk = 0; kk < K; kk += 2) {
+                    const double2 a = *reinterpret_cast<const double2 *>(As + kk), b = *reinterpret_cast<const double2 *>(Bs + kk);
+                    native_step(a.x, b.x, acc, comp);
+                    native_step(a.y, b.y, acc, comp);
+                }
+            } else {
+                for (int kk = 0; kk < kn; ++kk) native_step(As[kk], Bs[kk], acc, comp);
+            }
+            if (++stage == 3) stage = 0;
+        }
+        if (r0 + ty < rows && c0 + tx < p.n) native_store(p, p.list[r0 + ty], c0 + tx, acc, comp);
+        sync();                                  // the stages may be filled again
+    }
+}
+
+// Small tiles while they cost less: a tile of 8 x 16 takes an SM 27.5 cycles an inner index next to others, a round of 32 x 32 tiles over the resident
+// blocks 380, whether one or both blocks of an SM have a tile.  85 of 3000 rows x 3000 x 3000: 1648 us a call with the small ones, 1588 with the large, whose
+// one round is nearly full; 594 of 600 x 3000 x 300: 474 and 500; 60 of 2003 x 1999 x 1501: 461 and 580; 8000 x 8000 x 1500, every row: 68.1 and 63.8 ms.
+__device__ __forceinline__ bool small_tiles(int64_t rows, int64_t n, int64_t sms)
+{
+    const int64_t large = ((rows + kLarge - 1) / kLarge) * ((n + kLarge - 1) / kLarge), slots = kFbBlocksPerSm * sms;
+    const int64_t small = ((rows + kSmallRows - 1) / kSmallRows) * ((n + kSmallCols - 1) / kSmallCols);
+    return 55 * ((small + sms - 1) / sms) < 760 * ((large + slots - 1) / slots);
 }
 
 __global__ void __launch_bounds__(kFbThreads, kFbBlocksPerSm)
@@ -149,11 +215,9 @@ native_rows_kernel(const __grid_constant__ NativeParams p, int sms)
     dependency_wait();
     const int64_t rows = *p.count;
     if (rows == 0) return;
-    __shared__ __align__(16) double As[kFbStageDoubles];
-    __shared__ __align__(16) double Bs[kFbStageDoubles];
-    __shared__ int64_t row_of[32];
-    if (small_tiles(rows, p.n, static_cast<int64_t>(kFbBlocksPerSm) * sms)) native_tiles<16>(p, rows, As, Bs, row_of);
-    else native_tiles<32>(p, rows, As, Bs, row_of);
+    __shared__ int64_t row_of[kLarge];
+    if (small_tiles(rows, p.n, sms)) native_small(p, rows, static_cast<int>(threadIdx.x >> 7));
+    else native_large(p, rows, fb_shared, row_of);
 }
 
 }  // namespace
@@ -168,8 +232,11 @@ oz_status_t launch_native_rows(int64_t m, int64_t n, int64_t k, const double *A,
     const int sms = sm_count();
     NativeParams p{m, n, k, lda, ldb, ldc, A, B, list, count, shiftB, alpha, beta, C};
     // as many blocks as are resident at once, or fewer where even the smallest tiles are fewer
-    const int64_t most = ((m + 15) / 16) * ((n + 15) / 16), cap = static_cast<int64_t>(kFbBlocksPerSm) * sms;
-    OZ_CUDA_CHECK(launch(native_rows_kernel, dim3(static_cast<unsigned>(most < cap ? most : cap)), kFbThreads, 0, stream, p, sms));
+    const int64_t most = ((m + kSmallRows - 1) / kSmallRows) * ((n + kSmallCols - 1) / kSmallCols), cap = static_cast<int64_t>(kFbBlocksPerSm) * sms;
+    constexpr size_t shared = kFbSharedDoubles * sizeof(double);
+    static std::atomic<unsigned long long> ready{0};
+    OZ_CUDA_CHECK(allow_shared(native_rows_kernel, shared, ready));
+    OZ_CUDA_CHECK(launch(native_rows_kernel, dim3(static_cast<unsigned>(most < cap ? most : cap)), kFbThreads, shared, stream, p, sms));
     count_launch();
     OZ_CUDA_CHECK(cudaGetLastError());
     return OZ_OK;

@@ -170,3 +170,31 @@ def test_native_rows_tiles(m, n, k, sigma):
     want, flag = ozo.dgemm_fallback(A, B, ozo.SET_S, ozo.QUANT_RN, -1.0, 1.0, C0)
     assert st == 0 and oz.oz_query_fallback_rows() == int(flag.sum()) and flag.mean() > 0.9
     assert (got == want).all()
+
+
+@pytest.mark.parametrize("rows", [1, 8, 9, 17])
+@pytest.mark.parametrize("n,k", [(1, 64), (15, 63), (16, 65), (17, 129), (40, 193)])
+def test_native_tiles_and_stages(rows, n, k):
+    """Edges of the native path's small tiles (8 rows x 16 columns, stages of 64 indices, three of them): a few badly scaled
+    rows among flat ones, scattered."""
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(100 * rows + n + k)
+    m = 3 * rows + 2
+    A, B = np.asfortranarray(rng.choice([-1.0, 1.0], (m, k))), np.asfortranarray(rng.choice([-1.0, 1.0], (k, n)) * (1.0 + rng.random((k, n))))
+    A[1:3 * rows:3] = np.exp(6.0 * rng.standard_normal((rows, k))) * rng.standard_normal((rows, k))
+    C0 = np.asfortranarray(rng.standard_normal((m, n)))
+    got, st = gh.dgemm(A, B, "S", gh.route("fp8", fallback=True), -1.0, 1.0, C0)
+    want, flag = ozo.dgemm_fallback(A, B, ozo.SET_S, ozo.QUANT_RN, -1.0, 1.0, C0)
+    assert st == 0 and (rows == 1 or flag.sum() >= rows // 2)
+    assert (got == want).all()
+
+
+def test_native_large_tiles():
+    """Every row re-issued on tiles of 32 x 32: one round of them over the resident blocks, which the small tiles do not undercut."""
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(5)
+    A, B = _wide(rng, 511, 65, 3.0), _wide(rng, 65, 575, 3.0)
+    got, st = gh.dgemm(A, B, "S", gh.route("fp8", fallback=True))
+    want, flag = ozo.dgemm_fallback(A, B, ozo.SET_S, ozo.QUANT_RN)
+    assert st == 0 and flag.sum() >= 505
+    assert (got == want).all()
