@@ -180,10 +180,6 @@ constexpr ReconConst recon_constants()
 }
 __constant__ ReconConst c_recon[kNumSets] = {recon_constants<0>(), recon_constants<1>(), recon_constants<2>()};
 
-// Threads of a block of the private layout's kernel: one warp for each chunk of sixteen rows and, of two rows a thread, each half of it; eight columns.  1024
-// threads on an SM: numbers, sums and old values of C take 64 registers.  16384 x 16384 update, set S, in blocks of 256 threads 1709 us, of 128
-// 1611 us, the same with 896 threads on an SM (72 registers), 1893 with 1152 (56, spills).
-__host__ __device__ constexpr int tiled_threads(int rows) { return rows == 4 ? 128 : 256; }
 // Up to this many outputs two rows a thread (from 1200 x 1200 on four are faster): 512 x 512 on set S 23.7 us a call, with four rows 25.7; 700 x 700 x 300 29.3 and 30.6.
 constexpr int64_t kFewOutputs = 700000;
 // Public layout: blocks of 128 threads, nine an SM with two rows a thread (56 registers).  6000 x 6000 update, set E, with 8 / 9 / 10: 288 / 274 / 281 us
@@ -281,40 +277,49 @@ struct PublicLoader {
     int64_t stride;                  // bytes from modulus to modulus
     int nrows;
     bool words;                      // one 32-bit load covers the rows
-    __device__ __forceinline__ void load(Numbers &w) const
+    template <int I>
+    __device__ __forceinline__ void load_one(Numbers &w) const
     {
         constexpr int RB = residue_bytes(SET), ROWS = 4 / RB;
+        w.hi[I] = 0u;
+        const unsigned char *src = base + I * stride;
+        if (words) {
+            w.lo[I] = *reinterpret_cast<const uint32_t *>(src);        // ldr is a multiple of ROWS: in bounds
+        } else {
+            uint32_t v = 0;
 #pragma unroll
-        for (int i = 0; i < set_r(SET); ++i) {
-            w.hi[i] = 0u;
-            const unsigned char *src = base + i * stride;
-            if (words) {
-                w.lo[i] = *reinterpret_cast<const uint32_t *>(src);    // ldr is a multiple of ROWS: in bounds
-            } else {
-                uint32_t v = 0;
-#pragma unroll
-                for (int h = 0; h < ROWS; ++h) {
-                    if (h < nrows) {
-                        uint32_t e = RB == 2 ? reinterpret_cast<const uint16_t *>(src)[h] : src[h];
-                        v |= e << (8 * RB * h);
-                    }
+            for (int h = 0; h < ROWS; ++h) {
+                if (h < nrows) {
+                    uint32_t e = RB == 2 ? reinterpret_cast<const uint16_t *>(src)[h] : src[h];
+                    v |= e << (8 * RB * h);
                 }
-                w.lo[i] = v;
             }
+            w.lo[I] = v;
         }
     }
+    template <int I> __device__ __forceinline__ void finish_one(Numbers &) const {}
 };
 
-// From a patch of the private array: chunk c, column, word of the chunk; of two rows a thread, the half of the word
-template <int SET, int ROWS>
+// Threads of a block of the private layout's kernel: one warp for each chunk of sixteen rows and, of two rows a thread, each half of it; eight columns.  1024
+// threads on an SM: numbers, sums and old values of C take 64 registers.  16384 x 16384 update, set S, in blocks of 256 threads 1709 us, of 128
+// 1611 us, the same with 896 threads on an SM (72 registers), 1893 with 1152 (56, spills).
+__host__ __device__ constexpr int tiled_threads(int rows) { return rows == 4 ? 128 : 256; }
+constexpr int kPieces = 4;             // thread blocks to a patch
+
+// From a patch of the private array: chunk, column, word of the chunk; of two rows a thread, the half of the word.  Where a thread stands follows from its number.
+template <int SET, int ROWS, bool SPREAD>
 struct PatchLoader {
     static constexpr bool kPrivate = true;
     const unsigned char *patch;
-    uint32_t c, column, word, half;
+    static __device__ __forceinline__ uint32_t chunk() { return SPREAD ? (threadIdx.x >> 5) & 3u : (threadIdx.x >> 2) & 3u; }
+    static __device__ __forceinline__ uint32_t half_word() { return ROWS == 4 ? 0u : SPREAD ? threadIdx.x >> 7 : (threadIdx.x >> 4) & 1u; }
+    static __device__ __forceinline__ uint32_t column_of() { return blockIdx.x % kPieces * 8 + (SPREAD ? (threadIdx.x >> 2) & 7u : threadIdx.x / (64 / ROWS)); }
+    static __device__ __forceinline__ uint32_t word_of() { return threadIdx.x & 3u; }
     template <int I>
-    __device__ __forceinline__ void load_modulus(Numbers &w) const
+    __device__ __forceinline__ void load_one(Numbers &w) const
     {
         constexpr int form = stored_form(SET, I);
+        const uint32_t c = chunk(), half = half_word(), column = column_of(), word = word_of();
         const unsigned char *src = patch + stored_start(SET, I);           // a compile-time offset from one address
         w.hi[I] = 0u;
         if constexpr (form == kStoredPair) {
@@ -326,38 +331,49 @@ struct PatchLoader {
         }
     }
     template <int I>
-    __device__ __forceinline__ void own_rows(Numbers &w) const
+    __device__ __forceinline__ void finish_one(Numbers &w) const       // the thread's rows of what was loaded
     {
-        const uint32_t skip = ROWS == 2 ? 16 * half : 0u;
+        const uint32_t skip = 16 * half_word(), word = word_of();
         if constexpr (stored_form(SET, I) == kStoredTen) w.hi[I] = (w.hi[I] >> (2 * word + skip)) & 0x03030303u;        // the thread's bits
         if constexpr (stored_form(SET, I) != kStoredPair && ROWS == 2) w.lo[I] >>= skip;
     }
-    template <int... I>
-    __device__ __forceinline__ void load_all(std::integer_sequence<int, I...>, Numbers &w) const
-    {
-        (load_modulus<I>(w), ...);
-        (own_rows<I>(w), ...);
-    }
-    __device__ __forceinline__ void load(Numbers &w) const { load_all(std::make_integer_sequence<int, set_r(SET)>{}, w); }
 };
 
-// u_g where every residue is zero and stands there as 0 or as m
-template <int SET>
-__host__ __device__ constexpr int64_t group_of_moduli(int g)
+template <class Loader, int... I>
+__device__ __forceinline__ void load_numbers(std::integer_sequence<int, I...>, const Loader &from, Numbers &w)
 {
-    int64_t u = 0;
-    for (int e = 0; e < 3; ++e)
-        if (group_member(SET, g, e) >= 0) u += modulus(SET, group_member(SET, g, e)) % 1024 * member_weight(SET, g, e);
-    return u;
+    (from.template load_one<I>(w), ...);
+    (from.template finish_one<I>(w), ...);
 }
-template <int SET, bool MODULI>
-__device__ __forceinline__ bool no_residue(const int (&u)[kMaxGroups])
+
+// row h, no compile-time constant here, in the place of the first one
+template <int SET, bool PRIVATE>
+__device__ __forceinline__ void first_row(Numbers &w, int h)
 {
-    bool zero = u[0] == (MODULI ? static_cast<int>(group_of_moduli<SET>(0)) : 0);
-    zero = zero && u[1] == (MODULI ? static_cast<int>(group_of_moduli<SET>(1)) : 0) && u[2] == (MODULI ? static_cast<int>(group_of_moduli<SET>(2)) : 0) &&
-           u[3] == (MODULI ? static_cast<int>(group_of_moduli<SET>(3)) : 0) && u[4] == (MODULI ? static_cast<int>(group_of_moduli<SET>(4)) : 0);
-    if constexpr (set_groups(SET) == 6) zero = zero && u[5] == (MODULI ? static_cast<int>(group_of_moduli<SET>(5)) : 0);
-    return zero;
+#pragma unroll
+    for (int i = 0; i < set_r(SET); ++i) {
+        if (PRIVATE ? stored_form(SET, i) == kStoredPair : residue_bytes(SET) == 2) {
+            w.lo[i] = (h < 2 ? w.lo[i] : w.hi[i]) >> (16 * (h & 1));
+        } else {
+            w.lo[i] >>= 8 * h;
+            w.hi[i] >>= 8 * h;
+        }
+    }
+}
+
+// The thread's rows (bit h) whose c' is zero if it is below 2^(kRestErrorLog2 + 3) in magnitude: products with structural zeros have many.  It is zero where
+// the products of two groups, together larger than that, divide it.
+template <int SET, int ROWS, class Loader, int... H>
+__device__ __noinline__ uint32_t zero_rows(std::integer_sequence<int, H...>, Loader from)
+{
+    constexpr int64_t P0 = static_cast<int64_t>(group_product(SET, 0)), P1 = static_cast<int64_t>(group_product(SET, 1));
+    static_assert(static_cast<double>(P0) * static_cast<double>(P1) > pow2d(kRestErrorLog2<SET> + 4), "two groups tell");
+    constexpr int a2 = group_member(SET, 0, 2), b2 = group_member(SET, 1, 2);
+    Numbers w = {};
+    load_numbers(std::integer_sequence<int, group_member(SET, 0, 0), group_member(SET, 0, 1), group_member(SET, 1, 0), group_member(SET, 1, 1)>{}, from, w);
+    if constexpr (a2 >= 0) load_numbers(std::integer_sequence<int, a2>{}, from, w);
+    if constexpr (b2 >= 0) load_numbers(std::integer_sequence<int, b2>{}, from, w);
+    return ((group_value<SET, Loader::kPrivate, H, 0>(w) % static_cast<int>(P0) == 0 && group_value<SET, Loader::kPrivate, H, 1>(w) % static_cast<int>(P1) == 0 ? 1u << H : 0u) | ...);
 }
 
 // alpha 2^-(sa + sb) c' (alpha = 1 or -1, as a sign bit) where only the scale is out of reach: r is c' correctly rounded.  NaN for a line with
@@ -383,20 +399,10 @@ __device__ __noinline__ double row_value_exact(Loader from, int h, int sa, int s
     const double alpha = __hiloint2double(0x3FF00000 ^ alpha_sign, 0);
     if (marked(sa, sb)) return __longlong_as_double(0x7FF8000000000000ll) * alpha;
     Numbers w;
-    from.load(w);
-    // row h in the place of the first one
-#pragma unroll
-    for (int i = 0; i < set_r(SET); ++i) {
-        if (Loader::kPrivate ? stored_form(SET, i) == kStoredPair : residue_bytes(SET) == 2) {
-            w.lo[i] = (h < 2 ? w.lo[i] : w.hi[i]) >> (16 * (h & 1));
-        } else {
-            w.lo[i] >>= 8 * h;
-            w.hi[i] >>= 8 * h;
-        }
-    }
+    load_numbers(std::make_integer_sequence<int, set_r(SET)>{}, from, w);
+    first_row<SET, Loader::kPrivate>(w, h);
     int u[kMaxGroups] = {};
     group_values<SET, Loader::kPrivate, 0>(std::make_integer_sequence<int, set_groups(SET)>{}, w, u);
-    if (no_residue<SET, false>(u) || no_residue<SET, true>(u)) return 0.0 * alpha;       // structural zeros of a product
     constexpr Wide Mw = group_weight(SET, -1);
     const __int128 M = static_cast<__int128>((static_cast<unsigned __int128>(Mw.hi) << 64) | Mw.lo);
     const __int128 Mh = M >> 1;     // M is even for every set (each holds a power of two)
@@ -476,7 +482,7 @@ __device__ __forceinline__ void reconstruct_rows(std::integer_sequence<int, H...
     // all residue loads are issued before any arithmetic: independent requests in flight per
     // thread, kept packed so that they fit the register budget
     Numbers w;
-    from.load(w);
+    load_numbers(std::make_integer_sequence<int, set_r(SET)>{}, from, w);
     int sa[ROWS];
 #pragma unroll
     for (int h = 0; h < ROWS; ++h) sa[h] = row_of<PRIVATE>(h) < nrows ? shiftA[row + row_of<PRIVATE>(h)] : 0;
@@ -507,8 +513,18 @@ __device__ __forceinline__ void reconstruct_rows(std::integer_sequence<int, H...
         all = all && rounded[h];
     }
     if (!(all && far <= 1924u && wide < 1u << 31 && range < kRangeSpan<SET>)) {
+        constexpr uint32_t small = 2u * (static_cast<uint32_t>(1023 + kRestErrorLog2<SET> + 2) << 20);       // |c'| is below twice the bound of |r|
+        uint32_t least = 0xFFFFFFFFu, zeros = 0u;
+#pragma unroll
+        for (int h = 0; h < ROWS; ++h) least = min(least, 2u * static_cast<uint32_t>(__double2hiint(r[h])));
+        if (least < small) zeros = zero_rows<SET, ROWS>(std::integer_sequence<int, H...>{}, from);
         auto fix = [&](auto index) {
             constexpr int h = decltype(index)::value;
+            if (2u * static_cast<uint32_t>(__double2hiint(r[h])) < small && (zeros >> h & 1u) && !marked(sa[h], sb)) {
+                r[h] = 0.0;
+                scale[h] = 0x3FF00000u ^ static_cast<uint32_t>(alpha_sign);
+                return;
+            }
             const bool good = rounded[h] && range_word<SET>(r[h]) < kRangeSpan<SET>;
             const bool near = static_cast<uint32_t>(sa[h]) + static_cast<uint32_t>(sb) + 904u <= 1924u && static_cast<uint32_t>(sa[h]) + (1u << 30) < 1u << 31;
             if (good && near) return;
@@ -578,26 +594,20 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
 {
     dependency_release();
     dependency_wait();
-    constexpr int kColThreads = 64 / ROWS;                 // threads to a column of the patch
-    constexpr int kPieces = 32 * kColThreads / tiled_threads(ROWS);        // thread blocks per patch: 4
-    const uint32_t piece = blockIdx.x % kPieces;
+    constexpr bool spread = ACCESS != kSingleUpdates;
+    using Loader = PatchLoader<SET, ROWS, spread>;
     const uint32_t wi = (blockIdx.x / kPieces) & 15u;
     const uint32_t rank = blockIdx.x / (kPieces * 16);     // 0, or 0..1 with CTA pairs
     const uint32_t tn = static_cast<uint32_t>(tn0) + blockIdx.y, tm = blockIdx.z;
-    const uint32_t warp = threadIdx.x >> 5, sub = threadIdx.x & 3u;
-    constexpr bool spread = ACCESS != kSingleUpdates;
-    const uint32_t c = spread ? warp & 3u : (threadIdx.x >> 2) & 3u;               // four chunks of sixteen rows
-    const uint32_t half = ROWS == 4 ? 0u : spread ? warp >> 2 : (threadIdx.x >> 4) & 1u;
-    const uint32_t lane = piece * 8 + (spread ? (threadIdx.x >> 2) & 7u : threadIdx.x / kColThreads);      // column of the patch
     const uint32_t patch = ((tm * static_cast<uint32_t>(tiles_n) + tn) * static_cast<uint32_t>(cg) + rank) * 16 + wi;
-    if (ahead != 0 && threadIdx.x == 0 && piece == 0) {
+    if (ahead != 0 && threadIdx.x == 0 && blockIdx.x % kPieces == 0) {
         const uint32_t next = patch + ahead;
         if (next < static_cast<uint32_t>(tiles_n) * gridDim.z * static_cast<uint32_t>(cg) * 16)
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
                          ::"l"(static_cast<const unsigned char *>(Rv) + next * static_cast<int64_t>(patch_bytes(SET))), "r"(patch_bytes(SET)) : "memory");
     }
-    const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + c * 16 + half * 8 + sub * 2;
-    const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
+    const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + Loader::chunk() * 16 + Loader::half_word() * 8 + Loader::word_of() * 2;
+    const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + Loader::column_of();
     if (row >= m || j >= n || j < col0 || j >= col1) return;
     const int nrows = m - row < 16 ? static_cast<int>(m - row) : 16;
     uint32_t keep = 0xFu;
@@ -608,7 +618,7 @@ reconstruct_tiled_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int t
             if (row_of<true>(h) < nrows && !skip[row + row_of<true>(h)]) keep |= 1u << h;
         if (!keep) return;
     }
-    const PatchLoader<SET, ROWS> from{static_cast<const unsigned char *>(Rv) + patch * static_cast<int64_t>(patch_bytes(SET)), c, lane, sub, half};
+    const Loader from{static_cast<const unsigned char *>(Rv) + patch * static_cast<int64_t>(patch_bytes(SET))};
     reconstruct_rows<SET, ROWS>(std::make_integer_sequence<int, ROWS>{}, from, row, nrows, shiftB[j], shiftA, alpha, beta, C + row + j * ldc, ACCESS == kPairs, keep);
 }
 
@@ -646,10 +656,9 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     const int ntn = static_cast<int>((col1 + t.tile_cols - 1) / t.tile_cols) - tn0;
     // there the threads of four rows do not fill the chip
     const bool few = m * n <= kFewOutputs;
-    constexpr int pieces = 4;              // thread blocks per patch
     if (t.tiles_m > 65535 || ntn > 65535) return OZ_ERR_UNSUPPORTED;
     const int vecC = ((ldc & 1) == 0 && (reinterpret_cast<uintptr_t>(C) & 15u) == 0) ? 1 : 0;
-    const dim3 grid(static_cast<unsigned>(pieces * 16 * t.cg), static_cast<unsigned>(ntn),
+    const dim3 grid(static_cast<unsigned>(kPieces * 16 * t.cg), static_cast<unsigned>(ntn),
                     static_cast<unsigned>(t.tiles_m));
     // Blocks that become resident beside the GEMM's keep the multiprocessor's memory split at the GEMM's (28 KiB of L1) for
     // the whole kernel: worth the overlapped launch up to a million outputs only (16384 x 16384: 11.4 -> 11.9 ms a call)
@@ -657,7 +666,7 @@ oz_status_t launch_reconstruct_tiled(int64_t m, int64_t n, const void *R, const 
     // one round of resident blocks ahead; not for a panel, whose blocks do not walk the array from end to end
     const int64_t patches = static_cast<int64_t>(t.tiles_m) * t.tiles_n * t.cg * 16;
     if (patches > 0x7FFFFFFFll) return OZ_ERR_UNSUPPORTED;       // as the residue GEMM
-    const uint32_t ahead = ntn == t.tiles_n ? static_cast<uint32_t>(1024 / tiled_threads(few ? 2 : 4) * sm_count() / pieces) : 0u;
+    const uint32_t ahead = ntn == t.tiles_n ? static_cast<uint32_t>(1024 / tiled_threads(few ? 2 : 4) * sm_count() / kPieces) : 0u;
 #define OZ_RECON_KERNEL(SET_, SKIP_, ROWS_)                                             \
     (vecC          ? reconstruct_tiled_kernel<SET_, SKIP_, kPairs, ROWS_>               \
      : beta == 0.0 ? reconstruct_tiled_kernel<SET_, SKIP_, kSingleStores, ROWS_>        \
