@@ -500,7 +500,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         // Accurate mode: exponent scans, one magnitude plane per operand (kept in the first plane slot
         // of each operand, which the conversion overwrites afterwards), the bound product on the
         // tensor cores, the shifts from its row and column maxima, then the conversion as usual.
-        const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
+        const ScanJob ja{m, A, lda, a.shift, a.scratch, nullptr}, jb{n, B, ldb, b.shift, b.scratch, nullptr};
         st = launch_scan(&ja, &jb, k, set, rt, true, stream);
         if (st == OZ_OK) st = launch_bound_planes(ja, a.planes, jb, b.planes, k, a.pitch, stream);
         if (st == OZ_OK)
@@ -523,7 +523,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
         st = launch_deconstruct(1, n, k, B, ldb, set, rt, b.planes, private_planes(n, b.pitch), b.shift, b.scratch, false, side);
         if (st != OZ_OK) return st;
         OZ_CUDA_CHECK(cudaEventRecord(g_join[dev], side));
-        const ScanJob ja{m, A, lda, a.shift, a.scratch};
+        const ScanJob ja{m, A, lda, a.shift, a.scratch, nullptr};      // no planes of A
         st = launch_scan(&ja, nullptr, k, set, rt, false, stream);
         if (st != OZ_OK) return st;
         if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][1], stream));
@@ -543,7 +543,7 @@ oz_status_t dgemm_impl(int64_t m, int64_t n, int64_t k, double alpha, const doub
                                  {n, B, ldb, b.planes, private_planes(n, b.pitch), b.shift, b.scratch}, k, set, rt, &both, stream);
     if (st != OZ_OK) return st;
     if (!both) {
-        const ScanJob ja{m, A, lda, a.shift, a.scratch}, jb{n, B, ldb, b.shift, b.scratch};
+        const ScanJob ja{m, A, lda, a.shift, a.scratch, a.planes}, jb{n, B, ldb, b.shift, b.scratch, b.planes};
         const bool scans = three_passes(0, ja, k, set, rt) && three_passes(1, jb, k, set, rt);
         if (scans) {      // both operands in one launch per pass; the conversions then run side by side
             st = launch_scan(&ja, &jb, k, set, rt, true, stream);

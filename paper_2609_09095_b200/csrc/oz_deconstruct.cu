@@ -74,6 +74,10 @@ __device__ __forceinline__ int classify(double x, int *e)
     return 1;
 }
 
+// ceil(|x| scale), scale a power of two and a normal number.  The product is exact unless it leaves the normal range; rounded up there, a non-zero x
+// counts as 1 however small.
+__device__ __forceinline__ unsigned int magnitude(double x, double scale) { return __double2uint_ru(__dmul_ru(fabs(x), scale)); }
+
 // ceil(|x| 2^(9-E)) in integer arithmetic (lines of subnormals, where 2^(9-E) is no normal double)
 __device__ __forceinline__ unsigned int scaled_magnitude(double x, int E)
 {
@@ -89,6 +93,29 @@ __device__ __forceinline__ unsigned int scaled_magnitude(double x, int E)
     return static_cast<unsigned int>((sig >> sh) + ((sig & ((1ull << sh) - 1ull)) ? 1ull : 0ull));
 }
 
+// The norm sums of a line need its largest exponent, which is known only when the whole line has been read.  So the exponent is guessed low, from a sample
+// of kSamples elements, and the sums are taken for it and the next ones while the line is read for the first time: ceil(|x| 2^(9 - E - 1)) is
+// ceil(ceil(|x| 2^(9 - E)) / 2).  Lines whose exponent lies elsewhere are read again.  These arrays lie in the operand's planes, which the conversion
+// fills later; exponent null: two passes.
+constexpr int kGuesses = 3, kSamples = 32;
+struct ScanGuess {
+    unsigned long long *sumsq;  // [kGuesses][lines]
+    unsigned int *l1;           // [kGuesses][lines]
+    int *exponent;              // [lines]  INT32_MIN: none
+};
+constexpr int kGuessBytes = kGuesses * 12 + 4;       // a line
+__host__ __device__ inline ScanGuess carve_guess(void *spare, int64_t lines)
+{
+    char *base = static_cast<char *>(spare);
+    if (!spare) return {nullptr, nullptr, nullptr};
+    return {reinterpret_cast<unsigned long long *>(base), reinterpret_cast<unsigned int *>(base + 8 * kGuesses * lines),
+            reinterpret_cast<int *>(base + 12 * kGuesses * lines)};
+}
+__device__ __forceinline__ bool guessed(int exponent, int guess)
+{
+    return guess != INT32_MIN && exponent != INT32_MIN && static_cast<unsigned int>(exponent) - static_cast<unsigned int>(guess) < static_cast<unsigned int>(kGuesses);
+}
+
 // One operand of a scan.  lines = 0: none.
 struct ScanSide {
     const double *X;
@@ -97,6 +124,7 @@ struct ScanSide {
     uint32_t line_blocks;       // blocks across the lines
     uint32_t blocks;            // in all
     ScanScratch s;
+    ScanGuess g;
 };
 
 // The scans take one operand or both operands of a product in one launch: blocks [0, a.blocks) serve side 0, the others
@@ -115,7 +143,55 @@ __global__ void scan_init_kernel(ScanScratch sa, int64_t linesA, ScanScratch sb,
     s.nonfinite[i] = 0;
 }
 
-// One pass over the operand.  PASS 0: largest exponent + non-finite flag.  PASS 1: sum of squares.
+// The same and a guess of every line's exponent.  Blocks of 32 lines (side 0) or eight.
+__global__ void __launch_bounds__(256)
+scan_sample_kernel(const __grid_constant__ ScanSide a, const __grid_constant__ ScanSide b, int64_t k)
+{
+    __shared__ unsigned int tops[8][32];
+    dependency_release();
+    dependency_wait();
+    const uint32_t blocksA = static_cast<uint32_t>((a.lines + 31) / 32);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool side = blockIdx.x >= blocksA;
+    const ScanSide &p = side ? b : a;
+    unsigned int top = 0u;
+    int64_t line;
+    if (!side) {
+        line = static_cast<int64_t>(blockIdx.x) * 32 + lane;
+        double x[kSamples / 8];
+#pragma unroll
+        for (int u = 0; u < kSamples / 8; ++u)
+            x[u] = line < p.lines ? p.X[line + (warp * (kSamples / 8) + u) * k / kSamples * p.ldx] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kSamples / 8; ++u) top = max(top, static_cast<unsigned int>(__double2hiint(x[u])) & 0x7FFFFFFFu);
+        tops[warp][lane] = top;
+        __syncthreads();
+        if (warp != 0) return;
+#pragma unroll
+        for (int w = 1; w < 8; ++w) top = max(top, tops[w][lane]);
+    } else {
+        line = static_cast<int64_t>(blockIdx.x - blocksA) * 8 + warp;
+        static_assert(kSamples == 32, "one sample a lane");
+        if (line < p.lines) top = static_cast<unsigned int>(__double2hiint(p.X[lane * k / kSamples + line * p.ldx])) & 0x7FFFFFFFu;
+        top = __reduce_max_sync(0xFFFFFFFFu, top);
+        if (lane != 0) return;
+    }
+    if (line >= p.lines) return;
+    p.s.sumsq[line] = 0ull;
+    p.s.emax[line] = INT32_MIN;
+    p.s.nonfinite[line] = 0;
+    const int E = static_cast<int>(top >> 20) - 1023;
+    // 2^(9 - E) a normal number, as the sums' fast form needs it; no guess from zeros and subnormals, Inf or NaN
+    p.g.exponent[line] = top >= 0x00100000u && top < 0x7FF00000u && 9 - E >= -1000 && 9 - E <= 1000 - kGuesses ? E : INT32_MIN;
+#pragma unroll
+    for (int c = 0; c < kGuesses; ++c) {
+        p.g.sumsq[c * p.lines + line] = 0ull;
+        p.g.l1[c * p.lines + line] = 0u;
+    }
+}
+
+// One pass over the operand.  PASS 0: largest exponent + non-finite flag.  PASS 1: sum of squares, of the lines whose exponent was not guessed.
+// PASS 2: pass 0 and the sums for every guess.
 // side 0: thread = line, loop over a k-range (loads coalesced across lines).
 // side 1: warp = line, lanes stride over a k-range (loads coalesced along k), shuffle reduction.
 template <int SIDE, int PASS>
@@ -141,13 +217,19 @@ __device__ __forceinline__ void scan_block(const ScanSide &p, int64_t k, uint32_
     }
     bool live = line < lines;
     int emax = INT32_MIN;
-    unsigned int top = 0u;        // PASS 0: largest high word of |x|
+    unsigned int top = 0u;        // PASS 0, 2: largest high word of |x|
     unsigned long long acc = 0;
     unsigned int l1 = 0;          // sum of the magnitudes abar <= 2^10 (exponent-span check): below 2^30 for k <= 2^20
     int E = 0;
-    if (PASS == 1 && live) E = s.nonfinite[line] < 0 ? INT32_MIN : s.emax[line];      // INT32_MIN: nothing to add
+    if (PASS == 1 && live) {
+        E = s.nonfinite[line] < 0 ? INT32_MIN : s.emax[line];      // INT32_MIN: nothing to add
+        if (p.g.exponent && guessed(E, p.g.exponent[line])) live = false;
+    }
+    if (PASS == 2) E = live ? p.g.exponent[line] : INT32_MIN;
+    unsigned long long sums[kGuesses] = {};
+    unsigned int l1s[kGuesses] = {};
     // 2^(9-E) as a double, when it is a normal number (not for lines of subnormals only)
-    const bool fast_scale = PASS == 1 && E != INT32_MIN && 9 - E >= -1000 && 9 - E <= 1000;
+    const bool fast_scale = PASS >= 1 && E != INT32_MIN && 9 - E >= -1000 && 9 - E <= 1000;
     const double scale9 = __hiloint2double((1023 + (fast_scale ? 9 - E : 0)) << 20, 0);
     if (live && !(PASS == 1 && E == INT32_MIN)) {
         // batches of 8 independent loads keep enough bytes in flight to run at memory speed
@@ -158,20 +240,35 @@ __device__ __forceinline__ void scan_block(const ScanSide &p, int64_t k, uint32_
                 int64_t kk = kb + u * kstep;
                 xs[u] = kk < k1 ? *element(X, ldx, SIDE, line, kk) : 0.0;
             }
-            if (PASS == 0) {
+            if (PASS != 1) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u) top = max(top, static_cast<unsigned int>(__double2hiint(xs[u])) & 0x7FFFFFFFu);
-            } else {
+            }
+            if (PASS == 2) {
+                if (E != INT32_MIN) {
+                    // what is added for a guess below the line's exponent may wrap and is never read
+                    unsigned int part[kGuesses] = {};
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        const unsigned int abar = magnitude(xs[u], scale9);
+#pragma unroll
+                        for (int c = 0; c < kGuesses; ++c) {
+                            const unsigned int half = (abar + ((1u << c) - 1u)) >> c;
+                            part[c] += half * half;
+                            l1s[c] += half;
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < kGuesses; ++c) sums[c] += part[c];
+                }
+            } else if (PASS == 1) {
                 unsigned int part = 0u;           // eight terms of at most 2^20
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const double x = xs[u];
                     unsigned int abar;
                     if (fast_scale) {
-                        // ceil(|x| 2^(9-E)) through an exact FP64 scaling and a round-up conversion; a non-zero x whose
-                        // scaled value underflows to zero still counts as 1
-                        abar = __double2uint_ru(fabs(x) * scale9);
-                        if (abar == 0u && x != 0.0) abar = 1u;
+                        abar = magnitude(x, scale9);
                     } else {
                         abar = scaled_magnitude(x, E);
                     }
@@ -182,7 +279,7 @@ __device__ __forceinline__ void scan_block(const ScanSide &p, int64_t k, uint32_
             }
         }
     }
-    if (PASS == 0) {
+    if (PASS != 1) {
         // The high words order like the exponents; where only zeros and subnormals were seen, the exponents come
         // from the whole words.
         if (SIDE == 1) top = __reduce_max_sync(0xFFFFFFFFu, top);
@@ -200,8 +297,24 @@ __device__ __forceinline__ void scan_block(const ScanSide &p, int64_t k, uint32_
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
         l1 = __reduce_add_sync(0xFFFFFFFFu, l1);
     }
+    if (PASS == 2 && SIDE == 1) {
+#pragma unroll
+        for (int c = 0; c < kGuesses; ++c) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sums[c] += __shfl_xor_sync(0xFFFFFFFFu, sums[c], o);
+            l1s[c] = __reduce_add_sync(0xFFFFFFFFu, l1s[c]);
+        }
+    }
     if (!live || (SIDE == 1 && lane != 0)) return;
-    if (PASS == 0) {
+    if (PASS == 2 && E != INT32_MIN) {
+#pragma unroll
+        for (int c = 0; c < kGuesses; ++c)
+            if (sums[c]) {
+                atomicAdd(&p.g.sumsq[c * lines + line], sums[c]);
+                atomicAdd(&p.g.l1[c * lines + line], l1s[c]);
+            }
+    }
+    if (PASS != 1) {
         if (top >= 0x7FF00000u) atomicOr(&s.nonfinite[line], kNonfiniteBit);
         else if (emax != INT32_MIN) atomicMax(&s.emax[line], emax);
     } else if (acc) {
@@ -250,6 +363,7 @@ struct FinalizeSide {
     int64_t lines;
     int tbits;
     int32_t *shift;
+    ScanGuess g;
 };
 __global__ void scan_finalize_kernel(const __grid_constant__ FinalizeSide a, const __grid_constant__ FinalizeSide b, int64_t k, int rule,
                                      unsigned long long g2lo, unsigned long long g2hi,
@@ -274,6 +388,12 @@ __global__ void scan_finalize_kernel(const __grid_constant__ FinalizeSide a, con
         } else if (rule == 0) {
             shift[i] = (side ? b.tbits : a.tbits) - 1 - E;
         } else {
+            const ScanGuess g = side ? b.g : a.g;
+            if (g.exponent && guessed(E, g.exponent[i])) {       // the sums of the guess go where those of a second pass would be
+                const int64_t at = (E - g.exponent[i]) * (side ? b.lines : a.lines) + i;
+                s.sumsq[i] = g.sumsq[at];
+                s.nonfinite[i] = static_cast<int>(g.l1[at]);
+            }
             shift[i] = norm_exponent(s.sumsq[i], g2lo, g2hi) + 9 - E;
             flatness = line_flatness(static_cast<unsigned int>(s.nonfinite[i]), s.sumsq[i], k);
         }
@@ -396,9 +516,7 @@ __device__ __forceinline__ BoundLine bound_line(const ScanScratch &s, int64_t li
 __device__ __forceinline__ uint32_t bound_digit(double x, const BoundLine &b)
 {
     if (!b.fast) return bound_digit_exact(x, b.E);
-    // exact scaling and a round-up conversion; a non-zero x whose scaled value underflows to zero still counts as 1
-    uint32_t d = __double2uint_ru(fabs(x) * b.scale);
-    if (d == 0u && x != 0.0) d = 1u;
+    const uint32_t d = magnitude(x, b.scale);
     return d > 16u ? (d + 1u) & ~1u : d;
 }
 
@@ -937,8 +1055,7 @@ __device__ __forceinline__ void deconstruct_lines(const FusedParams &p, int bloc
                 if (fast_scale) {
                     for (int kk = k0 + lane; kk < k1; kk += 32) {
                         const double x = src[padded(kk)];
-                        unsigned int abar = __double2uint_ru(fabs(x) * scale9);
-                        if (abar == 0u && x != 0.0) abar = 1u;
+                        const unsigned int abar = magnitude(x, scale9);
                         acc += abar * abar;                              // at most 2^20
                         l1 += abar;
                     }
@@ -1257,8 +1374,7 @@ deconstruct_cluster_kernel(const __grid_constant__ ClusterParams cp)
                     for (int e = 0; e < 8; ++e) {
                         unsigned int abar;
                         if (fast_scale) {
-                            abar = __double2uint_ru(fabs(x[e]) * scale9);
-                            if (abar == 0u && x[e] != 0.0) abar = 1u;
+                            abar = magnitude(x[e], scale9);
                         } else {
                             abar = scaled_magnitude(x[e], E);
                         }
@@ -1455,11 +1571,13 @@ oz_status_t launch_convert(const double *X, int64_t ldx, int64_t lines, int64_t 
 // later from the bound product], of one operand or (both pointers) of both
 oz_status_t launch_scan(const ScanJob *a, const ScanJob *b, int64_t k, int set, const Route &rt, bool alone, cudaStream_t stream)
 {
+    const bool guesses = rt.rule == 1 && k >= kSamples && (!a || a->spare) && (!b || b->spare);
     auto scan_side = [&](const ScanJob *j, int side) {
         ScanSide p{};
         if (!j) return p;
         p.X = j->X; p.ldx = j->ldx; p.lines = j->lines;
         p.s = carve_scratch(j->scratch, j->lines);
+        p.g = carve_guess(guesses ? j->spare : nullptr, j->lines);
         // split the inner dimension so that the scan fills the machine even for few lines
         const int64_t line_blocks = side == 0 ? (j->lines + 255) / 256 : (j->lines + 7) / 8;
         const int64_t want_split = (148 * 8 + line_blocks - 1) / line_blocks, max_split = (k + 63) / 64;
@@ -1474,15 +1592,22 @@ oz_status_t launch_scan(const ScanJob *a, const ScanJob *b, int64_t k, int set, 
     };
     const ScanSide sa = scan_side(a, 0), sb = scan_side(b, 1);
     const unsigned blocks1d = static_cast<unsigned>((sa.lines + sb.lines + 255) / 256);
-    OZ_CUDA_CHECK(launch_if(alone, scan_init_kernel, dim3(blocks1d), 256, 0, stream, sa.s, sa.lines, sb.s, sb.lines));
-    count_launch();
-    if (k > 0) {
-        const dim3 grid(sa.blocks + sb.blocks);
-        OZ_CUDA_CHECK(launch_if(alone, scan_kernel<0>, grid, 256, 0, stream, sa, sb, k));
+    const dim3 grid(sa.blocks + sb.blocks);
+    if (guesses) {
+        OZ_CUDA_CHECK(launch_if(alone, scan_sample_kernel, dim3(static_cast<unsigned>((sa.lines + 31) / 32 + (sb.lines + 7) / 8)), 256, 0, stream, sa, sb, k));
+        OZ_CUDA_CHECK(launch_if(alone, scan_kernel<2>, grid, 256, 0, stream, sa, sb, k));
+        OZ_CUDA_CHECK(launch_if(alone, scan_kernel<1>, grid, 256, 0, stream, sa, sb, k));
+        count_launch(3);
+    } else {
+        OZ_CUDA_CHECK(launch_if(alone, scan_init_kernel, dim3(blocks1d), 256, 0, stream, sa.s, sa.lines, sb.s, sb.lines));
         count_launch();
-        if (rt.rule == 1) {
-            OZ_CUDA_CHECK(launch_if(alone, scan_kernel<1>, grid, 256, 0, stream, sa, sb, k));
+        if (k > 0) {
+            OZ_CUDA_CHECK(launch_if(alone, scan_kernel<0>, grid, 256, 0, stream, sa, sb, k));
             count_launch();
+            if (rt.rule == 1) {
+                OZ_CUDA_CHECK(launch_if(alone, scan_kernel<1>, grid, 256, 0, stream, sa, sb, k));
+                count_launch();
+            }
         }
     }
     if (rt.rule != 2) {
@@ -1490,7 +1615,7 @@ oz_status_t launch_scan(const ScanJob *a, const ScanJob *b, int64_t k, int set, 
         budget_maxexp(set, k, &tA, &tB);
         uint64_t g2lo = 0, g2hi = 0;
         cs_bound_squared(set, k, &g2lo, &g2hi);
-        const FinalizeSide fa{sa.s, sa.lines, tA, a ? a->shift : nullptr}, fb{sb.s, sb.lines, tB, b ? b->shift : nullptr};
+        const FinalizeSide fa{sa.s, sa.lines, tA, a ? a->shift : nullptr, sa.g}, fb{sb.s, sb.lines, tB, b ? b->shift : nullptr, sb.g};
         OZ_CUDA_CHECK(launch_if(alone, scan_finalize_kernel, dim3(blocks1d), 256, 0, stream, fa, fb, k, rt.rule, g2lo, g2hi,
                              esc_threshold(set), device_status_word()));
         count_launch();
@@ -1523,7 +1648,7 @@ unsigned int *bound_maxima(void *scratch, int64_t lines)
 // accurate rule: shifts from the maxima of the bound product
 oz_status_t launch_accurate_finalize(const ScanJob &a, const ScanJob &b, int budget_log2, cudaStream_t stream)
 {
-    const FinalizeSide fa{carve_scratch(a.scratch, a.lines), a.lines, 0, a.shift}, fb{carve_scratch(b.scratch, b.lines), b.lines, 0, b.shift};
+    const FinalizeSide fa{carve_scratch(a.scratch, a.lines), a.lines, 0, a.shift, {}}, fb{carve_scratch(b.scratch, b.lines), b.lines, 0, b.shift, {}};
     OZ_CUDA_CHECK(launch(accurate_finalize_kernel, dim3(static_cast<unsigned>((a.lines + b.lines + 255) / 256)), 256, 0, stream,
                          fa, fb, budget_log2, device_status_word()));
     count_launch();
@@ -1634,7 +1759,7 @@ oz_status_t launch_deconstruct(int side, int64_t lines, int64_t k, const double 
 #undef OZ_CLUSTER_SET
 #undef OZ_CLUSTER
     }
-    const ScanJob job{lines, X, ldx, shift, scratch};
+    const ScanJob job{lines, X, ldx, shift, scratch, geom.row_pitch >= kGuessBytes ? planes : nullptr};
     oz_status_t st = launch_scan(side == 0 ? &job : nullptr, side == 1 ? &job : nullptr, k, set, rt, alone, stream);
     if (st != OZ_OK) return st;
     return launch_convert_planes(side, lines, k, X, ldx, set, rt, planes, geom, shift, alone, stream);

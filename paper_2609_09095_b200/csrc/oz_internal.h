@@ -259,6 +259,7 @@ struct ScanJob {
     int64_t ldx;
     int32_t *shift;
     void *scratch;
+    void *spare;                // the operand's first plane, which the conversion fills after the scan, for sums in between; null: none
 };
 // whether launch_deconstruct() takes the scans and the conversion into private planes (else the one-kernel or the cluster form)
 bool three_passes(int side, const ScanJob &job, int64_t k, int set, const Route &rt);

@@ -112,3 +112,35 @@ def test_three_pass_deconstruction_of_columns(lines, k, set_name, sub):
     for a in range(0, lines, step):
         part, part_shift, _ = gh.deconstruct(1, np.asfortranarray(X[:, a:a + step]), set_name, rt)
         assert (shift[a:a + step] == part_shift).all() and (got[:, a:a + step] == part).all()
+
+
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("E", "int8"), ("A", "int8n")])
+@pytest.mark.parametrize("m,n,k", [(1003, 301, 5003), (33, 2049, 8193), (2600, 9, 4097)])
+def test_scan_by_guessed_exponents(set_name, sub, m, n, k):
+    """The scan of large operands guesses a line's largest exponent from a sample: lines whose largest element hides between the samples,
+    by no, one, two, three and many powers of two, lines of zeros, of subnormals, with samples of zeros only, with Inf and NaN."""
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m + n + k)
+    A, B = np.asfortranarray(rng.standard_normal((m, k))), np.asfortranarray(rng.standard_normal((k, n)))
+    hidden = k // 32 + 1                              # no sample: samples lie at the multiples of k / 32
+    for lines, axis in ((A, 0), (B, 1)):
+        count = lines.shape[axis]
+        rows = lines if axis == 0 else lines.T
+        for i, e in zip(range(count), (0, 1, 2, 3, 4, 60, -30, 900)):
+            rows[i] = np.clip(rows[i], -1.9, 1.9)
+            rows[i, hidden] = 1.5 * 2.0 ** e
+        if count > 20:
+            rows[9], rows[10] = 0.0, rows[10] * 2.0 ** -1060
+            rows[11, hidden + 1:], rows[11, :hidden] = 0.0, 0.0
+            rows[12] *= 2.0 ** -1000
+            rows[13] *= 2.0 ** 900
+            rows[14, ::k // 32] = 0.0
+            rows[15, hidden] = 5e-324
+            rows[16, 0] = 2.0 ** 300
+    if m > 100:
+        A[20, 5], A[21, hidden] = np.nan, np.inf
+    rt = gh.route(sub)
+    got, _ = gh.dgemm(A, B, set_name, rt)
+    want = ozo.dgemm(A, B, {"S": ozo.SET_S, "E": ozo.SET_E, "A": ozo.SET_A}[set_name], ozo.QUANT_RN, ozo.SCALE_CS)
+    assert (np.isnan(got) == np.isnan(want)).all()
+    assert (got[~np.isnan(want)] == want[~np.isnan(want)]).all()
