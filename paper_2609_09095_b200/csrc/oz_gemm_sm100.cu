@@ -523,6 +523,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     static_assert(SLIM == 0 || (CG == 1 && !DIRECT && TILED && !BOUND), "two-plane schedule: whole-method digit products");
     static_assert(BN == BLOCK_N || TILED, "narrow tiles: whole-method products");
     constexpr bool PACKED = TILED && RB == 2 && !BOUND;  // sets S and E in the private array
+    constexpr bool BIASED = TILED && SUB == 1 && !DIRECT;        // the combination starts at the bias that makes it non-negative
     using Slim = SlimTile<SLIM ? SLIM : 128, BN>;
     constexpr int STAGES = SLIM ? Slim::STAGES : Tile<CG, BN>::STAGES;
     constexpr int STAGE_BYTES = SLIM ? Slim::STAGE_BYTES : Tile<CG, BN>::STAGE_BYTES;
@@ -776,7 +777,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             // running combination per element: FP32 (FP8 route) or INT32 (INT8 routes), as raw bits
             uint32_t comb[COLS_PER_WARP];
             if constexpr (!DIRECT) {
-                const uint32_t start = PACKED && SUB == 0 ? __float_as_uint(-mi.centre) : 0u;
+                const uint32_t start = SUB == 0 ? (PACKED ? __float_as_uint(-mi.centre) : 0u) : (BIASED ? ibias : 0u);
 #pragma unroll
                 for (int c = 0; c < COLS_PER_WARP; ++c) comb[c] = start;
             }
@@ -898,9 +899,9 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     uint32_t u = cv + mi.bias30;                          // in (0, 2^31 + 256)
                     return u - (__umulhi(u, mi.magic39) >> 7) * im;      // exact quotient: canonical [0, m)
                 } else {
-                    uint32_t u = cv + ibias;
+                    uint32_t u = BIASED ? cv : cv + ibias;
                     uint32_t r = u - __umulhi(u, imagic) * im;           // in [0, 2m)
-                    return min(r, r - im);                               // canonical [0, m)
+                    return __viaddmin_u32(r, 0u - im, r);                // canonical [0, m)
                 }
             };
             // same for two values at once; the balanced FP32 form is done with packed pairs
@@ -945,7 +946,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                             pack_rows(8 * c + 4, 8 * c + 6, val.z, val.w);
                             *reinterpret_cast<uint4 *>(base + (2 * chunk0 + c) * 512) = val;
                         }
-                    } else {
+                    } else if (mi.store_form == kStoredTen) {
                         uint32_t high[COLS_PER_WARP / 16];           // bits 8 and 9 of sixteen rows
 #pragma unroll
                         for (int g = 0; g < COLS_PER_WARP / 16; ++g) {
@@ -955,14 +956,26 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                                 uint32_t w0, w1;
                                 pack_rows(16 * g + 2 * h, 16 * g + 2 * h + 8, w0, w1);
                                 lo[h] = __byte_perm(w0, w1, 0x6420);
-                                hi[h] = __byte_perm(w0, w1, 0x7531) & 0x03030303u;   // 1024 is 0 modulo 1024
+                                hi[h] = __byte_perm(w0, w1, 0x7531);
+                                if constexpr (SUB == 0) hi[h] &= 0x03030303u;        // 1024 is 0 modulo 1024
                             }
                             *reinterpret_cast<uint4 *>(base + (chunk0 + g) * 512) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                             high[g] = (hi[0] + 4u * hi[1]) + 16u * (hi[2] + 4u * hi[3]);
                         }
-                        if (mi.store_form == kStoredTen) {
-                            if constexpr (COLS_PER_WARP == 64) *reinterpret_cast<uint4 *>(base + 2048) = make_uint4(high[0], high[1], high[2], high[3]);
-                            else *reinterpret_cast<uint32_t *>(base + 2048 + 4 * chunk0) = high[0];
+                        if constexpr (COLS_PER_WARP == 64) *reinterpret_cast<uint4 *>(base + 2048) = make_uint4(high[0], high[1], high[2], high[3]);
+                        else *reinterpret_cast<uint32_t *>(base + 2048 + 4 * chunk0) = high[0];
+                    } else {
+#pragma unroll
+                        for (int g = 0; g < COLS_PER_WARP / 16; ++g) {
+                            uint32_t lo[4];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                uint32_t b0, b1, b8, b9;
+                                final_bits2(comb[16 * g + 2 * h], comb[16 * g + 2 * h + 1], b0, b1);
+                                final_bits2(comb[16 * g + 2 * h + 8], comb[16 * g + 2 * h + 9], b8, b9);
+                                lo[h] = __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b8, b9, 0x0040), 0x5410);
+                            }
+                            *reinterpret_cast<uint4 *>(base + (chunk0 + g) * 512) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
                         }
                     }
                 } else {
