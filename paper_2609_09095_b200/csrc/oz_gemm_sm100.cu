@@ -30,7 +30,7 @@
 //   warp 0       TMA producer: 128-byte-swizzled K-major tiles of B (128 lines) and A (256 lines,
 //                or this CTA's half of them in a pair) into a shared-memory ring of 192 KiB
 //                (4 stages of 48 KiB, or 6 of 32 KiB in a pair), no multicast
-//   warp 1       MMA issuer: one lane issues tcgen05.mma (M=128 or 256 across the pair, N=256,
+//   warp 1       MMA issuer: an elected lane issues tcgen05.mma (M=128 or 256 across the pair, N=256,
 //                K=32); accumulators live in TMEM, two slots of 256 columns used alternately per job
 //   warps 2..17  epilogue (4 per TMEM lane quarter, 64 columns each): tcgen05.ld the finished slot,
 //                reduce each accumulator modulo m_i in FP32 (all values are integers below 2^24,
@@ -207,6 +207,14 @@ __device__ __forceinline__ void mbar_arrive_relaxed(uint32_t bar)
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+}
+
+// one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
 }
 
 // all threads of both CTAs of the pair (no time limit: every thread reaches it on every path)
@@ -548,7 +556,9 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     volatile uint32_t *tmem_base_ptr = reinterpret_cast<volatile uint32_t *>(gen + 16 * STAGES + 32);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + 16 * STAGES + 40);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // Broadcast, the warp number and the TMEM base are the same in a warp by construction and need no register of a thread:
+    // the epilogue's 64 running values then fit its 96 registers without spills in all but two of the variants.
+    const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     dependency_release();
     if (threadIdx.x == 0) {
@@ -571,10 +581,17 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     if (CG == 2) cluster_sync_all();      // the peer's barriers exist before anything signals them
     tc_fence_after();
     dependency_wait();                    // the planes are there, and the previous readers of the residues are done
-    const uint32_t tmem_base = *tmem_base_ptr;
+    const uint32_t tmem_base = __shfl_sync(0xFFFFFFFFu, *tmem_base_ptr, 0);
 
     if (warp < FIRST_EPI_WARP) {
-        if (warp == 0 && lane == 0) {
+        // The whole warp walks the loops of its role and one elected lane issues: with nothing that depends on the thread, what a
+        // copy or an MMA takes is computed in uniform registers, where these instructions want it.  A single thread that walks them
+        // moves every descriptor over instead and falls behind the tensor cores (us, single threads -> issuer -> both):
+        // 8192 x 8192 x 1024 set S FP8 1900 -> 1781 -> 1627, 3000 x 3000 x 500 150 -> 134 -> 123, 6144 x 6144 x 3072 native INT8
+        // 1086 -> 1074 -> 994, 10007 x 9973 x 5003 at the power cap 14286 -> 13977 -> 13664.
+        const bool leader = elect_one();
+        auto wait = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, p.status)) != 0; };
+        if (warp == 0) {
             // -------------------------------------------------------- TMA producer
             int stage = 0;
             uint32_t phase = 0;
@@ -584,14 +601,14 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 const ModInfo &mi = p.mod[it.mod];
                 // one stage: 128 bytes of K of plane pa of A and pb of B
                 auto load = [&](int pa, int pb, int kc) {
-                    if (!mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status)) return false;
+                    if (!wait(empty_bar + 8 * stage, phase ^ 1u)) return false;
                     uint32_t fb = full_bar + 8 * stage;
                     uint32_t sa = tiles + stage * STAGE_BYTES;
-                    if (CG == 1) {
+                    if (leader && CG == 1) {
                         mbar_expect_tx(fb, STAGE_BYTES);
                         tma_load_3d(sa, &mapB, fb, kc * p.kc_x, it.tn * BLOCK_M, pb * p.plane_z + kc * p.kc_z);
                         tma_load_3d(sa + A_BYTES, &mapA, fb, kc * p.kc_x, it.tm * BN, pa * p.plane_z + kc * p.kc_z);
-                    } else {
+                    } else if (leader) {
                         // both CTAs' copies complete on the leader's barrier
                         if (rank == 0) mbar_expect_tx(fb, 2 * STAGE_BYTES);
                         const uint32_t fb_leader = map_to_cta(fb, 0);
@@ -606,16 +623,18 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 if constexpr (SLIM != 0) {
                     for (int kc = 0; ok && kc < p.nk; ++kc)
                         for (int h = 0; ok && h < 2; ++h) {
-                            ok = mbar_wait(empty_bar + 8 * stage, phase ^ 1u, abort_flag, p.status);
+                            ok = wait(empty_bar + 8 * stage, phase ^ 1u);
                             if (!ok) break;
                             const uint32_t fb = full_bar + 8 * stage, sa = tiles + stage * STAGE_BYTES;
                             int first, second;
                             slim_stage(mi, h, &first, &second);
-                            mbar_expect_tx(fb, first >= 0 ? STAGE_BYTES : STAGE_BYTES - Slim::B_BYTES);
                             const int x = kc * p.kc_x, z = kc * p.kc_z;
-                            tma_load_3d(sa + 2 * Slim::B_BYTES, &mapA, fb, x, it.tm * BN, (mi.planeA0 + h) * p.plane_z + z);
-                            if (first >= 0) tma_load_3d(sa, &mapB, fb, x, it.tn * BLOCK_M, first * p.plane_z + z);
-                            tma_load_3d(sa + Slim::B_BYTES, &mapB, fb, x, it.tn * BLOCK_M, second * p.plane_z + z);
+                            if (leader) {
+                                mbar_expect_tx(fb, first >= 0 ? STAGE_BYTES : STAGE_BYTES - Slim::B_BYTES);
+                                tma_load_3d(sa + 2 * Slim::B_BYTES, &mapA, fb, x, it.tm * BN, (mi.planeA0 + h) * p.plane_z + z);
+                                if (first >= 0) tma_load_3d(sa, &mapB, fb, x, it.tn * BLOCK_M, first * p.plane_z + z);
+                                tma_load_3d(sa + Slim::B_BYTES, &mapB, fb, x, it.tn * BLOCK_M, second * p.plane_z + z);
+                            }
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                         }
                     continue;
@@ -642,7 +661,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 unsigned long long t0 = global_timer_ns();
                 while (global_timer_ns() - t0 < 2000000ull) { }
             }
-        } else if (warp == 1 && lane == 0 && rank == 0) {
+        } else if (warp == 1 && rank == 0) {
             // -------------------------------------------------------- MMA issuer (pair: leader CTA only)
             constexpr uint32_t idesc = instr_desc<SUB, CG, BN>();
             int stage = 0;
@@ -658,30 +677,34 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     const uint32_t idesc1 = mi.kind == 5 ? idesc | kNegateB : idesc;
                     for (int seg = 0; ok && seg < mi.nseg_all; ++seg) {
                         for (int h = 0; ok && h < 2; ++h)
-                            ok = mbar_wait(tempty_bar + 8 * h, ((slot_phase >> h) & 1u) ^ 1u, abort_flag, p.status);
+                            ok = wait(tempty_bar + 8 * h, ((slot_phase >> h) & 1u) ^ 1u);
                         if (!ok) break;
                         tc_fence_after();
                         const int kc0 = seg * mi.seg_len_all, kc1 = min(p.nk, kc0 + mi.seg_len_all);
                         for (int st = 0; st < 2 * (kc1 - kc0); ++st) {
                             const int h = st & 1;
-                            ok = mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status);
+                            ok = wait(full_bar + 8 * stage, phase);
                             if (!ok) break;
                             tc_fence_after();
                             const uint32_t sa = tiles + stage * STAGE_BYTES;
                             const uint64_t e0 = smem_desc(sa), e1 = smem_desc(sa + Slim::B_BYTES), a = smem_desc(sa + 2 * Slim::B_BYTES);
+                            if (leader) {
 #pragma unroll
-                            for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
-                                const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
-                                const uint32_t accumulate = st > 0 || ks > 0 ? 1u : 0u, id = h ? idesc1 : idesc;
-                                if (mi.kind != 0 || h == 0) umma<SUB, CG>(tmem_base, e0 + o, a + o, id, accumulate);
-                                umma<SUB, CG>(tmem_base + BLOCK_N, e1 + o, a + o, id, accumulate);
+                                for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
+                                    const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
+                                    const uint32_t accumulate = st > 0 || ks > 0 ? 1u : 0u, id = h ? idesc1 : idesc;
+                                    if (mi.kind != 0 || h == 0) umma<SUB, CG>(tmem_base, e0 + o, a + o, id, accumulate);
+                                    umma<SUB, CG>(tmem_base + BLOCK_N, e1 + o, a + o, id, accumulate);
+                                }
+                                umma_commit<CG>(empty_bar + 8 * stage);
                             }
-                            umma_commit<CG>(empty_bar + 8 * stage);
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                         }
                         if (!ok) break;
-                        umma_commit<CG>(tfull_bar);
-                        umma_commit<CG>(tfull_bar + 8);
+                        if (leader) {
+                            umma_commit<CG>(tfull_bar);
+                            umma_commit<CG>(tfull_bar + 8);
+                        }
                         slot_phase ^= 3u;
                     }
                     continue;
@@ -689,67 +712,70 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 if (!DIRECT && p.pair_squares && mi.kind == 0) {
                     // d0 e0 into one slot, d1 e0 + d0 e1 into the other, from the four tiles of a chunk
                     for (int h = 0; ok && h < 2; ++h)
-                        ok = mbar_wait(tempty_bar + 8 * (slot ^ h), ((slot_phase >> (slot ^ h)) & 1u) ^ 1u, abort_flag, p.status);
+                        ok = wait(tempty_bar + 8 * (slot ^ h), ((slot_phase >> (slot ^ h)) & 1u) ^ 1u);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d0 = tmem_base + static_cast<uint32_t>(slot * BLOCK_N);
                     const uint32_t d1 = tmem_base + static_cast<uint32_t>((slot ^ 1) * BLOCK_N);
                     for (int kc = 0; kc < p.nk; ++kc) {
                         const int s0 = stage, s1 = stage + 1 == STAGES ? 0 : stage + 1;
-                        ok = mbar_wait(full_bar + 8 * s0, phase, abort_flag, p.status);
+                        ok = wait(full_bar + 8 * s0, phase);
                         if (!ok) break;
-                        ok = mbar_wait(full_bar + 8 * s1, s1 == 0 ? phase ^ 1u : phase, abort_flag, p.status);
+                        ok = wait(full_bar + 8 * s1, s1 == 0 ? phase ^ 1u : phase);
                         if (!ok) break;
                         tc_fence_after();
                         const uint32_t t0 = tiles + s0 * STAGE_BYTES, t1 = tiles + s1 * STAGE_BYTES;
                         const uint64_t e0 = smem_desc(t0), a0 = smem_desc(t0 + A_BYTES), e1 = smem_desc(t1), a1 = smem_desc(t1 + A_BYTES);
+                        if (leader) {
 #pragma unroll
-                        for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
-                            const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
-                            const uint32_t accumulate = kc > 0 || ks > 0 ? 1u : 0u;
-                            umma<SUB, CG>(d0, e0 + o, a0 + o, idesc, accumulate);
-                            umma<SUB, CG>(d1, e0 + o, a1 + o, idesc, accumulate);
-                            umma<SUB, CG>(d1, e1 + o, a0 + o, idesc, 1u);
+                            for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
+                                const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
+                                const uint32_t accumulate = kc > 0 || ks > 0 ? 1u : 0u;
+                                umma<SUB, CG>(d0, e0 + o, a0 + o, idesc, accumulate);
+                                umma<SUB, CG>(d1, e0 + o, a1 + o, idesc, accumulate);
+                                umma<SUB, CG>(d1, e1 + o, a0 + o, idesc, 1u);
+                            }
+                            umma_commit<CG>(empty_bar + 8 * s0);
+                            umma_commit<CG>(empty_bar + 8 * s1);
                         }
-                        umma_commit<CG>(empty_bar + 8 * s0);
-                        umma_commit<CG>(empty_bar + 8 * s1);
                         for (int h = 0; h < 2; ++h)
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                     }
                     if (!ok) break;
-                    umma_commit<CG>(tfull_bar + 8 * slot);
-                    umma_commit<CG>(tfull_bar + 8 * (slot ^ 1));
+                    if (leader) {
+                        umma_commit<CG>(tfull_bar + 8 * slot);
+                        umma_commit<CG>(tfull_bar + 8 * (slot ^ 1));
+                    }
                     slot_phase ^= 3u;
                     continue;
                 }
                 for (int job = 0; ok && job < mi.njobs; ++job)
                 for (int seg = 0, nseg = job_segments(mi, job); ok && seg < nseg; ++seg) {
-                    ok = mbar_wait(tempty_bar + 8 * slot, ((slot_phase >> slot) & 1u) ^ 1u, abort_flag, p.status);
+                    ok = wait(tempty_bar + 8 * slot, ((slot_phase >> slot) & 1u) ^ 1u);
                     if (!ok) break;
                     tc_fence_after();
                     const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(slot * BLOCK_N);
-                    uint32_t accumulate = 0;
                     int kc0, kc1;
                     segment_range(mi, job, seg, p.nk, &kc0, &kc1);
                     int steps = job_pairs(mi, job) * (kc1 - kc0);
                     for (int st = 0; st < steps; ++st) {
-                        ok = mbar_wait(full_bar + 8 * stage, phase, abort_flag, p.status);
+                        ok = wait(full_bar + 8 * stage, phase);
                         if (!ok) break;
                         tc_fence_after();
                         uint32_t sa = tiles + stage * STAGE_BYTES;
                         uint64_t da = smem_desc(sa), db = smem_desc(sa + A_BYTES);
+                        if (leader) {
 #pragma unroll
-                        for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
-                            // advancing K inside the 128-byte swizzle atom: +32 bytes = +2 in the address field
-                            umma<SUB, CG>(d_tmem, da + static_cast<uint64_t>(ks * (UMMA_K >> 4)),
-                                      db + static_cast<uint64_t>(ks * (UMMA_K >> 4)), idesc, accumulate);
-                            accumulate = 1;
+                            for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks)
+                                // advancing K inside the 128-byte swizzle atom: +32 bytes = +2 in the address field
+                                umma<SUB, CG>(d_tmem, da + static_cast<uint64_t>(ks * (UMMA_K >> 4)),
+                                          db + static_cast<uint64_t>(ks * (UMMA_K >> 4)), idesc, st > 0 || ks > 0 ? 1u : 0u);
+                            umma_commit<CG>(empty_bar + 8 * stage);     // frees the stage when these MMAs finish
                         }
-                        umma_commit<CG>(empty_bar + 8 * stage);     // frees the stage when these MMAs finish
                         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                     }
                     if (!ok) break;
-                    umma_commit<CG>(tfull_bar + 8 * slot);           // accumulator complete
+                    if (leader) umma_commit<CG>(tfull_bar + 8 * slot);           // accumulator complete
                     slot_phase ^= 1u << slot;
                     slot ^= 1;
                 }
@@ -782,7 +808,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                 for (int c = 0; c < COLS_PER_WARP; ++c) comb[c] = start;
             }
             // SLIM: both jobs of a K segment before the next segment.  (The bound is read where it is compared: in a register of its
-            // own it costs the public FP8 variants 144 bytes of spills instead of 48, 4096 x 4096 x 1024: 516 us against 485.)
+            // own it costs the public FP8 pair 72 bytes of spills instead of 40.)
             for (int o = 0; ok && o < (SLIM ? mi.nseg_all : mi.njobs); ++o)
             for (int i = 0, inner = SLIM ? 2 : job_segments(mi, o); ok && i < inner; ++i) {
                 const int job = SLIM ? i : o;
@@ -1001,6 +1027,9 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     pack_rows(c, c + 2, packed[c >> 2], unused);
                 }
             }
+            // all are packed before the first is stored: the unpacked ones in between cost 72 bytes of spills
+#pragma unroll
+            for (int c = 0; c < COLS_PER_WARP * RB / 4; ++c) asm volatile("" : "+r"(packed[c]));
             unsigned char *rbase = static_cast<unsigned char *>(p.R) + it.mod * p.mod_stride * RB;
             if (p.vec_store && i0 + COLS_PER_WARP <= p.m) {
                 // Transpose through a per-warp shared buffer so that one store instruction writes
