@@ -710,42 +710,66 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     continue;
                 }
                 if (!DIRECT && p.pair_squares && mi.kind == 0) {
-                    // d0 e0 into one slot, d1 e0 + d0 e1 into the other, from the four tiles of a chunk
-                    for (int h = 0; ok && h < 2; ++h)
-                        ok = wait(tempty_bar + 8 * (slot ^ h), ((slot_phase >> (slot ^ h)) & 1u) ^ 1u);
-                    if (!ok) break;
-                    tc_fence_after();
+                    // d0 e0 into one slot, d1 e0 + d0 e1 into the other, from the four tiles of a chunk: first all that goes into
+                    // the first slot, so that it is complete while the last chunk's other products run, and the next product's
+                    // can begin in it while the epilogue still empties the second.  That takes longer than one chunk's 4 MMAs, so
+                    // a pair starts with those of two chunks.  (Two at a time throughout leave two of the six stages to prefetch
+                    // into.)  Both slots waited for and complete together -> in turn: 8192 x 8192 x 512 set E INT8 1003 -> 909 us,
+                    // 8192 x 8192 x 1024 set S FP8 1707 -> 1621, 16384 x 16384 x 1024 7510 -> 7100, 4096 x 4096 x 4096
+                    // 1596 -> 1578; in turn -> two chunks at the start (two at a time): 955 -> 923 (915), 1721 -> 1691 (1732),
+                    // 7182 -> 7036 (7237), 1689 -> 1678 (1691).
                     const uint32_t d0 = tmem_base + static_cast<uint32_t>(slot * BLOCK_N);
                     const uint32_t d1 = tmem_base + static_cast<uint32_t>((slot ^ 1) * BLOCK_N);
-                    for (int kc = 0; kc < p.nk; ++kc) {
-                        const int s0 = stage, s1 = stage + 1 == STAGES ? 0 : stage + 1;
-                        ok = wait(full_bar + 8 * s0, phase);
-                        if (!ok) break;
-                        ok = wait(full_bar + 8 * s1, s1 == 0 ? phase ^ 1u : phase);
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint32_t t0 = tiles + s0 * STAGE_BYTES, t1 = tiles + s1 * STAGE_BYTES;
-                        const uint64_t e0 = smem_desc(t0), a0 = smem_desc(t0 + A_BYTES), e1 = smem_desc(t1), a1 = smem_desc(t1 + A_BYTES);
-                        if (leader) {
+                    constexpr int GROUP = CG == 2 ? 2 : 1;           // chunks
+                    for (int kc = 0, count; ok && kc < p.nk; kc += count) {
+                        const int start = stage;
+                        count = kc == 0 ? min(GROUP, p.nk) : 1;
+                        const uint32_t start_phase = phase;
+                        if (kc == 0) ok = wait(tempty_bar + 8 * slot, ((slot_phase >> slot) & 1u) ^ 1u);
+                        for (int c = 0; ok && c < count; ++c) {
+                            ok = wait(full_bar + 8 * stage, phase);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t t0 = tiles + stage * STAGE_BYTES;
+                            const uint64_t e0 = smem_desc(t0), a0 = smem_desc(t0 + A_BYTES);
+                            if (leader) {
 #pragma unroll
-                            for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
-                                const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
-                                const uint32_t accumulate = kc > 0 || ks > 0 ? 1u : 0u;
-                                umma<SUB, CG>(d0, e0 + o, a0 + o, idesc, accumulate);
-                                umma<SUB, CG>(d1, e0 + o, a1 + o, idesc, accumulate);
-                                umma<SUB, CG>(d1, e1 + o, a0 + o, idesc, 1u);
+                                for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
+                                    const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
+                                    umma<SUB, CG>(d0, e0 + o, a0 + o, idesc, kc > 0 || c > 0 || ks > 0 ? 1u : 0u);
+                                }
                             }
-                            umma_commit<CG>(empty_bar + 8 * s0);
-                            umma_commit<CG>(empty_bar + 8 * s1);
+                            for (int h = 0; h < 2; ++h)
+                                if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                         }
-                        for (int h = 0; h < 2; ++h)
+                        if (!ok) break;
+                        if (leader && kc + count >= p.nk) umma_commit<CG>(tfull_bar + 8 * slot);
+                        if (kc == 0) ok = wait(tempty_bar + 8 * (slot ^ 1), ((slot_phase >> (slot ^ 1)) & 1u) ^ 1u);
+                        stage = start;
+                        phase = start_phase;
+                        for (int c = 0; ok && c < count; ++c) {
+                            const int s0 = stage;
                             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                            ok = wait(full_bar + 8 * stage, phase);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t t0 = tiles + s0 * STAGE_BYTES, t1 = tiles + stage * STAGE_BYTES;
+                            const uint64_t e0 = smem_desc(t0), a0 = smem_desc(t0 + A_BYTES), e1 = smem_desc(t1), a1 = smem_desc(t1 + A_BYTES);
+                            if (leader) {
+#pragma unroll
+                                for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
+                                    const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
+                                    umma<SUB, CG>(d1, e0 + o, a1 + o, idesc, kc > 0 || c > 0 || ks > 0 ? 1u : 0u);
+                                    umma<SUB, CG>(d1, e1 + o, a0 + o, idesc, 1u);
+                                }
+                                umma_commit<CG>(empty_bar + 8 * s0);
+                                umma_commit<CG>(empty_bar + 8 * stage);
+                            }
+                            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+                        }
                     }
                     if (!ok) break;
-                    if (leader) {
-                        umma_commit<CG>(tfull_bar + 8 * slot);
-                        umma_commit<CG>(tfull_bar + 8 * (slot ^ 1));
-                    }
+                    if (leader) umma_commit<CG>(tfull_bar + 8 * (slot ^ 1));
                     slot_phase ^= 3u;
                     continue;
                 }
@@ -1421,8 +1445,8 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(m, n, k, set, sms)));
     fill_mod_info(p, set, rt, k, slim);
     // Squares in one K-loop: the products of a square read d0 and e0 twice, so job after job a K chunk costs six tiles;
-    // with both accumulators open it costs four.  The drains of the two slots no longer hide behind each other's K-loop,
-    // which costs less than the tiles at every size measured: 10240 x 64 x 10240 with a kept operator (DRAM) 680 -> 620 us a
+    // with both accumulators open it costs four.  The drains of the two slots hide behind less of the K-loop than job after
+    // job, which costs less than the tiles at every size measured, with the slots still filled and emptied together: 10240 x 64 x 10240 with a kept operator (DRAM) 680 -> 620 us a
     // call, 131072 x 128 x 4096 9159 -> 8801, 16384 x 16384 x 1024 (power) 11.52 -> 11.10 ms, 4096^3 2371 -> 2358 us.  Not
     // with K segments, whose accumulators take the slots in turn.
     p.pair_squares = !rt.native() && p.mod[0].nseg_all == 1;

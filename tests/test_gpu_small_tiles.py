@@ -53,3 +53,17 @@ def test_three_pass_conversion_on_views(m, n, k, pad, offset):
     got = gh.from_dev(dC)
     assert (np.isnan(got) == np.isnan(want)).all()
     assert (got[~np.isnan(want)] == want[~np.isnan(want)]).all()
+
+
+@pytest.mark.parametrize("k", [1, 128, 129, 384, 385, 896, 1025])
+@pytest.mark.parametrize("m,n", [(700, 600), (700, 100), (1100, 1290)])
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("E", "int8"), ("A", "fp8")])
+def test_square_chains(set_name, sub, m, n, k):
+    """The two chains of a square modulus over 1, 2, 3, 4, 7 and 9 chunks of k (a pair starts with two chunks and goes on one at a time;
+    its ring holds three), several products per pair of blocks, in one block where there are few columns."""
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(k + m + n)
+    A, B = syn._draw(rng, m, k, "normal"), syn._draw(rng, k, n, "lognormal:0.5")
+    got, st = gh.dgemm(A, B, set_name, gh.route(sub) | oz.OZ_ACC_SEPARATE)
+    assert st == 0 and (got == ozo.dgemm(A, B, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS)).all()
