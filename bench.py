@@ -39,6 +39,9 @@ sys.path.insert(0, ROOT)
 
 import synth_inputs as syn  # noqa: E402
 
+# Residues of an output as the whole-method calls store them: 8, 10 or 16 bits each by their modulus (set A: 8).
+STORED_BYTES = {"S": 15.75, "E": 15.25, "A": 15.0}
+
 # DRAM traffic of the residue GEMM relative to its algorithmic bytes (reads / plane bytes, writes /
 # residue bytes) comes from the table in profiles/residue_gemm_dram_traffic.md: ncu captures of a
 # smaller launch, one row per kernel variant, scaled here to the full-size launch by the units.
@@ -457,10 +460,10 @@ def main():
         roof_nominal = 4500.0 / (passes + 1)               # P_low/(3r+1), or P_low/(r+1) native INT8, at B200's dense 8-bit rate
         hbm = peaks["hbm_gbs"]
         dec_bytes = 8 * (m * k + k * n) + (p_store_a * m + p_store * n) * k    # operands read once, planes written, whatever form is taken
-        rb = oz.oz_residue_elem_bytes(modset)                 # bytes per stored residue
-        rec_bytes = (rb * r + 8 + (8 if cfg.beta else 0)) * m * n
+        rb = STORED_BYTES[args.set_name]                      # bytes of all residues of an output
+        rec_bytes = (rb + 8 + (8 if cfg.beta else 0)) * m * n
         plane_bytes = float((p_store_a * m + p_store * n) * k)
-        residue_bytes = float(rb) * r * m * n
+        residue_bytes = float(rb) * m * n
         amp = gemm_dram_amplification(args.set_name, args.substrate)
         lib_peak = lib8["fp8" if args.substrate == "fp8" else "int8"]
         line = {
@@ -472,7 +475,7 @@ def main():
                        "modulus_set": args.set_name, "r": r, "substrate": args.substrate, "quantiser": "RN",
                        "scale_rule": "CS", "storage_mode": "F (A converted inside the product kernel)" if args.fused else "M (materialised planes)",
                        "l2": "inputs larger than L2 (126 MB): A+B %.0f MB, C %.0f MB, planes %.0f MB, residues %.0f MB"
-                             % (8e-6 * (m * k + k * n), 8e-6 * m * n, 1e-6 * p_store * (m + n) * k, 1e-6 * rb * r * m * n),
+                             % (8e-6 * (m * k + k * n), 8e-6 * m * n, 1e-6 * p_store * (m + n) * k, 1e-6 * rb * m * n),
                        "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
             "roof": {"definition": "P_low/(3r+1)" if passes == 3 * r else "P_low/(r+1)", "nominal_tflops": roof_nominal,
                      "frac_of_nominal": value / world / roof_nominal,

@@ -85,8 +85,8 @@ struct Tile {
     static constexpr int TILE_J = BLOCK_M * CG;                  // columns of C per work item
 };
 // Two-plane schedule (SLIM, one tile of columns): a stage holds one of A's planes and the two tiles of B's planes that it
-// meets, one per accumulator.  SLIM is the number of lines of B that are loaded: with 64 a fourth stage fits.  The MMA
-// reads 128 lines all the same; those behind the 64 are whatever follows in the stage and end in columns that no one reads.
+// meets, one per accumulator.  SLIM is the number of lines of B that are loaded: with 64 a fourth stage fits, and the two
+// tiles, one behind the other, are the 128 lines of ONE MMA: both accumulators in one slot, the first in TMEM lanes 0 to 63.
 template <int SLIM, int BN = BLOCK_N>
 struct SlimTile {
     static constexpr int B_BYTES = SLIM * BLOCK_K;
@@ -103,7 +103,7 @@ constexpr int EPI_WARPS = 16;
 constexpr int DRAIN_W = OZ_DRAIN_W;                // accumulator columns per tcgen05.ld of a drain: 64 running
                                                    // values + 16 loaded ones stay inside the 96 registers
 constexpr int XPOSE_BYTES = 16 * 128;                // per epilogue warp: 16 lines x 128 bytes
-constexpr size_t SMEM_BYTES = RING_BYTES + EPI_WARPS * XPOSE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+constexpr size_t SMEM_BYTES = RING_BYTES + EPI_WARPS * XPOSE_BYTES + 1024 /*alignment slack*/ + 384 /*barriers*/;
 
 struct ModInfo {
     float m, inv_m;
@@ -204,6 +204,10 @@ __device__ __forceinline__ void mbar_arrive_relaxed(uint32_t bar)
     asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_addr)
 {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
@@ -318,6 +322,19 @@ __device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t da, uint64_t db, 
     if (SUB == 0 && CG == 2) OZ_UMMA("2", "f8f6f4");
     if (SUB == 1 && CG == 1) OZ_UMMA("1", "i8");
     if (SUB == 1 && CG == 2) OZ_UMMA("2", "i8");
+#undef OZ_UMMA
+}
+
+// the same for one CTA, always accumulating, into TMEM lanes 64 to 127 only
+template <int SUB>
+__device__ __forceinline__ void umma_upper(uint32_t d_tmem, uint64_t da, uint64_t db, uint32_t idesc)
+{
+#define OZ_UMMA(KIND)                                                                             \
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"                               \
+                 "tcgen05.mma.cta_group::1.kind::" KIND " [%0], %1, %2, %3, {%4, %4, %5, %5}, p;\n\t}" \
+                 ::"r"(d_tmem), "l"(da), "l"(db), "r"(idesc), "r"(0xFFFFFFFFu), "r"(0u) : "memory")
+    if (SUB == 0) OZ_UMMA("f8f6f4");
+    else OZ_UMMA("i8");
 #undef OZ_UMMA
 }
 
@@ -536,7 +553,13 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     constexpr int STAGES = SLIM ? Slim::STAGES : Tile<CG, BN>::STAGES;
     constexpr int STAGE_BYTES = SLIM ? Slim::STAGE_BYTES : Tile<CG, BN>::STAGE_BYTES;
     constexpr int COLS_PER_WARP = BN / 4;                // four warps share a TMEM lane quarter
-    static_assert(16 * STAGES + 48 <= 256, "barriers");
+    // Both accumulators of a modulus in one slot, one above the other: half the MMAs, which bound a block whose SM is not waiting for
+    // memory (a stage of 48 KiB takes 512 cycles instead of 1024), and the other slot free for the next product.  GEMM in us, two MMAs -> one:
+    // 10240 x 64 x 10240 482 -> 416 (the last of its 3.24 rounds over the SMs 98 -> 61), 9472 rows (3 rounds) 384 -> 355; calls on kept
+    // operands: set E 1104 x 18 x 2754 47.0 -> 36.7, A 1402 x 26 x 7026 125 -> 92.  For it half of the epilogue hands its sums to the other half.
+    constexpr bool STACKED = SLIM == 64;
+    constexpr int NUM_HANDS = 8;                         // pairs of epilogue warps that hand over the second accumulator
+    static_assert(16 * STAGES + 48 + 16 * NUM_HANDS <= 384, "barriers");
     // CTA pair: rank 0 leads (issues the MMAs, owns the `full` and `tmem-empty` barriers that both
     // CTAs signal); work items are dealt to pairs, so both CTAs walk the same item sequence.
     const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
@@ -551,6 +574,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     const uint32_t tfull_bar = bars + 16 * STAGES;                    // 2 x 8
     const uint32_t tempty_bar = tfull_bar + 16;                       // 2 x 8
     const uint32_t tmem_slot = tempty_bar + 16;                       // 4 bytes: TMEM base address
+    const uint32_t hand_bar = tmem_slot + 16;                         // NUM_HANDS x (written, taken)
     unsigned char *xpose_base = smem_raw + (tiles - raw) + RING_BYTES;
     unsigned char *gen = xpose_base + EPI_WARPS * XPOSE_BYTES;
     volatile uint32_t *tmem_base_ptr = reinterpret_cast<volatile uint32_t *>(gen + 16 * STAGES + 32);
@@ -572,6 +596,8 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             mbar_init(tfull_bar + 8 * s, 1);
             mbar_init(tempty_bar + 8 * s, EPI_WARPS * CG);   // pair: the peer's epilogue warps arrive too
         }
+        if constexpr (STACKED)
+            for (int s = 0; s < 2 * NUM_HANDS; ++s) mbar_init(hand_bar + 8 * s, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -676,10 +702,15 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     // kind 5: A's second plane is -16 d1, which the tensor core negates
                     const uint32_t idesc1 = mi.kind == 5 ? idesc | kNegateB : idesc;
                     for (int seg = 0; ok && seg < mi.nseg_all; ++seg) {
-                        for (int h = 0; ok && h < 2; ++h)
-                            ok = wait(tempty_bar + 8 * h, ((slot_phase >> h) & 1u) ^ 1u);
+                        if constexpr (STACKED) {
+                            ok = wait(tempty_bar + 8 * slot, ((slot_phase >> slot) & 1u) ^ 1u);
+                        } else {
+                            for (int h = 0; ok && h < 2; ++h)
+                                ok = wait(tempty_bar + 8 * h, ((slot_phase >> h) & 1u) ^ 1u);
+                        }
                         if (!ok) break;
                         tc_fence_after();
+                        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(slot * BLOCK_N);
                         const int kc0 = seg * mi.seg_len_all, kc1 = min(p.nk, kc0 + mi.seg_len_all);
                         for (int st = 0; st < 2 * (kc1 - kc0); ++st) {
                             const int h = st & 1;
@@ -693,8 +724,14 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                                 for (int ks = 0; ks < BLOCK_K / UMMA_K; ++ks) {
                                     const uint64_t o = static_cast<uint64_t>(ks * (UMMA_K >> 4));
                                     const uint32_t accumulate = st > 0 || ks > 0 ? 1u : 0u, id = h ? idesc1 : idesc;
-                                    if (mi.kind != 0 || h == 0) umma<SUB, CG>(tmem_base, e0 + o, a + o, id, accumulate);
-                                    umma<SUB, CG>(tmem_base + BLOCK_N, e1 + o, a + o, id, accumulate);
+                                    if constexpr (STACKED) {
+                                        // d1 of a square meets e0 only, in the second accumulator
+                                        if (mi.kind != 0 || h == 0) umma<SUB, CG>(d_tmem, e0 + o, a + o, id, accumulate);
+                                        else umma_upper<SUB>(d_tmem, e0 + o, a + o, idesc);
+                                    } else {
+                                        if (mi.kind != 0 || h == 0) umma<SUB, CG>(tmem_base, e0 + o, a + o, id, accumulate);
+                                        umma<SUB, CG>(tmem_base + BLOCK_N, e1 + o, a + o, id, accumulate);
+                                    }
                                 }
                                 umma_commit<CG>(empty_bar + 8 * stage);
                             }
@@ -702,10 +739,11 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                         }
                         if (!ok) break;
                         if (leader) {
-                            umma_commit<CG>(tfull_bar);
-                            umma_commit<CG>(tfull_bar + 8);
+                            umma_commit<CG>(tfull_bar + 8 * slot);
+                            if constexpr (!STACKED) umma_commit<CG>(tfull_bar + 8 * (slot ^ 1));
                         }
-                        slot_phase ^= 3u;
+                        if constexpr (STACKED) { slot_phase ^= 1u << slot; slot ^= 1; }
+                        else slot_phase ^= 3u;
                     }
                     continue;
                 }
@@ -814,6 +852,9 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
         const int q = warp & 3;                              // TMEM lane quarter this warp may read
         const int part = (warp - FIRST_EPI_WARP) >> 2;       // which 64 of the tile's 256 TMEM columns (any four
                                                              // consecutive warps cover the four lane quarters)
+        // STACKED: warps of lanes 64 to 127 drain the second accumulator and hand it to those of lanes 0 to 63
+        const bool second = STACKED && q >= 2;
+        uint32_t hand_phase = 0;
         int slot = 0;
         uint32_t slot_phase = 0;   // bit s = phase of slot s
         bool ok = true;
@@ -827,15 +868,15 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             // running combination per element: FP32 (FP8 route) or INT32 (INT8 routes), as raw bits
             uint32_t comb[COLS_PER_WARP];
             if constexpr (!DIRECT) {
-                const uint32_t start = SUB == 0 ? (PACKED ? __float_as_uint(-mi.centre) : 0u) : (BIASED ? ibias : 0u);
+                const uint32_t start = second ? 0u : SUB == 0 ? (PACKED ? __float_as_uint(-mi.centre) : 0u) : (BIASED ? ibias : 0u);
 #pragma unroll
                 for (int c = 0; c < COLS_PER_WARP; ++c) comb[c] = start;
             }
             // SLIM: both jobs of a K segment before the next segment.  (The bound is read where it is compared: in a register of its
             // own it costs the public FP8 pair 72 bytes of spills instead of 40.)
             for (int o = 0; ok && o < (SLIM ? mi.nseg_all : mi.njobs); ++o)
-            for (int i = 0, inner = SLIM ? 2 : job_segments(mi, o); ok && i < inner; ++i) {
-                const int job = SLIM ? i : o;
+            for (int i = 0, inner = STACKED ? 1 : SLIM ? 2 : job_segments(mi, o); ok && i < inner; ++i) {
+                const int job = STACKED ? q >> 1 : SLIM ? i : o;
                 // every lane polls for itself; the outcome is made warp-uniform before anything that
                 // contains a warp barrier depends on it
                 ok = __all_sync(0xFFFFFFFFu, mbar_wait(tfull_bar + 8 * slot, (slot_phase >> slot) & 1u, abort_flag, p.status));
@@ -917,6 +958,35 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             const int64_t jw = static_cast<int64_t>(it.tn) * Tile<CG>::TILE_J + rank * BLOCK_M + q * 32;   // first column of the warp
             const int64_t j = jw + lane;
             const int64_t i0 = static_cast<int64_t>(it.tm) * BN + part * COLS_PER_WARP;
+            if constexpr (STACKED) {
+                // through 4 KiB of shared memory a pair of warps, a word of every lane at a time: no bank conflicts
+                constexpr int PIECE = COLS_PER_WARP < 32 ? COLS_PER_WARP : 32;
+                const int pair = part * 2 + (q & 1);
+                if (i0 < p.m && (q & 1) * 32 < p.n) {
+                    uint32_t *box = reinterpret_cast<uint32_t *>(xpose_base + pair * (2 * XPOSE_BYTES)) + lane;
+                    const uint32_t written = hand_bar + 16 * pair, taken = written + 8;
+#pragma unroll
+                    for (int c0 = 0; c0 < COLS_PER_WARP; c0 += PIECE) {
+                        ok = ok && __all_sync(0xFFFFFFFFu, mbar_wait(second ? taken : written, second ? hand_phase ^ 1u : hand_phase, abort_flag, p.status));
+                        if (ok) {
+                            if (second) {
+#pragma unroll
+                                for (int c = 0; c < PIECE; ++c) box[32 * c] = comb[c0 + c];
+                            } else {
+#pragma unroll
+                                for (int c = 0; c < PIECE; ++c) {
+                                    if constexpr (SUB == 0) comb[c0 + c] = __float_as_uint(__uint_as_float(comb[c0 + c]) + __uint_as_float(box[32 * c]));
+                                    else comb[c0 + c] += box[32 * c];
+                                }
+                            }
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(second ? written : taken);
+                        }
+                        hand_phase ^= 1u;
+                    }
+                    if (!ok) break;
+                }
+            }
             if (i0 >= p.m || jw >= p.n) continue;                                 // warp-uniform
             if constexpr (BOUND) {
                 // The accumulators are non-negative integers held exactly in FP32: their bit patterns
@@ -1396,15 +1466,11 @@ bool two_plane_applies(int64_t m, int64_t n, const Route &rt)
     return rt.automatic && rt.merged() && !rt.fused && n <= BLOCK_M && m >= n;
 }
 
-// Kept operands (planes of the merged layouts): a fifth less of A from memory for a sixth more products, and K segments on set S.
-// Taken up to 64 columns, and where the tiles cover the SMs or one segment holds k (the call with three planes and with two, S:
-// 10240 x 64 x 10240 558 -> 541 us, 10240 x 16 x 10240 558 -> 523; 6000 x 32 x 3000 on A 158 -> 139; 4000 x 64 x 4000 the same; 1500 x 16 x 6000
-// on E 95 -> 97; not 1000 x 32 x 12000 on S: 138 -> 146, nor 100 columns: 4000 x 100 x 4000 119 -> 118).
-static bool slim_merged(int64_t m, int64_t n, int64_t k, int set, int sms)
-{
-    const int64_t tiles = set_r(set) * ((m + BLOCK_N - 1) / BLOCK_N);
-    return n <= 64 && (tiles >= sms || k <= (set == 0 ? 3840 : 15360));
-}
+// Kept operands (planes of the merged layouts): a fifth less of A from memory for a sixth more products, which up to 64 columns both
+// accumulators share.  Calls with three planes and with two, us: set S 2126 x 9 x 8360 109 -> 89, 1200 x 64 x 9000 113 -> 87, 3000 x 64 x 30000
+// (eight K segments) 457 -> 373; E 1900 x 50 x 20000 247 -> 196; A 800 x 50 x 16000 193 -> 144.  Not with more columns, whose
+// accumulators need products of their own: 4000 x 100 x 4000 119 -> 118.
+static bool slim_merged(int64_t n) { return n <= 64; }
 
 ResidueTiling residue_tiling(int64_t m, int64_t n, int set)
 {
@@ -1442,7 +1508,7 @@ oz_status_t launch_residue_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *
     p.patch_bytes = patch_bytes(set);
     p.stall_producer = take_stall_flag();
     p.status = device_status_word();
-    const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(m, n, k, set, sms)));
+    const bool slim = tiled && cg == 1 && p.tiles_n == 1 && (rt.two_plane() || (rt.merged() && rt.substrate == 0 && slim_merged(n)));
     fill_mod_info(p, set, rt, k, slim);
     // Squares in one K-loop: the products of a square read d0 and e0 twice, so job after job a K chunk costs six tiles;
     // with both accumulators open it costs four.  The drains of the two slots hide behind less of the K-loop than job after

@@ -53,3 +53,27 @@ def test_depth_with_like_signs(set_name, m, n, k):
     dC = torch.zeros((n, m), dtype=torch.float64, device="cuda")
     oz.check(oz.oz_dgemm_prepared(m, n, k, 1.0, *ops, 0.0, dC, m, sid, rt), "oz_dgemm_prepared")
     assert gh.sync_status() == 0 and (gh.from_dev(dC) == want).all()
+
+
+@pytest.mark.parametrize("sub", ["fp8", "int8"])
+@pytest.mark.parametrize("m,n,k", [(40, 1, 33), (200, 31, 300), (300, 32, 129), (2000, 33, 260), (700, 63, 1000), (9600, 64, 130), (500, 64, 4300)])
+def test_stacked_accumulators(sub, m, n, k):
+    """At most 64 columns: both accumulators of a modulus from one chain, handed from one half of the epilogue to the other.  Edges of the
+    warps' 32 columns, tiles of 64 and of 256 rows, several products a block and several K segments; whole calls and kept operands."""
+    import torch
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m + n + k)
+    A, B = syn._draw(rng, m, k, "normal"), syn._draw(rng, k, n, "lognormal:0.5")
+    rt = gh.route(sub)
+    for set_name, sid in gh.SETS.items():
+        want = ozo.dgemm(A, B, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS)
+        got, st = gh.dgemm(A, B, set_name, rt)
+        assert st == 0 and (got == want).all()
+        block = [torch.empty(oz.oz_operand_bytes(side, lines, k, sid, rt), dtype=torch.uint8, device="cuda") for side, lines in ((0, m), (1, n))]
+        oz.check(oz.oz_prepare_operand(0, m, k, gh.to_dev(A), m, sid, rt, block[0]), "oz_prepare_operand A")
+        oz.check(oz.oz_prepare_operand(1, n, k, gh.to_dev(B), k, sid, rt, block[1]), "oz_prepare_operand B")
+        gh.ensure_workspace(oz.oz_product_workspace_bytes(m, n, sid))
+        dC = gh.to_dev(np.zeros((m, n), order="F"))
+        oz.check(oz.oz_dgemm_prepared(m, n, k, 1.0, *block, 0.0, dC, m, sid, rt), "oz_dgemm_prepared")
+        assert gh.sync_status() == 0 and (gh.from_dev(dC) == want).all()
