@@ -393,7 +393,7 @@ oz_status_t product_impl(int64_t m, int64_t n, int64_t k, double alpha, const Op
 {
     const bool ev = g_stage_events_on[dev];
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][2], stream));
-    // the residues stay inside this call: tile-ordered, and the two-byte sets skip the canonicalisation
+    // the residues stay inside this call: tile-ordered, in the bits of their moduli
     oz_status_t st = launch_residue_gemm(m, n, k, a.planes, a.stride, a.pitch, b.planes, b.stride, b.pitch, set,
                                          rt, R, 0, 0, true, stream);
     if (st != OZ_OK) return st;
