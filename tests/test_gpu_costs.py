@@ -1,0 +1,62 @@
+"""What a call must not pay for: device times of the same work on other data or another leading dimension, as ratios.  The bounds
+leave about half as much again as the ratios that the kernels show; the forms that they guard against lie above them."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROUTES = [("S", "fp8"), ("E", "fp8"), ("A", "int8n")]
+
+
+def _ratio(slow, fast, tries=12):
+    """Least device time of `slow` over that of `fast`, taken in turn."""
+    import torch
+    ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    best = [float("inf"), float("inf")]
+    for t in range(tries + 2):
+        for i, f in enumerate((slow, fast)):
+            ev[0].record()
+            for _ in range(3):
+                f()
+            ev[1].record()
+            ev[1].synchronize()
+            if t >= 2:
+                best[i] = min(best[i], ev[0].elapsed_time(ev[1]))
+    return best[0] / best[1]
+
+
+def _normal(rows, cols, seed):
+    import torch
+    return torch.randn((cols, rows), dtype=torch.float64, device="cuda", generator=torch.Generator(device="cuda").manual_seed(seed))
+
+
+def _residues(set_name, n, ldr, numbers, seed):
+    """Random residues (numbers None), or those of whole numbers up to `numbers` in magnitude, for n columns of ldr rows."""
+    import torch
+
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    moduli = oz.oz_set_info(gh.SETS[set_name])[2]
+    dt = gh.residue_dtype(set_name)[0]
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    if numbers is None:
+        return torch.stack([torch.randint(0, mm, (n, ldr), device="cuda", generator=g, dtype=torch.int32).to(dt) for mm in moduli])
+    x = torch.randint(-numbers, numbers + 1, (n, ldr), device="cuda", generator=g, dtype=torch.int64)
+    return torch.stack([(x % mm).to(torch.int32).to(dt) for mm in moduli])
+
+
+@pytest.mark.parametrize("set_name,sub", ROUTES)
+@pytest.mark.parametrize("beta", [0.0, 1.0])
+def test_odd_leading_dimension_of_the_residues(set_name, sub, beta):
+    """Residues element by element, against the words that the next even leading dimension allows."""
+    import torch
+
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    m, n = 3001, 2999
+    sA, sB = torch.zeros(m, dtype=torch.int32, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    C = _normal(m, n, 1)
+    calls = []
+    for ldr in (3001, 3008):
+        R = _residues(set_name, n, ldr, None, 2)
+        calls.append(lambda R=R, ldr=ldr: oz.check(oz.oz_reconstruct(m, n, R, ldr, n * ldr, sA, sB, gh.SETS[set_name], -1.0, beta, C, m)))
+    assert _ratio(*calls) < 1.8
