@@ -10,8 +10,8 @@
 // into a high and a middle part of at most 21 signed bits and the rest: the sums of the first two are integers below 2^53
 // (group_bounds()) and formed EXACTLY by FP64 fused multiply-adds, that of the third is off by less than kRestError.
 // kappa = round(S/M) comes from a floating estimate; error-free additions then give the correctly rounded FP64 value unless
-// c' lies within kRestError of a rounding boundary, is so small that this error counts, or lies near +-M/2 -- those rare
-// outputs take an exact path: the 128-bit integer, an exact range test for the lift to [-M/2, M/2), and one
+// c' lies within kRestError of a rounding boundary, is so small that this error counts, or lies near +-M/2.  The first two kinds are settled
+// from c' modulo 2^64 (settle_rows()); for the last, an exact path: the 128-bit integer, an exact range test for the lift to [-M/2, M/2), and one
 // round-to-nearest-even done in integer arithmetic.  A term for every modulus, three parts of 38 or 40 bits each, took 36 (S) to 45 (A)
 // FP64 multiply-adds and 12 to 15 conversions an output where this takes 18 and 6 (A: 15 and 5).
 // A thread handles four rows of a column, two where the outputs are few.
@@ -358,10 +358,64 @@ __device__ __forceinline__ void first_row(Numbers &w, int h)
     }
 }
 
-// The thread's rows (bit h) whose c' is zero if it is below 2^(kRestErrorLog2 + 3) in magnitude: products with structural zeros have many.  It is zero where
-// the products of two groups, together larger than that, divide it.
+// ---- results that a floating sum with an inexact rest leaves undecided: near a rounding boundary, or small ----
+// r is an integer near c', and c' modulo 2^64 takes two integer multiply-adds a group: c' - r is the difference modulo 2^64 with its sign,
+// exact as a double, and r + (c' - r) is c' correctly rounded by that one addition.  For |r| below 2^kSettledLog2: the difference, the rest's error and half an
+// ulp of r, stays below 2^53, and kappa is far from a tie.  Products with structural zeros, decaying or graded operands have such results by the
+// million: 4000 x 4000 x 500 updates of graded operands (N(0,1) exp(-|i - j| / 5), results 2^-30 to 2^-80 of the bound) by the 128-bit sum below, row after
+// row, 604 us a call on S, 601 on E, 434 on A, by this form 416, 410 and 299, where every result settled by the floating sum takes 380, 400 and 270.
+constexpr int kSettledLog2 = 104;
+template <int SET> constexpr bool kSettles = kRestErrorLog2<SET> < 50 && static_cast<double>(half_M_word(SET) >> 20) > 1023.0 + kSettledLog2 + 4.0;
+static_assert(kSettles<0> && kSettles<1> && kSettles<2>, "a difference that a double holds, kappa within a tenth of an integer");
+__device__ __forceinline__ bool settles(double r) { return 2u * static_cast<uint32_t>(__double2hiint(r)) < 2u * (static_cast<uint32_t>(1023 + kSettledLog2) << 20); }
+
+// kappa = round(sum of u_g / P_g) by integers: 2^share_bits() / P_g fits 31 bits
+__host__ __device__ constexpr int share_bits(int set)
+{
+    uint64_t least = group_product(set, 0);
+    for (int g = 1; g < set_groups(set); ++g) least = group_product(set, g) < least ? group_product(set, g) : least;
+    int b = 31;
+    while (b < 50 && ((2ull << b) / least) >> 31 == 0) ++b;
+    return b;
+}
+__host__ __device__ constexpr int32_t share_factor(int set, int g) { return static_cast<int32_t>((1ull << share_bits(set)) / group_product(set, g)); }
+template <int SET> constexpr bool kShares = group_bounds(SET).kappa * pow2d(share_bits(SET)) < pow2d(62) &&
+                                            set_groups(SET) * pow2d(31) < pow2d(share_bits(SET) - 3);
+static_assert(kShares<0> && kShares<1> && kShares<2>, "the sum of the shares fits 63 bits and is within an eighth");
+
+// + u w modulo 2^64, the low word of w balanced
+__device__ __forceinline__ void add_low(int u, uint64_t w, uint64_t &low, uint32_t &high)
+{
+    const int32_t l = static_cast<int32_t>(static_cast<uint32_t>(w));
+    low += static_cast<uint64_t>(static_cast<int64_t>(u) * l);
+    high += static_cast<uint32_t>(u) * static_cast<uint32_t>((w - static_cast<uint64_t>(static_cast<int64_t>(l))) >> 32);
+}
+
+// an integer r, |r| < 2^116, modulo 2^64
+__device__ __forceinline__ uint64_t low_bits(double r)
+{
+    const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(r)), sig = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const int e = (__double2hiint(r) >> 20 & 0x7FF) - 1075;
+    const uint64_t v = e >= 0 ? sig << (e & 63) : e >= -52 ? sig >> (-e & 63) : 0ull;
+    return __double2hiint(r) < 0 ? 0ull - v : v;
+}
+
+template <int SET, int... G>
+__device__ __forceinline__ double settled(std::integer_sequence<int, G...>, const int (&u)[kMaxGroups], double r)
+{
+    int64_t share = 1ll << (share_bits(SET) - 1);
+    ((share += static_cast<int64_t>(u[G]) * share_factor(SET, G)), ...);
+    uint64_t low = 0ull;
+    uint32_t high = 0u;
+    (add_low(u[G], group_weight(SET, G).lo, low, high), ...);
+    add_low(-static_cast<int>(share >> share_bits(SET)), group_weight(SET, -1).lo, low, high);
+    return r + static_cast<double>(static_cast<int64_t>(low + (static_cast<uint64_t>(high) << 32) - low_bits(r)));
+}
+
+// The thread's rows (bit h) whose c' is zero if it is below 2^(kRestErrorLog2 + 3) in magnitude.  It is zero where the products of two
+// groups, together larger than that, divide it: a third of the work of settle_rows(), for products with structural zeros.
 template <int SET, int ROWS, class Loader, int... H>
-__device__ __noinline__ uint32_t zero_rows(std::integer_sequence<int, H...>, Loader from)
+__device__ __forceinline__ uint32_t zero_rows(std::integer_sequence<int, H...>, const Loader &from)
 {
     constexpr int64_t P0 = static_cast<int64_t>(group_product(SET, 0)), P1 = static_cast<int64_t>(group_product(SET, 1));
     static_assert(static_cast<double>(P0) * static_cast<double>(P1) > pow2d(kRestErrorLog2<SET> + 4), "two groups tell");
@@ -371,6 +425,21 @@ __device__ __noinline__ uint32_t zero_rows(std::integer_sequence<int, H...>, Loa
     if constexpr (a2 >= 0) load_numbers(std::integer_sequence<int, a2>{}, from, w);
     if constexpr (b2 >= 0) load_numbers(std::integer_sequence<int, b2>{}, from, w);
     return ((group_value<SET, Loader::kPrivate, H, 0>(w) % static_cast<int>(P0) == 0 && group_value<SET, Loader::kPrivate, H, 1>(w) % static_cast<int>(P1) == 0 ? 1u << H : 0u) | ...);
+}
+
+template <int SET, int ROWS, class Loader, int... H>
+__device__ __forceinline__ void settle_rows(std::integer_sequence<int, H...>, const Loader &from, double (&r)[ROWS])
+{
+    Numbers w;
+    load_numbers(std::make_integer_sequence<int, set_r(SET)>{}, from, w);
+    auto one = [&](auto index) {
+        constexpr int h = decltype(index)::value;
+        constexpr auto groups = std::make_integer_sequence<int, set_groups(SET)>{};
+        int u[kMaxGroups] = {};
+        group_values<SET, Loader::kPrivate, h>(groups, w, u);
+        r[h] = settles(r[h]) ? settled<SET>(groups, u, r[h]) : r[h];
+    };
+    (one(std::integral_constant<int, H>{}), ...);
 }
 
 // alpha 2^-(sa + sb) c' (alpha = 1 or -1, as a sign bit) where only the scale is out of reach: r is c' correctly rounded.  NaN for a line with
@@ -458,6 +527,56 @@ template <int SET> constexpr uint32_t kRangeSpan = 2u * (half_M_word(SET) - smal
 template <int SET>
 __device__ __forceinline__ uint32_t range_word(double r) { return 2u * static_cast<uint32_t>(__double2hiint(r)) - 2u * small_word(SET); }
 
+template <bool PRIVATE> __device__ __forceinline__ constexpr int row_of(int h) { return (h & 1) + (PRIVATE ? 8 : 2) * (h >> 1); }
+// alpha 2^-(sa + sb) c' for all rows of a thread, one of which at least is not as row_value() leaves it.  sure: the rows that
+// row_value() calls rounded (bit h).
+template <int ROWS> struct Results { double r[ROWS]; };
+template <int ROWS> struct Shifts { int s[ROWS]; };
+template <int SET, int ROWS, class Loader, int... H>
+__device__ __forceinline__ Results<ROWS> finish_rows(std::integer_sequence<int, H...> rows, const Loader &from, Results<ROWS> v, const Shifts<ROWS> &sa, int sb,
+                                                     int alpha_sign, int nrows, uint32_t sure)
+{
+    // rows of C whose result is not known to be rounded; those among them near zero
+    uint32_t open = 0u, least = 0u;
+    constexpr uint32_t small = 2u * (static_cast<uint32_t>(1023 + kRestErrorLog2<SET> + 2) << 20);       // |c'| is below twice the bound of |r|
+#pragma unroll
+    for (int h = 0; h < ROWS; ++h) {
+        if (((sure >> h & 1u) && range_word<SET>(v.r[h]) < kRangeSpan<SET>) || marked(sa.s[h], sb) || row_of<Loader::kPrivate>(h) >= nrows) continue;
+        open |= 1u << h;
+        if (2u * static_cast<uint32_t>(__double2hiint(v.r[h])) < small) least |= 1u << h;
+    }
+    if (open != 0u && open == least) {
+        const uint32_t zeros = zero_rows<SET, ROWS>(rows, from) & open;
+#pragma unroll
+        for (int h = 0; h < ROWS; ++h) v.r[h] = zeros >> h & 1u ? 0.0 : v.r[h];
+        open &= ~zeros;
+    }
+    if (open != 0u) {
+        settle_rows<SET, ROWS>(rows, from, v.r);
+#pragma unroll
+        for (int h = 0; h < ROWS; ++h)
+            if (settles(v.r[h])) open &= ~(1u << h);
+    }
+#pragma unroll
+    for (int h = 0; h < ROWS; ++h) {
+        const uint32_t sum = static_cast<uint32_t>(sa.s[h]) + static_cast<uint32_t>(sb);
+        if (open >> h & 1u) v.r[h] = row_value_exact<SET>(from, h, sa.s[h], sb, alpha_sign);
+        else if (sum + 904u <= 1924u && static_cast<uint32_t>(sa.s[h]) + (1u << 30) < 1u << 31)
+            v.r[h] *= __hiloint2double(static_cast<int>((1023u - sum) << 20) ^ alpha_sign, 0);
+        else v.r[h] = row_value_far(v.r[h], sa.s[h], sb, alpha_sign);
+    }
+    return v;
+}
+
+// Out of line for four rows a thread of the private layout, whose registers are full: what it needs then costs the common case none of them (all but
+// two variants without spills; inline, which keeps the numbers from the first load, 20 to 50 bytes: plain 4000 x 4000 x 500 updates 2 percent slower).
+template <int SET, int ROWS, class Loader, int... H>
+__device__ __noinline__ Results<ROWS> finish_rows_call(std::integer_sequence<int, H...> rows, Loader from, Results<ROWS> v, Shifts<ROWS> sa, int sb,
+                                                       int alpha_sign, int nrows, uint32_t sure)
+{
+    return finish_rows<SET, ROWS>(rows, from, v, sa, sb, alpha_sign, nrows, sure);
+}
+
 // scalar stores of up to two consecutive rows; `first` / `second`: which of them are written
 __device__ __forceinline__ void store_pair(double *out, double p0, double p1, bool first, bool second, double beta)
 {
@@ -469,7 +588,6 @@ __device__ __forceinline__ void store_pair(double *out, double p0, double p1, bo
 // For beta = 1 the old values of C are requested before the arithmetic starts, so that their latency
 // hides behind it.  nrows: rows of C from `row` on.  `keep`: bit h set = the thread's row h is written (rows that go to the native FP64 path are not).
 // The tests of a thread's rows are taken together: one branch a thread, which almost none takes.
-template <bool PRIVATE> __device__ __forceinline__ constexpr int row_of(int h) { return (h & 1) + (PRIVATE ? 8 : 2) * (h >> 1); }
 template <int SET, int ROWS, class Loader, int... H>
 __device__ __forceinline__ void reconstruct_rows(std::integer_sequence<int, H...>, const Loader &from, int64_t row, int nrows, int sb,
                                                  const int32_t *__restrict__ shiftA, double alpha, double beta,
@@ -510,29 +628,17 @@ __device__ __forceinline__ void reconstruct_rows(std::integer_sequence<int, H...
         all = all && rounded[h];
     }
     if (!(all && far <= 1924u && wide < 1u << 31 && range < kRangeSpan<SET>)) {
-        constexpr uint32_t small = 2u * (static_cast<uint32_t>(1023 + kRestErrorLog2<SET> + 2) << 20);       // |c'| is below twice the bound of |r|
-        uint32_t least = 0xFFFFFFFFu, zeros = 0u;
+        uint32_t sure = 0u;
 #pragma unroll
-        for (int h = 0; h < ROWS; ++h) least = min(least, 2u * static_cast<uint32_t>(__double2hiint(r[h])));
-        if (least < small) zeros = zero_rows<SET, ROWS>(std::integer_sequence<int, H...>{}, from);
-        auto fix = [&](auto index) {
-            constexpr int h = decltype(index)::value;
-            if (2u * static_cast<uint32_t>(__double2hiint(r[h])) < small && (zeros >> h & 1u) && !marked(sa[h], sb)) {
-                r[h] = 0.0;
-                scale[h] = 0x3FF00000u ^ static_cast<uint32_t>(alpha_sign);
-                return;
-            }
-            const bool good = rounded[h] && range_word<SET>(r[h]) < kRangeSpan<SET>;
-            const bool near = static_cast<uint32_t>(sa[h]) + static_cast<uint32_t>(sb) + 904u <= 1924u && static_cast<uint32_t>(sa[h]) + (1u << 30) < 1u << 31;
-            if (good && near) return;
-            if (good) {
-                r[h] = row_value_far(r[h], sa[h], sb, alpha_sign);
-            } else if (row_of<PRIVATE>(h) < nrows) {
-                r[h] = row_value_exact<SET>(from, h, sa[h], sb, alpha_sign);
-            }
+        for (int h = 0; h < ROWS; ++h) sure |= rounded[h] ? 1u << h : 0u;
+        Results<ROWS> v;
+        if constexpr (PRIVATE && ROWS == 4) v = finish_rows_call<SET, ROWS>(std::integer_sequence<int, H...>{}, from, {{r[H]...}}, {{sa[H]...}}, sb, alpha_sign, nrows, sure);
+        else v = finish_rows<SET, ROWS>(std::integer_sequence<int, H...>{}, from, {{r[H]...}}, {{sa[H]...}}, sb, alpha_sign, nrows, sure);
+#pragma unroll
+        for (int h = 0; h < ROWS; ++h) {
+            r[h] = v.r[h];
             scale[h] = 0x3FF00000u;
-        };
-        (fix(std::integral_constant<int, H>{}), ...);
+        }
     }
 #pragma unroll
     for (int p = 0; p < ROWS / 2; ++p) {

@@ -45,6 +45,48 @@ def _residues(set_name, n, ldr, numbers, seed):
 
 
 @pytest.mark.parametrize("set_name,sub", ROUTES)
+@pytest.mark.parametrize("numbers", [0, 2 ** 60])
+def test_small_results_of_the_stage(set_name, sub, numbers):
+    """Results that are zero or far below the bound of their row and column, by the public layout."""
+    import torch
+
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    m = n = 4000
+    sA, sB = (torch.zeros(m, dtype=torch.int32, device="cuda") for _ in range(2))
+    C = _normal(m, n, 1)
+    calls = []
+    for top in (numbers, None):
+        R = _residues(set_name, n, m, top, 2)
+        calls.append(lambda R=R: oz.check(oz.oz_reconstruct(m, n, R, m, n * m, sA, sB, gh.SETS[set_name], -1.0, 1.0, C, m)))
+    assert _ratio(*calls) < (1.3 if numbers == 0 else 1.7)
+
+
+@pytest.mark.parametrize("set_name,sub", ROUTES)
+def test_small_results_of_a_product(set_name, sub):
+    """One large entry in every row of A and column of B, so that nearly every result lies far below its bound."""
+    import torch
+
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    m = n = 4000
+    k, rt = 128, gh.route(sub)
+    gh.ensure_workspace(oz.oz_product_workspace_bytes(m, n, gh.SETS[set_name]))
+    C = _normal(m, n, 1)
+    calls = []
+    for spike in (1e6, 1.0):
+        A, B = _normal(m, k, 2), _normal(k, n, 3)
+        A[torch.arange(m, device="cuda") % k, torch.arange(m, device="cuda")] *= spike
+        B[torch.arange(n, device="cuda"), (torch.arange(n, device="cuda") * 7 + 3) % k] *= spike
+        ops = [torch.empty(oz.oz_operand_bytes(s, m, k, gh.SETS[set_name], rt), dtype=torch.uint8, device="cuda") for s in (0, 1)]
+        oz.check(oz.oz_prepare_operand(0, m, k, A, m, gh.SETS[set_name], rt, ops[0]))
+        oz.check(oz.oz_prepare_operand(1, n, k, B, k, gh.SETS[set_name], rt, ops[1]))
+        calls.append(lambda ops=ops: oz.check(oz.oz_dgemm_prepared(m, n, k, -1.0, ops[0], ops[1], 1.0, C, m, gh.SETS[set_name], rt)))
+    assert _ratio(*calls) < 1.6
+    gh.sync_status()
+
+
+@pytest.mark.parametrize("set_name,sub", ROUTES)
 @pytest.mark.parametrize("beta", [0.0, 1.0])
 def test_odd_leading_dimension_of_the_residues(set_name, sub, beta):
     """Residues element by element, against the words that the next even leading dimension allows."""

@@ -97,3 +97,48 @@ def test_stored_forms_and_small_results(set_name, sub, recon, m, n, k):
         got = gh.from_dev(dC)
         want = ozo.dgemm(Af, Bf, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS, alpha=alpha, beta=beta, C0=C0)
         assert (got[:m] == want).all() and (got[m:] == 3.0).all()
+
+
+@pytest.mark.parametrize("set_name", ["S", "E", "A"])
+@pytest.mark.parametrize("ldr", [None, 1024, 1025])
+def test_integers_of_every_magnitude(set_name, ldr):
+    """c' of every bit length up to M/2: a power of two and its neighbours, the ties of every length above 53 bits and theirs, random ones; four
+    shifts each, so that rows that the floating sum settles lie beside rows that it leaves open."""
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(11)
+    ms = ozo.modset(OSET[set_name])
+    M = int(np.prod([int(v) for v in ms], dtype=object))
+    xs = [0]
+    for e in range(M.bit_length() - 1):
+        tie = 2 ** e + 2 ** max(e - 53, 0)
+        x = 2 ** e + int(rng.integers(0, 2 ** 62)) * 2 ** max(e - 62, 0) % 2 ** e + int(rng.integers(0, 2 ** 40)) % 2 ** min(e, 40)
+        xs += [s * v for s in (1, -1) for v in (2 ** e, 2 ** e - 1, tie, tie - 1, tie + 1, x)]
+    xs = [x for x in xs if -(M // 2) <= x < M // 2]
+    m = 1023 if ldr else len(xs)
+    xs = (xs * 2)[:m]
+    sB = np.array([0, 57, -900, 900], dtype=np.int32)
+    row = np.array([[x % int(mm) for x in xs] for mm in ms], dtype=np.uint16)
+    R = np.ascontiguousarray(np.broadcast_to(row[:, None, :], (len(ms), 4, m)))
+    R[:, 1] = R[:, 1, rng.permutation(m)]                                             # small ones next to large ones
+    sA = np.zeros(m, dtype=np.int32)
+    C0 = np.asfortranarray(rng.standard_normal((m, 4)))
+    for alpha, beta in ((1.0, 0.0), (-1.0, 1.0)):
+        got, _ = gh.reconstruct(R, sA, sB, set_name, alpha, beta, C0, ldr=ldr)
+        assert (got == ozo.output(ozo.crt(R, OSET[set_name]), sA, sB, alpha, beta, C0)).all()
+
+
+@pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("E", "int8"), ("A", "int8n")])
+@pytest.mark.parametrize("m,n", [(200, 300), (1001, 900)])
+@pytest.mark.parametrize("fall", [2.0, 5.0, 20.0])
+def test_graded_operands(set_name, sub, m, n, fall):
+    """Whole calls on operands that fall off from the diagonal: results of every size below the bound of their row and column, two rows a
+    thread and four."""
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m + int(fall))
+    k = 150
+    away = lambda p, q: np.exp(-np.abs(np.arange(p)[:, None] * (q / p) - np.arange(q)[None, :]) / fall)     # noqa: E731
+    A, B = np.asfortranarray(rng.standard_normal((m, k)) * away(m, k)), np.asfortranarray(rng.standard_normal((k, n)) * away(k, n))
+    C0 = np.asfortranarray(rng.standard_normal((m, n)) * 1e-9)
+    for alpha, beta in ((1.0, 0.0), (-1.0, 1.0)):
+        got, st = gh.dgemm(A, B, set_name, gh.route(sub), alpha, beta, C0)
+        assert st == 0 and (got == ozo.dgemm(A, B, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS, alpha=alpha, beta=beta, C0=C0)).all()
