@@ -115,14 +115,16 @@ def test_three_pass_deconstruction_of_columns(lines, k, set_name, sub):
 
 
 @pytest.mark.parametrize("set_name,sub", [("S", "fp8"), ("E", "int8"), ("A", "int8n")])
-@pytest.mark.parametrize("m,n,k", [(1003, 301, 5003), (33, 2049, 8193), (2600, 9, 4097)])
+@pytest.mark.parametrize("m,n,k", [(1003, 301, 5003), (33, 2049, 8193), (2600, 9, 4097),
+                                   (450, 640, 9601)])            # both operands in three passes, in one launch each
 def test_scan_by_guessed_exponents(set_name, sub, m, n, k):
     """The scan of large operands guesses a line's largest exponent from a sample: lines whose largest element hides between the samples,
-    by no, one, two, three and many powers of two, lines of zeros, of subnormals, with samples of zeros only, with Inf and NaN."""
+    by no, one, two, three and many powers of two, lines of zeros, of subnormals, with samples of zeros only, with Inf and NaN, and lines whose
+    samples spread so far that there is no guess."""
     import tests.gpu_helpers as gh
     rng = np.random.default_rng(m + n + k)
     A, B = np.asfortranarray(rng.standard_normal((m, k))), np.asfortranarray(rng.standard_normal((k, n)))
-    hidden = k // 32 + 1                              # no sample: samples lie at the multiples of k / 32
+    hidden = k // 32 + 5                              # no sample: samples lie at the multiples of k / 32, or four behind each of k / 8
     for lines, axis in ((A, 0), (B, 1)):
         count = lines.shape[axis]
         rows = lines if axis == 0 else lines.T
@@ -134,9 +136,14 @@ def test_scan_by_guessed_exponents(set_name, sub, m, n, k):
             rows[11, hidden + 1:], rows[11, :hidden] = 0.0, 0.0
             rows[12] *= 2.0 ** -1000
             rows[13] *= 2.0 ** 900
-            rows[14, ::k // 32] = 0.0
+            for sample in [i * k // 32 for i in range(32)] + [i * k // 8 + u for i in range(8) for u in range(4)]:
+                rows[14, sample] = 0.0
             rows[15, hidden] = 5e-324
             rows[16, 0] = 2.0 ** 300
+            rows[17] *= np.exp(3.0 * rng.standard_normal(k))
+            rows[18] *= np.exp(1.2 * rng.standard_normal(k))
+        if count > 200:
+            rows[96:128] *= np.exp(2.0 * rng.standard_normal((32, k)))
     if m > 100:
         A[20, 5], A[21, hidden] = np.nan, np.inf
     rt = gh.route(sub)

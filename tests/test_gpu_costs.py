@@ -1,5 +1,5 @@
 """What a call must not pay for: device times of the same work on other data or another leading dimension, as ratios.  The bounds
-leave about half as much again as the ratios that the kernels show; the forms that they guard against lie above them."""
+leave room above the ratios that the kernels show; the forms that they guard against lie above them."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -102,3 +102,18 @@ def test_odd_leading_dimension_of_the_residues(set_name, sub, beta):
         R = _residues(set_name, n, ldr, None, 2)
         calls.append(lambda R=R, ldr=ldr: oz.check(oz.oz_reconstruct(m, n, R, ldr, n * ldr, sA, sB, gh.SETS[set_name], -1.0, beta, C, m)))
     assert _ratio(*calls) < 1.8
+
+
+def test_wide_columns_of_a_small_operand():
+    """Columns whose exponents spread, below the size from which a guess of their largest exponent pays."""
+    import torch
+
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    n, k, rt, S = 2647, 1700, gh.route("int8n"), gh.SETS["A"]
+    block = torch.empty(oz.oz_operand_bytes(1, n, k, S, rt), dtype=torch.uint8, device="cuda")
+    calls = []
+    for sigma in (2.0, 0.0):
+        X = _normal(k, n, 1) * torch.exp(sigma * _normal(k, n, 2))
+        calls.append(lambda X=X: oz.check(oz.oz_prepare_operand(1, n, k, X, k, S, rt, block)))
+    assert _ratio(*calls) < 1.05
