@@ -321,9 +321,16 @@ __device__ __forceinline__ void scan_block(const ScanSide &p, int64_t k, uint32_
         if (top >= 0x00100000u) {
             emax = static_cast<int>(top >> 20) - 1023;
         } else if (live) {
-            for (int64_t kk = kstart; kk < k1; kk += kstep) {
-                int e;
-                if (classify(*element(X, ldx, SIDE, line, kk), &e) == 1 && e > emax) emax = e;
+            // (zeros in every tenth row of A, 131072 x 4096: one load at a time 6579 us a deconstruction, by eight 5355)
+            for (int64_t kb = kstart; kb < k1; kb += 8 * kstep) {
+                double xs[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) xs[u] = kb + u * kstep < k1 ? *element(X, ldx, SIDE, line, kb + u * kstep) : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    int e;
+                    if (classify(xs[u], &e) == 1 && e > emax) emax = e;
+                }
             }
             if (SIDE == 1) emax = __reduce_max_sync(0xFFFFFFFFu, emax);
         }

@@ -117,3 +117,16 @@ def test_wide_columns_of_a_small_operand():
         X = _normal(k, n, 1) * torch.exp(sigma * _normal(k, n, 2))
         calls.append(lambda X=X: oz.check(oz.oz_prepare_operand(1, n, k, X, k, S, rt, block)))
     assert _ratio(*calls) < 1.05
+
+
+def test_rows_of_zeros():
+    """Rows of A without a normal number are read again for subnormals."""
+    import torch
+
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    m, k, rt, S = 6000, 12000, gh.route("int8n"), gh.SETS["A"]
+    block = torch.empty(oz.oz_operand_bytes(0, m, k, S, rt), dtype=torch.uint8, device="cuda")
+    X, Z = _normal(m, k, 1), _normal(m, k, 1)
+    Z[:, ::10] = 0.0
+    assert _ratio(*(lambda Y=Y: oz.check(oz.oz_prepare_operand(0, m, k, Y, m, S, rt, block)) for Y in (Z, X))) < 1.28
