@@ -1096,7 +1096,8 @@ __device__ __forceinline__ void deconstruct_lines(const FusedParams &p, int bloc
                 if (fast_scale) {
                     for (int kk = k0 + lane; kk < k1; kk += 32) {
                         const double x = src[padded(kk)];
-                        const unsigned int abar = magnitude(x, scale9);
+                        unsigned int abar = __double2uint_ru(fabs(x) * scale9);     // (magnitude(): 128^3 from cold caches 11.2 us, like this 10.4)
+                        if (abar == 0u && x != 0.0) abar = 1u;
                         acc += abar * abar;                              // at most 2^20
                         l1 += abar;
                     }
