@@ -36,19 +36,15 @@ __host__ __device__ constexpr int residue_bytes(int set) { return set == 2 ? 1 :
 // How the private residue array of the whole-method calls stores a residue of modulus i: some representative in [0, m + 1], modulo 2^10
 // or 2^8 where m is that, in one byte, in ten bits (moduli up to 1024) or in two bytes.  (Set A: canonical.)
 enum { kStoredByte, kStoredTen, kStoredPair };
-__host__ __device__ constexpr int stored_form(int set, int i)
-{
-    return modulus(set, i) <= 256 ? kStoredByte : modulus(set, i) <= 1024 ? kStoredTen : kStoredPair;
-}
-// bytes of one modulus' residues of a 32 x 64 patch of the output (see ResidueTiling), of those before it, and of a whole patch
-__host__ __device__ constexpr int stored_bytes(int set, int i)
-{
-    return stored_form(set, i) == kStoredByte ? 2048 : stored_form(set, i) == kStoredTen ? 2560 : 4096;
-}
+__host__ __device__ constexpr int form_of(int m) { return m <= 256 ? kStoredByte : m <= 1024 ? kStoredTen : kStoredPair; }
+__host__ __device__ constexpr int form_bytes(int form) { return form == kStoredByte ? 2048 : form == kStoredTen ? 2560 : 4096; }
+__host__ __device__ constexpr int stored_form(int set, int i) { return form_of(modulus(set, i)); }
+// where a modulus' residues of a 32 x 64 patch of the output (see ResidueTiling) begin, form_bytes() each, and bytes of a whole patch.  (Sums over the moduli
+// before it, for constants: the host takes them along, fill_mod_info().)
 __host__ __device__ constexpr int stored_start(int set, int i)
 {
     int o = 0;
-    for (int j = 0; j < i; ++j) o += stored_bytes(set, j);
+    for (int j = 0; j < i; ++j) o += form_bytes(stored_form(set, j));
     return o;
 }
 __host__ __device__ constexpr int patch_bytes(int set) { return stored_start(set, set_r(set)); }
