@@ -17,14 +17,19 @@
 // even, through the 64 leading bits and a sticky bit).  No FP64 arithmetic except the update of C.
 //
 // The residues come in the tile-ordered private layout of the whole-method calls (ResidueTiling): a
-// thread block of 128 threads takes ROWS = 2 (sets S and E) or 4 rows of 128 neighbouring pieces of columns of a 32 x 64 patch,
-// ROWS outputs per thread, ROWS small products per step.
+// thread block of 128 threads takes a chunk of sixteen rows of a 32 x 64 patch, four outputs a thread and four small products per step.  (Two
+// outputs a thread on sets S and E, whose ten-bit residues then take a load of high bits for every two: 10000 x 8000 x 128 2245 us a call on S and 2532 on
+// E, with four 1615 and 1618.)
 //
 // Every wait is bounded; on expiry the block records OZ_ERR_TIMEOUT, frees its TMEM and returns.
+#include <utility>
+
 #include "oz_internal.h"
 
 namespace oz {
 namespace {
+
+constexpr int kPieces = 4;             // chunks of sixteen rows: steps of a patch
 
 struct HostedConst {
     unsigned char B[16][32];   // B[s][K]
@@ -201,22 +206,29 @@ __device__ __forceinline__ double finish_from_sums(const uint32_t (&P)[16], int 
     return neg ? -d : d;
 }
 
-// The residues of modulus i in two rows (sets S and E; row even) or four of a column of the patch (see ResidueTiling) as the numbers that are
-// stored: two 16-bit halves, or four bytes
-template <int SET>
-__device__ __forceinline__ uint32_t stored_rows(const unsigned char *patch, int i, uint32_t column, uint32_t row)
+// The residues of modulus i in a thread's four rows (word `word` of chunk c of a column of the patch, see ResidueTiling): low bytes and, of sets S
+// and E, the bytes above them
+template <int SET, int I>
+__device__ __forceinline__ void stored_rows(const unsigned char *patch, uint32_t column, uint32_t c, uint32_t word, uint32_t &low, uint32_t &high)
 {
-    const unsigned char *src = patch + stored_start(SET, i);
-    const int form = stored_form(SET, i);
-    const uint32_t word = (row & 7u) >> 1, half = (row >> 2) & 2u;                // word of the chunk; its lower or upper two bytes
-    const unsigned char *low = src + ((row >> 4) * 32 + column) * 16 + word * 4;
-    if (residue_bytes(SET) == 1) return *reinterpret_cast<const uint32_t *>(low);
-    if (form == kStoredPair) return *reinterpret_cast<const uint32_t *>(src + ((row >> 3) * 32 + column) * 16 + (row & 7u) * 2);
-    const uint32_t two = *reinterpret_cast<const uint16_t *>(low + half);
-    uint32_t high = 0u;
-    if (form == kStoredTen)
-        high = (*reinterpret_cast<const uint32_t *>(src + 2048 + column * 16 + (row >> 4) * 4) >> (2 * word + 8 * half)) & 0x0303u;
-    return __byte_perm(two, high, 0x5140);
+    constexpr int form = stored_form(SET, I);
+    const unsigned char *src = patch + stored_start(SET, I);
+    high = 0u;
+    if constexpr (form == kStoredPair) {
+        const uint32_t first = *reinterpret_cast<const uint32_t *>(src + (2 * c * 32 + column) * 16 + word * 4);
+        const uint32_t second = *reinterpret_cast<const uint32_t *>(src + ((2 * c + 1) * 32 + column) * 16 + word * 4);
+        low = __byte_perm(first, second, 0x6420);
+        high = __byte_perm(first, second, 0x7531);
+    } else {
+        low = *reinterpret_cast<const uint32_t *>(src + (c * 32 + column) * 16 + word * 4);
+        if constexpr (form == kStoredTen) high = (*reinterpret_cast<const uint32_t *>(src + 2048 + column * 16 + c * 4) >> (2 * word)) & 0x03030303u;
+    }
+}
+template <int SET, int... I>
+__device__ __forceinline__ void stored_numbers(std::integer_sequence<int, I...>, const unsigned char *patch, uint32_t column, uint32_t c, uint32_t word,
+                                               uint32_t (&low)[16], uint32_t (&high)[16])
+{
+    (stored_rows<SET, I>(patch, column, c, word, low[I], high[I]), ...);
 }
 
 template <int SET>
@@ -227,10 +239,8 @@ reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int 
                           double alpha, double beta, double *__restrict__ C, int64_t ldc, int vecC,
                           unsigned int *status)
 {
-    constexpr int RB = residue_bytes(SET), ROWS = 4 / RB, r = set_r(SET);
-    constexpr int kBlockWords = 64 * 32 * RB / 4;          // words of one 32 x 64 patch per modulus
-    constexpr int kPieces = kBlockWords / 128;             // 128-word pieces of a patch: 8 or 4
-    constexpr uint32_t kTmemCols = ROWS * 16 < 32 ? 32 : ROWS * 16;
+    constexpr int RB = residue_bytes(SET), ROWS = 4, r = set_r(SET);
+    constexpr uint32_t kTmemCols = ROWS * 16;
     __shared__ __align__(128) unsigned char tileA[ROWS][128 * 32];
     __shared__ __align__(128) unsigned char tileB[16 * 32];
     __shared__ __align__(8) unsigned long long bar_storage;
@@ -268,19 +278,16 @@ reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int 
         const uint32_t wi = u & 15u, rank = u >> 4;
         const uint32_t tn = static_cast<uint32_t>(tn0) + static_cast<uint32_t>(tile % ntn);
         const uint32_t tm = static_cast<uint32_t>(tile / ntn);
-        const uint32_t w_idx = piece * 128u + t;
-        const uint32_t lane = (w_idx >> 2) & 31u, sub = w_idx & 3u;
-        // the thread's rows: row, row + 1 and, of set A, row + 8, row + 9
-        const uint32_t row0 = piece * (16 / RB) + sub * 2;
-        const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + row0;
+        const uint32_t lane = t >> 2, sub = t & 3u;
+        // the thread's rows: row, row + 1, row + 8 and row + 9
+        const int64_t row = static_cast<int64_t>(tm) * 256 + (wi >> 2) * 64 + piece * 16 + sub * 2;
         auto row_of = [](int h) { return (h & 1) + 8 * (h >> 1); };
         const int64_t j = (static_cast<int64_t>(tn) * cg + rank) * 128 + (wi & 3u) * 32 + lane;
         const bool valid = row < m && j < n && j >= col0 && j < col1;
         const int64_t wb = ((static_cast<int64_t>(tm) * tiles_n + tn) * cg + rank) * 16 + wi;
         const unsigned char *patch = static_cast<const unsigned char *>(Rv) + wb * patch_bytes(SET);
-        uint32_t w[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) w[i] = (i < r && valid) ? stored_rows<SET>(patch, i, lane, row0) : 0u;
+        uint32_t w[16] = {}, above[16] = {};
+        if (valid) stored_numbers<SET>(std::make_integer_sequence<int, r>{}, patch, lane, piece, sub, w, above);
         // old values of C and the shifts travel while the tensor core works
         const int64_t left = valid ? m - row : 0;
         const bool whole = vecC != 0 && left > row_of(ROWS - 1);
@@ -301,13 +308,15 @@ reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int 
 #pragma unroll
         for (int h = 0; h < ROWS; ++h) {
             uint32_t kw[8];
+            // byte h of every modulus' words
+            const uint32_t sel = static_cast<uint32_t>(((4 + h) << 4) | h);
             if constexpr (RB == 2) {
                 // K = 2 i + a: the two bytes of modulus i; word q holds moduli 2q, 2q+1
 #pragma unroll
-                for (int q = 0; q < 8; ++q) kw[q] = __byte_perm(w[2 * q], w[2 * q + 1], h ? 0x7632 : 0x5410);
+                for (int q = 0; q < 8; ++q)
+                    kw[q] = __byte_perm(__byte_perm(w[2 * q], above[2 * q], sel), __byte_perm(w[2 * q + 1], above[2 * q + 1], sel), 0x5410);
             } else {
-                // K = i: byte h of every modulus' word; word q holds moduli 4q .. 4q+3
-                const uint32_t sel = static_cast<uint32_t>(((4 + h) << 4) | h);
+                // K = i; word q holds moduli 4q .. 4q+3
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     kw[q] = __byte_perm(__byte_perm(w[4 * q], w[4 * q + 1], sel), __byte_perm(w[4 * q + 2], w[4 * q + 3], sel), 0x5410);
@@ -438,11 +447,9 @@ oz_status_t launch_reconstruct_hosted(int64_t m, int64_t n, const void *R, const
     int dev = 0, sms = 148;
     OZ_CUDA_CHECK(cudaGetDevice(&dev));
     OZ_CUDA_CHECK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int pieces = 64 * 32 * residue_bytes(set) / 4 / 128;
-    const int64_t total = static_cast<int64_t>(t.tiles_m) * ntn * t.cg * 16 * pieces;
-    // persistent blocks: TMEM (512 columns per SM) admits 16 blocks of 32 columns, 8 of 64
-    const int per_sm = residue_bytes(set) == 2 ? 12 : 8;
-    const int64_t cap = static_cast<int64_t>(sms) * per_sm;
+    const int64_t total = static_cast<int64_t>(t.tiles_m) * ntn * t.cg * 16 * kPieces;
+    // persistent blocks: TMEM (512 columns per SM) admits 8 of 64 columns
+    const int64_t cap = static_cast<int64_t>(sms) * 8;
     const unsigned grid = static_cast<unsigned>(total < cap ? total : cap);
     unsigned int *status = device_status_word();
 #define OZ_RECON_HOSTED(SET_)                                                                               \
