@@ -927,6 +927,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                         }
                     } else {
                         // INT32 accumulators: exact integer arithmetic, no conversions
+                        // (added modulo 2^32: a combination that starts at its bias, above 2^31, is no int)
                         const int iwj = mi.iw[job];
                         if (reduce_first) {
 #pragma unroll
@@ -934,13 +935,13 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                                 uint32_t u = v[e] + ibias;                       // non-negative, same residue
                                 uint32_t r = u - __umulhi(u, imagic) * im;       // in [0, 2m)
                                 r = min(r, r - im);
-                                comb[c0 + e] = static_cast<uint32_t>(static_cast<int>(r) * iwj + static_cast<int>(comb[c0 + e]));
+                                comb[c0 + e] += static_cast<uint32_t>(static_cast<int>(r) * iwj);
                             }
                         } else {
                             // the host has checked that the weighted sum stays inside INT32 for this k
 #pragma unroll
                             for (int e = 0; e < DRAIN_W; ++e)
-                                comb[c0 + e] = static_cast<uint32_t>(static_cast<int>(v[e]) * iwj + static_cast<int>(comb[c0 + e]));
+                                comb[c0 + e] += static_cast<uint32_t>(static_cast<int>(v[e]) * iwj);
                         }
                     }
                 }
