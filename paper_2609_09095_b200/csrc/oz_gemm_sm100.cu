@@ -25,7 +25,7 @@
 // contiguous in the column-major residue array; a warp transposes its 32 x 64 block through a
 // small swizzled shared-memory buffer so that each store instruction writes whole lines.
 //
-// Kernel structure (one persistent CTA per SM, 576 threads, up to 112 registers each; launched as
+// Kernel structure (one persistent CTA per SM, 576 threads, up to 96 registers each; launched as
 // clusters of two CTAs that share one tcgen05.mma.cta_group::2 unless n pads badly to 256):
 //   warp 0       TMA producer: 128-byte-swizzled K-major tiles of B (128 lines) and A (256 lines,
 //                or this CTA's half of them in a pair) into a shared-memory ring of 192 KiB
@@ -94,7 +94,7 @@ struct SlimTile {
     static constexpr int STAGES = RING_BYTES / STAGE_BYTES;                  // 3 or 4, narrow tiles 4 or 8
 };
 constexpr int TMEM_COLS = 512;                     // two accumulator slots of BLOCK_N columns
-constexpr int NUM_THREADS = 576;                   // 18 warps: 112 registers each fit the register file
+constexpr int NUM_THREADS = 576;                   // 18 warps, five on one of the schedulers: 96 registers each
 constexpr int FIRST_EPI_WARP = 2;                  // warp 0: producer, warp 1: MMA issuer
 constexpr int EPI_WARPS = 16;
 #ifndef OZ_DRAIN_W
@@ -581,7 +581,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + 16 * STAGES + 40);
 
     // Broadcast, the warp number and the TMEM base are the same in a warp by construction and need no register of a thread:
-    // the epilogue's 64 running values then fit its 96 registers without spills in all but two of the variants.
+    // the epilogue's 64 running values then fit its 96 registers without spills in all but one of the variants.
     const int warp = __shfl_sync(0xFFFFFFFFu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
     dependency_release();
@@ -1010,12 +1010,8 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     float t = __uint_as_float(cv);
                     float quot = fmaf(t, inv_m, 12582912.0f) - 12582912.0f;
                     float res = fmaf(-quot, mm, t);                      // |res| <= ~m/2
-                    if constexpr (PACKED) {
-                        return __float_as_uint(res + centre_big);        // in the low mantissa bits
-                    } else {
-                        res = res < 0.0f ? res + mm : res;               // canonical [0, m)
-                        return __float_as_uint(res + 8388608.0f);        // integer in the low mantissa bits
-                    }
+                    res = res < 0.0f ? res + mm : res;                   // canonical [0, m) (PACKED: final_bits2)
+                    return __float_as_uint(res + 8388608.0f);            // integer in the low mantissa bits
                 } else if constexpr (DIRECT) {
                     uint32_t u = cv + mi.bias30;                          // in (0, 2^31 + 256)
                     return u - (__umulhi(u, mi.magic39) >> 7) * im;      // exact quotient: canonical [0, m)

@@ -305,7 +305,7 @@ oz_status_t launch_reconstruct(int64_t m, int64_t n, const void *R, int64_t ldr,
                                int set, double alpha, double beta, double *C, int64_t ldc,
                                cudaStream_t stream);
 
-// uploads the reconstruction constants of every set to the current device
+// uploads the constants of the reconstruction on the tensor pipe, of every set, to the current device
 oz_status_t upload_hosted_constants();
 
 // reconstruction from the tile-ordered array with the CRT recombination on the INT8 tensor pipe
