@@ -39,13 +39,16 @@ sys.path.insert(0, ROOT)
 
 import synth_inputs as syn  # noqa: E402
 
-# Residues of an output as the whole-method calls store them: 8, 10 or 16 bits each by their modulus (set A: 8).
-STORED_BYTES = {"S": 15.75, "E": 15.25, "A": 15.0}
-
 # DRAM traffic of the residue GEMM relative to its algorithmic bytes (reads / plane bytes, writes /
 # residue bytes) comes from the table in profiles/residue_gemm_dram_traffic.md: ncu captures of a
 # smaller launch, one row per kernel variant, scaled here to the full-size launch by the units.
 TRAFFIC_TABLE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "profiles", "residue_gemm_dram_traffic.md")
+
+
+def residue_bytes_per_output(moduli, elem_bytes, fused):
+    """Bytes of all residues of an output between the residue GEMM and the reconstruction: in the public layout (storage mode F) one element
+    a modulus, in the whole-method calls' own 8, 10 or 16 bits each by the modulus."""
+    return float(elem_bytes * len(moduli)) if fused else sum(8 if m <= 256 else 10 if m <= 1024 else 16 for m in moduli) / 8
 
 
 def gemm_dram_amplification(set_name: str, substrate: str):
@@ -460,7 +463,7 @@ def main():
         roof_nominal = 4500.0 / (passes + 1)               # P_low/(3r+1), or P_low/(r+1) native INT8, at B200's dense 8-bit rate
         hbm = peaks["hbm_gbs"]
         dec_bytes = 8 * (m * k + k * n) + (p_store_a * m + p_store * n) * k    # operands read once, planes written, whatever form is taken
-        rb = STORED_BYTES[args.set_name]                      # bytes of all residues of an output
+        rb = residue_bytes_per_output(oz.oz_set_info(modset)[2], oz.oz_residue_elem_bytes(modset), args.fused)
         rec_bytes = (rb + 8 + (8 if cfg.beta else 0)) * m * n
         plane_bytes = float((p_store_a * m + p_store * n) * k)
         residue_bytes = float(rb) * m * n

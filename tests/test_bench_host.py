@@ -72,6 +72,15 @@ def test_traffic_table_lookup():
     assert bench.gemm_dram_amplification("no such set", "fp8") is None
 
 
+def test_residue_bytes_of_an_output():
+    import paper_2609_09095_b200 as oz
+    packed, public = {"S": 15.75, "E": 15.25, "A": 15.0}, {"S": 24.0, "E": 26.0, "A": 15.0}
+    for name, modset in (("S", oz.OZ_SET_S), ("E", oz.OZ_SET_E), ("A", oz.OZ_SET_A)):
+        moduli, elem = oz.oz_set_info(modset)[2], oz.oz_residue_elem_bytes(modset)
+        assert bench.residue_bytes_per_output(moduli, elem, False) == packed[name]
+        assert bench.residue_bytes_per_output(moduli, elem, True) == public[name]
+
+
 def test_clock_sample_parser():
     s = bench.ClockSampler(0)
     s.proc = type("P", (), {"terminate": lambda self: None, "wait": lambda self, timeout=None: 0})()
