@@ -199,13 +199,14 @@ __device__ __noinline__ void native_small(const NativeParams &p, int64_t rows, i
 }
 
 // Small tiles while they cost less: a tile of 8 x 16 takes an SM 27.5 cycles an inner index next to others, a round of 32 x 32 tiles over the resident
-// blocks 380, whether one or both blocks of an SM have a tile.  85 of 3000 rows x 3000 x 3000: 1648 us a call with the small ones, 1588 with the large, whose
-// one round is nearly full; 594 of 600 x 3000 x 300: 474 and 500; 60 of 2003 x 1999 x 1501: 461 and 580; 8000 x 8000 x 1500, every row: 68.1 and 63.8 ms.
+// blocks 365, whether one or both blocks of an SM have a tile (a last round of a few tiles somewhat less).  Calls with the small and the large ones, us, by
+// rounds: 600 rows x 3000 x 300, 96 and 7: 473, 435; 150 x 5000 x 400, 41 and 3: 354, 339; 400 x 3000 x 600, 64 and 5: 595, 578; 450 x 3200 x 500, 78 and 6: 651, 676;
+// 225 x 2000 x 1000, 25 and 2: 423, 448; 300 x 3000 x 1500, 49 and 4: 1182, 1315; 1200 x 1600 x 400, 102 and 7: 647, 607.
 __device__ __forceinline__ bool small_tiles(int64_t rows, int64_t n, int64_t sms)
 {
     const int64_t large = ((rows + kLarge - 1) / kLarge) * ((n + kLarge - 1) / kLarge), slots = kFbBlocksPerSm * sms;
     const int64_t small = ((rows + kSmallRows - 1) / kSmallRows) * ((n + kSmallCols - 1) / kSmallCols);
-    return 55 * ((small + sms - 1) / sms) < 760 * ((large + slots - 1) / slots);
+    return 3 * ((small + sms - 1) / sms) < 40 * ((large + slots - 1) / slots);
 }
 
 __global__ void __launch_bounds__(kFbThreads, kFbBlocksPerSm)
