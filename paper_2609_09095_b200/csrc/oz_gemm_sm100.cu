@@ -119,7 +119,6 @@ struct ModInfo {
     int nseg, seg_len;
     int nseg_all, seg_len_all;
     // integer epilogue of the INT8 routes (INT32 accumulators):
-    int iw[3];            // weights as integers
     uint32_t mi;          // the modulus
     uint32_t magic;       // floor(2^32 / m)
     uint32_t bias;        // a multiple of m just above 2^31: makes a signed combination non-negative
@@ -130,8 +129,9 @@ struct ModInfo {
     int store_form;       // kStoredByte, kStoredTen or kStoredPair
     int store_start;      // the byte of a patch where this modulus' residues begin
     float centre;         // (m + 1) / 2 (FP32 epilogue)
-    int reserved;         // whole 16-byte pieces: a size of 108 cost the public native variant spills
 };
+// The parameters travel with every launch, and calls of up to about 128^3 follow one another as fast as launches do: 64^3 13.8 us a call with 112 bytes, 13.4 with 96.
+static_assert(sizeof(ModInfo) <= 96, "parameters of a launch");
 
 struct GemmParams {
     int64_t m, n, k;
@@ -928,7 +928,7 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     } else {
                         // INT32 accumulators: exact integer arithmetic, no conversions
                         // (added modulo 2^32: a combination that starts at its bias, above 2^31, is no int)
-                        const int iwj = mi.iw[job];
+                        const int iwj = __float2int_rn(wj);
                         if (reduce_first) {
 #pragma unroll
                             for (int e = 0; e < DRAIN_W; ++e) {
@@ -1118,9 +1118,9 @@ residue_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
                     pack_rows(c, c + 2, packed[c >> 2], unused);
                 }
             }
-            // all are packed before the first is stored: the unpacked ones in between cost 72 bytes of spills.  (Native residues in single CTAs have none that way
-            // and 56 bytes packed first: 300^3 12.1 us against 10.8, 200 x 300 x 1000 11.9 against 10.1.)
-            if constexpr (!(DIRECT && CG == 1)) {
+            // all are packed before the first is stored: the unpacked ones in between cost 72 bytes of spills.  (Native residues have none that way and up to 56 bytes
+            // packed first: in single CTAs 300^3 12.1 us against 10.8, 200 x 300 x 1000 11.9 against 10.1.)
+            if constexpr (!DIRECT) {
 #pragma unroll
                 for (int c = 0; c < COLS_PER_WARP * RB / 4; ++c) asm volatile("" : "+r"(packed[c]));
             }
@@ -1461,7 +1461,6 @@ static void fill_mod_info(GemmParams &p, int set, const Route &rt, int64_t k, bo
             mo.reduce[1] = skip01 ? 0 : 1;
             mo.reduce[2] = skip_all ? 0 : 1;
         }
-        for (int j = 0; j < 3; ++j) mo.iw[j] = static_cast<int>(mo.w[j]);
     }
 }
 
@@ -1631,7 +1630,6 @@ oz_status_t launch_bound_gemm(int64_t m, int64_t n, int64_t k, const uint8_t *GA
     mo.njobs = 1;
     mo.kind = 2;                       // one plane, one K-loop
     mo.w[0] = 1.0f;
-    mo.iw[0] = 1;
     mo.reduce[0] = 0;
     mo.planeA0 = mo.planeB0 = 0;
     mo.nseg = mo.nseg_all = 1;
