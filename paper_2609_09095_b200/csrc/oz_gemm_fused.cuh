@@ -247,8 +247,8 @@ fused_gemm_kernel(const __grid_constant__ CUtensorMap mapB, const __grid_constan
                         for (int c = 0; c < 32; ++c) comb[c] = 0u;
 #pragma unroll
                         for (int job = 0; job < 2; ++job) {
-                            const float wj = mi.w[job];
-                            const int iwj = __float2int_rn(wj);
+                            const float wj = __uint_as_float(mi.w[job]);
+                            const int iwj = static_cast<int>(mi.w[job]);
                             const bool reduce_first = mi.reduce[job] != 0;
                             const uint32_t taddr = tmem_base + (static_cast<uint32_t>(q * 32) << 16) +
                                                    static_cast<uint32_t>(s * 2 * F_LINES + job * F_LINES + half * 32);
