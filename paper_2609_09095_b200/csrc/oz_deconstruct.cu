@@ -2,9 +2,12 @@
 // 8-bit residue planes.
 //
 // Kernels of the three-pass form, in launch order (the scans serve both operands of a product at once where both take it):
-//   scan_init      clears the per-line scratch (largest exponent, non-finite flag, sum of squares)
-//   scan pass 0    largest floor(log2|x|) of every line, Inf/NaN detection
-//   scan pass 1    CS rule only: exact integer sum of ceil(|x| 2^(9-E))^2 per line
+//   scan_sample    clears the per-line scratch (largest exponent, non-finite flag, sums) and guesses every line's largest exponent from 32 samples
+//   scan pass 2    largest floor(log2|x|) of every line, Inf/NaN detection, and for the guess and the next two exponents the exact integer sum of
+//                  ceil(|x| 2^(9-E))^2
+//   scan pass 1    the sums of the lines whose exponent was not among those
+// (scan_init, pass 0 without sums and pass 1 of all lines where there is no room for the guesses' sums, too few elements for them to pay, or no need of
+// sums: rule MAXEXP and the accurate one, which end with pass 0)
 //   scan_finalize  shift[line] (sigma_i or tau_j of Eq. 1)
 //   convert        quantise, reduce modulo every modulus, split into digits, store the planes
 // Small operands take one kernel instead of the five, both operands of a product together where they fit; lines that fit a
