@@ -577,11 +577,11 @@ __device__ __noinline__ Results<ROWS> finish_rows_call(std::integer_sequence<int
     return finish_rows<SET, ROWS>(rows, from, v, sa, sb, alpha_sign, nrows, sure);
 }
 
-// scalar stores of up to two consecutive rows; `first` / `second`: which of them are written
+// scalar stores of up to two consecutive rows; `first` / `second`: which of them are written.  A zero without an old value is +0, as in the stores of pairs.
 __device__ __forceinline__ void store_pair(double *out, double p0, double p1, bool first, bool second, double beta)
 {
-    if (first) out[0] = beta != 0.0 ? out[0] + p0 : p0;
-    if (second) out[1] = beta != 0.0 ? out[1] + p1 : p1;
+    if (first) out[0] = (beta != 0.0 ? out[0] : 0.0) + p0;
+    if (second) out[1] = (beta != 0.0 ? out[1] : 0.0) + p1;
 }
 
 // ROWS rows of a column, row_of(0) .. from `row` on: reconstruct, update C with fast alpha 2^-(sa + sb) c'.

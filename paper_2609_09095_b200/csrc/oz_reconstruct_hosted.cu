@@ -374,7 +374,7 @@ reconstruct_hosted_kernel(const void *__restrict__ Rv, int cg, int tiles_n, int 
         } else {
 #pragma unroll
             for (int h = 0; h < ROWS; ++h)
-                if (row_of(h) < left) out[row_of(h)] = beta != 0.0 ? out[row_of(h)] + val[h] : val[h];
+                if (row_of(h) < left) out[row_of(h)] = (beta != 0.0 ? out[row_of(h)] : 0.0) + val[h];      // a zero is +0, as above
         }
         // the next step's products overwrite the accumulators: every thread has read its rows
     }

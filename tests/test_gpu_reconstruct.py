@@ -142,3 +142,24 @@ def test_graded_operands(set_name, sub, m, n, fall):
     for alpha, beta in ((1.0, 0.0), (-1.0, 1.0)):
         got, st = gh.dgemm(A, B, set_name, gh.route(sub), alpha, beta, C0)
         assert st == 0 and (got == ozo.dgemm(A, B, OSET[set_name], ozo.QUANT_RN, ozo.SCALE_CS, alpha=alpha, beta=beta, C0=C0)).all()
+
+
+@pytest.mark.parametrize("set_name,sub,recon", [("S", "fp8", None), ("E", "int8", None), ("A", "int8n", None), ("S", "fp8", "tensor"), ("A", "int8n", "tensor")])
+@pytest.mark.parametrize("m,pad", [(64, 0), (75, 0), (75, 1), (1003, 0), (1002, 1)])
+def test_zeros_are_positive(set_name, sub, recon, m, pad):
+    """C = - A B without an old value: results that are zero, or too small and negative, are +0 in whatever group of rows and form of store they lie."""
+    import paper_2609_09095_b200 as oz
+    import tests.gpu_helpers as gh
+    rng = np.random.default_rng(m + pad)
+    n, k = 800, 40
+    A, B = np.asfortranarray(rng.standard_normal((m, k))), np.asfortranarray(rng.standard_normal((k, n)))
+    A[::3, : k // 2], B[k // 2:, ::2] = 0.0, 0.0
+    A[1::6] *= 2.0 ** -1000
+    B[:, 1::4] *= 2.0 ** -900
+    rt = gh.route(sub, recon=recon)
+    gh.ensure_workspace(oz.oz_workspace_bytes(m, n, k, gh.SETS[set_name], rt))
+    dC = gh.to_dev(np.asfortranarray(np.full((m + pad, n), 3.0)))
+    oz.check(oz.oz_dgemm_ex(m, n, k, -1.0, gh.to_dev(A), m, gh.to_dev(B), k, 0.0, dC, m + pad, gh.SETS[set_name], rt), "oz_dgemm_ex")
+    assert gh.sync_status() == 0
+    got = gh.from_dev(dC)[:m]
+    assert (got == 0.0).mean() > 0.2 and not np.signbit(got[got == 0.0]).any()
