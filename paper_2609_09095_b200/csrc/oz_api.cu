@@ -398,7 +398,7 @@ oz_status_t product_impl(int64_t m, int64_t n, int64_t k, double alpha, const Op
                                          rt, R, 0, 0, true, stream);
     if (st != OZ_OK) return st;
     if (ev) OZ_CUDA_CHECK(cudaEventRecord(g_stage_events[dev][3], stream));
-    // the CRT recombination: exact FP64 chunk sums on the FP64 pipe, or (OZ_RECON_TENSOR) one small
+    // the CRT recombination: sums over groups of moduli on the integer and FP64 pipes, or (OZ_RECON_TENSOR) one small
     // unsigned 8-bit product per 128 outputs on the tensor pipe and an integer tail
     auto reconstruct = [&](int64_t m_, int64_t n_, const void *R_, const int32_t *sa, const int32_t *sb, int set_,
                            double alpha_, double beta_, double *C_, int64_t ldc_, int64_t c0, int64_t c1,
